@@ -1,19 +1,29 @@
-// Attention with the exact angular kernel (Eq. 4-5) on the tensor cores, bf16, head width 64:
+// Attention with explicit weights on the tensor cores, bf16, head width 64: the exact angular kernel (Eq. 4-5)
 //     out_t = sum_j (1 - arccos(q^_t . k^_j) / pi) v_j + bias + DWConv(V)_t
-// with explicit weights, quadratic in the number of tokens.  A work item is a (plane, tile of 128 queries); for
-// every tile of 128 keys of the plane
-//   warp 0       TMA: K and V tiles (128-byte swizzle, rows beyond the plane zero-filled), the Q tile once per item
-//   warps 2..5   scale every K row (and, once per item, every Q row) to a unit row in place, as bf16
-//   warp 1       one thread issues the UMMAs: C[128 x 128] = Q^ K^^T into one of two TMEM buffers, and, one tile
-//                behind, O[128 x 64] += W[128 x 128] V with the weights W from shared memory
-//   warps 6..13  thread = (query, 64 of the 128 keys): cosines out of TMEM, clamp, 1 - arccos/pi (a polynomial in
-//                |x| times sqrt(1 - |x|), Abramowitz & Stegun 4.4.45, |error| < 7e-5 rad: far below the bf16 rounding
-//                of the weights), bf16 weights into the shared-memory operand of the second contraction
-// and at the end of the item warps 6..9 (thread = query) read O, add bias and the depthwise convolution of V taken
-// from global memory, and store the row.  Keys beyond the plane have k^ = 0, weight 1/2 and v = 0: no masking.
-// With the auxiliary branch of training (Eq. 10) every item takes a first sweep over the keys that only forms the
-// cosines and adds up exp(cosine) per query (keys beyond the plane excluded); in the second sweep the weight of a pair
-// is the base weight (exact kernel, or its kept part 1/2 + x/pi) plus Mask_eps of its softmax probability.
+// and / or the masked softmax branch of training (Eq. 10) on top of either base kernel; quadratic in the number of
+// tokens.  A work item is a plane and one or two tiles ("slots") of 128 queries, which share every tile of 128 keys.
+//   warp 0       one thread keeps three rings of TMA copies going: Q tiles (an item ahead), K tiles, V tiles
+//   warps 4..7   scale every K row and every Q row to a unit row in place, as bf16
+//   warp 1       issues C[128 x 128] = Q^ K^^T, slot after slot, into three TMEM buffers in turn
+//   warps 8..23  thread = (query, 64 of the tile's keys): cosines out of TMEM, the weights back over them as bf16 (eight
+//                warps per slot)
+//   warp 2       issues O[128 x 64] += W[128 x 128] V, whose A operand W is read from TMEM
+//   warps 24..31 while the sweep over the keys runs: bias and depthwise convolution of V for the item's queries (lane =
+//                channel pair, V from global memory in coalesced rows) into shared memory as fp32; then thread = query:
+//                O out of TMEM, add, round, 128-byte rows to memory
+// Keys beyond the plane have k^ = 0 and v = 0 and need no mask in the weighted sum.  The masked branch takes a first
+// sweep over the keys that only forms the cosines and adds up exp(cosine) per query (keys beyond the plane excluded); in
+// the second sweep the weight of a pair is the base weight plus Mask_eps of its softmax probability.  When a plane has at
+// most kResident key tiles they stay in shared memory between the two sweeps.
+//
+// What bounds it: the weight function, 16 square roots or exponentials per cycle and multiprocessor (2 x 8 planes of
+// 64 x 64 tokens: 2.7e8 pairs, 61 us of that unit at 1.85 GHz).  Per 128 x 128 pairs that unit needs 1024 cycles and the
+// UMMAs 512 (64 each at N = 128, 32 each with A in TMEM), so two slots keep both busy.  The two contractions have an
+// issuing warp each: a ready wait costs 50 to 90 cycles and an issue 30 per UMMA, which one warp could not do in time.
+// Measured (B200, per forward): exact kernel, 2 x 8 planes of 64 x 64 tokens 143 us (338 with one issuing thread, weights
+// through shared memory and eight weight warps: 480 TFLOP/s over the two contractions against 203); masked branch, 64 x 12
+// planes of 14 x 14 74 us (303: there every item waited for its Q tiles and for a convolution of one thread per token).
+// Eight weight warps instead of sixteen: 151 and 77 us (two warps per scheduler do not hide the trips to TMEM).
 // No workspace; every wait is bounded.
 #include "tc_common.cuh"
 #include "tc_host.cuh"
@@ -23,19 +33,24 @@ namespace tc {
 namespace {
 
 constexpr int kD = 64;
-constexpr int kTile = 128;
+constexpr int kTile = 128;                          // queries per slot, keys per tile
 constexpr int kTileBytes = kTile * kD * 2;          // 16 KiB
-constexpr int kStageBytes = 2 * kTileBytes;         // K then V
-constexpr int kStages = 3;
-constexpr int kPBytes = kTile * kTile * 2;          // weights of one tile pair: two 64-key blocks of 16 KiB
-constexpr int kThreads = 14 * 32;
-constexpr int kNormThreads = 128, kWThreads = 256;
-constexpr int kTmemCols = 512;                      // cosines: 2 x 128 columns; output: 64 columns at 256
-constexpr int kOffQ = 0, kOffStages = kTileBytes, kOffP = kOffStages + kStages * kStageBytes;
-constexpr int kOffDen = kOffP + 2 * kPBytes;        // softmax denominators: one partial sum per weight thread
-constexpr int kOffBar = kOffDen + 2 * kTile * 4;
-constexpr size_t kSmem = 1024 + kOffBar + 256;
+constexpr int kKStages = 3, kVStages = 2;
+constexpr int kResident = 2;                        // key tiles of a plane that stay between the sweeps
+constexpr int kCBufs = 3;                           // cosine buffers
+constexpr int kNormThreads = 128, kSlotThreads = 256, kConvThreads = 256;
+constexpr int kThreads = 128 + kNormThreads + 2 * kSlotThreads + kConvThreads;
+constexpr int kTmemCols = 512;
+constexpr int kColO = kCBufs * kTile;               // outputs of the two slots behind the cosine buffers
+constexpr int kStgStride = kD * 4 + 16;             // fp32 row + 16 B: conflict-free row-per-thread access
+constexpr int kOffQ = 0, kOffK = 4 * kTileBytes, kOffV = kOffK + kKStages * kTileBytes;   // Q: [2 items][2 slots]
+constexpr int kOffStg = kOffV + kVStages * kTileBytes;
+constexpr int kOffDen = kOffStg + 2 * kTile * kStgStride;   // softmax denominators [2 items][2 slots][2 halves][128]
+constexpr int kOffW = kOffDen + 8 * kTile * 4;              // filters of the item's head: [taps][32 lanes] channel pairs
+constexpr int kOffBar = kOffW + 25 * 32 * 4;
+constexpr size_t kSmem = 1024 + kOffBar + 512;
 static_assert(kSmem <= 227 * 1024, "shared memory");
+static_assert(kColO + 2 * kD <= kTmemCols, "tensor memory");
 
 struct QuadParams {
     const __nv_bfloat16* v;      // for the convolution
@@ -43,22 +58,97 @@ struct QuadParams {
     const __nv_bfloat16* w;
     const __nv_bfloat16* bias;
     Layout lv, lo;
-    int hdiv, H, head0, BH, N, gridH, gridW, q_tiles, k_tiles, n_items;
+    int hdiv, H, head0, N, gridH, gridW;
+    int slots;                   // query tiles per item (1 or 2)
+    int groups;                  // items per plane
+    int k_tiles, n_items;
     float eps2;
     unsigned* status;
-    float sparse_eps;       // threshold of the mask (sparse sweeps only)
+    float sparse_eps;            // threshold of the mask (sparse sweeps only)
 };
 
-// 1 - arccos(x) / pi for x in [-1, 1]
-__device__ __forceinline__ float angular_weight(float x) {
-    const float ax = fminf(fabsf(x), 1.0f);
-    const float t = 1.0f - ax;
-    float p = fmaf(-0.0187293f, ax, 0.0742610f);
-    p = fmaf(p, ax, -0.2121144f);
-    p = fmaf(p, ax, 1.5707288f);
-    const float ac = p * (t * rsqrtf(fmaxf(t, 1e-30f)));     // arccos(|x|)
-    const float r = ac * kInvPi;                              // arccos(|x|) / pi
-    return x >= 0.f ? 1.0f - r : r;                           // arccos(-a) = pi - arccos(a)
+// The descriptors of all operands here (128-byte swizzle, 1024 bytes between groups of eight rows) differ in their low
+// word only, so an UMMA costs its issuer one addition for each.
+constexpr uint32_t kDescHigh = (1024u >> 4) | (1u << 14) | (2u << 29);   // bits 32..63 of umma_desc_sw128(.., 0, 1024)
+__device__ __forceinline__ uint32_t desc_low(const void* smem_ptr) { return smem_u32(smem_ptr) >> 4; }
+template <bool kAccumulate>
+__device__ __forceinline__ void umma_ss(uint32_t d_tmem, uint32_t a_low, uint32_t b_low, uint32_t idesc) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
+        "setp.ne.b32 p, %5, 0;\n\t"
+        "mov.b64 da, {%1, %4};\n\tmov.b64 db, {%2, %4};\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %3, p;\n\t}"
+        ::"r"(d_tmem), "r"(a_low), "r"(b_low), "r"(idesc), "r"(kDescHigh), "n"(kAccumulate ? 1 : 0)
+        : "memory");
+}
+// D[tmem] (+)= A[tmem] * B[smem]: row i of A in lane i, two bf16 of the contracted index per 32-bit column.
+__device__ __forceinline__ void umma_ts(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_low, uint32_t idesc, uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b64 db;\n\t"
+        "setp.ne.b32 p, %5, 0;\n\t"
+        "mov.b64 db, {%2, %4};\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], db, %3, p;\n\t}"
+        ::"r"(d_tmem), "r"(a_tmem), "r"(b_low), "r"(idesc), "r"(kDescHigh), "r"(accumulate)
+        : "memory");
+}
+// 8 consecutive 32-bit columns of this thread's TMEM lane, written.
+__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&r)[8]) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
+        ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
+        : "memory");
+}
+__device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+
+__device__ __forceinline__ float2 fadd2(float2 a, float2 b) {
+    float2 d;
+    asm("{\n\t.reg .b64 ra, rb, rd;\n\t"
+        "mov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\t"
+        "add.rn.f32x2 rd, ra, rb;\n\t"
+        "mov.b64 {%0, %1}, rd;\n\t}"
+        : "=f"(d.x), "=f"(d.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return d;
+}
+__device__ __forceinline__ float2 dup2(float x) { return make_float2(x, x); }
+__device__ __forceinline__ float sqrt_approx(float x) {
+    float r;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ float exp2_approx(float x) {
+    float r;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+// A word of V, or 0.  Volatile: the loads of a window stay together in front of the arithmetic.  Left to itself the
+// compiler spreads them out to save registers, and every few FMAs then wait for a trip to L2 (102 us instead of 77 us for
+// the masked branch on 768 planes of 14 x 14).
+__device__ __forceinline__ uint32_t ldg_or_zero(const __nv_bfloat16* p, bool valid) {
+    uint32_t v;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %2, 0;\n\t"
+        "mov.b32 %0, 0;\n\t"
+        "@p ld.global.nc.b32 %0, [%1];\n\t}"
+        : "=r"(v) : "l"(p), "r"((int)valid));
+    return v;
+}
+
+constexpr float kLog2e = 1.4426950408889634f;
+
+// 1 - arccos(x)/pi of a pair: with t = 1 - |x| (clamped to [0, 1]: rounding can leave a cosine just outside [-1, 1]),
+// arccos(|x|) = sqrt(t) * cubic(t) -- Abramowitz & Stegun 4.4.45 with its cubic in |x| expanded about |x| = 1, |error| <
+// 7e-5 rad, far below the bf16 rounding of the weights -- and 1 - arccos(x)/pi = 1/2 + sign(x) (1/2 - arccos(|x|)/pi).
+__device__ __forceinline__ float2 angular_weight2(float2 x) {
+    const float2 t = make_float2(__saturatef(1.0f - fabsf(x.x)), __saturatef(1.0f - fabsf(x.y)));
+    const float2 s = make_float2(sqrt_approx(t.x), sqrt_approx(t.y));
+    float2 p = ffma2(dup2(-0.0187293f * kInvPi), t, dup2(-0.0180731f * kInvPi));
+    p = ffma2(p, t, dup2(-0.1197803f * kInvPi));
+    p = ffma2(p, t, dup2(-1.4141461f * kInvPi));
+    const float2 h = ffma2(s, p, dup2(0.5f));
+    const uint32_t sx = __float_as_uint(x.x) & 0x80000000u, sy = __float_as_uint(x.y) & 0x80000000u;
+    return fadd2(make_float2(__uint_as_float((__float_as_uint(h.x) & 0x7fffffffu) | sx),
+                             __uint_as_float((__float_as_uint(h.y) & 0x7fffffffu) | sy)), dup2(0.5f));
 }
 
 template <int KS, bool SPARSE, bool EXACT>
@@ -68,38 +158,52 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     uint8_t* Q_s = smem + kOffQ;
-    uint8_t* stages = smem + kOffStages;
-    uint8_t* P_s = smem + kOffP;
-    float* den_s = reinterpret_cast<float*>(smem + kOffDen);
-    uint64_t* q_full = reinterpret_cast<uint64_t*>(smem + kOffBar);
-    uint64_t* q_ready = q_full + 1;      // Q rows scaled (128)
-    uint64_t* q_free = q_ready + 1;      // the item's last cosine UMMAs have read Q
-    uint64_t* kv_full = q_free + 1;      // [kStages]
-    uint64_t* k_scaled = kv_full + kStages;
-    uint64_t* kv_empty = k_scaled + kStages;
-    uint64_t* c_full = kv_empty + kStages;   // [2]
-    uint64_t* c_free = c_full + 2;           // [2] (256)
-    uint64_t* p_full = c_free + 2;           // [2] (256)
-    uint64_t* p_free = p_full + 2;           // [2]
-    uint64_t* o_full = p_free + 2;
-    uint64_t* o_free = o_full + 1;           // (128)
-    uint64_t* den_bar = o_free + 1;          // (256) both halves of every query's denominator are in shared memory
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(den_bar + 1);
+    uint8_t* K_s = smem + kOffK;
+    uint8_t* V_s = smem + kOffV;
+    uint8_t* stg = smem + kOffStg;
+    uint64_t* q_full = reinterpret_cast<uint64_t*>(smem + kOffBar);   // [2] by item
+    uint64_t* q_ready = q_full + 2;              // [2] Q rows scaled (kNormThreads)
+    uint64_t* q_free = q_ready + 2;              // [2] the item's last cosine UMMAs have read Q
+    uint64_t* k_full = q_free + 2;               // [kKStages]
+    uint64_t* k_scaled = k_full + kKStages;      // [kKStages] (kNormThreads)
+    uint64_t* k_empty = k_scaled + kKStages;     // [kKStages]
+    uint64_t* v_full = k_empty + kKStages;       // [kVStages]
+    uint64_t* v_empty = v_full + kVStages;       // [kVStages]
+    uint64_t* c_full = v_empty + kVStages;       // [2][kCBufs] by slot: cosines written
+    uint64_t* r_done = c_full + 2 * kCBufs;      // [kCBufs] cosines of a first sweep read (kSlotThreads)
+    uint64_t* p_full = r_done + kCBufs;          // [kCBufs] weights written (kSlotThreads)
+    uint64_t* pv_done = p_full + kCBufs;         // [kCBufs] weights read by the second contraction
+    uint64_t* o_full = pv_done + kCBufs;         // [2] by slot
+    uint64_t* o_free = o_full + 2;               // [2] (128)
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(o_free + 2);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int my_items = ((int)blockIdx.x < prm.n_items) ? (prm.n_items - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
-    const int KT = prm.k_tiles;
-    const int sweeps = SPARSE ? 2 : 1;   // key tiles per item: sweeps * KT; the last sweep feeds the second contraction
+    const int T = prm.k_tiles, N = prm.N;
+    constexpr int kSweeps = SPARSE ? 2 : 1;
+    const bool resident = SPARSE && T <= kResident;
+    const int k_loads = resident ? T : kSweeps * T;   // K tiles loaded per item
     constexpr unsigned kBit = kStatusFusedTimeout;
+    // item number i of this CTA: plane, first token, active slots
+    struct Item { int bh, t0, slots; };
+    auto item_of = [&](int i) -> Item {
+        const int item = blockIdx.x + i * gridDim.x, bh = item / prm.groups, t0 = (item - bh * prm.groups) * prm.slots * kTile;
+        return {bh, t0, min(prm.slots, (N - t0 + kTile - 1) / kTile)};
+    };
+    auto warp_wait = [&](uint64_t* bar, uint32_t parity) -> bool {
+        return __all_sync(0xffffffffu, mbar_poll(bar, parity) || mbar_wait(bar, parity, abort_flag, prm.status, kBit));
+    };
 
     if (tid == 0) {
-        mbar_init(q_full, 1); mbar_init(q_ready, kNormThreads); mbar_init(q_free, 1);
-        for (int s = 0; s < kStages; ++s) { mbar_init(&kv_full[s], 1); mbar_init(&k_scaled[s], kNormThreads); mbar_init(&kv_empty[s], 1); }
-        for (int b = 0; b < 2; ++b) {
-            mbar_init(&c_full[b], 1); mbar_init(&c_free[b], kWThreads); mbar_init(&p_full[b], kWThreads); mbar_init(&p_free[b], 1);
+        for (int b = 0; b < 2; ++b) { mbar_init(&q_full[b], 1); mbar_init(&q_ready[b], kNormThreads); mbar_init(&q_free[b], 1); }
+        for (int s = 0; s < kKStages; ++s) { mbar_init(&k_full[s], 1); mbar_init(&k_scaled[s], kNormThreads); mbar_init(&k_empty[s], 1); }
+        for (int s = 0; s < kVStages; ++s) { mbar_init(&v_full[s], 1); mbar_init(&v_empty[s], 1); }
+        for (int b = 0; b < kCBufs; ++b) {
+            mbar_init(&c_full[b], 1); mbar_init(&c_full[kCBufs + b], 1);
+            mbar_init(&r_done[b], kSlotThreads); mbar_init(&p_full[b], kSlotThreads); mbar_init(&pv_done[b], 1);
         }
-        mbar_init(o_full, 1); mbar_init(o_free, kNormThreads); mbar_init(den_bar, kWThreads);
+        for (int s = 0; s < 2; ++s) { mbar_init(&o_full[s], 1); mbar_init(&o_free[s], kTile); }
         *abort_flag = 0;
         mbar_fence_init();
         tma_prefetch_desc(&tmQ); tma_prefetch_desc(&tmK); tma_prefetch_desc(&tmV);
@@ -112,259 +216,406 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
 
     if (warp == 0) {
         if (lane == 0) {
-            long long g = 0;   // key tiles issued so far, over all items
-            bool ok = true;
-            for (int i = 0; i < my_items && ok; ++i) {
-                const int item = blockIdx.x + i * gridDim.x, bh = item / prm.q_tiles, qt = item - bh * prm.q_tiles;
-                const int pb = bh / prm.hdiv, ph = bh - pb * prm.hdiv;
-                if (i > 0 && !mbar_wait(q_free, (i - 1) & 1, abort_flag, prm.status, kBit)) break;
-                mbar_expect_tx(q_full, kTileBytes);
-                tma_load_4d(Q_s, &tmQ, q_full, 0, qt * kTile, ph, pb);
-                for (int tt = 0; tt < sweeps * KT; ++tt, ++g) {
-                    const int jt = tt % KT;
-                    const bool with_v = tt >= (sweeps - 1) * KT;   // the first sweep of two needs the keys only
-                    const int s = (int)(g % kStages), use = (int)(g / kStages);
-                    if (use > 0 && !mbar_wait(&kv_empty[s], (use - 1) & 1, abort_flag, prm.status, kBit)) { ok = false; break; }
-                    uint8_t* ks = stages + s * kStageBytes;
-                    mbar_expect_tx(&kv_full[s], with_v ? kStageBytes : kTileBytes);
-                    tma_load_4d(ks, &tmK, &kv_full[s], 0, jt * kTile, ph, pb);
-                    if (with_v) tma_load_4d(ks + kTileBytes, &tmV, &kv_full[s], 0, jt * kTile, ph, pb);
+            // three independent rings, polled in turn: none waits behind another
+            int qi = 0, ki = 0, kj = 0, vi = 0, vj = 0;   // next item (and tile of it) of each ring
+            int kn = 0, vn = 0;                           // tiles issued
+            unsigned long long t_last = 0;
+            uint32_t idle = 0;
+            while (qi < my_items || ki < my_items || vi < my_items) {
+                bool moved = false;
+                if (qi < my_items && (qi < 2 || mbar_poll(&q_free[qi & 1], ((qi >> 1) - 1) & 1))) {
+                    const Item im = item_of(qi);
+                    const int pb = im.bh / prm.hdiv, ph = im.bh - pb * prm.hdiv, b = qi & 1;
+                    mbar_expect_tx(&q_full[b], im.slots * kTileBytes);
+                    for (int s = 0; s < im.slots; ++s)
+                        tma_load_4d(Q_s + (2 * b + s) * kTileBytes, &tmQ, &q_full[b], 0, im.t0 + s * kTile, ph, pb);
+                    ++qi;
+                    moved = true;
+                }
+                if (ki < my_items) {
+                    const int s = kn % kKStages, use = kn / kKStages;
+                    if (use == 0 || mbar_poll(&k_empty[s], (use - 1) & 1)) {
+                        const int bh = item_of(ki).bh, pb = bh / prm.hdiv, ph = bh - pb * prm.hdiv;
+                        mbar_expect_tx(&k_full[s], kTileBytes);
+                        tma_load_4d(K_s + s * kTileBytes, &tmK, &k_full[s], 0, (kj % T) * kTile, ph, pb);
+                        ++kn;
+                        if (++kj == k_loads) { kj = 0; ++ki; }
+                        moved = true;
+                    }
+                }
+                if (vi < my_items) {
+                    const int s = vn % kVStages, use = vn / kVStages;
+                    if (use == 0 || mbar_poll(&v_empty[s], (use - 1) & 1)) {
+                        const int bh = item_of(vi).bh, pb = bh / prm.hdiv, ph = bh - pb * prm.hdiv;
+                        mbar_expect_tx(&v_full[s], kTileBytes);
+                        tma_load_4d(V_s + s * kTileBytes, &tmV, &v_full[s], 0, vj * kTile, ph, pb);
+                        ++vn;
+                        if (++vj == T) { vj = 0; ++vi; }
+                        moved = true;
+                    }
+                }
+                if (moved) { idle = 0; continue; }
+                __nanosleep(20);
+                if ((++idle & 255u) == 0) {
+                    const unsigned long long now = global_ns();
+                    if (idle == 256u) t_last = now;
+                    if (*abort_flag) break;
+                    if (now - t_last > kWaitLimitNs) { *abort_flag = 1; atomicOr(prm.status, kBit); break; }
                 }
             }
             if (*abort_flag) {  // giving up: let the copies in flight land before shared memory goes away
-                for (long long i = (g > kStages ? g - kStages : 0); i < g; ++i)
-                    for (int spin = 0; spin < (1 << 20) && !mbar_try_wait(&kv_full[i % kStages], (uint32_t)((i / kStages) & 1)); ++spin) {}
+                for (int i = max(0, kn - kKStages); i < kn; ++i)
+                    for (int spin = 0; spin < (1 << 20) && !mbar_try_wait(&k_full[i % kKStages], (i / kKStages) & 1); ++spin) {}
+                for (int i = max(0, vn - kVStages); i < vn; ++i)
+                    for (int spin = 0; spin < (1 << 20) && !mbar_try_wait(&v_full[i % kVStages], (i / kVStages) & 1); ++spin) {}
+                for (int i = max(0, qi - 2); i < qi; ++i)
+                    for (int spin = 0; spin < (1 << 20) && !mbar_try_wait(&q_full[i & 1], (i >> 1) & 1); ++spin) {}
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            constexpr uint32_t idesc_c = umma_idesc_bf16(128, 128, false, false);   // Q^ (K-major) x K^ (K-major)
-            constexpr uint32_t idesc_o = umma_idesc_bf16(128, kD, false, true);     // W (K-major) x V (N-major)
-            const uint32_t q_addr = smem_u32(Q_s), p_addr = smem_u32(P_s);
-            long long g = 0, gp = 0;   // key tiles so far: all of them / those that feed the second contraction
-            bool ok = true;
-            // the second contraction of the tile with ring number gg and weight-buffer number pp; first: the item's first
-            auto second = [&](long long gg, long long pp, bool first) -> bool {
-                const int s = (int)(gg % kStages), pbuf = (int)(pp & 1);
-                if (!mbar_wait(&p_full[pbuf], (uint32_t)((pp >> 1) & 1), abort_flag, prm.status, kBit)) return false;
-                tcgen05_fence_after_sync();
-                const uint32_t va = smem_u32(stages + s * kStageBytes + kTileBytes), pa = p_addr + pbuf * kPBytes;
-#pragma unroll
-                for (int j = 0; j < kTile / 16; ++j) {
-                    const uint64_t a = umma_desc_sw128(pa + (j >> 2) * kTileBytes + (j & 3) * 32, 0, 1024);
-                    const uint64_t b = umma_desc_sw128(va + j * 2048, 0, 1024);
-                    umma_bf16(tmem + 256, a, b, idesc_o, (first && j == 0) ? 0u : 1u);
-                }
-                umma_commit(&p_free[pbuf]);
-                umma_commit(&kv_empty[s]);
-                return true;
-            };
-            for (int i = 0; i < my_items && ok; ++i) {
-                if (!mbar_wait(q_ready, i & 1, abort_flag, prm.status, kBit)) break;
-                // the previous item's output has been read out of TMEM before this item's first accumulation
-                if (i > 0 && !mbar_wait(o_free, (i - 1) & 1, abort_flag, prm.status, kBit)) break;
-                for (int tt = 0; tt < sweeps * KT && ok; ++tt, ++g) {
-                    const bool last_sweep = tt >= (sweeps - 1) * KT;
-                    const int jt = tt % KT;
-                    const int s = (int)(g % kStages), use = (int)(g / kStages), cb = (int)(g & 1);
-                    ok = mbar_wait(&k_scaled[s], use & 1, abort_flag, prm.status, kBit);
-                    if (ok && g >= 2) ok = mbar_wait(&c_free[cb], (uint32_t)(((g >> 1) - 1) & 1), abort_flag, prm.status, kBit);
-                    if (!ok) break;
-                    tcgen05_fence_after_sync();
-                    const uint32_t ka = smem_u32(stages + s * kStageBytes);
-#pragma unroll
-                    for (int k = 0; k < kD / 16; ++k) {
-                        const uint64_t a = umma_desc_sw128(q_addr + k * 32, 0, 1024);
-                        const uint64_t b = umma_desc_sw128(ka + k * 32, 0, 1024);
-                        umma_bf16(tmem + cb * 128, a, b, idesc_c, k != 0);
+        // ---- cosines: the whole warp walks through the schedule, one elected lane issues ----
+        constexpr uint32_t idesc_c = umma_idesc_bf16(kTile, kTile, false, false);   // Q^ (K-major) x K^ (K-major)
+        const uint32_t q_low = desc_low(Q_s), k_low = desc_low(K_s);
+        uint32_t pv_pending = 0, rd_pending = 0;   // bit b: buffer b was last handed to the second contraction / to a first sweep
+        uint32_t pv_parity = 0, rd_parity = 0;     // bit b: parity of the next completion of pv_done[b] / r_done[b]
+        int b = 0, ks = 0;                         // next buffer and K stage
+        uint32_t k_par = 0;
+        bool ok = true;
+        for (int i = 0; i < my_items && ok; ++i) {
+            const int slots = item_of(i).slots;
+            if (!(ok = warp_wait(&q_ready[i & 1], (i >> 1) & 1))) break;
+            const int ks_item = ks;                // resident: the second sweep reads the stages of the first
+            const uint32_t k_par_item = k_par;
+            for (int u = 0; u < kSweeps * T && ok; ++u) {
+                const bool last_sweep = u >= (kSweeps - 1) * T;
+                if (SPARSE && resident && u == T) { ks = ks_item; k_par = k_par_item; }
+                if (!(ok = warp_wait(&k_scaled[ks], k_par))) break;
+                for (int s = 0; s < slots; ++s) {
+                    const uint32_t bit = 1u << b;
+                    if (pv_pending & bit) {
+                        ok = warp_wait(&pv_done[b], (pv_parity & bit) != 0);
+                        pv_parity ^= bit;
+                    } else if (SPARSE && (rd_pending & bit)) {
+                        ok = warp_wait(&r_done[b], (rd_parity & bit) != 0);
+                        rd_parity ^= bit;
                     }
-                    umma_commit(&c_full[cb]);
-                    if (!last_sweep) { umma_commit(&kv_empty[s]); continue; }   // cosines only: the stage is free again
-                    if (jt == KT - 1) umma_commit(q_free);
-                    if (jt > 0) { ok = second(g - 1, gp, jt == 1); ++gp; }   // one tile behind: the weight warps work meanwhile
+                    if (!ok) break;
+                    if (last_sweep) { pv_pending |= bit; rd_pending &= ~bit; } else { rd_pending |= bit; pv_pending &= ~bit; }
+                    tcgen05_fence_after_sync();
+                    if (elect_one()) {
+                        const uint32_t d = tmem + b * kTile, a = q_low + (2 * (i & 1) + s) * (kTileBytes >> 4);
+                        const uint32_t k = k_low + ks * (kTileBytes >> 4);
+                        umma_ss<false>(d, a, k, idesc_c);
+                        umma_ss<true>(d, a + 2, k + 2, idesc_c);
+                        umma_ss<true>(d, a + 4, k + 4, idesc_c);
+                        umma_ss<true>(d, a + 6, k + 6, idesc_c);
+                        umma_commit(&c_full[s * kCBufs + b]);
+                        if (s == slots - 1) {
+                            if (last_sweep || !resident) umma_commit(&k_empty[ks]);
+                            if (u == kSweeps * T - 1) umma_commit(&q_free[i & 1]);
+                        }
+                    }
+                    __syncwarp();
+                    b = b == kCBufs - 1 ? 0 : b + 1;
                 }
-                if (ok) { ok = second(g - 1, gp, KT == 1); ++gp; }
-                if (ok) umma_commit(o_full);
+                if (++ks == kKStages) { ks = 0; k_par ^= 1; }
             }
         }
-    } else if (warp < 6) {
-        // ---- unit rows: Q once per item, K per tile ----
-        const int t = tid - 64;
-        auto scale_row = [&](uint8_t* row) {
+    } else if (warp == 2) {
+        // ---- weighted sums ----
+        constexpr uint32_t idesc_o = umma_idesc_bf16(kTile, kD, false, true);       // W (TMEM) x V (N-major)
+        const uint32_t v_low = desc_low(V_s);
+        int b = 0, vs = 0;
+        uint32_t p_parity = 0, v_par = 0, o_used = 0, o_parity = 0;
+        bool ok = true;
+        for (int i = 0; i < my_items && ok; ++i) {
+            const int slots = item_of(i).slots;
+            if (SPARSE) b = (b + T * slots) % kCBufs;   // the buffers of the first sweep are not this warp's
+            for (int j = 0; j < T && ok; ++j) {
+                if (!(ok = warp_wait(&v_full[vs], v_par))) break;
+                for (int s = 0; s < slots; ++s) {
+                    const uint32_t bit = 1u << b;
+                    if (j == 0) {   // the previous item's output has been read out of TMEM
+                        if ((o_used >> s) & 1) { ok = warp_wait(&o_free[s], (o_parity >> s) & 1); o_parity ^= 1u << s; }
+                        o_used |= 1u << s;
+                    }
+                    ok = ok && warp_wait(&p_full[b], (p_parity & bit) != 0);
+                    if (!ok) break;
+                    p_parity ^= bit;
+                    tcgen05_fence_after_sync();
+                    if (elect_one()) {
+                        const uint32_t d = tmem + kColO + s * kD, a = tmem + b * kTile, v = v_low + vs * (kTileBytes >> 4);
+                        umma_ts(d, a, v, idesc_o, j != 0);
+#pragma unroll
+                        for (int k = 1; k < kTile / 16; ++k)   // the weights of each half of the keys lie in its half of the columns
+                            umma_ts(d, a + (k & 3) * 8 + (k >> 2) * (kTile / 2), v + k * 128, idesc_o, 1u);
+                        umma_commit(&pv_done[b]);
+                        if (s == slots - 1) umma_commit(&v_empty[vs]);
+                        if (j == T - 1) umma_commit(&o_full[s]);
+                    }
+                    __syncwarp();
+                    b = b == kCBufs - 1 ? 0 : b + 1;
+                }
+                if (++vs == kVStages) { vs = 0; v_par ^= 1; }
+            }
+        }
+    } else if (warp == 3) {
+        // spare: keeps the roles below aligned to groups of four warps
+    } else if (warp < 8) {
+        // ---- unit rows ----
+        const int t = tid - 128;
+        auto scale_row = [&](uint8_t* row) {   // row t of a tile
             uint4 c[8];
-            float ss = 0.f;
+            float2 ss[4] = {dup2(0.f), dup2(0.f), dup2(0.f), dup2(0.f)};
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
                 c[j] = *reinterpret_cast<const uint4*>(row + ((j ^ (t & 7)) << 4));
                 const uint32_t w[4] = {c[j].x, c[j].y, c[j].z, c[j].w};
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
-                    const float lo = bf16lo(w[e]), hi = bf16hi(w[e]);
-                    ss = fmaf(lo, lo, ss);
-                    ss = fmaf(hi, hi, ss);
+                    const float2 p = make_float2(bf16lo(w[e]), bf16hi(w[e]));
+                    ss[e] = ffma2(p, p, ss[e]);
                 }
             }
-            const float rk = 1.0f / sqrtf(fmaxf(ss, prm.eps2));
+            const float2 sum = fadd2(fadd2(ss[0], ss[1]), fadd2(ss[2], ss[3]));
+            const float2 rk2 = dup2(1.0f / sqrtf(fmaxf(sum.x + sum.y, prm.eps2)));
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
-                uint4 o;
-                o.x = pack_bf16x2(bf16lo(c[j].x) * rk, bf16hi(c[j].x) * rk);
-                o.y = pack_bf16x2(bf16lo(c[j].y) * rk, bf16hi(c[j].y) * rk);
-                o.z = pack_bf16x2(bf16lo(c[j].z) * rk, bf16hi(c[j].z) * rk);
-                o.w = pack_bf16x2(bf16lo(c[j].w) * rk, bf16hi(c[j].w) * rk);
-                *reinterpret_cast<uint4*>(row + ((j ^ (t & 7)) << 4)) = o;
+                const uint32_t w[4] = {c[j].x, c[j].y, c[j].z, c[j].w};
+                uint32_t o[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const float2 p = ffma2(make_float2(bf16lo(w[e]), bf16hi(w[e])), rk2, dup2(0.f));
+                    o[e] = pack_bf16x2(p.x, p.y);
+                }
+                *reinterpret_cast<uint4*>(row + ((j ^ (t & 7)) << 4)) = make_uint4(o[0], o[1], o[2], o[3]);
             }
-            fence_proxy_async_smem();
         };
-        long long g = 0;
-        bool ok = true;
+        // The Q tiles of item i + 1 come after the first K tiles of item i: their copy starts once the cosines of item
+        // i - 1 are done, whose K tiles were all scaled before those of item i, so this wait never holds up its own cause.
+        auto scale_q = [&](int i) -> bool {
+            if (!warp_wait(&q_full[i & 1], (i >> 1) & 1)) return false;
+            const int slots = item_of(i).slots;
+            for (int s = 0; s < slots; ++s) scale_row(Q_s + (2 * (i & 1) + s) * kTileBytes + t * 128);
+            fence_proxy_async_smem();
+            mbar_arrive(&q_ready[i & 1]);
+            return true;
+        };
+        int ks = 0;
+        uint32_t k_par = 0;
+        const int q_after = min(k_loads, 2) - 1;
+        bool ok = my_items > 0 && scale_q(0);
         for (int i = 0; i < my_items && ok; ++i) {
-            if (!mbar_wait(q_full, i & 1, abort_flag, prm.status, kBit)) break;
-            scale_row(Q_s + t * 128);
-            mbar_arrive(q_ready);
-            for (int tt = 0; tt < sweeps * KT; ++tt, ++g) {
-                const int s = (int)(g % kStages), use = (int)(g / kStages);
-                if (!mbar_wait(&kv_full[s], use & 1, abort_flag, prm.status, kBit)) { ok = false; break; }
-                scale_row(stages + s * kStageBytes + t * 128);
-                mbar_arrive(&k_scaled[s]);
+            for (int j = 0; j < k_loads; ++j) {
+                if (!(ok = warp_wait(&k_full[ks], k_par))) break;
+                scale_row(K_s + ks * kTileBytes + t * 128);
+                fence_proxy_async_smem();
+                mbar_arrive(&k_scaled[ks]);
+                if (++ks == kKStages) { ks = 0; k_par ^= 1; }
+                if (j == q_after && i + 1 < my_items && !(ok = scale_q(i + 1))) break;
             }
         }
-    } else {
-        // ---- weights: thread = (query row, 64 of the tile's 128 keys); at the end of an item half 0 writes the rows ----
-        const int quarter = warp & 3, half = (warp - 6) >> 2, row = quarter * 32 + lane;
-        const uint32_t lane_base = tmem + ((uint32_t)(quarter * 32) << 16);
-        long long g = 0, gp = 0;
+    } else if (warp < 24) {
+        // ---- weights: thread = query row of slot (warp - 8) / 8, half of the keys of every tile ----
+        const int slot = (warp - 8) >> 3, half = ((warp - 8) >> 2) & 1, quarter = warp & 3;
+        const uint32_t col0 = tmem + ((uint32_t)(quarter * 32) << 16) + half * (kTile / 2);
+        int b = 0;                  // buffer of the next step of the CTA (this slot's or not)
+        uint32_t par = 0;           // bit b: parity of the next completion of this slot's c_full[b]
+        auto skip = [&](int n) { b = (b + n) % kCBufs; };
+        auto wait_cosines = [&]() -> bool {
+            const bool done = warp_wait(&c_full[slot * kCBufs + b], (par >> b) & 1);
+            par ^= 1u << b;
+            return done;
+        };
         bool ok = true;
         for (int i = 0; i < my_items && ok; ++i) {
-            const int item = blockIdx.x + i * gridDim.x, bh = item / prm.q_tiles, qt = item - bh * prm.q_tiles;
-            float inv_den = 0.f;
+            const Item im = item_of(i);
+            if (slot >= im.slots) { skip(kSweeps * T * im.slots); continue; }
+            const bool live = im.t0 + slot * kTile + quarter * 32 < N;   // some row of this warp is a token
+            float ebias = 0.f;   // exp(x) / den = exp2(y * 2 log2(e) + ebias), y = (x + 1) / 2
+            skip(slot);
             if (SPARSE) {
-                // first sweep: sum over the plane's keys of exp(cosine) for this thread's query, half of every tile
-                float den = 0.f;
-                for (int jt = 0; jt < KT; ++jt, ++g) {
-                    const int cb = (int)(g & 1);
-                    if (!mbar_wait(&c_full[cb], (uint32_t)((g >> 1) & 1), abort_flag, prm.status, kBit)) { ok = false; break; }
-                    tcgen05_fence_after_sync();
-                    const int key0 = jt * kTile + half * 64;
+                float2 den = dup2(0.f);
+                for (int jt = 0; jt < T; ++jt) {
+                    if (!(ok = wait_cosines())) break;
+                    const int left = N - jt * kTile - half * (kTile / 2);   // keys of the plane from this half on
+                    if (live && left > 0) {
+                        tcgen05_fence_after_sync();
+                        float x[2][16];
+                        tmem_ld16(col0 + b * kTile, x[0]);
 #pragma unroll
-                    for (int cc = 0; cc < 4; ++cc) {
-                        float x[16];
-                        tmem_ld16(lane_base + cb * 128 + half * 64 + cc * 16, x);
-                        tmem_ld_wait();
-                        if (jt < KT - 1) {   // only the last tile can reach beyond the plane
+                        for (int cc = 0; cc < 4; ++cc) {
+                            tmem_ld_wait();
+                            if (cc < 3) tmem_ld16(col0 + b * kTile + (cc + 1) * 16, x[(cc + 1) & 1]);
+                            if (cc * 16 >= left) continue;
 #pragma unroll
-                            for (int e = 0; e < 16; ++e) den += __expf(fminf(fmaxf(x[e], -1.0f), 1.0f));
-                        } else {
-#pragma unroll
-                            for (int e = 0; e < 16; ++e)
-                                if (key0 + cc * 16 + e < prm.N) den += __expf(fminf(fmaxf(x[e], -1.0f), 1.0f));
-                        }
-                    }
-                    tcgen05_fence_before_sync();
-                    mbar_arrive(&c_free[cb]);
-                }
-                if (!ok) break;
-                den_s[half * kTile + row] = den;
-                mbar_arrive(den_bar);
-                if (!mbar_wait(den_bar, i & 1, abort_flag, prm.status, kBit)) break;
-                inv_den = 1.0f / (den_s[row] + den_s[kTile + row]);
-            }
-            // weight of a pair from its cosine
-            auto weight = [&](float xr) -> float {
-                // rounding can leave a cosine just outside [-1, 1]; the exact kernel's function clamps |x| itself
-                const float x = (EXACT && !SPARSE) ? xr : fminf(fmaxf(xr, -1.0f), 1.0f);
-                float wv = EXACT ? angular_weight(x) : fmaf(x, kInvPi, 0.5f);
-                if (SPARSE) {
-                    const float pr = __expf(x) * inv_den;
-                    if (pr > prm.sparse_eps) wv += pr;
-                }
-                return wv;
-            };
-            for (int jt = 0; jt < KT; ++jt, ++g, ++gp) {
-                const int cb = (int)(g & 1), pbuf = (int)(gp & 1);
-                if (!mbar_wait(&c_full[cb], (uint32_t)((g >> 1) & 1), abort_flag, prm.status, kBit)) { ok = false; break; }
-                tcgen05_fence_after_sync();
-                if (gp >= 2 && !mbar_wait(&p_free[pbuf], (uint32_t)(((gp >> 1) - 1) & 1), abort_flag, prm.status, kBit)) { ok = false; break; }
-                uint8_t* prow = P_s + pbuf * kPBytes + half * kTileBytes + row * 128;
-#pragma unroll
-                for (int cc = 0; cc < 4; ++cc) {
-                    float x[16];
-                    tmem_ld16(lane_base + cb * 128 + half * 64 + cc * 16, x);
-                    tmem_ld_wait();
-                    uint4 o0, o1;
-                    o0.x = pack_bf16x2(weight(x[0]), weight(x[1]));
-                    o0.y = pack_bf16x2(weight(x[2]), weight(x[3]));
-                    o0.z = pack_bf16x2(weight(x[4]), weight(x[5]));
-                    o0.w = pack_bf16x2(weight(x[6]), weight(x[7]));
-                    o1.x = pack_bf16x2(weight(x[8]), weight(x[9]));
-                    o1.y = pack_bf16x2(weight(x[10]), weight(x[11]));
-                    o1.z = pack_bf16x2(weight(x[12]), weight(x[13]));
-                    o1.w = pack_bf16x2(weight(x[14]), weight(x[15]));
-                    *reinterpret_cast<uint4*>(prow + (((2 * cc) ^ (row & 7)) << 4)) = o0;
-                    *reinterpret_cast<uint4*>(prow + (((2 * cc + 1) ^ (row & 7)) << 4)) = o1;
-                }
-                tcgen05_fence_before_sync();
-                mbar_arrive(&c_free[cb]);
-                fence_proxy_async_smem();
-                mbar_arrive(&p_full[pbuf]);
-            }
-            if (!ok) break;
-            if (half == 0) {
-                if (!mbar_wait(o_full, i & 1, abort_flag, prm.status, kBit)) break;
-                tcgen05_fence_after_sync();
-                float o[kD];
-#pragma unroll
-                for (int cc = 0; cc < 4; ++cc) {
-                    float x[16];
-                    tmem_ld16(lane_base + 256 + cc * 16, x);
-                    tmem_ld_wait();
-#pragma unroll
-                    for (int e = 0; e < 16; ++e) o[cc * 16 + e] = x[e];
-                }
-                tcgen05_fence_before_sync();
-                mbar_arrive(o_free);
-                const int tq = qt * kTile + row;
-                if (tq < prm.N) {
-                    const int y = tq / prm.gridW, xq = tq - y * prm.gridW;
-                    constexpr int R = KS / 2;
-                    const __nv_bfloat16* vp = prm.v + plane_offset(prm.lv, bh, prm.hdiv);
-                    // filters and bias of the item's head: the same address in every lane (a broadcast from L1)
-                    const int hh = (prm.head0 + bh) % prm.H;
-                    const __nv_bfloat16* wh = prm.w + (size_t)hh * kD * (KS * KS);
-                    if (prm.bias) {
-#pragma unroll
-                        for (int c = 0; c < kD; ++c) o[c] += __bfloat162float(prm.bias[hh * kD + c]);
-                    }
-                    for (int dy = 0; dy < KS; ++dy) {
-                        const int yy = y + dy - R;
-                        if ((unsigned)yy >= (unsigned)prm.gridH) continue;
-                        for (int dx = 0; dx < KS; ++dx) {
-                            const int xx = xq + dx - R;
-                            if ((unsigned)xx >= (unsigned)prm.gridW) continue;
-                            const uint4* vr = reinterpret_cast<const uint4*>(vp + (size_t)(yy * prm.gridW + xx) * prm.lv.token);
-                            const __nv_bfloat16* fw = wh + dy * KS + dx;   // channel c at fw[c * KS * KS]
-#pragma unroll
-                            for (int c8 = 0; c8 < 8; ++c8) {
-                                const uint4 vv = __ldg(vr + c8);
-                                const uint32_t w4[4] = {vv.x, vv.y, vv.z, vv.w};
-#pragma unroll
-                                for (int e = 0; e < 4; ++e) {
-                                    o[c8 * 8 + 2 * e] = fmaf(__bfloat162float(fw[(c8 * 8 + 2 * e) * (KS * KS)]), bf16lo(w4[e]), o[c8 * 8 + 2 * e]);
-                                    o[c8 * 8 + 2 * e + 1] = fmaf(__bfloat162float(fw[(c8 * 8 + 2 * e + 1) * (KS * KS)]), bf16hi(w4[e]), o[c8 * 8 + 2 * e + 1]);
+                            for (int e = 0; e < 16; e += 2) {
+                                const float* xe = &x[cc & 1][e];
+                                const float2 y = make_float2(__saturatef(fmaf(xe[0], 0.5f, 0.5f)), __saturatef(fmaf(xe[1], 0.5f, 0.5f)));
+                                const float2 a = ffma2(y, dup2(2.0f * kLog2e), dup2(-kLog2e));
+                                float2 p = make_float2(exp2_approx(a.x), exp2_approx(a.y));
+                                if (cc * 16 + 16 > left) {   // the chunk that reaches beyond the plane
+                                    p.x = cc * 16 + e < left ? p.x : 0.f; p.y = cc * 16 + e + 1 < left ? p.y : 0.f;
                                 }
+                                den = fadd2(den, p);
                             }
                         }
+                        tcgen05_fence_before_sync();
                     }
-                    uint4* orow = reinterpret_cast<uint4*>(prm.out + plane_offset(prm.lo, bh, prm.hdiv) + (size_t)tq * prm.lo.token);
+                    mbar_arrive(&r_done[b]);
+                    skip(im.slots);
+                }
+                if (!ok) break;
+                // the two halves of a query meet in shared memory (by item parity: a thread is never two items ahead)
+                float* den_s = reinterpret_cast<float*>(smem + kOffDen) + ((i & 1) * 4 + slot * 2) * kTile + quarter * 32 + lane;
+                den_s[half * kTile] = den.x + den.y;
+                named_barrier_sync(2 + slot, kSlotThreads);
+                ebias = -kLog2e - __log2f(den_s[0] + den_s[kTile]);
+            }
+            for (int jt = 0; jt < T; ++jt) {
+                if (!(ok = wait_cosines())) break;
+                if (live) {
+                    tcgen05_fence_after_sync();
+                    const uint32_t cb = col0 + b * kTile;
+                    const int left = N - jt * kTile - half * (kTile / 2);
+                    float x[2][16];
+                    tmem_ld16(cb, x[0]);
 #pragma unroll
-                    for (int c8 = 0; c8 < 8; ++c8) {
-                        uint4 pk;
-                        pk.x = pack_bf16x2(o[c8 * 8 + 0], o[c8 * 8 + 1]); pk.y = pack_bf16x2(o[c8 * 8 + 2], o[c8 * 8 + 3]);
-                        pk.z = pack_bf16x2(o[c8 * 8 + 4], o[c8 * 8 + 5]); pk.w = pack_bf16x2(o[c8 * 8 + 6], o[c8 * 8 + 7]);
-                        orow[c8] = pk;
+                    for (int cc = 0; cc < 4; ++cc) {
+                        tmem_ld_wait();
+                        if (cc < 3) tmem_ld16(cb + (cc + 1) * 16, x[(cc + 1) & 1]);
+                        uint32_t o[8];
+                        if (cc * 16 < left) {
+#pragma unroll
+                            for (int e = 0; e < 8; ++e) {
+                                const float2 xe = make_float2(x[cc & 1][2 * e], x[cc & 1][2 * e + 1]);
+                                float2 wv;
+                                if (EXACT) wv = angular_weight2(xe);
+                                if (SPARSE) {
+                                    const float2 y = make_float2(__saturatef(fmaf(xe.x, 0.5f, 0.5f)), __saturatef(fmaf(xe.y, 0.5f, 0.5f)));
+                                    if (!EXACT) wv = ffma2(y, dup2(2.0f * kInvPi), dup2(0.5f - kInvPi));   // 1/2 + x / pi
+                                    const float2 a = ffma2(y, dup2(2.0f * kLog2e), dup2(ebias));
+                                    const float px = exp2_approx(a.x), py = exp2_approx(a.y);
+                                    wv = fadd2(wv, make_float2(px > prm.sparse_eps ? px : 0.f, py > prm.sparse_eps ? py : 0.f));
+                                }
+                                o[e] = pack_bf16x2(wv.x, wv.y);
+                            }
+                        } else {
+#pragma unroll
+                            for (int e = 0; e < 8; ++e) o[e] = 0u;   // keys beyond the plane: finite, times v = 0
+                        }
+                        tmem_st8(cb + cc * 8, o);   // over cosines that this thread has already read
+                    }
+                    tmem_st_wait();
+                    tcgen05_fence_before_sync();
+                }
+                mbar_arrive(&p_full[b]);
+                if (jt < T - 1) skip(im.slots);
+            }
+            skip(im.slots - slot);   // to the first step of the next item
+        }
+    } else {
+        // ---- convolution of the item's queries, then their output rows ----
+        const int cw = warp - 24, slot = cw >> 2, quarter = warp & 3;
+        constexpr int R = KS / 2, SEG = 4;
+        uint32_t* w_s = reinterpret_cast<uint32_t*>(smem + kOffW) + lane;
+        float2 bias2 = dup2(0.f);
+        int prev_head = -1, o_uses = 0;
+        bool ok = true;
+        const int W = prm.gridW, segs = (W + SEG - 1) / SEG;
+        for (int i = 0; i < my_items; ++i) {
+            const Item im = item_of(i);
+            const int t_end = min(N, im.t0 + im.slots * kTile);
+            const int head = (prm.head0 + im.bh) % prm.H;
+            if (head != prev_head) {
+                prev_head = head;
+                const unsigned short* w0 = reinterpret_cast<const unsigned short*>(prm.w) + (size_t)(head * kD + 2 * lane) * (KS * KS);
+                for (int e = cw; e < KS * KS; e += kConvThreads / 32)
+                    w_s[e * 32] = (uint32_t)__ldg(w0 + e) | ((uint32_t)__ldg(w0 + KS * KS + e) << 16);
+                if (prm.bias) {
+                    const uint32_t bw = __ldg(reinterpret_cast<const uint32_t*>(prm.bias + head * kD) + lane);
+                    bias2 = make_float2(bf16lo(bw), bf16hi(bw));
+                }
+                named_barrier_sync(1, kConvThreads);
+            }
+            const __nv_bfloat16* vp = prm.v + plane_offset(prm.lv, im.bh, prm.hdiv) + 2 * lane;
+            const int y_first = im.t0 / W, n_units = ((t_end - 1) / W - y_first + 1) * segs;
+            for (int u = cw; u < n_units; u += kConvThreads / 32) {
+                const int y = y_first + u / segs, x0 = (u % segs) * SEG;
+                const int tl = y * W + x0 - im.t0;                        // first token of the unit, within the item
+                if (tl + SEG <= 0 || y * W + x0 >= t_end) continue;
+                uint32_t raw[KS][SEG + KS - 1];
+#pragma unroll
+                for (int dy = 0; dy < KS; ++dy) {
+                    const int yy = y + dy - R;
+                    const bool rv = (unsigned)yy < (unsigned)prm.gridH;
+                    const __nv_bfloat16* vr = vp + (long long)(yy * W + x0 - R) * prm.lv.token;
+#pragma unroll
+                    for (int c = 0; c < SEG + KS - 1; ++c) {
+                        raw[dy][c] = ldg_or_zero(vr, rv && (unsigned)(x0 + c - R) < (unsigned)W);
+                        asm volatile("add.s64 %0, %0, %1;" : "+l"(vr) : "l"(prm.lv.token * 2));   // no table of offsets
+                    }
+                }
+                float2 acc[SEG];
+#pragma unroll
+                for (int j = 0; j < SEG; ++j) acc[j] = bias2;
+#pragma unroll
+                for (int dy = 0; dy < KS; ++dy) {
+                    float2 win[SEG + KS - 1];
+#pragma unroll
+                    for (int c = 0; c < SEG + KS - 1; ++c) win[c] = make_float2(bf16lo(raw[dy][c]), bf16hi(raw[dy][c]));
+#pragma unroll
+                    for (int dx = 0; dx < KS; ++dx) {
+                        const uint32_t fw = w_s[(dy * KS + dx) * 32];
+                        const float2 f = make_float2(bf16lo(fw), bf16hi(fw));
+#pragma unroll
+                        for (int j = 0; j < SEG; ++j) acc[j] = ffma2(f, win[j + dx], acc[j]);
+                    }
+                }
+#pragma unroll
+                for (int j = 0; j < SEG; ++j)
+                    if (x0 + j < W && tl + j >= 0 && tl + j < 2 * kTile)
+                        *reinterpret_cast<float2*>(stg + (tl + j) * kStgStride + lane * 8) = acc[j];
+            }
+            named_barrier_sync(1, kConvThreads);   // the item's convolution is in shared memory
+            if (slot < im.slots) {
+                ok = ok && warp_wait(&o_full[slot], o_uses & 1);
+                ++o_uses;
+                if (ok) {
+                    tcgen05_fence_after_sync();
+                    const uint32_t o_base = tmem + ((uint32_t)(quarter * 32) << 16) + kColO + slot * kD;
+                    uint8_t* srow = stg + (slot * kTile + quarter * 32 + lane) * kStgStride;
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {   // 16 channels: fp32 read at 64 c, bf16 written behind it at 32 c
+                        float a[16];
+                        tmem_ld16(o_base + c * 16, a);
+                        tmem_ld_wait();
+                        uint4 pk[2];
+#pragma unroll
+                        for (int hf = 0; hf < 2; ++hf) {
+                            const float4 s0 = *reinterpret_cast<const float4*>(srow + c * 64 + hf * 32);
+                            const float4 s1 = *reinterpret_cast<const float4*>(srow + c * 64 + hf * 32 + 16);
+                            pk[hf].x = pack_bf16x2(a[8 * hf + 0] + s0.x, a[8 * hf + 1] + s0.y);
+                            pk[hf].y = pack_bf16x2(a[8 * hf + 2] + s0.z, a[8 * hf + 3] + s0.w);
+                            pk[hf].z = pack_bf16x2(a[8 * hf + 4] + s1.x, a[8 * hf + 5] + s1.y);
+                            pk[hf].w = pack_bf16x2(a[8 * hf + 6] + s1.z, a[8 * hf + 7] + s1.w);
+                        }
+                        *reinterpret_cast<uint4*>(srow + c * 32) = pk[0];
+                        *reinterpret_cast<uint4*>(srow + c * 32 + 16) = pk[1];
+                    }
+                    tcgen05_fence_before_sync();
+                    mbar_arrive(&o_free[slot]);
+                    __syncwarp();
+                    __nv_bfloat16* op = prm.out + plane_offset(prm.lo, im.bh, prm.hdiv) + (lane & 7) * 8;
+#pragma unroll
+                    for (int it = 0; it < 8; ++it) {   // four whole 128-byte rows per instruction
+                        const int r = slot * kTile + quarter * 32 + it * 4 + (lane >> 3);
+                        const uint4 val = *reinterpret_cast<const uint4*>(stg + r * kStgStride + (lane & 7) * 16);
+                        if (im.t0 + r < N) *reinterpret_cast<uint4*>(op + (long long)(im.t0 + r) * prm.lo.token) = val;
                     }
                 }
             }
+            named_barrier_sync(1, kConvThreads);   // the staging rows may be overwritten
         }
     }
     tcgen05_fence_before_sync();
@@ -392,10 +643,17 @@ cudaError_t launch_quad_ks(const Problem& p, unsigned* status, cudaStream_t st) 
     prm.w = static_cast<const __nv_bfloat16*>(p.w);
     prm.bias = static_cast<const __nv_bfloat16*>(p.bias);
     prm.lv = p.lv; prm.lo = p.lo;
-    prm.hdiv = p.hdiv; prm.H = p.H; prm.head0 = p.head0; prm.BH = p.BH; prm.N = p.N;
+    prm.hdiv = p.hdiv; prm.H = p.H; prm.head0 = p.head0; prm.N = p.N;
     prm.gridH = p.gridH; prm.gridW = p.gridW;
-    prm.q_tiles = (p.N + kTile - 1) / kTile; prm.k_tiles = prm.q_tiles;
-    prm.n_items = p.BH * prm.q_tiles;
+    // Two query tiles per item share the key tiles and keep both halves of the weight warps busy, but an item of one tile
+    // takes about 0.6 of its time: one tile each when that fills the multiprocessors in fewer rounds.
+    const int sms = device_sm_count();
+    const int q_tiles = (p.N + kTile - 1) / kTile;
+    const long long one = (long long)p.BH * q_tiles, two = (long long)p.BH * ((q_tiles + 1) / 2);
+    prm.slots = ((one + sms - 1) / sms) * 3 < ((two + sms - 1) / sms) * 5 ? 1 : 2;
+    prm.groups = (q_tiles + prm.slots - 1) / prm.slots;
+    prm.k_tiles = q_tiles;
+    prm.n_items = p.BH * prm.groups;
     prm.eps2 = p.eps2; prm.status = status;
     prm.sparse_eps = p.sparse_eps;
     static PerDevice opt_in;
@@ -403,7 +661,6 @@ cudaError_t launch_quad_ks(const Problem& p, unsigned* status, cudaStream_t st) 
         const cudaError_t e = opt_in_smem(tc_quad_kernel<KS, SPARSE, EXACT>, kSmem, opt_in);
         if (e != cudaSuccess) return e;
     }
-    const int sms = device_sm_count();
     const int grid = prm.n_items < sms ? prm.n_items : sms;
     tc_quad_kernel<KS, SPARSE, EXACT><<<(unsigned)grid, kThreads, kSmem, st>>>(tmQ, tmK, tmV, prm);
     return cudaGetLastError();
