@@ -171,32 +171,31 @@ tc_apply_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            constexpr uint32_t idesc = umma_idesc_bf16(128, kAccN, false, true);
-            const uint32_t s_addr = smem_u32(S_s);
-            const uint32_t lbo = RN ? smem_u32(S2_s) - s_addr : 0;     // to the operand's second 64-wide block
-            int prev_bh = -1, seg = 0;
-            PatchWalk pw(g_begin, prm.tilesX, prm.tilesY);
-            for (int it = 0; it < my_tiles; ++it, pw.step(prm.tilesX, prm.tilesY)) {
-                const int s = it % NS, use = it / NS, b = it & 1, ub = it >> 1;
-                const int bh = pw.bh;
-                if (bh != prev_bh) {
-                    if (!mbar_wait(s_ready, seg & 1, abort_flag, prm.status, kBit)) break;
-                    ++seg; prev_bh = bh;
-                }
-                if (!mbar_wait(&full[s], use & 1, abort_flag, prm.status, kBit)) break;
-                if (ub > 0 && !mbar_wait(&buf_free[b], (ub - 1) & 1, abort_flag, prm.status, kBit)) break;
-                tcgen05_fence_after_sync();
-                const uint32_t q_addr = smem_u32(stages + s * G::kStage);
+        // the whole warp walks through the patches, one elected lane issues
+        constexpr uint32_t idesc = umma_idesc_bf16(128, kAccN, false, true);
+        const uint32_t s_addr = smem_u32(S_s);
+        const uint32_t s_low = desc_low(s_addr, RN ? smem_u32(S2_s) - s_addr : 0);   // lbo: to the operand's second 64-wide block
+        int prev_bh = -1, seg = 0;
+        PatchWalk pw(g_begin, prm.tilesX, prm.tilesY);
+        for (int it = 0; it < my_tiles; ++it, pw.step(prm.tilesX, prm.tilesY)) {
+            const int s = it % NS, use = it / NS, b = it & 1, ub = it >> 1;
+            const int bh = pw.bh;
+            if (bh != prev_bh) {
+                if (!mbar_wait_warp(s_ready, seg & 1, abort_flag, prm.status, kBit)) break;
+                ++seg; prev_bh = bh;
+            }
+            if (!mbar_wait_warp(&full[s], use & 1, abort_flag, prm.status, kBit)) break;
+            if (ub > 0 && !mbar_wait_warp(&buf_free[b], (ub - 1) & 1, abort_flag, prm.status, kBit)) break;
+            tcgen05_fence_after_sync();
+            if (elect_one()) {
+                const uint32_t q_low = desc_low(smem_u32(stages + s * G::kStage));   // K-major rows of 128 B
 #pragma unroll
-                for (int k = 0; k < kD / 16; ++k) {
-                    const uint64_t a = umma_desc_sw128(q_addr + k * 32, 0, 1024);        // K-major rows of 128 B
-                    const uint64_t bd = umma_desc_sw128(s_addr + k * 2048, lbo, 1024);   // N-major, 16 K-rows per step
-                    umma_bf16(tmem + b * kAcc, a, bd, idesc, k != 0);
-                }
+                for (int k = 0; k < kD / 16; ++k)   // the operand is N-major, 16 K-rows per step
+                    umma_bf16_low(tmem + b * kAcc, q_low + k * 2, s_low + k * (2048u >> 4), idesc, k != 0);
                 umma_commit(&acc_full[b]);
                 umma_commit(&empty[s]);  // the same UMMAs have finished reading the Q patch
             }
+            __syncwarp();
         }
     } else if (warp < 2 + kEpiWarps) {
         // ------- epilogue: thread = (token of the patch, half of the channels) -------

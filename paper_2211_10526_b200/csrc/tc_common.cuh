@@ -76,7 +76,7 @@ __device__ __forceinline__ bool mbar_poll(uint64_t* bar, uint32_t parity) {
 // thread of the CTA has already given up; the caller then leaves its loop for the common exit.
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
                                           unsigned* status, unsigned bit, unsigned long long limit_ns = kWaitLimitNs) {
-    if (mbar_try_wait(bar, parity)) return true;
+    if (mbar_poll(bar, parity)) return true;
     const unsigned long long t0 = global_ns();
     uint32_t spins = 0;
     while (true) {
@@ -90,6 +90,12 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
             }
         }
     }
+}
+
+// The same for a converged warp; the result is the same in every lane.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, volatile int* abort_flag, unsigned* status,
+                                               unsigned bit) {
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, status, bit));
 }
 
 // ---- fences ---------------------------------------------------------------------------
@@ -292,6 +298,22 @@ __device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t a_desc, uint
         "setp.ne.b32 p, %4, 0;\n\t"
         "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
         ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+// The same with the descriptors given by their low words.  Every operand of these kernels has a 128-byte swizzle and 1024
+// bytes between groups of eight rows, so the high word is a constant and stepping along an operand is one addition.
+constexpr uint32_t kDescHigh = (1024u >> 4) | (1u << 14) | (2u << 29);   // bits 32..63 of umma_desc_sw128(.., .., 1024)
+__device__ __forceinline__ uint32_t desc_low(uint32_t smem_addr, uint32_t lbo_bytes = 0) {
+    return ((smem_addr >> 4) & 0x3fffu) | (((lbo_bytes >> 4) & 0x3fffu) << 16);
+}
+__device__ __forceinline__ void umma_bf16_low(uint32_t d_tmem, uint32_t a_low, uint32_t b_low, uint32_t idesc,
+                                              uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
+        "setp.ne.b32 p, %5, 0;\n\t"
+        "mov.b64 da, {%1, %4};\n\tmov.b64 db, {%2, %4};\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %3, p;\n\t}"
+        ::"r"(d_tmem), "r"(a_low), "r"(b_low), "r"(idesc), "r"(kDescHigh), "r"(accumulate)
         : "memory");
 }
 // All UMMAs issued so far by this thread arrive on `bar` when they have completed.

@@ -157,37 +157,48 @@ tc_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        {   // the whole warp walks through the planes, one elected lane issues
             constexpr uint32_t idesc_state = umma_idesc_bf16(128, kD, true, true);
             constexpr uint32_t idesc_apply = umma_idesc_bf16(128, kD, false, true);
             const uint32_t k_addr = smem_u32(K_s), v_addr = smem_u32(V_s), q_addr = smem_u32(Q_s);
             const uint32_t s_addr = smem_u32(S_s), ones_addr = smem_u32(ones);
             for (int it = 0; it < n_planes; ++it) {
                 const uint32_t ph = it & 1;
-                if (!mbar_wait(k_scaled, ph, abort_flag, prm.status, kBit)) break;
-                if (!mbar_wait(v_full, ph, abort_flag, prm.status, kBit)) break;
+                if (!mbar_wait_warp(v_full, ph, abort_flag, prm.status, kBit)) break;
                 // the previous plane's output accumulators share TMEM columns with this plane's state
-                if (it > 0 && !mbar_wait(tm_free, (it - 1) & 1, abort_flag, prm.status, kBit)) break;
+                if (it > 0 && !mbar_wait_warp(tm_free, (it - 1) & 1, abort_flag, prm.status, kBit)) break;
+                if (!mbar_wait_warp(k_scaled, ph, abort_flag, prm.status, kBit)) break;
                 tcgen05_fence_after_sync();
-                for (int t = 0; t < tiles; ++t) {
+                if (elect_one()) {
+                    // A: stepping 16 tokens adds to the address of K and takes the same off the distance to the constant block
+                    constexpr uint32_t kStep = (2048u >> 4) - ((2048u >> 4) << 16);
+                    const uint32_t a = desc_low(k_addr, ones_addr - k_addr), b = desc_low(v_addr);
 #pragma unroll
-                    for (int j = 0; j < kTile / 16; ++j) {  // one UMMA per 16 tokens (K = 16)
-                        const uint32_t a0 = k_addr + t * kTileBytes + j * 2048, b0 = v_addr + t * kTileBytes + j * 2048;
-                        umma_bf16(tmem, umma_desc_sw128(a0, ones_addr - a0, 1024), umma_desc_sw128(b0, 0, 1024),
-                                  idesc_state, (t | j) != 0);
+                    for (int j = 0; j < kTile / 16; ++j)  // one UMMA per 16 tokens (K = 16)
+                        umma_bf16_low(tmem, a + j * kStep, b + j * (2048u >> 4), idesc_state, j != 0);
+                    if (tiles > 1) {
+#pragma unroll
+                        for (int j = kTile / 16; j < 2 * kTile / 16; ++j)
+                            umma_bf16_low(tmem, a + j * kStep, b + j * (2048u >> 4), idesc_state, 1u);
                     }
+                    umma_commit(s_done);
                 }
-                umma_commit(s_done);
-                if (!mbar_wait(sp_ready, ph, abort_flag, prm.status, kBit)) break;
-                if (!mbar_wait(q_full, ph, abort_flag, prm.status, kBit)) break;
+                __syncwarp();
+                if (!mbar_wait_warp(q_full, ph, abort_flag, prm.status, kBit)) break;
+                if (!mbar_wait_warp(sp_ready, ph, abort_flag, prm.status, kBit)) break;
                 tcgen05_fence_after_sync();
-                for (int t = 0; t < tiles; ++t) {
+                if (elect_one()) {
+                    const uint32_t q = desc_low(q_addr), sl = desc_low(s_addr);
 #pragma unroll
-                    for (int k = 0; k < kD / 16; ++k)
-                        umma_bf16(tmem + t * kD, umma_desc_sw128(q_addr + t * kTileBytes + k * 32, 0, 1024),
-                                  umma_desc_sw128(s_addr + k * 2048, 0, 1024), idesc_apply, k != 0);
+                    for (int k = 0; k < kD / 16; ++k) umma_bf16_low(tmem, q + k * 2, sl + k * (2048u >> 4), idesc_apply, k != 0);
+                    if (tiles > 1) {
+#pragma unroll
+                        for (int k = 0; k < kD / 16; ++k)
+                            umma_bf16_low(tmem + kD, q + (kTileBytes >> 4) + k * 2, sl + k * (2048u >> 4), idesc_apply, k != 0);
+                    }
+                    umma_commit(o_done);
                 }
-                umma_commit(o_done);
+                __syncwarp();
             }
         }
     } else {

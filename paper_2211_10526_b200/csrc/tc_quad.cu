@@ -67,20 +67,6 @@ struct QuadParams {
     float sparse_eps;            // threshold of the mask (sparse sweeps only)
 };
 
-// The descriptors of all operands here (128-byte swizzle, 1024 bytes between groups of eight rows) differ in their low
-// word only, so an UMMA costs its issuer one addition for each.
-constexpr uint32_t kDescHigh = (1024u >> 4) | (1u << 14) | (2u << 29);   // bits 32..63 of umma_desc_sw128(.., 0, 1024)
-__device__ __forceinline__ uint32_t desc_low(const void* smem_ptr) { return smem_u32(smem_ptr) >> 4; }
-template <bool kAccumulate>
-__device__ __forceinline__ void umma_ss(uint32_t d_tmem, uint32_t a_low, uint32_t b_low, uint32_t idesc) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
-        "setp.ne.b32 p, %5, 0;\n\t"
-        "mov.b64 da, {%1, %4};\n\tmov.b64 db, {%2, %4};\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %3, p;\n\t}"
-        ::"r"(d_tmem), "r"(a_low), "r"(b_low), "r"(idesc), "r"(kDescHigh), "n"(kAccumulate ? 1 : 0)
-        : "memory");
-}
 // D[tmem] (+)= A[tmem] * B[smem]: row i of A in lane i, two bf16 of the contracted index per 32-bit column.
 __device__ __forceinline__ void umma_ts(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_low, uint32_t idesc, uint32_t accumulate) {
     asm volatile(
@@ -192,7 +178,7 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
         return {bh, t0, min(prm.slots, (N - t0 + kTile - 1) / kTile)};
     };
     auto warp_wait = [&](uint64_t* bar, uint32_t parity) -> bool {
-        return __all_sync(0xffffffffu, mbar_poll(bar, parity) || mbar_wait(bar, parity, abort_flag, prm.status, kBit));
+        return mbar_wait_warp(bar, parity, abort_flag, prm.status, kBit);
     };
 
     if (tid == 0) {
@@ -275,7 +261,7 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     } else if (warp == 1) {
         // ---- cosines: the whole warp walks through the schedule, one elected lane issues ----
         constexpr uint32_t idesc_c = umma_idesc_bf16(kTile, kTile, false, false);   // Q^ (K-major) x K^ (K-major)
-        const uint32_t q_low = desc_low(Q_s), k_low = desc_low(K_s);
+        const uint32_t q_low = desc_low(smem_u32(Q_s)), k_low = desc_low(smem_u32(K_s));
         uint32_t pv_pending = 0, rd_pending = 0;   // bit b: buffer b was last handed to the second contraction / to a first sweep
         uint32_t pv_parity = 0, rd_parity = 0;     // bit b: parity of the next completion of pv_done[b] / r_done[b]
         int b = 0, ks = 0;                         // next buffer and K stage
@@ -305,10 +291,10 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                     if (elect_one()) {
                         const uint32_t d = tmem + b * kTile, a = q_low + (2 * (i & 1) + s) * (kTileBytes >> 4);
                         const uint32_t k = k_low + ks * (kTileBytes >> 4);
-                        umma_ss<false>(d, a, k, idesc_c);
-                        umma_ss<true>(d, a + 2, k + 2, idesc_c);
-                        umma_ss<true>(d, a + 4, k + 4, idesc_c);
-                        umma_ss<true>(d, a + 6, k + 6, idesc_c);
+                        umma_bf16_low(d, a, k, idesc_c, 0u);
+                        umma_bf16_low(d, a + 2, k + 2, idesc_c, 1u);
+                        umma_bf16_low(d, a + 4, k + 4, idesc_c, 1u);
+                        umma_bf16_low(d, a + 6, k + 6, idesc_c, 1u);
                         umma_commit(&c_full[s * kCBufs + b]);
                         if (s == slots - 1) {
                             if (last_sweep || !resident) umma_commit(&k_empty[ks]);
@@ -324,7 +310,7 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     } else if (warp == 2) {
         // ---- weighted sums ----
         constexpr uint32_t idesc_o = umma_idesc_bf16(kTile, kD, false, true);       // W (TMEM) x V (N-major)
-        const uint32_t v_low = desc_low(V_s);
+        const uint32_t v_low = desc_low(smem_u32(V_s));
         int b = 0, vs = 0;
         uint32_t p_parity = 0, v_par = 0, o_used = 0, o_parity = 0;
         bool ok = true;

@@ -133,30 +133,33 @@ tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            constexpr uint32_t idesc = umma_idesc_bf16(128, kAcc, true, true);
-            const uint32_t ones_addr = smem_u32(ones);
-            bool ok = true;
-            int gt = 0;  // tiles issued so far, over all items
-            for (int item = 0; item < n_items && ok; ++item) {
-                const int buf = item & 1;
-                if (item >= 2) ok = mbar_wait(&acc_free[buf], ((item >> 1) - 1) & 1, abort_flag, status, kStatusStateTimeout);
-                for (int it = 0; it < n_tiles && ok; ++it, ++gt) {
-                    const int s = gt % kStages, use = gt / kStages;
-                    ok = mbar_wait(&scaled[s], use & 1, abort_flag, status, kStatusStateTimeout);
-                    if (!ok) break;
-                    tcgen05_fence_after_sync();
+        // the whole warp walks through the tiles, one elected lane issues
+        constexpr uint32_t idesc = umma_idesc_bf16(128, kAcc, true, true);
+        const uint32_t ones_addr = smem_u32(ones);
+        // A: 128 bytes of K per token and, lbo bytes on, the constant block; stepping to the next 16 tokens adds to the
+        // address and takes the same off the distance
+        constexpr uint32_t kStep = (2048u >> 4) - ((2048u >> 4) << 16);
+        bool ok = true;
+        int s = 0;
+        uint32_t par = 0;
+        for (int item = 0; item < n_items && ok; ++item) {
+            const int buf = item & 1;
+            if (item >= 2) ok = mbar_wait_warp(&acc_free[buf], ((item >> 1) - 1) & 1, abort_flag, status, kStatusStateTimeout);
+            for (int it = 0; it < n_tiles && ok; ++it) {
+                ok = mbar_wait_warp(&scaled[s], par, abort_flag, status, kStatusStateTimeout);
+                if (!ok) break;
+                tcgen05_fence_after_sync();
+                if (elect_one()) {
                     const uint32_t ka = smem_u32(smem + s * kStageBytes), va = ka + kTileBytes;
+                    const uint32_t a = desc_low(ka, ones_addr - ka), b = desc_low(va, RN ? ones_addr - va : 0);
 #pragma unroll
-                    for (int j = 0; j < kTile / 16; ++j) {  // one UMMA per 16 tokens (K = 16)
-                        const uint32_t a0 = ka + j * 2048, b0 = va + j * 2048;
-                        const uint64_t a = umma_desc_sw128(a0, ones_addr - a0, 1024);
-                        const uint64_t b = umma_desc_sw128(b0, RN ? ones_addr - b0 : 0, 1024);
-                        umma_bf16(tmem + buf * kAcc, a, b, idesc, (it | j) != 0);
-                    }
+                    for (int j = 0; j < kTile / 16; ++j)  // one UMMA per 16 tokens (K = 16)
+                        umma_bf16_low(tmem + buf * kAcc, a + j * kStep, b + j * (RN ? kStep : (2048u >> 4)), idesc, (it | j) != 0);
                     umma_commit(&empty[s]);
+                    if (it == n_tiles - 1) umma_commit(&accum[buf]);
                 }
-                if (ok) umma_commit(&accum[buf]);
+                __syncwarp();
+                if (++s == kStages) { s = 0; par ^= 1; }
             }
         }
     } else {
