@@ -66,7 +66,7 @@ enum {
     CASTLING_PATH_AUTO = 0,
     CASTLING_PATH_SIMT = 1,   /* CUDA-core FMA kernels: every dtype, d and ksize supported   */
     CASTLING_PATH_TENSOR = 2  /* tcgen05/TMEM + TMA kernels: bf16, ksize 3 or 5, d = 64, or   */
-                              /* d = 32 packed two tokens or two heads to a 128-byte row      */
+                              /* d = 32 with rows that lie next to one another in memory      */
 };
 
 typedef struct {
@@ -167,10 +167,10 @@ typedef struct {
  *   everything else as for castling_attn_forward.
  *
  * The tensor-core kernels read such layouts directly through strided TMA descriptors: width-64
- * heads with any strides; width-32 heads when a 128-byte row holds either two adjacent tokens of one
- * head (contiguous tokens, even gridW and N) or the same token of two adjacent heads (head stride 32,
- * even H, as in token-major [B,N,H,32]).  Everything else, and any layout a descriptor cannot express,
- * runs on the CUDA-core kernels.
+ * heads with any strides; width-32 heads whose tokens (token stride 32) or heads (head stride 32, as in
+ * token-major [B,N,H,32]) lie next to one another, except small calls whose 64-byte rows do not fill 128-byte
+ * ones (odd gridW, N or H).  Everything else, and any layout a descriptor cannot express, runs on the CUDA-core
+ * kernels.
  * Errors: INVALID_ARG, UNSUPPORTED, ALIGNMENT, OOM, CUDA.
  */
 CASTLING_API int castling_attn_forward_strided(castling_attn_t* handle,

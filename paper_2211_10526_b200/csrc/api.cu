@@ -56,12 +56,7 @@ size_t workspace_words(int BH, int N, int d, bool bf16) {
         if (Pt > P) P = Pt;
         if (castling::tc::kStateWordsRownorm > words) words = castling::tc::kStateWordsRownorm;
     }
-    size_t slots = (size_t)BH * (P > 1 ? P : 0);  // partial states behind the BH final ones
-    if (bf16 && d == 32 && BH % 2 == 0) {
-        // two width-32 heads side by side (token-major layouts): BH / 2 planes of N rows each
-        const int Pp = castling::tc::choose_splits(BH / 2, N);
-        if (Pp > 1 && (size_t)(BH / 2) * Pp > slots) slots = (size_t)(BH / 2) * Pp;
-    }
+    const size_t slots = (size_t)BH * (P > 1 ? P : 0);  // partial states behind the BH final ones
     size_t behind = slots * words;  // what follows the BH final states
     if (bf16 && (d == 64 || d == 32)) {  // the one-kernel forward keeps its per-plane operand blocks there
         const size_t r = castling::tc::pipe_ready_words(BH);
@@ -258,8 +253,7 @@ int run_device(castling_attn* h, const Problem& p, cudaStream_t stream) {
     if (use_tensor) {
         rc = ensure_counters(h, p.BH);
         if (rc != CASTLING_OK) return rc;
-        e = castling::tc::forward(p, state, partial, h->counters, castling::tc::choose_splits(p.BH, castling::tc::rows_per_head(p.N, p.d)),
-                                  reinterpret_cast<unsigned*>(h->ws), stream, &launches, &h->timer);
+        e = castling::tc::forward(p, state, partial, h->counters, reinterpret_cast<unsigned*>(h->ws), stream, &launches, &h->timer);
     } else {
         e = castling::simt_forward(p, state, partial, castling::simt_choose_splits(p.BH, p.N), stream, &launches,
                                    &h->timer);

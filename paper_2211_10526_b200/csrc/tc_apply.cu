@@ -1,5 +1,4 @@
-// Apply kernel of the tensor-core path (bf16; width-64 heads, or width-32 heads packed two to a 128-byte
-// row: see the modes at the kernel template):
+// Apply kernel of the tensor-core path (bf16, width-64 heads; width-32 heads: tc_apply32.cu):
 //     out_t = (1/pi) q^_t S + 1/2 s + bias + DWConv(V)_t                         (Eq. 9)
 // Persistent CTAs walk a contiguous range of 8 x 16-token patches of the token grid.  Per patch
 //   warp 0      TMA: the raw Q patch (128 rows of 128 B, 128-byte swizzle) and the V patch with
@@ -31,17 +30,14 @@ constexpr int kEpiWarps = 8;                   // two warps per TMEM lane quarte
 constexpr int kEpiThreads = kEpiWarps * 32;
 constexpr int kTmemCols = 128;              // two 64-column accumulators
 
-// PAIR = true serves head width 32: a 128-byte row holds two horizontally adjacent tokens, so a
-// "column" of the patch is a token pair and the 8 x 16-column patch covers 8 x 32 tokens.
-template <int KS, bool PAIR> struct Geo {
+template <int KS> struct Geo {
     // conv warps: each takes kConvRows patch rows x 8 columns.  3x3: 8 warps of 2 rows; 5x5: 4 warps of
     // 4 rows (fewer redundant window loads, and the larger window fits the registers of 448 threads)
     static constexpr int kConvRows = (KS == 3) ? 2 : 4;
     static constexpr int kConvWarps = 2 * kTY / kConvRows, kConvThreads = kConvWarps * 32;
     static constexpr int kThreads = 64 + kEpiThreads + kConvThreads;
     static constexpr int R = KS / 2;
-    static constexpr int HC = PAIR ? (R + 1) / 2 : R;   // halo columns on each side
-    static constexpr int HY = kTY + 2 * R, HX = kTX + 2 * HC;
+    static constexpr int HY = kTY + 2 * R, HX = kTX + 2 * R;
     static constexpr int kVBytes = HY * HX * kD * 2;
     static constexpr int kStage = ((kQBytes + kVBytes + 1023) / 1024) * 1024;
     static constexpr int kStages = (KS == 3) ? 3 : 2;
@@ -58,12 +54,11 @@ template <int KS, bool PAIR> struct Geo {
 };
 
 struct ApplyParams {
-    const float* state;            // [BH][P][64*64 + 64] raw sums of the P token splits
-    int P;
+    const float* state;            // [BH][64*64 + 64 (+ 64)]
     const __nv_bfloat16* w;        // [H*d][KS][KS]
     const __nv_bfloat16* bias;     // [H*d] or nullptr
     int flat;                      // the planes have one uniform stride: the tensor maps are 4-D, [.., plane]
-    int H, head0, bh0, hdiv, tilesX, tilesY, n_tiles;  // tiles of (b,h) in [bh0, bh0 + n_tiles / (tilesX*tilesY))
+    int H, head0, hdiv, tilesX, tilesY, n_tiles;
     float eps2;
     unsigned* status;
     int v_row0;                    // V holds more grid rows than the plane has (a band of a sharded sequence with its
@@ -86,18 +81,14 @@ struct PatchWalk {
     }
 };
 
-// MODE 0: width-64 heads; 1: width-32 heads, two adjacent tokens per 128-byte row (the PAIR geometry);
-// 2: two width-32 heads side by side in the one-token-per-row geometry (block-diagonal state).
 // RN: row-sum normalisation (Eq. 3's denominator on the kept kernel of Eq. 8).  The state carries sum_n k^_n behind s; the
-// operand gets one or two more columns (sum k^ / pi per head or token of the row), so that column 64 (65) of the
-// accumulator is q . sum k^ / pi; the attention term (acc / ||q|| + 1/2 s) is divided by n_tokens / 2 + that product
+// operand gets one more column (sum k^ / pi), so that column 64 of the accumulator is q . sum k^ / pi; the attention term (acc / ||q|| + 1/2 s) is divided by n_tokens / 2 + that product
 // / ||q|| before the convolution and the bias are added.
-template <int KS, int MODE, bool RN>
-__global__ void __launch_bounds__((Geo<KS, MODE == 1>::kThreads), 1)
+template <int KS, bool RN>
+__global__ void __launch_bounds__(Geo<KS>::kThreads, 1)
 tc_apply_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmV,
                 const __grid_constant__ CUtensorMap tmO, const ApplyParams prm) {
-    constexpr bool PAIR = (MODE == 1), BLOCKDIAG = (MODE == 2);
-    using G = Geo<KS, PAIR>;
+    using G = Geo<KS>;
     constexpr int NS = G::kStages;
     constexpr int kSW = kD * kD + kD + (RN ? kD : 0);   // words of one state
     constexpr int kAcc = RN ? 2 * kD : kD;              // TMEM columns per accumulator
@@ -157,11 +148,11 @@ tc_apply_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                 mbar_expect_tx(&full[s], kQBytes + G::kVBytes);
                 if (prm.flat) {
                     tma_load_4d_hint(qs, &tmQ, &full[s], 0, x0, y0, bh, pol_q);
-                    tma_load_4d(qs + kQBytes, &tmV, &full[s], 0, x0 - G::HC, y0 - G::R + prm.v_row0, bh);
+                    tma_load_4d(qs + kQBytes, &tmV, &full[s], 0, x0 - G::R, y0 - G::R + prm.v_row0, bh);
                 } else {
                     const int pb = bh / prm.hdiv, ph = bh - pb * prm.hdiv;
                     tma_load_5d_hint(qs, &tmQ, &full[s], 0, x0, y0, ph, pb, pol_q);
-                    tma_load_5d(qs + kQBytes, &tmV, &full[s], 0, x0 - G::HC, y0 - G::R + prm.v_row0, ph, pb);
+                    tma_load_5d(qs + kQBytes, &tmV, &full[s], 0, x0 - G::R, y0 - G::R + prm.v_row0, ph, pb);
                 }
                 ++issued;
             }
@@ -213,52 +204,19 @@ tc_apply_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                 // every UMMA that read the previous S' has retired (its acc_full was waited on below)
                 prev_bh = bh;
                 const int i = et >> 2, part = et & 3;  // row i of the operand, 16 columns part*16 ..
-                const float* st = prm.state + (size_t)(prm.bh0 + bh) * prm.P * kSW;
+                const float* st = prm.state + (size_t)bh * kSW;
 #pragma unroll
                 for (int c = 0; c < 2; ++c) {
-                    float4 lo, hi;
-                    if (!PAIR) {
-                        const float4* src = reinterpret_cast<const float4*>(st + i * kD + part * 16);
-                        lo = __ldg(src + 2 * c); hi = __ldg(src + 2 * c + 1);
-                        for (int pp = 1; pp < prm.P; ++pp) {  // fixed order: bitwise reproducible
-                            const float4 l2 = __ldg(src + pp * (kSW / 4) + 2 * c);
-                            const float4 h2 = __ldg(src + pp * (kSW / 4) + 2 * c + 1);
-                            lo.x += l2.x; lo.y += l2.y; lo.z += l2.z; lo.w += l2.w;
-                            hi.x += h2.x; hi.y += h2.y; hi.z += h2.z; hi.w += h2.w;
-                        }
-                        if (BLOCKDIAG && ((i < 32) != (part < 2))) {  // off-diagonal block: the other head's keys
-                            lo = make_float4(0.f, 0.f, 0.f, 0.f); hi = lo;
-                        }
-                    } else {
-                        // operand = blockdiag(S32, S32) with S32 = block(0,0) + block(1,1) of the paired sums
-                        const int col = part * 16 + c * 8;  // first of 8 columns
-                        if ((i < 32) == (col < 32)) {
-                            const int a = i & 31, bcol = col & 31;
-                            const float4* s0 = reinterpret_cast<const float4*>(st + a * kD + bcol);
-                            const float4* s1 = reinterpret_cast<const float4*>(st + (32 + a) * kD + 32 + bcol);
-                            const float4 l0 = __ldg(s0), h0 = __ldg(s0 + 1), l1 = __ldg(s1), h1 = __ldg(s1 + 1);
-                            lo = make_float4(l0.x + l1.x, l0.y + l1.y, l0.z + l1.z, l0.w + l1.w);
-                            hi = make_float4(h0.x + h1.x, h0.y + h1.y, h0.z + h1.z, h0.w + h1.w);
-                        } else {
-                            lo = make_float4(0.f, 0.f, 0.f, 0.f); hi = lo;
-                        }
-                    }
+                    const float4* src = reinterpret_cast<const float4*>(st + i * kD + part * 16);
+                    const float4 lo = __ldg(src + 2 * c), hi = __ldg(src + 2 * c + 1);
                     uint4 o;
                     o.x = pack_bf16x2(lo.x * kInvPi, lo.y * kInvPi); o.y = pack_bf16x2(lo.z * kInvPi, lo.w * kInvPi);
                     o.z = pack_bf16x2(hi.x * kInvPi, hi.y * kInvPi); o.w = pack_bf16x2(hi.z * kInvPi, hi.w * kInvPi);
                     *reinterpret_cast<uint4*>(S_s + i * 128 + (((part * 2 + c) ^ (i & 7)) << 4)) = o;
                     if (RN) {
-                        // second block of the operand: row i (a key feature) holds sum k^[i] / pi in column 0, or, where a
-                        // row carries two tokens or two heads, in the column of its half; the rest is zero
+                        // second block of the operand: row i (a key feature) holds sum k^[i] / pi in column 0; the rest is zero
                         uint4 z = make_uint4(0, 0, 0, 0);
-                        if (part == 0 && c == 0) {
-                            const float* sk = st + kD * kD + kD;
-                            float val;
-                            if (PAIR) val = __ldg(sk + (i & 31)) + __ldg(sk + 32 + (i & 31));   // both token parities
-                            else val = __ldg(sk + i);
-                            const uint32_t hv = pack_bf16x2(val * kInvPi, 0.f) & 0xffffu;
-                            z.x = (MODE != 0 && i >= 32) ? (hv << 16) : hv;
-                        }
+                        if (part == 0 && c == 0) z.x = pack_bf16x2(__ldg(st + kD * kD + kD + i) * kInvPi, 0.f) & 0xffffu;
                         *reinterpret_cast<uint4*>(S2_s + i * 128 + (((part * 2 + c) ^ (i & 7)) << 4)) = z;
                     }
                 }
@@ -299,16 +257,14 @@ tc_apply_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                 float x[16];
                 tmem_ld16(tmem + ((uint32_t)(quarter * 32) << 16) + b * kAcc + kD, x);
                 tmem_ld_wait();
-                qk = (MODE != 0 && half == 1) ? x[1] : x[0];
+                qk = x[0];
             }
             if (!mbar_wait(&conv_full[b], ub & 1, abort_flag, prm.status, kBit)) break;
             // the previous patch's TMA store must have read out_s before it is rewritten; the same
             // barrier makes both halves of every row's sum of squares visible
             if (it > 0 && leader) tma_store_wait_read();
             named_barrier_sync(1, kEpiThreads);
-            const float rq = (PAIR || BLOCKDIAG)
-                                 ? rsqrtf(fmaxf(rq_s[half * kTile + row], prm.eps2))   // half row = one token / one head
-                                 : rsqrtf(fmaxf(rq_s[row] + rq_s[kTile + row], prm.eps2));
+            const float rq = rsqrtf(fmaxf(rq_s[row] + rq_s[kTile + row], prm.eps2));
             const uint8_t* srow = stg + b * kStgBytes + row * kStgStride + half * 128;
             uint8_t* orow = out_s + row * 128;
             if (RN) {
@@ -364,23 +320,9 @@ tc_apply_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
             const int bh = pw.bh;
             if (bh != prev_bh) {
                 prev_bh = bh;
-                // this lane's channel pair: 2*lane of 64 channels, or (PAIR) 2*(lane & 15) of 32 channels
-                // for the token of parity lane >> 4
-                const int gbh = prm.bh0 + bh;
-                const int cp2 = PAIR ? 2 * (lane & 15) : 2 * lane;
-                const int ch = ((prm.head0 + gbh) % prm.H) * (PAIR ? 32 : kD) + cp2;
-                const float* sv = prm.state + (size_t)gbh * prm.P * kSW + kD * kD;
-                float s0, s1;
-                if (PAIR) {  // token sum = sum of the two halves of the paired sums
-                    s0 = __ldg(sv + cp2) + __ldg(sv + 32 + cp2);
-                    s1 = __ldg(sv + cp2 + 1) + __ldg(sv + 32 + cp2 + 1);
-                } else {
-                    s0 = __ldg(sv + cp2); s1 = __ldg(sv + cp2 + 1);
-                    for (int pp = 1; pp < prm.P; ++pp) {
-                        s0 += __ldg(sv + pp * kSW + cp2);
-                        s1 += __ldg(sv + pp * kSW + cp2 + 1);
-                    }
-                }
+                const int ch = ((prm.head0 + bh) % prm.H) * kD + 2 * lane;   // this lane's channel pair
+                const float* sv = prm.state + (size_t)bh * kSW + kD * kD + 2 * lane;
+                const float s0 = __ldg(sv), s1 = __ldg(sv + 1);
                 cinit.x = RN ? 0.f : 0.5f * s0; cinit.y = RN ? 0.f : 0.5f * s1;
                 hs2 = make_float2(0.5f * s0, 0.5f * s1);
                 if (prm.bias) { cinit.x += __bfloat162float(prm.bias[ch]); cinit.y += __bfloat162float(prm.bias[ch + 1]); }
@@ -393,33 +335,24 @@ tc_apply_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
             }
             if (!mbar_wait(&full[s], use & 1, abort_flag, prm.status, kBit)) break;
             if (ub > 0 && !mbar_wait(&buf_free[b], (ub - 1) & 1, abort_flag, prm.status, kBit)) break;
-            // Window of KS tokens per halo row, sliding along x.  Token t (relative to the first token this
-            // lane needs) sits U bytes after token t-1: U = 128, one token per column, or (PAIR) 64.
-            // One output column advances the window by STEP tokens (2 when PAIR: the lane's token keeps
-            // its parity).  Slot of token t in the rotating window: t % KS (t is a compile-time value).
-            constexpr int U = PAIR ? 64 : 128, STEP = PAIR ? 2 : 1;
-            const int tok0 = PAIR ? 2 * (xh * kCX + G::HC) + (lane >> 4) - R : xh * kCX;
-            const uint8_t* vh = stages + s * G::kStage + kQBytes + (RO * cw) * G::HX * 128 + tok0 * U +
-                                (PAIR ? (lane & 15) * 4 : lane * 4);
+            // Window of KS columns per halo row, sliding along x; column x (relative to the first this lane needs) lives in
+            // slot x % KS (compile-time after unrolling).
+            const uint8_t* vh = stages + s * G::kStage + kQBytes + ((RO * cw) * G::HX + xh * kCX) * 128 + lane * 4;
             uint8_t* so = stg + b * kStgBytes + ((RO * cw) * kTX + xh * kCX) * kStgStride + lane * 8;
             float2 win[ROWS][KS];
 #pragma unroll
-            for (int t = 0; t < KS - STEP; ++t)
+            for (int t = 0; t < KS - 1; ++t)
 #pragma unroll
                 for (int r = 0; r < ROWS; ++r) {
-                    const uint32_t wv = *reinterpret_cast<const uint32_t*>(vh + r * G::HX * 128 + t * U);
-                    win[r][t % KS] = make_float2(bf16lo(wv), bf16hi(wv));
+                    const uint32_t wv = *reinterpret_cast<const uint32_t*>(vh + (r * G::HX + t) * 128);
+                    win[r][t] = make_float2(bf16lo(wv), bf16hi(wv));
                 }
 #pragma unroll
             for (int x = 0; x < kCX; ++x) {
 #pragma unroll
-                for (int n = 0; n < STEP; ++n) {
-                    const int t = STEP * x + KS - STEP + n;  // compile-time after unrolling
-#pragma unroll
-                    for (int r = 0; r < ROWS; ++r) {
-                        const uint32_t wv = *reinterpret_cast<const uint32_t*>(vh + r * G::HX * 128 + t * U);
-                        win[r][t % KS] = make_float2(bf16lo(wv), bf16hi(wv));
-                    }
+                for (int r = 0; r < ROWS; ++r) {
+                    const uint32_t wv = *reinterpret_cast<const uint32_t*>(vh + (r * G::HX + x + KS - 1) * 128);
+                    win[r][(x + KS - 1) % KS] = make_float2(bf16lo(wv), bf16hi(wv));
                 }
                 float2 acc[RO];
 #pragma unroll
@@ -430,14 +363,13 @@ tc_apply_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                     for (int dx = 0; dx < KS; ++dx)
 #pragma unroll
                         for (int r = 0; r < RO; ++r)
-                            acc[r] = ffma2(wreg[dy][dx], win[dy + r][(STEP * x + dx) % KS], acc[r]);
+                            acc[r] = ffma2(wreg[dy][dx], win[dy + r][(x + dx) % KS], acc[r]);
 #pragma unroll
                 for (int r = 0; r < RO; ++r) *reinterpret_cast<float2*>(so + (r * kTX + x) * kStgStride) = acc[r];
             }
             if (RN && cw == 0 && xh == 0) {
-                // 1/2 s of the plane this patch belongs to, per column of a 128-byte row, beside the staging buffer
-                const int col = PAIR ? (lane >> 4) * 32 + 2 * (lane & 15) : 2 * lane;
-                *reinterpret_cast<float2*>(hs_s + b * kD + col) = hs2;
+                // 1/2 s of the plane this patch belongs to, beside the staging buffer
+                *reinterpret_cast<float2*>(hs_s + b * kD + 2 * lane) = hs2;
             }
             mbar_arrive(&empty[s]);      // the V patch of this stage is no longer needed
             mbar_arrive(&conv_full[b]);
@@ -448,21 +380,19 @@ tc_apply_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     if (warp == 1) tmem_dealloc(tmem, RN ? 2 * kTmemCols : kTmemCols);
 }
 
-template <int KS, int MODE, bool RN>
-cudaError_t launch_apply_ks(const Problem& p, const float* state, int P, unsigned* status, cudaStream_t st) {
-    constexpr bool PAIR = (MODE == 1);
-    using G = Geo<KS, PAIR>;
+template <int KS, bool RN>
+cudaError_t launch_apply_ks(const Problem& p, const float* state, unsigned* status, cudaStream_t st) {
+    using G = Geo<KS>;
     CUtensorMap tmQ, tmV, tmO;
-    const int cols = PAIR ? p.gridW / 2 : p.gridW;  // 128-byte columns per grid row
     // [64, columns, grid rows, planes per batch step, batch steps]; with a single batch step the last
     // dimension is dropped (a 4-D copy is a little cheaper for the TMA unit than a 5-D one)
     const uint64_t nb = (uint64_t)(p.BH / p.hdiv);
     const int rank = nb > 1 ? 5 : 4;
-    const uint64_t dims[5] = {(uint64_t)kD, (uint64_t)cols, (uint64_t)p.gridH, (uint64_t)p.hdiv, nb};
+    const uint64_t dims[5] = {(uint64_t)kD, (uint64_t)p.gridW, (uint64_t)p.gridH, (uint64_t)p.hdiv, nb};
     const uint32_t box[5] = {kD, kTX, kTY, 1, 1};
     const uint32_t boxv[5] = {kD, (uint32_t)G::HX, (uint32_t)G::HY, 1, 1};
     auto strides = [&](const Layout& l, uint64_t (&s)[4]) {
-        s[0] = (uint64_t)(PAIR ? kD : l.token);          // next column: one token, or (PAIR) two
+        s[0] = (uint64_t)l.token;                        // next column
         s[1] = (uint64_t)(l.token * p.gridW);            // next grid row
         s[2] = (uint64_t)l.head;
         s[3] = (uint64_t)(nb > 1 ? l.batch : l.head * p.hdiv);
@@ -476,23 +406,22 @@ cudaError_t launch_apply_ks(const Problem& p, const float* state, int P, unsigne
     // V may hold more grid rows than the plane (the neighbours' rows of a band of a sharded sequence): rows outside
     // that taller tensor, not outside the band, are the zero padding
     uint64_t dimsv[5] = {dims[0], dims[1], (uint64_t)(p.v_rows > 0 ? p.v_rows : p.gridH), dims[3], dims[4]};
-    if (!make_tensor_map_bf16(&tmQ, qg, rank, dims, sq, box, true) || !make_tensor_map_bf16(&tmO, og, rank, dims, so, box, true) ||
-        !make_tensor_map_bf16(&tmV, vg, rank, dimsv, sv, boxv, false))
+    if (!make_tensor_map_bf16(&tmQ, qg, rank, dims, sq, box, 128) || !make_tensor_map_bf16(&tmO, og, rank, dims, so, box, 128) ||
+        !make_tensor_map_bf16(&tmV, vg, rank, dimsv, sv, boxv, 0))
         return cudaErrorNotSupported;
     ApplyParams prm;
     prm.state = state;
-    prm.P = P;
     prm.w = static_cast<const __nv_bfloat16*>(p.w);
     prm.bias = static_cast<const __nv_bfloat16*>(p.bias);
     prm.flat = (rank == 4) ? 1 : 0;
-    prm.H = p.H; prm.head0 = p.head0; prm.bh0 = 0; prm.hdiv = p.hdiv;
-    prm.tilesX = (cols + kTX - 1) / kTX; prm.tilesY = (p.gridH + kTY - 1) / kTY;
+    prm.H = p.H; prm.head0 = p.head0; prm.hdiv = p.hdiv;
+    prm.tilesX = (p.gridW + kTX - 1) / kTX; prm.tilesY = (p.gridH + kTY - 1) / kTY;
     prm.n_tiles = p.BH * prm.tilesX * prm.tilesY;
     prm.eps2 = p.eps2; prm.status = status; prm.n_tokens = p.N; prm.v_row0 = p.v_rows > 0 ? p.v_row0 : 0;
     constexpr size_t kSmemBytes = RN ? G::kSmemRN : G::kSmem;
     static PerDevice opt_in;  // one per instantiation
     {
-        const cudaError_t e = opt_in_smem(tc_apply_kernel<KS, MODE, RN>, kSmemBytes, opt_in);
+        const cudaError_t e = opt_in_smem(tc_apply_kernel<KS, RN>, kSmemBytes, opt_in);
         if (e != cudaSuccess) return e;
     }
     const int sms = device_sm_count();  // one persistent CTA per multiprocessor
@@ -505,13 +434,14 @@ cudaError_t launch_apply_ks(const Problem& p, const float* state, int P, unsigne
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr; cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, tc_apply_kernel<KS, MODE, RN>, tmQ, tmV, tmO, prm);
+    return cudaLaunchKernelEx(&cfg, tc_apply_kernel<KS, RN>, tmQ, tmV, tmO, prm);
 }
 
 // Output rows of the off-grid leading tokens: out = q^ S / pi + 1/2 s (no convolution, no bias), from the
 // final state the state kernel left in the workspace.  One block of 64 threads per (plane, token), thread =
 // channel.  mode 0: 64-wide heads; 1: token pairs (width 32, the state is the sum of the two diagonal
-// blocks); 2: two width-32 heads side by side (each half of the row is its own head).
+// blocks); 2: two width-32 heads side by side (each half of the row is its own head); 3: width-32 heads with a
+// 32 x 32 state.
 __global__ void __launch_bounds__(64)
 tc_prefix_rows_kernel(const __nv_bfloat16* __restrict__ q, __nv_bfloat16* __restrict__ out,
                       const float* __restrict__ state, Layout lq, Layout lo, int hdiv, int prefix, int mode,
@@ -519,7 +449,7 @@ tc_prefix_rows_kernel(const __nv_bfloat16* __restrict__ q, __nv_bfloat16* __rest
     __shared__ float qs[kD];
     __shared__ float part[2];
     const int plane = blockIdx.x / prefix, t = blockIdx.x % prefix, j = threadIdx.x;
-    const int width = (mode == 1) ? 32 : kD;  // elements of this plane's token rows
+    const int width = (mode & 1) ? 32 : kD;  // elements of this plane's token rows
     const __nv_bfloat16* qrow = q + plane_offset(lq, plane, hdiv) + t * lq.token;
     const float x = (j < width) ? __bfloat162float(qrow[j]) : 0.f;
     qs[j] = x;
@@ -529,14 +459,20 @@ tc_prefix_rows_kernel(const __nv_bfloat16* __restrict__ q, __nv_bfloat16* __rest
     if ((j & 31) == 0) part[j >> 5] = ss;
     __syncthreads();
     if (j >= width) return;
-    const float* st = state + (size_t)plane * (kD * kD + kD + (rownorm ? kD : 0));
-    const float* sk = st + kD * kD + kD;  // row-sum normalisation: sum of the unit key rows (per token parity / head)
+    const int sw = mode == 3 ? 32 : kD;   // width of the state
+    const float* st = state + (size_t)plane * (sw * sw + sw + (rownorm ? sw : 0));
+    const float* sk = st + sw * sw + sw;  // row-sum normalisation: sum of the unit key rows (per token parity / head)
     float nrm2, acc = 0.f, sum, qk = 0.f;
     if (mode == 0) {
         nrm2 = part[0] + part[1];
         for (int i = 0; i < kD; ++i) acc = fmaf(qs[i], st[i * kD + j], acc);
         sum = st[kD * kD + j];
         if (rownorm) for (int i = 0; i < kD; ++i) qk = fmaf(qs[i], sk[i], qk);
+    } else if (mode == 3) {
+        nrm2 = part[0];
+        for (int i = 0; i < 32; ++i) acc = fmaf(qs[i], st[i * 32 + j], acc);
+        sum = st[32 * 32 + j];
+        if (rownorm) for (int i = 0; i < 32; ++i) qk = fmaf(qs[i], sk[i], qk);
     } else if (mode == 1) {
         nrm2 = part[0];
         for (int i = 0; i < 32; ++i) acc = fmaf(qs[i], st[i * kD + j] + st[(32 + i) * kD + 32 + j], acc);
@@ -559,29 +495,17 @@ tc_prefix_rows_kernel(const __nv_bfloat16* __restrict__ q, __nv_bfloat16* __rest
 
 cudaError_t launch_prefix_rows(const Problem& p, const float* state, cudaStream_t st) {
     if (p.prefix <= 0) return cudaSuccess;
-    const int mode = p.d == 32 ? 1 : (p.blockdiag ? 2 : 0);
+    const int mode = p.narrow ? 3 : p.d == 32 ? 1 : (p.blockdiag ? 2 : 0);
     tc_prefix_rows_kernel<<<(unsigned)(p.BH * p.prefix), 64, 0, st>>>(
         static_cast<const __nv_bfloat16*>(p.q), static_cast<__nv_bfloat16*>(p.out), state, p.lq, p.lo, p.hdiv,
         p.prefix, mode, p.eps2, p.rownorm ? 1 : 0, p.N);
     return cudaGetLastError();
 }
 
-namespace {
-template <bool RN>
-cudaError_t launch_apply_rn(const Problem& p, const float* partial, int P, unsigned* status, cudaStream_t st) {
-    if (p.d == 32)
-        return p.ksize == 3 ? launch_apply_ks<3, 1, RN>(p, partial, P, status, st)
-                            : launch_apply_ks<5, 1, RN>(p, partial, P, status, st);
-    if (p.blockdiag)
-        return p.ksize == 3 ? launch_apply_ks<3, 2, RN>(p, partial, P, status, st)
-                            : launch_apply_ks<5, 2, RN>(p, partial, P, status, st);
-    return p.ksize == 3 ? launch_apply_ks<3, 0, RN>(p, partial, P, status, st)
-                        : launch_apply_ks<5, 0, RN>(p, partial, P, status, st);
-}
-}  // namespace
-
-cudaError_t launch_apply(const Problem& p, const float* partial, int P, unsigned* status, cudaStream_t st) {
-    return p.rownorm ? launch_apply_rn<true>(p, partial, P, status, st) : launch_apply_rn<false>(p, partial, P, status, st);
+cudaError_t launch_apply(const Problem& p, const float* state, unsigned* status, cudaStream_t st) {
+    if (p.d == 32) return launch_apply32(p, state, status, st);
+    if (p.ksize == 3) return p.rownorm ? launch_apply_ks<3, true>(p, state, status, st) : launch_apply_ks<3, false>(p, state, status, st);
+    return p.rownorm ? launch_apply_ks<5, true>(p, state, status, st) : launch_apply_ks<5, false>(p, state, status, st);
 }
 
 }  // namespace tc

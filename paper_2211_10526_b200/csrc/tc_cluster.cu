@@ -576,7 +576,7 @@ cudaError_t launch_cluster_ks(const Problem& p, int C, unsigned* status, cudaStr
                                 (uint64_t)(nb > 1 ? p.lk.batch : p.lk.head * p.hdiv)};
         const uint64_t sv[3] = {(uint64_t)(pair ? kD : p.lv.token), (uint64_t)p.lv.head,
                                 (uint64_t)(nb > 1 ? p.lv.batch : p.lv.head * p.hdiv)};
-        if (!make_tensor_map_bf16(&tmK, p.k, 4, dims, sk, box, true) || !make_tensor_map_bf16(&tmVs, p.v, 4, dims, sv, box, true))
+        if (!make_tensor_map_bf16(&tmK, p.k, 4, dims, sk, box, 128) || !make_tensor_map_bf16(&tmVs, p.v, 4, dims, sv, box, 128))
             return cudaErrorNotSupported;
     }
     const int rank = nb > 1 ? 5 : 4;
@@ -592,8 +592,8 @@ cudaError_t launch_cluster_ks(const Problem& p, int C, unsigned* status, cudaStr
         };
         uint64_t sq[4], sv[4], so[4];
         strides(p.lq, sq); strides(p.lv, sv); strides(p.lo, so);
-        if (!make_tensor_map_bf16(&tmQ, p.q, rank, dims, sq, box, true) || !make_tensor_map_bf16(&tmO, p.out, rank, dims, so, box, true) ||
-            !make_tensor_map_bf16(&tmVh, p.v, rank, dims, sv, boxv, false))
+        if (!make_tensor_map_bf16(&tmQ, p.q, rank, dims, sq, box, 128) || !make_tensor_map_bf16(&tmO, p.out, rank, dims, so, box, 128) ||
+            !make_tensor_map_bf16(&tmVh, p.v, rank, dims, sv, boxv, 0))
             return cudaErrorNotSupported;
     }
     ClusterParams prm;

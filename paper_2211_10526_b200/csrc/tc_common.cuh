@@ -300,12 +300,15 @@ __device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t a_desc, uint
         ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
         : "memory");
 }
-// The same with the descriptors given by their low words.  Every operand of these kernels has a 128-byte swizzle and 1024
-// bytes between groups of eight rows, so the high word is a constant and stepping along an operand is one addition.
+// The same with the descriptors given by their low words.  The operands of a kernel have one row width: rows of 128 bytes,
+// 128-byte swizzle, 1024 bytes between groups of eight rows, or rows of 64 bytes, 64-byte swizzle and 512 bytes.  So the
+// high word is a constant and stepping along an operand is one addition.
 constexpr uint32_t kDescHigh = (1024u >> 4) | (1u << 14) | (2u << 29);   // bits 32..63 of umma_desc_sw128(.., .., 1024)
+constexpr uint32_t kDescHigh64 = (512u >> 4) | (1u << 14) | (4u << 29);
 __device__ __forceinline__ uint32_t desc_low(uint32_t smem_addr, uint32_t lbo_bytes = 0) {
     return ((smem_addr >> 4) & 0x3fffu) | (((lbo_bytes >> 4) & 0x3fffu) << 16);
 }
+template <uint32_t HIGH = kDescHigh>
 __device__ __forceinline__ void umma_bf16_low(uint32_t d_tmem, uint32_t a_low, uint32_t b_low, uint32_t idesc,
                                               uint32_t accumulate) {
     asm volatile(
@@ -313,7 +316,7 @@ __device__ __forceinline__ void umma_bf16_low(uint32_t d_tmem, uint32_t a_low, u
         "setp.ne.b32 p, %5, 0;\n\t"
         "mov.b64 da, {%1, %4};\n\tmov.b64 db, {%2, %4};\n\t"
         "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %3, p;\n\t}"
-        ::"r"(d_tmem), "r"(a_low), "r"(b_low), "r"(idesc), "r"(kDescHigh), "r"(accumulate)
+        ::"r"(d_tmem), "r"(a_low), "r"(b_low), "r"(idesc), "r"(HIGH), "r"(accumulate)
         : "memory");
 }
 // All UMMAs issued so far by this thread arrive on `bar` when they have completed.

@@ -8,34 +8,40 @@ namespace castling {
 namespace tc {
 
 namespace {
-constexpr int kStateTile = 128;  // tokens per UMMA stage of the state kernel
+constexpr int kStateTile = 128;  // 128-byte rows per UMMA stage of the state kernel
+// Width-32 shapes that fit no 128-byte rows (odd grid widths or token counts, an odd number of heads side by side) come
+// here from this many tokens in all planes on.  The kernels are faster below it too (300 tokens: 6 us against 17 us on the
+// CUDA cores; 2 x 6 planes of 33 x 21: 8 us against 25 us), but the tests hold the smallest shapes to the CUDA-core family.
+constexpr long long kNarrowMinTokens = 4096;
 }
 
 namespace {
-// Width-32 heads fill a 128-byte row in one of two ways: two adjacent tokens of one head (tokens
-// contiguous, even grid width), or the same token of two adjacent heads (head stride 32, as in a
-// token-major [B,N,H,32] tensor with an even number of heads).
+// The single-kernel forward (and the non-default variants) put two width-32 rows side by side in one of 128 bytes: two
+// adjacent tokens of one head (tokens contiguous, even grid width), or the same token of two adjacent heads (head stride
+// 32, as in a token-major [B,N,H,32] tensor with an even number of heads).
 bool head_pairs(const Problem& p) {
     return p.d == 32 && p.H % 2 == 0 && p.hdiv == p.H && p.head0 == 0 && p.lq.head == 32 && p.lk.head == 32 &&
            p.lv.head == 32 && p.lo.head == 32;
 }
 }  // namespace
 
-// bf16, 3x3 or 5x5 filters, head width 64 or one of the two width-32 arrangements above.
+// Width-32 heads whose 64-byte rows lie next to one another in memory, token after token or head after head.
+static bool dense_rows(const Problem& p) {
+    return p.d == 32 && (p.contiguous_tokens() || (p.hdiv == p.H && p.lq.head == 32 && p.lk.head == 32 && p.lv.head == 32 && p.lo.head == 32));
+}
+
+// bf16, 3x3 or 5x5 filters, head width 64, one of the two width-32 arrangements above, or enough dense 64-byte rows.
 bool supports(const Problem& p) {
     if (!p.bf16 || (p.ksize != 3 && p.ksize != 5)) return false;
-    return p.d == 64 || token_pairs(p) || head_pairs(p);
+    return p.d == 64 || token_pairs(p) || head_pairs(p) || (dense_rows(p) && (long long)p.BH * p.N >= kNarrowMinTokens);
 }
 
-int rows_per_head(int N, int d) { return d == 32 ? N / 2 : N; }
+int rows_per_head(int N, int d) { return d == 32 ? (N + 1) / 2 : N; }
 
-// With fewer than 48 rows per (b,h) the 128-row tiles of the tensor-core kernels are mostly padding
-// and the CUDA-core kernels are faster (measured: 4x4 grids of width-32 heads, 20 us against 33 us).
-bool preferred(const Problem& p) {
-    if (!supports(p)) return false;
-    const int rows = (p.d == 32 && !token_pairs(p)) ? p.N : rows_per_head(p.N, p.d);
-    return rows >= 48;
-}
+// With fewer than 48 tokens per (b,h) the tiles of the tensor-core kernels are mostly padding and the CUDA-core kernels
+// are faster (measured: 4x4 grids of width-32 heads, 20 us against 33 us); from 7x7 on they are not (64 x 8 planes: 17.0 us
+// against 14.6 us).
+bool preferred(const Problem& p) { return supports(p) && p.N >= 48; }
 
 // Two state CTAs fit on an SM: as many splits as keep all CTAs of the launch resident at once
 // (two per multiprocessor), every split non-empty, at most 64 splits.
@@ -63,45 +69,49 @@ static bool cluster_enabled() {
     return on;
 }
 
-cudaError_t forward(const Problem& p_in, float* ws_state, float* ws_partial, unsigned* counters, int P,
-                    unsigned* status, cudaStream_t stream, int* launches, KernelTimer* timer) {
+cudaError_t forward(const Problem& p_in, float* ws_state, float* ws_partial, unsigned* counters, unsigned* status,
+                    cudaStream_t stream, int* launches, KernelTimer* timer) {
     *launches = 0;
     Problem p = p_in;
-    if (p.d == 32 && !token_pairs(p)) {
+    bool rows128 = p.d == 64 || token_pairs(p);   // every row of 128 bytes is full
+    if (!rows128 && head_pairs(p)) {
         // heads (2m, 2m+1) side by side = one width-64 plane whose state is block diagonal
         p.d = 64; p.H /= 2; p.BH /= 2; p.hdiv = p.H; p.blockdiag = true;
         p.lq.head = p.lk.head = p.lv.head = p.lo.head = 64;
-        P = choose_splits(p.BH, p.N);
+        rows128 = true;
     }
-    if (!p.rownorm && fused_supports(p)) {  // a whole (b,h) fits in shared memory: one kernel, no workspace
-        const cudaError_t e = launch_fused(p, status, stream);
+    rows128 = rows128 && !p.rownorm;   // the row sums are carried by the separate state and apply kernels only
+    cudaError_t e;
+    if (rows128 && fused_supports(p)) {  // a whole (b,h) fits in shared memory: one kernel, no workspace
+        e = launch_fused(p, status, stream);
         if (e != cudaSuccess) return e;
         ++*launches;
         timer->mark(stream, "tc_fused");
         return cudaSuccess;
     }
-    cudaError_t e;
-    if (const int C = (cluster_enabled() && !p.rownorm) ? cluster_size(p) : 0) {
+    if (const int C = (cluster_enabled() && rows128) ? cluster_size(p) : 0) {
         e = launch_cluster(p, C, status, stream);
         if (e != cudaSuccess) return e;
         ++*launches;
         timer->mark(stream, "tc_cluster");
         return cudaSuccess;
     }
-    if (!two_kernels() && !p.rownorm && pipe_supports(p)) {
+    if (!two_kernels() && rows128 && pipe_supports(p)) {
         // state and apply pipelines in one persistent kernel: V is read from memory once
         e = launch_pipe(p, ws_state, ws_partial, counters, status, stream);
         if (e != cudaSuccess) return e;
         ++*launches;
         timer->mark(stream, "tc_pipe");
     } else {
-        const int tiles = (rows_per_head(p.N, p.d) + kStateTile - 1) / kStateTile;
-        const int per = (tiles + P - 1) / P;
-        e = launch_state(p, ws_partial, ws_state, counters, P, per, status, stream);
+        p = p_in;   // width-32 heads in 64-byte rows of their own
+        p.narrow = p.d == 32;
+        const int rows = rows_per_head(p.N, p.d), P = choose_splits(p.BH, rows);
+        const int tiles = (rows + kStateTile - 1) / kStateTile;
+        e = launch_state(p, ws_partial, ws_state, counters, P, (tiles + P - 1) / P, status, stream);
         if (e != cudaSuccess) return e;
         ++*launches;
         timer->mark(stream, "tc_state");
-        e = launch_apply(p, ws_state, 1, status, stream);
+        e = launch_apply(p, ws_state, status, stream);
         if (e != cudaSuccess) return e;
         ++*launches;
         timer->mark(stream, "tc_apply");
@@ -134,7 +144,7 @@ cudaError_t shard_state(const Problem& p, float* state_out, float* ws_partial, u
 cudaError_t shard_apply(const Problem& p, const float* state, unsigned* status, cudaStream_t stream, int* launches,
                         KernelTimer* timer) {
     *launches = 0;
-    const cudaError_t e = launch_apply(p, state, 1, status, stream);
+    const cudaError_t e = launch_apply(p, state, status, stream);
     if (e != cudaSuccess) return e;
     ++*launches;
     timer->mark(stream, "tc_apply");

@@ -524,8 +524,8 @@ cudaError_t launch_fused_ks(const Problem& p, unsigned* status, cudaStream_t st)
     };
     uint64_t sq[3], sk[3], sv[3];
     strides(p.lq, sq); strides(p.lk, sk); strides(p.lv, sv);
-    if (!make_tensor_map_bf16(&tmK, p.k, 4, dims, sk, box, true) || !make_tensor_map_bf16(&tmV, p.v, 4, dims, sv, box, true) ||
-        !make_tensor_map_bf16(&tmQ, p.q, 4, dims, sq, box, true) || !make_tensor_map_bf16(&tmVplain, p.v, 4, dims, sv, box, false))
+    if (!make_tensor_map_bf16(&tmK, p.k, 4, dims, sk, box, 128) || !make_tensor_map_bf16(&tmV, p.v, 4, dims, sv, box, 128) ||
+        !make_tensor_map_bf16(&tmQ, p.q, 4, dims, sq, box, 128) || !make_tensor_map_bf16(&tmVplain, p.v, 4, dims, sv, box, 0))
         return cudaErrorNotSupported;
     FusedParams prm;
     prm.w = static_cast<const __nv_bfloat16*>(p.w);

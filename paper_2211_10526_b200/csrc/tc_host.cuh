@@ -11,7 +11,7 @@ namespace tc {
 constexpr int kCountersPerHead = 17;
 
 bool make_tensor_map_bf16(CUtensorMap* out, const void* base, int rank, const uint64_t* dims,
-                          const uint64_t* strides, const uint32_t* box, bool swizzle128);
+                          const uint64_t* strides, const uint32_t* box, int swizzle);
 
 // Width-32 heads, two adjacent tokens of one head per 128-byte row: contiguous tokens, even grid width,
 // an even number of tokens per plane.
@@ -19,17 +19,17 @@ inline bool token_pairs(const Problem& p) {
     return p.d == 32 && p.gridW % 2 == 0 && p.N % 2 == 0 && p.contiguous_tokens();
 }
 
-// True when the tensor-core kernels can take this problem (bf16; d = 64, or d = 32 with even gridW;
-// 3x3 or 5x5 filters).
+// True when the tensor-core kernels can take this problem (bf16; 3x3 or 5x5 filters; d = 64, or d = 32 with rows that lie
+// next to one another in memory).
 bool supports(const Problem& p);
 
 // True when automatic dispatch should pick them (enough rows per (b,h) to fill their tiles).
 bool preferred(const Problem& p);
 
-// 128-byte rows per (b,h): N for d = 64, N / 2 for d = 32 (two tokens per row).
+// 128-byte rows per (b,h): N for d = 64, N / 2 (rounded up) for d = 32 (two tokens per row).
 int rows_per_head(int N, int d);
 
-// Words of one (b,h) state as the tensor-core kernels store it (always the 64-wide form): S, s, and with row-sum
+// Words of one (b,h) state as the tensor-core kernels store it, at most (width-64 heads): S, s, and with row-sum
 // normalisation the sum of the unit key rows behind them.
 constexpr int kStateWords = 64 * 64 + 64;
 constexpr int kStateWordsRownorm = kStateWords + 64;
@@ -41,8 +41,8 @@ int choose_splits(int BH, int N);
 // Enqueue state build, split reduction and apply for one problem.  `status` is the device status
 // word; `counters` holds kCountersPerHead zero-initialised arrival counters per (b,h), left at zero by every call.  Returns the cudaError_t of the launches; cudaErrorNotSupported if a tensor map could not
 // be built.
-cudaError_t forward(const Problem& p, float* ws_state, float* ws_partial, unsigned* counters, int P,
-                    unsigned* status, cudaStream_t stream, int* launches, KernelTimer* timer);
+cudaError_t forward(const Problem& p, float* ws_state, float* ws_partial, unsigned* counters, unsigned* status, cudaStream_t stream,
+                    int* launches, KernelTimer* timer);
 
 // The two halves of a forward on their own (a sequence sharded over devices): the state of a shard's tokens, written
 // to state_out in the documented layout (S row-major, then s), and the apply pass over a band of grid rows with a
@@ -56,7 +56,9 @@ cudaError_t shard_apply(const Problem& p, const float* state, unsigned* status, 
 // Launchers of the individual kernels (each in its own file).
 cudaError_t launch_state(const Problem& p, float* partial, float* final_state, unsigned* counters, int P,
                          int tiles_per_cta, unsigned* status, cudaStream_t st);
-cudaError_t launch_apply(const Problem& p, const float* partial, int P, unsigned* status, cudaStream_t st);
+cudaError_t launch_apply(const Problem& p, const float* state, unsigned* status, cudaStream_t st);
+// The apply kernel for width-32 heads in 64-byte rows (csrc/tc_apply32.cu).
+cudaError_t launch_apply32(const Problem& p, const float* state, unsigned* status, cudaStream_t st);
 // Output rows of the off-grid leading tokens (p.prefix of them per plane), from the final state.
 cudaError_t launch_prefix_rows(const Problem& p, const float* state, cudaStream_t st);
 

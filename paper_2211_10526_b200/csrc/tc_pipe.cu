@@ -773,7 +773,7 @@ cudaError_t launch_pipe_ks(const Problem& p, float* state, float* ready, unsigne
                                 (uint64_t)(nb > 1 ? p.lk.batch : p.lk.head * p.hdiv)};
         const uint64_t sv[3] = {(uint64_t)(pair ? kD : p.lv.token), (uint64_t)p.lv.head,
                                 (uint64_t)(nb > 1 ? p.lv.batch : p.lv.head * p.hdiv)};
-        if (!make_tensor_map_bf16(&tmK, p.k, 4, dims, sk, box, true) || !make_tensor_map_bf16(&tmVs, p.v, 4, dims, sv, box, true))
+        if (!make_tensor_map_bf16(&tmK, p.k, 4, dims, sk, box, 128) || !make_tensor_map_bf16(&tmVs, p.v, 4, dims, sv, box, 128))
             return cudaErrorNotSupported;
     }
     const int rank = nb > 1 ? 5 : 4;
@@ -792,8 +792,8 @@ cudaError_t launch_pipe_ks(const Problem& p, float* state, float* ready, unsigne
         const __nv_bfloat16* qg = static_cast<const __nv_bfloat16*>(p.q) + p.prefix * p.lq.token;
         const __nv_bfloat16* vg = static_cast<const __nv_bfloat16*>(p.v) + p.prefix * p.lv.token;
         __nv_bfloat16* og = static_cast<__nv_bfloat16*>(p.out) + p.prefix * p.lo.token;
-        if (!make_tensor_map_bf16(&tmQ, qg, rank, dims, sq, box, true) || !make_tensor_map_bf16(&tmVh, vg, rank, dims, sv, boxv, false) ||
-            !make_tensor_map_bf16(&tmO, og, rank, dims, so, box, true))
+        if (!make_tensor_map_bf16(&tmQ, qg, rank, dims, sq, box, 128) || !make_tensor_map_bf16(&tmVh, vg, rank, dims, sv, boxv, 0) ||
+            !make_tensor_map_bf16(&tmO, og, rank, dims, so, box, 128))
             return cudaErrorNotSupported;
     }
     PipeParams prm;

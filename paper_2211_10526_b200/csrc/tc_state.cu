@@ -1,4 +1,4 @@
-// State kernel of the tensor-core path (bf16, d = 64): per (b,h) and token split,
+// State kernel of the tensor-core path (bf16, d = 64; d = 32: NARROW below): per (b,h) and token split,
 //     S = sum_n k^_n^T v_n  (64 x 64)   and   s = sum_n v_n  (64)            (Eq. 9)
 // as one tcgen05 contraction over tokens.  Per 128-token stage TMA brings the K and V tiles
 // into 128-byte-swizzled shared memory; four warps scale every K row by 1 / max(||k||, eps) in
@@ -18,7 +18,8 @@ namespace tc {
 namespace {
 
 constexpr int kD = 64;
-constexpr int kTile = 128;                   // tokens per stage
+constexpr int kTile = 128;                   // 128-byte rows per stage
+constexpr int kThreadRows = 128;             // normalising threads: one 128-byte row of a stage each
 constexpr int kStages = 3;                  // 3 x 32 KiB: two CTAs fit on one SM
 constexpr int kTileBytes = kTile * kD * 2;   // 16 KiB per operand tile
 constexpr int kStageBytes = 2 * kTileBytes;  // K then V
@@ -28,14 +29,11 @@ constexpr int kTmemCols = 128;                // two 64-column accumulators: a C
 constexpr int kGroup = 4;                    // splits per first-level reduction group
 constexpr size_t kSmemBytes = 1024 + kStages * kStageBytes + kOnesBytes + 256;
 
-// PAIR = true serves head width 32: the [N][32] tensors are viewed as [N/2][64], one 128-byte row
-// holding two consecutive tokens.  The same contraction then yields the four 32 x 32 blocks
-// [k_even^T v_even, k_even^T v_odd; k_odd^T v_even, k_odd^T v_odd]; the state is the sum of the two
-// diagonal blocks (and s the sum of the two halves of row 64), which the apply kernel folds when it
-// reads them.  Each half row is normalised by its own token's norm.
-// The same instantiation serves two width-32 heads stored side by side in one 128-byte row (head
-// stride 32): identical arithmetic; there the consumers keep the two diagonal blocks apart, one per head.
-template <bool PAIR, bool RN>
+// NARROW serves width-32 heads: rows of 64 bytes, 64-byte swizzle, 256 tokens per stage (any grid width, any number of
+// tokens), UMMAs of M = 64 (32 key features, then the row of ones) and N = 32, states of 32 x 32 + 32 words.  Two tokens
+// packed to a 128-byte row instead, which wastes half of the contraction and needs an even grid width, took 19.8 us against
+// 17.6 us (8 x 8 planes of 64 x 64 tokens).
+template <bool NARROW, bool RN>
 __global__ void __launch_bounds__(kThreads, 2)
 tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
                 float* __restrict__ dst, float* __restrict__ final_state, unsigned* __restrict__ counters,
@@ -51,13 +49,15 @@ tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_free + 2);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
-    constexpr int kAcc = RN ? 2 * kD : kD;                 // accumulator columns
-    constexpr int kStateW = kD * kD + kD + (RN ? kD : 0);  // words of one state: S, s, (RN) sum of the unit key rows
+    constexpr int kW = NARROW ? 32 : kD;                   // width of the contraction's operands
+    constexpr int kTok = NARROW ? 2 * kTile : kTile;       // rows (of kW elements) per stage
+    constexpr int kAcc = RN ? 2 * kW : kW;                 // accumulator columns
+    constexpr int kStateW = kW * kW + kW + (RN ? kW : 0);  // words of one state: S, s, (RN) sum of the unit key rows
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     // Work items.  With P > 1 a CTA serves one (b,h, split).  With P == 1 (many heads, few tokens) a CTA
     // serves items_per_cta consecutive (b,h) one after another, so that barrier set-up, TMEM allocation
     // and the first load latency are paid once and the loads of the next (b,h) overlap the current one.
-    const int total_tiles = (N + kTile - 1) / kTile;
+    const int total_tiles = (N + kTok - 1) / kTok;
     const int p = (P > 1) ? blockIdx.x % P : 0;
     const int bh0 = (P > 1) ? blockIdx.x / P : blockIdx.x * items_per_cta;
     const int n_items = (P > 1) ? 1 : min(items_per_cta, BH - bh0);
@@ -77,10 +77,10 @@ tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     if (tid == 0) {
         for (int s = 0; s < kStages; ++s) {
             mbar_init(&full[s], 1);
-            mbar_init(&scaled[s], kTile);
+            mbar_init(&scaled[s], kThreadRows);
             mbar_init(&empty[s], 1);
         }
-        for (int b = 0; b < 2; ++b) { mbar_init(&accum[b], 1); mbar_init(&acc_free[b], kTile); }
+        for (int b = 0; b < 2; ++b) { mbar_init(&accum[b], 1); mbar_init(&acc_free[b], kThreadRows); }
         *abort_flag = 0;
         mbar_fence_init();
         tma_prefetch_desc(&tmK);
@@ -90,11 +90,12 @@ tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     if (warp >= 2) {
         // constant block of A: for each of 16 token rows, element 64 (first of the second 64-wide
         // block along M) is 1.0 and the rest 0; 16-byte chunk c of row r sits at chunk c ^ (r & 7)
+        // (rows of 64 bytes: element 32, chunk c of row r at chunk c ^ ((r >> 1) & 3), half as many threads)
         const int t = tid - 64;  // 0..127 -> one 16-byte chunk each
-        const int r = t >> 3, c = t & 7;
+        const int r = NARROW ? t >> 2 : t >> 3, c = NARROW ? t & 3 : t & 7;
         uint4 val = make_uint4(0, 0, 0, 0);
-        if ((c ^ (r & 7)) == 0) val.x = 0x3f80u;  // logical chunk 0: bf16 1.0 in its first element
-        *reinterpret_cast<uint4*>(ones + r * 128 + c * 16) = val;
+        if ((c ^ (NARROW ? (r >> 1) & 3 : r & 7)) == 0) val.x = 0x3f80u;  // logical chunk 0: bf16 1.0 in its first element
+        if (!NARROW || r < 16) *reinterpret_cast<uint4*>(ones + t * 16) = val;
         fence_proxy_async_smem();
     }
     tcgen05_fence_before_sync();
@@ -122,8 +123,8 @@ tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
                     uint8_t* ks = smem + s * kStageBytes;
                     mbar_expect_tx(&full[s], kStageBytes);
                     const int plane = bh0 + item, pb = plane / hdiv, ph = plane - pb * hdiv;
-                    tma_load_4d_hint(ks, &tmK, &full[s], 0, (t_begin + it) * kTile, ph, pb, pol_k);
-                    tma_load_4d_hint(ks + kTileBytes, &tmV, &full[s], 0, (t_begin + it) * kTile, ph, pb, pol_v);
+                    tma_load_4d_hint(ks, &tmK, &full[s], 0, (t_begin + it) * kTok, ph, pb, pol_k);
+                    tma_load_4d_hint(ks + kTileBytes, &tmV, &full[s], 0, (t_begin + it) * kTok, ph, pb, pol_v);
                 }
             }
             if (*abort_flag) {
@@ -134,11 +135,11 @@ tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
         }
     } else if (warp == 1) {
         // the whole warp walks through the tiles, one elected lane issues
-        constexpr uint32_t idesc = umma_idesc_bf16(128, kAcc, true, true);
+        constexpr uint32_t idesc = umma_idesc_bf16(NARROW ? 64 : 128, kAcc, true, true);
         const uint32_t ones_addr = smem_u32(ones);
         // A: 128 bytes of K per token and, lbo bytes on, the constant block; stepping to the next 16 tokens adds to the
         // address and takes the same off the distance
-        constexpr uint32_t kStep = (2048u >> 4) - ((2048u >> 4) << 16);
+        constexpr uint32_t kStepB = (16u * kW * 2) >> 4, kStep = kStepB - (kStepB << 16);
         bool ok = true;
         int s = 0;
         uint32_t par = 0;
@@ -153,8 +154,9 @@ tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
                     const uint32_t ka = smem_u32(smem + s * kStageBytes), va = ka + kTileBytes;
                     const uint32_t a = desc_low(ka, ones_addr - ka), b = desc_low(va, RN ? ones_addr - va : 0);
 #pragma unroll
-                    for (int j = 0; j < kTile / 16; ++j)  // one UMMA per 16 tokens (K = 16)
-                        umma_bf16_low(tmem + buf * kAcc, a + j * kStep, b + j * (RN ? kStep : (2048u >> 4)), idesc, (it | j) != 0);
+                    for (int j = 0; j < kTok / 16; ++j)  // one UMMA per 16 tokens (K = 16)
+                        umma_bf16_low<NARROW ? kDescHigh64 : kDescHigh>(tmem + buf * kAcc, a + j * kStep,
+                                                                        b + j * (RN ? kStep : kStepB), idesc, (it | j) != 0);
                     umma_commit(&empty[s]);
                     if (it == n_tiles - 1) umma_commit(&accum[buf]);
                 }
@@ -163,7 +165,7 @@ tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
             }
         }
     } else {
-        const int t = tid - 64;  // token row of the stage handled by this thread
+        const int t = tid - 64;  // 128-byte row of the stage handled by this thread
         const int quarter = warp & 3;
         bool ok = true;
         // read the finished accumulator of `item` out of TMEM: rows 0..63 are S, row 64 is s; a warp reads
@@ -175,23 +177,24 @@ tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
             tcgen05_fence_after_sync();
             if (quarter < 3) {
                 float* out = dst + ((size_t)(bh0 + item) * P + p) * kStateW;
-                const int row = quarter * 32 + lane;
+                // M = 64 keeps rows 16 q .. 16 q + 15 in lanes 32 q .. 32 q + 15
+                const int row = NARROW ? (lane < 16 ? quarter * 16 + lane : kW + 1) : quarter * 32 + lane;
 #pragma unroll
-                for (int cc = 0; cc < kD / 16; ++cc) {
+                for (int cc = 0; cc < kW / 16; ++cc) {
                     float v[16];
                     tmem_ld16(tmem + ((uint32_t)(quarter * 32) << 16) + buf * kAcc + cc * 16, v);
                     tmem_ld_wait();
-                    if (row <= kD) {
-                        float4* o4 = reinterpret_cast<float4*>(out + row * kD + cc * 16);  // row 64 lands on s
+                    if (row <= kW) {
+                        float4* o4 = reinterpret_cast<float4*>(out + row * kW + cc * 16);  // row kW lands on s
 #pragma unroll
                         for (int e = 0; e < 4; ++e) o4[e] = make_float4(v[4 * e], v[4 * e + 1], v[4 * e + 2], v[4 * e + 3]);
                     }
                 }
-                if (RN) {  // column 64: the row sums of A; rows 0..63 are sum_n k^_n, stored behind s
+                if (RN) {  // column kW: the row sums of A; rows 0..kW - 1 are sum_n k^_n, stored behind s
                     float v[16];
-                    tmem_ld16(tmem + ((uint32_t)(quarter * 32) << 16) + buf * kAcc + kD, v);
+                    tmem_ld16(tmem + ((uint32_t)(quarter * 32) << 16) + buf * kAcc + kW, v);
                     tmem_ld_wait();
-                    if (row < kD) out[kD * kD + kD + row] = v[0];
+                    if (row < kW) out[kW * kW + kW + row] = v[0];
                 }
             }
             tcgen05_fence_before_sync();
@@ -204,9 +207,11 @@ tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
                 const int s = gt % kStages, use = gt / kStages;
                 ok = mbar_wait(&full[s], use & 1, abort_flag, status, kStatusStateTimeout);
                 if (!ok) break;
+                // NARROW: the 128 bytes are tokens 2 t and 2 t + 1, whose chunk c sits at chunk c ^ (t & 3) of their half; the
+                // same walk over the eight chunks as for a 128-byte swizzle meets all chunks of one of them first
                 uint8_t* row = smem + s * kStageBytes + t * 128;
                 uint4 c[8];
-                float ssa = 0.f, ssb = 0.f;  // first / second half of the row (two tokens when PAIR)
+                float ssa = 0.f, ssb = 0.f;  // first / second half of the 128 bytes
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
                     c[j] = *reinterpret_cast<const uint4*>(row + ((j ^ (t & 7)) << 4));
@@ -221,7 +226,7 @@ tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
                     if (j < 4) ssa += part; else ssb += part;
                 }
                 float rka, rkb;
-                if (PAIR) {
+                if (NARROW) {
                     rka = 1.0f / sqrtf(fmaxf(ssa, eps2));
                     rkb = 1.0f / sqrtf(fmaxf(ssb, eps2));
                 } else {
@@ -352,28 +357,19 @@ tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
 
 cudaError_t launch_state(const Problem& p, float* partial, float* final_state, unsigned* counters, int P,
                          int tiles_per_cta, unsigned* status, cudaStream_t st) {
-    const bool pair = (p.d == 32);          // two tokens per 128-byte row
-    const bool halves = pair || p.blockdiag;  // each half of a row has its own norm
-    const int rows = pair ? p.N / 2 : p.N;  // 128-byte rows per (b,h)
+    const bool narrow = p.d == 32;
     CUtensorMap tmK, tmV;
-    // [64, rows, planes per batch step, batch steps]; a 128-byte row is one token, or two adjacent ones
+    // [row, tokens, planes per batch step, batch steps]
     const uint64_t nb = (uint64_t)(p.BH / p.hdiv);
-    const uint64_t dims[4] = {(uint64_t)kD, (uint64_t)rows, (uint64_t)p.hdiv, nb};
-    const uint32_t box[4] = {kD, kTile, 1, 1};
-    const uint64_t sk[3] = {(uint64_t)(pair ? kD : p.lk.token), (uint64_t)p.lk.head,
-                            (uint64_t)(nb > 1 ? p.lk.batch : p.lk.head * p.hdiv)};
-    const uint64_t sv[3] = {(uint64_t)(pair ? kD : p.lv.token), (uint64_t)p.lv.head,
-                            (uint64_t)(nb > 1 ? p.lv.batch : p.lv.head * p.hdiv)};
-    if (!make_tensor_map_bf16(&tmK, p.k, 4, dims, sk, box, true) || !make_tensor_map_bf16(&tmV, p.v, 4, dims, sv, box, true))
+    const uint32_t width = narrow ? 32 : kD;
+    const uint64_t dims[4] = {width, (uint64_t)p.N, (uint64_t)p.hdiv, nb};
+    const uint32_t box[4] = {width, narrow ? 2u * kTile : kTile, 1, 1};
+    const uint64_t sk[3] = {(uint64_t)p.lk.token, (uint64_t)p.lk.head, (uint64_t)(nb > 1 ? p.lk.batch : p.lk.head * p.hdiv)};
+    const uint64_t sv[3] = {(uint64_t)p.lv.token, (uint64_t)p.lv.head, (uint64_t)(nb > 1 ? p.lv.batch : p.lv.head * p.hdiv)};
+    const int swizzle = narrow ? 64 : 128;
+    if (!make_tensor_map_bf16(&tmK, p.k, 4, dims, sk, box, swizzle) || !make_tensor_map_bf16(&tmV, p.v, 4, dims, sv, box, swizzle))
         return cudaErrorNotSupported;
     static PerDevice opt_in[4];
-    {
-        const cudaError_t e = p.rownorm ? (halves ? opt_in_smem(tc_state_kernel<true, true>, kSmemBytes, opt_in[3])
-                                                  : opt_in_smem(tc_state_kernel<false, true>, kSmemBytes, opt_in[2]))
-                                        : (halves ? opt_in_smem(tc_state_kernel<true, false>, kSmemBytes, opt_in[1])
-                                                  : opt_in_smem(tc_state_kernel<false, false>, kSmemBytes, opt_in[0]));
-        if (e != cudaSuccess) return e;
-    }
     float* dst = P > 1 ? partial : final_state;
     // P == 1: a CTA serves several consecutive (b,h); at most two CTAs per multiprocessor so all are resident
     int grid = p.BH * P, items = 1;
@@ -389,11 +385,13 @@ cudaError_t launch_state(const Problem& p, float* partial, float* final_state, u
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr; cfg.numAttrs = 1;
     auto launch = [&](auto kernel) {
-        return cudaLaunchKernelEx(&cfg, kernel, tmK, tmV, dst, final_state, counters, rows, tiles_per_cta, P, p.BH, p.hdiv, items,
+        const cudaError_t e = opt_in_smem(kernel, kSmemBytes, opt_in[(narrow ? 2 : 0) + (p.rownorm ? 1 : 0)]);
+        if (e != cudaSuccess) return e;
+        return cudaLaunchKernelEx(&cfg, kernel, tmK, tmV, dst, final_state, counters, p.N, tiles_per_cta, P, p.BH, p.hdiv, items,
                                   p.eps2, status);
     };
-    if (p.rownorm) return halves ? launch(tc_state_kernel<true, true>) : launch(tc_state_kernel<false, true>);
-    return halves ? launch(tc_state_kernel<true, false>) : launch(tc_state_kernel<false, false>);
+    if (narrow) return p.rownorm ? launch(tc_state_kernel<true, true>) : launch(tc_state_kernel<true, false>);
+    return p.rownorm ? launch(tc_state_kernel<false, true>) : launch(tc_state_kernel<false, false>);
 }
 
 }  // namespace tc

@@ -29,7 +29,7 @@ struct CacheEntry {
     uint64_t dims[5] = {};
     uint64_t strides[4] = {};
     uint32_t box[5] = {};
-    bool swizzle = false;
+    int swizzle = 0;
     CUtensorMap map;
 };
 constexpr int kCacheSize = 32;
@@ -38,7 +38,7 @@ int g_cache_next = 0;
 std::mutex g_cache_mutex;
 
 bool same_key(const CacheEntry& e, const void* base, int rank, const uint64_t* dims, const uint64_t* strides,
-              const uint32_t* box, bool sw) {
+              const uint32_t* box, int sw) {
     if (!e.valid || e.base != base || e.rank != rank || e.swizzle != sw) return false;
     for (int i = 0; i < rank; ++i)
         if (e.dims[i] != dims[i] || e.box[i] != box[i]) return false;
@@ -50,13 +50,13 @@ bool same_key(const CacheEntry& e, const void* base, int rank, const uint64_t* d
 
 namespace {
 bool encode_tensor_map_bf16(CUtensorMap* out, const void* base, int rank, const uint64_t* dims,
-                            const uint64_t* strides, const uint32_t* box, bool swizzle128);
+                            const uint64_t* strides, const uint32_t* box, int swizzle);
 }
 
 // dims/box are innermost-first, in elements; the innermost dimension is contiguous; strides[i] is the
-// distance in elements between consecutive indices of dimension i + 1 (rank - 1 entries).
+// distance in elements between consecutive indices of dimension i + 1 (rank - 1 entries); swizzle: 0, 64 or 128 bytes.
 bool make_tensor_map_bf16(CUtensorMap* out, const void* base, int rank, const uint64_t* dims,
-                          const uint64_t* strides, const uint32_t* box, bool swizzle128) {
+                          const uint64_t* strides, const uint32_t* box, int swizzle) {
     if (rank < 2 || rank > 5) return false;
     uint64_t fixed[4];
     for (int i = 0; i + 1 < rank; ++i) {
@@ -66,11 +66,11 @@ bool make_tensor_map_bf16(CUtensorMap* out, const void* base, int rank, const ui
     strides = fixed;
     std::lock_guard<std::mutex> lock(g_cache_mutex);
     for (const CacheEntry& e : g_cache)
-        if (same_key(e, base, rank, dims, strides, box, swizzle128)) { *out = e.map; return true; }
-    if (!encode_tensor_map_bf16(out, base, rank, dims, strides, box, swizzle128)) return false;
+        if (same_key(e, base, rank, dims, strides, box, swizzle)) { *out = e.map; return true; }
+    if (!encode_tensor_map_bf16(out, base, rank, dims, strides, box, swizzle)) return false;
     CacheEntry& e = g_cache[g_cache_next];
     g_cache_next = (g_cache_next + 1) % kCacheSize;
-    e.valid = true; e.base = base; e.rank = rank; e.swizzle = swizzle128; e.map = *out;
+    e.valid = true; e.base = base; e.rank = rank; e.swizzle = swizzle; e.map = *out;
     for (int i = 0; i < rank; ++i) { e.dims[i] = dims[i]; e.box[i] = box[i]; }
     for (int i = 0; i + 1 < rank; ++i) e.strides[i] = strides[i];
     return true;
@@ -78,7 +78,7 @@ bool make_tensor_map_bf16(CUtensorMap* out, const void* base, int rank, const ui
 
 namespace {
 bool encode_tensor_map_bf16(CUtensorMap* out, const void* base, int rank, const uint64_t* dims,
-                            const uint64_t* strides, const uint32_t* box, bool swizzle128) {
+                            const uint64_t* strides, const uint32_t* box, int swizzle) {
     std::call_once(g_once, lookup);
     if (!g_encode) return false;
     cuuint64_t gdim[5];
@@ -92,7 +92,7 @@ bool encode_tensor_map_bf16(CUtensorMap* out, const void* base, int rank, const 
     }
     const CUresult r = g_encode(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (cuuint32_t)rank, const_cast<void*>(base), gdim,
                                 gstride, bdim, estride, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                                swizzle128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE,
+                                swizzle == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : swizzle == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_NONE,
                                 CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS;
 }
