@@ -73,7 +73,6 @@ tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
         return;
     }
 
-    pdl_launch_dependents();  // the apply kernel may begin its prologue while this grid drains
     if (tid == 0) {
         for (int s = 0; s < kStages; ++s) {
             mbar_init(&full[s], 1);
@@ -116,6 +115,9 @@ tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
             // Global memory is first touched here; the partial states and arrival counters are written only after
             // these loads have landed.
             pdl_wait_primary();
+            // Only now may the apply kernel begin its prologue: it loads Q and V, which may be the output of the kernel
+            // this grid has just waited for, as soon as it runs.
+            pdl_launch_dependents();
             for (int item = 0; item < n_items && ok; ++item) {
                 for (int it = 0; it < n_tiles; ++it, ++issued) {
                     const int s = issued % kStages, use = issued / kStages;
