@@ -49,7 +49,7 @@ size_t elem_bytes(castling_dtype_t t) { return t == CASTLING_F32 ? 4 : 2; }
 
 // header | state [BH] | partial [BH][P] (only when the token range is split)
 size_t workspace_words(int BH, int N, int d, bool bf16) {
-    int P = castling::simt_choose_splits(BH, N);
+    int P = castling::simt_choose_splits(BH, N, d, bf16);
     size_t words = castling::state_words_rownorm(d);  // the CUDA-core kernels' state, with room for the key-row sum
     if (bf16 && (d == 64 || d == 32)) {  // shapes the tensor-core kernels may take: they keep 64-wide states
         const int Pt = castling::tc::choose_splits(BH, castling::tc::rows_per_head(N, d));
@@ -255,7 +255,7 @@ int run_device(castling_attn* h, const Problem& p, cudaStream_t stream) {
         if (rc != CASTLING_OK) return rc;
         e = castling::tc::forward(p, state, partial, h->counters, reinterpret_cast<unsigned*>(h->ws), stream, &launches, &h->timer);
     } else {
-        e = castling::simt_forward(p, state, partial, castling::simt_choose_splits(p.BH, p.N), stream, &launches,
+        e = castling::simt_forward(p, state, partial, castling::simt_choose_splits(p.BH, p.N, p.d, p.bf16), stream, &launches,
                                    &h->timer);
     }
     if (use_tensor && e == cudaErrorNotSupported && h->cfg.force_path == CASTLING_PATH_AUTO) {
@@ -264,7 +264,7 @@ int run_device(castling_attn* h, const Problem& p, cudaStream_t stream) {
         use_tensor = false;
         partial = state + (size_t)p.BH * simt_words;
         h->timer.begin(stream);
-        e = castling::simt_forward(p, state, partial, castling::simt_choose_splits(p.BH, p.N), stream, &launches, &h->timer);
+        e = castling::simt_forward(p, state, partial, castling::simt_choose_splits(p.BH, p.N, p.d, p.bf16), stream, &launches, &h->timer);
     }
     if (e != cudaSuccess) return fail_cuda(h, e);
     h->last_path = use_tensor ? CASTLING_PATH_TENSOR : CASTLING_PATH_SIMT;
@@ -521,7 +521,7 @@ int castling_attn_shard_state(castling_attn_t* h, const void* k, const void* v, 
     }
     if (!tensor) {
         partial = h->ws + castling::kHeaderWords + (size_t)p.BH * castling::state_words(p.d);
-        e = castling::simt_forward(p, state_out, partial, castling::simt_choose_splits(p.BH, p.N),
+        e = castling::simt_forward(p, state_out, partial, castling::simt_choose_splits(p.BH, p.N, p.d, p.bf16),
                                    static_cast<cudaStream_t>(stream), &launches, &h->timer);
     }
     if (e != cudaSuccess) return fail_cuda(h, e);

@@ -119,7 +119,14 @@ int device_sm_count();
 // CUDA-core path.  simt_forward returns the cudaError_t of its launches.
 cudaError_t simt_forward(const Problem& p, float* ws_state, float* ws_partial, int P,
                          cudaStream_t stream, int* launches, KernelTimer* timer);
-int simt_choose_splits(int BH, int N);
+int simt_choose_splits(int BH, int N, int d, bool bf16);
+// fp32 kernels for head widths 32, 64 and 128 and 3x3 or 5x5 filters (csrc/f32_kernels.cu); simt_forward takes them where
+// they apply.
+inline bool f32_width(int d) { return d == 32 || d == 64 || d == 128; }
+bool f32_supports(const Problem& p);
+int f32_choose_splits(int BH, int N);
+cudaError_t f32_forward(const Problem& p, float* ws_state, float* ws_partial, int P, cudaStream_t stream, int* launches,
+                        KernelTimer* timer);
 // Explicit-weights forward (csrc/quad_kernels.cu): exact kernel and / or masked softmax branch; O(N^2 d).
 cudaError_t quad_forward(const Problem& p, cudaStream_t stream, int* launches, KernelTimer* timer);
 bool simt_supports(int d, int ksize);

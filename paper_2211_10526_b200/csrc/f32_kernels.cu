@@ -1,0 +1,437 @@
+// fp32 kernels of the linear-angular attention core for head widths 32, 64 and 128 and 3x3 or 5x5 filters (the 1e-5
+// tolerance rules out bf16 operands; every other fp32 shape runs on simt_kernels.cu):
+//   state kernel  S += k^^T v, s += v per (plane, token split): 64-token tiles, K scaled to unit rows on its way to shared
+//                 memory, the next tile's loads in flight; a thread owns 8 x 8 of S and every G-th token (G groups of
+//                 (D/8)^2 threads), the groups meet in shared memory at the end
+//   apply kernel  a patch of 8 rows x TX columns of tokens: Q, V with halo and S' = S / pi in shared memory (asynchronous
+//                 copies; Q and V before the state kernel has finished); a thread owns a run of 8 tokens x 4 channels: the
+//                 contraction over the key features, then the convolution, its window sliding along the run
+// Bound: fp32 FMA issue (4 d^2 flop per token and head at 128 FMA per cycle and multiprocessor: 62 us for 2 x 8 planes of
+// 128 x 128, d = 64), which needs register tiles large enough for shared memory: 64 FMAs per four 16-byte loads in the state
+// kernel, 128 per twelve in the apply kernel.
+// Measured: 2 x 8 planes of 128 x 128, d = 64: 155 us per forward (392 on the kernels of simt_kernels.cu, whose threads issued 28
+// instructions and eight 4-byte loads for 16 FMAs and read the convolution's window from global memory); 2 x 4 planes of 14 x 14,
+// d = 32: 8.5 us in a replayed graph (22.7: one CTA per plane walked through seven tiles with three barriers and a trip to
+// memory each).
+#include "tc_common.cuh"
+#include "tc_host.cuh"
+
+namespace castling {
+namespace {
+
+using tc::ffma2;
+using tc::pdl_launch_dependents;
+using tc::pdl_wait_primary;
+using tc::smem_u32;
+
+constexpr int kThreads = 256;
+constexpr int kTok = 64;          // tokens per tile of the state kernel
+constexpr int kF32ApplyParts = 4; // partial states that the apply kernel adds up itself
+
+__device__ __forceinline__ void cp_async16(void* dst, const void* src, bool valid) {   // zero-filled when not valid
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(valid ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+// ---------------------------------------------------------------------------
+// state kernel: grid (BH * P); CTA bh * P + p covers tokens [p * chunk, min(N, (p + 1) * chunk))
+// ---------------------------------------------------------------------------
+template <int D> struct StateGeo {
+    static constexpr int kSide = D / 8, kGroup = kSide * kSide, G = kThreads / kGroup;   // threads per group, groups
+    static constexpr int kChunks = D / 4, kRowsPass = kThreads / kChunks, kPasses = kTok / kRowsPass;   // 16-byte chunks
+    static constexpr int kTileBytes = kTok * D * 4;
+    static constexpr size_t kSmem = (size_t)(4 * kTileBytes > G * D * D * 4 ? 4 * kTileBytes : G * D * D * 4);   // K, V twice
+};
+
+template <int D, bool RN>
+__global__ void __launch_bounds__(kThreads, D == 128 ? 1 : 2)
+f32_state_kernel(const float* __restrict__ k, const float* __restrict__ v, float* __restrict__ dst, int N, int chunk, int P,
+                 float eps2, Layout lk, Layout lv, int hdiv) {
+    using G = StateGeo<D>;
+    constexpr int kWords = D * D + D + (RN ? D : 0);
+    extern __shared__ __align__(16) float smem[];
+    const int tid = threadIdx.x, p = blockIdx.x % P, bh = blockIdx.x / P;
+    const int n_begin = p * chunk, n_end = min(N, n_begin + chunk);
+    // loading: thread = 16-byte chunk lc of rows lr, lr + kRowsPass, ...
+    const int lc = tid % G::kChunks, lr = tid / G::kChunks;
+    const float* kb = k + plane_offset(lk, bh, hdiv) + lc * 4;
+    const float* vb = v + plane_offset(lv, bh, hdiv) + lc * 4;
+    float4 kreg[G::kPasses];
+    float4 vsum = make_float4(0.f, 0.f, 0.f, 0.f), ksum = vsum;
+    auto fetch = [&](int n0, int buf) {   // V straight to shared memory, K to registers
+        float* vs = smem + (2 * buf + 1) * (kTok * D);
+#pragma unroll
+        for (int r = 0; r < G::kPasses; ++r) {
+            const int row = lr + r * G::kRowsPass, n = n0 + row;
+            const bool ok = n < n_end;
+            const long long off = ok ? n : n_begin;
+            kreg[r] = ok ? __ldg(reinterpret_cast<const float4*>(kb + off * lk.token)) : make_float4(0.f, 0.f, 0.f, 0.f);
+            cp_async16(vs + row * D + lc * 4, vb + off * lv.token, ok);
+        }
+        cp_async_commit();
+    };
+    auto store_k = [&](int buf) {   // unit rows to shared memory
+        float* ks = smem + 2 * buf * (kTok * D);
+#pragma unroll
+        for (int r = 0; r < G::kPasses; ++r) {
+            float4 x = kreg[r];
+            float ss = fmaf(x.x, x.x, fmaf(x.y, x.y, fmaf(x.z, x.z, x.w * x.w)));
+#pragma unroll
+            for (int o = G::kChunks / 2; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+            const float rk = 1.0f / sqrtf(fmaxf(ss, eps2));
+            x.x *= rk; x.y *= rk; x.z *= rk; x.w *= rk;
+            if (RN) { ksum.x += x.x; ksum.y += x.y; ksum.z += x.z; ksum.w += x.w; }
+            *reinterpret_cast<float4*>(ks + (lr + r * G::kRowsPass) * D + lc * 4) = x;
+        }
+    };
+    // computing: group g takes tokens g, g + G, ...; a thread owns rows 8 ti .. and columns {4 tj .., D/2 + 4 tj ..} of S
+    const int g = tid / G::kGroup, t = tid % G::kGroup, ti = t / G::kSide, tj = t % G::kSide;
+    // where a warp holds two groups (D = 32), whose rows lie in the same banks, the odd one takes its halves in reverse order
+    const bool flip = G::kGroup < 32 && (g & 1);
+    const int row_a = ti * 8 + (flip ? 4 : 0), row_b = ti * 8 + (flip ? 0 : 4);
+    const int col_a = tj * 4 + (flip ? D / 2 : 0), col_b = tj * 4 + (flip ? 0 : D / 2);
+    float2 acc[8][4];
+#pragma unroll
+    for (int a = 0; a < 8; ++a)
+#pragma unroll
+        for (int b = 0; b < 4; ++b) acc[a][b] = make_float2(0.f, 0.f);
+
+    pdl_wait_primary();
+    pdl_launch_dependents();
+    fetch(n_begin, 0);
+    int buf = 0;
+    for (int n0 = n_begin; n0 < n_end; n0 += kTok, buf ^= 1) {
+        store_k(buf);
+        cp_async_wait<0>();
+        __syncthreads();   // this tile is in shared memory; every thread has left the previous one
+        if (n0 + kTok < n_end) fetch(n0 + kTok, buf ^ 1);
+        const float* ks = smem + 2 * buf * (kTok * D);
+        const float* vs = ks + kTok * D;
+#pragma unroll 2
+        for (int n = g; n < kTok; n += G::G) {
+            const float4 a0 = *reinterpret_cast<const float4*>(ks + n * D + row_a);
+            const float4 a1 = *reinterpret_cast<const float4*>(ks + n * D + row_b);
+            const float4 b0 = *reinterpret_cast<const float4*>(vs + n * D + col_a);
+            const float4 b1 = *reinterpret_cast<const float4*>(vs + n * D + col_b);
+            const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+            const float2 b[4] = {make_float2(b0.x, b0.y), make_float2(b0.z, b0.w), make_float2(b1.x, b1.y), make_float2(b1.z, b1.w)};
+#pragma unroll
+            for (int x = 0; x < 8; ++x)
+#pragma unroll
+                for (int y = 0; y < 4; ++y) acc[x][y] = ffma2(make_float2(a[x], a[x]), b[y], acc[x][y]);
+        }
+        // the thread's own columns of V: rows it loaded itself, so its asynchronous copies are complete
+#pragma unroll
+        for (int r = 0; r < G::kPasses; ++r) {
+            const float4 x = *reinterpret_cast<const float4*>(vs + (lr + r * G::kRowsPass) * D + lc * 4);
+            vsum.x += x.x; vsum.y += x.y; vsum.z += x.z; vsum.w += x.w;
+        }
+    }
+    float* out = dst + ((size_t)bh * P + p) * kWords;
+    // groups meet in shared memory, in their order
+    __syncthreads();
+#pragma unroll
+    for (int x = 0; x < 8; ++x) {
+        float* row = smem + (g * D + (x < 4 ? row_a + x : row_b + x - 4)) * D;
+        *reinterpret_cast<float4*>(row + col_a) = make_float4(acc[x][0].x, acc[x][0].y, acc[x][1].x, acc[x][1].y);
+        *reinterpret_cast<float4*>(row + col_b) = make_float4(acc[x][2].x, acc[x][2].y, acc[x][3].x, acc[x][3].y);
+    }
+    __syncthreads();
+    for (int i = tid * 4; i < D * D; i += kThreads * 4) {
+        float4 s = *reinterpret_cast<const float4*>(smem + i);
+#pragma unroll
+        for (int h = 1; h < G::G; ++h) {
+            const float4 x = *reinterpret_cast<const float4*>(smem + h * D * D + i);
+            s.x += x.x; s.y += x.y; s.z += x.z; s.w += x.w;
+        }
+        *reinterpret_cast<float4*>(out + i) = s;
+    }
+    __syncthreads();
+    *reinterpret_cast<float4*>(smem + lr * D + lc * 4) = vsum;
+    if (RN) *reinterpret_cast<float4*>(smem + (G::kRowsPass + lr) * D + lc * 4) = ksum;
+    __syncthreads();
+    if (tid < (RN ? 2 * D : D)) {
+        const float* src = smem + (tid / D) * G::kRowsPass * D + tid % D;
+        float s = 0.f;
+#pragma unroll
+        for (int r = 0; r < G::kRowsPass; ++r) s += src[r * D];
+        out[D * D + tid] = s;
+    }
+}
+
+// Sums P partial states per plane in index order; grid (BH, words / 256 rounded up).
+__global__ void __launch_bounds__(kThreads)
+f32_reduce_kernel(const float* __restrict__ partial, float* __restrict__ state, int words, int P) {
+    pdl_wait_primary();
+    pdl_launch_dependents();
+    const int i = blockIdx.y * kThreads + threadIdx.x;
+    if (i >= words) return;
+    const float* src = partial + (size_t)blockIdx.x * P * words + i;
+    float s = 0.f;
+#pragma unroll 8
+    for (int p = 0; p < P; ++p) s += __ldcg(src + (size_t)p * words);
+    state[(size_t)blockIdx.x * words + i] = s;
+}
+
+// ---------------------------------------------------------------------------
+// apply kernel: grid (BH * patches of a plane)
+// ---------------------------------------------------------------------------
+template <int D, int KS> struct ApplyGeo {
+    static constexpr int kCG = D / 4;                     // channel groups of four
+    static constexpr int kRuns = kThreads / kCG;          // runs of eight tokens
+    static constexpr int TX = kRuns, TY = 8;              // patch: 8 rows x TX columns (TX / 8 runs per row)
+    static constexpr int R = KS / 2, HX = TX + 2 * R, HY = TY + 2 * R;
+    static constexpr int kTokens = TX * TY;
+    static constexpr int LQ = D + 4;                      // padded Q rows: consecutive rows start 16 bytes apart in the banks
+    // S' | 1/2 s | bias | sum k^ | filters (tap-major) | 1/||q|| | 1 / row sum | Q | V
+    static constexpr int kOffC = D * D, kOffB = kOffC + D, kOffZ = kOffB + D, kOffW = kOffZ + D, kOffRq = kOffW + KS * KS * D;
+    static constexpr int kOffDen = kOffRq + kTokens, kOffQ = kOffDen + kTokens, kOffV = kOffQ + kTokens * LQ;
+    static constexpr size_t kSmem = sizeof(float) * (kOffV + HX * HY * D);
+    static_assert(kSmem <= 227 * 1024, "shared memory");
+};
+
+struct F32ApplyParams {
+    const float *q, *v, *w, *bias, *state;
+    float* out;
+    Layout lq, lv, lo;
+    int H, head0, hdiv, prefix, gridH, gridW, tilesX, patches;   // patches per plane: tiles, then one of leading tokens
+    int P;                 // partial states per plane to be summed here (1: the state is final)
+    float eps2;
+    int v_row0, v_rows;    // V holds v_rows grid rows, of which row v_row0 is grid row 0
+};
+
+template <int D, int KS, bool RN>
+__global__ void __launch_bounds__(kThreads, D == 128 ? 1 : 2)
+f32_apply_kernel(const F32ApplyParams prm) {
+    using G = ApplyGeo<D, KS>;
+    constexpr int kWords = D * D + D + (RN ? D : 0);
+    extern __shared__ __align__(16) float smem[];
+    float* S_sm = smem;
+    float* q_s = smem + G::kOffQ;
+    float* v_s = smem + G::kOffV;
+    const int tid = threadIdx.x, bh = blockIdx.x / prm.patches, patch = blockIdx.x % prm.patches;
+    const int h = (prm.head0 + bh) % prm.H, W = prm.gridW;
+    // the last patch of a plane with leading tokens holds those: no grid position, no convolution
+    const bool lead = prm.prefix > 0 && patch == prm.patches - 1;
+    const int py = patch / prm.tilesX, y0 = py * G::TY, x0 = (patch - py * prm.tilesX) * G::TX;
+    // token of the patch: row y, column x; in shared memory the j-th tokens of all runs are neighbours (row j * kRuns + run)
+    auto token_of = [&](int j, int run) -> int {   // token index of the sequence, or -1
+        if (lead) { const int n = run * 8 + j; return n < prm.prefix ? n : -1; }
+        const int y = y0 + run / (G::TX / 8), x = x0 + (run % (G::TX / 8)) * 8 + j;
+        return (y < prm.gridH && x < W) ? prm.prefix + y * W + x : -1;
+    };
+    const float* qp = prm.q + plane_offset(prm.lq, bh, prm.hdiv);
+    const float* vp = prm.v + plane_offset(prm.lv, bh, prm.hdiv) + prm.prefix * prm.lv.token;
+    // Q, V and the filters were there before the state kernel started
+    for (int c = tid; c < G::kTokens * G::kCG; c += kThreads) {
+        const int r = c / G::kCG, ch = (c % G::kCG) * 4, n = token_of(r / G::kRuns, r % G::kRuns);
+        cp_async16(q_s + r * G::LQ + ch, qp + (n < 0 ? 0 : n) * prm.lq.token + ch, n >= 0);
+    }
+    if (!lead) {
+        for (int c = tid; c < G::HX * G::HY * G::kCG; c += kThreads) {
+            const int r = c / G::kCG, ch = (c % G::kCG) * 4, vy = r / G::HX, y = y0 + vy - G::R + prm.v_row0, x = x0 + r - vy * G::HX - G::R;
+            const bool ok = (unsigned)y < (unsigned)prm.v_rows && (unsigned)x < (unsigned)W;
+            cp_async16(v_s + r * D + ch, vp + (ok ? y * W + x : 0) * prm.lv.token + ch, ok);
+        }
+    }
+    cp_async_commit();
+    for (int i = tid; i < KS * KS * D; i += kThreads)
+        smem[G::kOffW + i] = __ldg(prm.w + ((size_t)(h * D + i % D)) * (KS * KS) + i / D);
+    if (tid < D) smem[G::kOffB + tid] = prm.bias ? __ldg(prm.bias + h * D + tid) : 0.f;
+    pdl_wait_primary();
+    pdl_launch_dependents();
+    {
+        const float* st = prm.state + (size_t)bh * prm.P * kWords;
+        for (int i = tid * 4; i < kWords; i += kThreads * 4) {
+            float4 s = __ldcg(reinterpret_cast<const float4*>(st + i));
+            for (int p = 1; p < prm.P; ++p) {
+                const float4 x = __ldcg(reinterpret_cast<const float4*>(st + (size_t)p * kWords + i));
+                s.x += x.x; s.y += x.y; s.z += x.z; s.w += x.w;
+            }
+            const float f = i < D * D ? kInvPi : i < D * D + D ? 0.5f : 1.0f;   // S / pi, 1/2 s, sum k^
+            float* dst = smem + (i < D * D + D ? i : G::kOffZ + i - D * D - D);
+            *reinterpret_cast<float4*>(dst) = make_float4(s.x * f, s.y * f, s.z * f, s.w * f);
+        }
+    }
+    cp_async_wait<0>();
+    __syncthreads();
+    {   // 1 / max(||q||, eps) of every token, two threads (or four, or eight) each
+        constexpr int L = kThreads / G::kTokens > 0 ? kThreads / G::kTokens : 1;
+        const int r = tid / L, l = tid % L;
+        float ss = 0.f, dot = 0.f;
+#pragma unroll 4
+        for (int i = l * 4; i < D; i += L * 4) {
+            const float4 x = *reinterpret_cast<const float4*>(q_s + r * G::LQ + i);
+            ss = fmaf(x.x, x.x, fmaf(x.y, x.y, fmaf(x.z, x.z, fmaf(x.w, x.w, ss))));
+            if (RN) {
+                const float* z = smem + G::kOffZ + i;
+                dot = fmaf(x.x, z[0], fmaf(x.y, z[1], fmaf(x.z, z[2], fmaf(x.w, z[3], dot))));
+            }
+        }
+#pragma unroll
+        for (int o = L / 2; o > 0; o >>= 1) {
+            ss += __shfl_xor_sync(0xffffffffu, ss, o);
+            if (RN) dot += __shfl_xor_sync(0xffffffffu, dot, o);
+        }
+        if (l == 0) {
+            const float rq = 1.0f / sqrtf(fmaxf(ss, prm.eps2));
+            smem[G::kOffRq + r] = rq;
+            // Eq. 3's denominator for the kept kernel of Eq. 8: N/2 + q^ . (sum_j k^_j) / pi
+            if (RN) smem[G::kOffDen + r] = 1.0f / fmaf(dot * rq, kInvPi, 0.5f * (float)(prm.prefix + prm.gridH * W));
+        }
+    }
+    __syncthreads();
+
+    const int cg = tid % G::kCG, run = tid / G::kCG;
+    float2 acc[8][2];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) acc[j][0] = acc[j][1] = make_float2(0.f, 0.f);
+#pragma unroll 2
+    for (int i = 0; i < D; i += 4) {
+        float4 a[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) a[j] = *reinterpret_cast<const float4*>(q_s + (j * G::kRuns + run) * G::LQ + i);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const float4 s = *reinterpret_cast<const float4*>(S_sm + (i + u) * D + cg * 4);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const float x = u == 0 ? a[j].x : u == 1 ? a[j].y : u == 2 ? a[j].z : a[j].w;
+                acc[j][0] = ffma2(make_float2(x, x), make_float2(s.x, s.y), acc[j][0]);
+                acc[j][1] = ffma2(make_float2(x, x), make_float2(s.z, s.w), acc[j][1]);
+            }
+        }
+    }
+    const float4 cs = *reinterpret_cast<const float4*>(smem + G::kOffC + cg * 4);
+    float4 bs = *reinterpret_cast<const float4*>(smem + G::kOffB + cg * 4);
+    if (lead) bs = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        const float rq = smem[G::kOffRq + j * G::kRuns + run], inv = RN ? smem[G::kOffDen + j * G::kRuns + run] : 1.0f;
+        if (RN) {
+            acc[j][0].x = fmaf(fmaf(acc[j][0].x, rq, cs.x), inv, bs.x); acc[j][0].y = fmaf(fmaf(acc[j][0].y, rq, cs.y), inv, bs.y);
+            acc[j][1].x = fmaf(fmaf(acc[j][1].x, rq, cs.z), inv, bs.z); acc[j][1].y = fmaf(fmaf(acc[j][1].y, rq, cs.w), inv, bs.w);
+        } else {
+            acc[j][0].x = fmaf(acc[j][0].x, rq, cs.x + bs.x); acc[j][0].y = fmaf(acc[j][0].y, rq, cs.y + bs.y);
+            acc[j][1].x = fmaf(acc[j][1].x, rq, cs.z + bs.z); acc[j][1].y = fmaf(acc[j][1].y, rq, cs.w + bs.w);
+        }
+    }
+    if (!lead) {
+        const float* vw = v_s + ((run / (G::TX / 8)) * G::HX + (run % (G::TX / 8)) * 8) * D + cg * 4;   // halo row 0, column 0
+#pragma unroll 1
+        for (int dy = 0; dy < KS; ++dy) {
+            float4 f[KS];
+#pragma unroll
+            for (int dx = 0; dx < KS; ++dx) f[dx] = *reinterpret_cast<const float4*>(smem + G::kOffW + (dy * KS + dx) * D + cg * 4);
+#pragma unroll
+            for (int c = 0; c < 8 + KS - 1; ++c) {
+                const float4 x = *reinterpret_cast<const float4*>(vw + (dy * G::HX + c) * D);
+#pragma unroll
+                for (int dx = 0; dx < KS; ++dx) {
+                    const int j = c - dx;   // compile-time after unrolling
+                    if (j < 0 || j >= 8) continue;
+                    acc[j][0] = ffma2(make_float2(f[dx].x, f[dx].y), make_float2(x.x, x.y), acc[j][0]);
+                    acc[j][1] = ffma2(make_float2(f[dx].z, f[dx].w), make_float2(x.z, x.w), acc[j][1]);
+                }
+            }
+        }
+    }
+    float* op = prm.out + plane_offset(prm.lo, bh, prm.hdiv) + cg * 4;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        const int n = token_of(j, run);
+        if (n >= 0) *reinterpret_cast<float4*>(op + n * prm.lo.token) = make_float4(acc[j][0].x, acc[j][0].y, acc[j][1].x, acc[j][1].y);
+    }
+}
+
+template <typename Kernel, typename... Args>
+cudaError_t launch_pdl(Kernel kernel, dim3 grid, size_t smem, cudaStream_t st, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid; cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = smem; cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+template <int D, int KS, bool RN>
+cudaError_t launch_f32(const Problem& p, float* ws_state, float* ws_partial, int P, cudaStream_t st, int* launches, KernelTimer* timer) {
+    constexpr int kWords = D * D + D + (RN ? D : 0);
+    const float* state = ws_state;
+    int apply_parts = 1;
+    cudaError_t e;
+    if (p.phase != kPhaseApplyOnly) {
+        const int tiles = (p.N + kTok - 1) / kTok, per = (tiles + P - 1) / P;
+        P = (tiles + per - 1) / per;   // every split has tokens
+        using G = StateGeo<D>;
+        static PerDevice opt_in;
+        e = opt_in_smem(f32_state_kernel<D, RN>, G::kSmem, opt_in);
+        if (e != cudaSuccess) return e;
+        e = launch_pdl(f32_state_kernel<D, RN>, dim3((unsigned)(p.BH * P)), G::kSmem, st, static_cast<const float*>(p.k),
+                       static_cast<const float*>(p.v), P > 1 ? ws_partial : ws_state, p.N, per * kTok, P, p.eps2, p.lk, p.lv, p.hdiv);
+        if (e != cudaSuccess) return e;
+        ++*launches;
+        timer->mark(st, "f32_state");
+        if (P > kF32ApplyParts || (P > 1 && p.phase == kPhaseStateOnly)) {
+            e = launch_pdl(f32_reduce_kernel, dim3((unsigned)p.BH, (kWords + kThreads - 1) / kThreads), 0, st, ws_partial, ws_state, kWords, P);
+            if (e != cudaSuccess) return e;
+            ++*launches;
+            timer->mark(st, "f32_reduce");
+        } else if (P > 1) {
+            state = ws_partial;   // few parts: the apply kernel adds them as it reads them
+            apply_parts = P;
+        }
+        if (p.phase == kPhaseStateOnly) return cudaSuccess;
+    }
+    using A = ApplyGeo<D, KS>;
+    F32ApplyParams prm;
+    prm.q = static_cast<const float*>(p.q); prm.v = static_cast<const float*>(p.v);
+    prm.w = static_cast<const float*>(p.w); prm.bias = static_cast<const float*>(p.bias);
+    prm.state = state; prm.out = static_cast<float*>(p.out);
+    prm.lq = p.lq; prm.lv = p.lv; prm.lo = p.lo;
+    prm.H = p.H; prm.head0 = p.head0; prm.hdiv = p.hdiv; prm.prefix = p.prefix; prm.gridH = p.gridH; prm.gridW = p.gridW;
+    prm.tilesX = (p.gridW + A::TX - 1) / A::TX;
+    prm.patches = prm.tilesX * ((p.gridH + A::TY - 1) / A::TY) + (p.prefix > 0 ? 1 : 0);
+    prm.P = apply_parts; prm.eps2 = p.eps2;
+    prm.v_row0 = p.v_row0; prm.v_rows = p.v_rows > 0 ? p.v_rows : p.gridH;
+    static PerDevice opt_in;
+    e = opt_in_smem(f32_apply_kernel<D, KS, RN>, A::kSmem, opt_in);
+    if (e != cudaSuccess) return e;
+    e = launch_pdl(f32_apply_kernel<D, KS, RN>, dim3((unsigned)(p.BH * prm.patches)), A::kSmem, st, prm);
+    if (e != cudaSuccess) return e;
+    ++*launches;
+    timer->mark(st, "f32_apply");
+    return cudaSuccess;
+}
+
+template <int D>
+cudaError_t launch_f32_d(const Problem& p, float* s, float* part, int P, cudaStream_t st, int* n, KernelTimer* t) {
+    if (p.ksize == 3) return p.rownorm ? launch_f32<D, 3, true>(p, s, part, P, st, n, t) : launch_f32<D, 3, false>(p, s, part, P, st, n, t);
+    return p.rownorm ? launch_f32<D, 5, true>(p, s, part, P, st, n, t) : launch_f32<D, 5, false>(p, s, part, P, st, n, t);
+}
+
+}  // namespace
+
+bool f32_supports(const Problem& p) { return !p.bf16 && f32_width(p.d) && (p.ksize == 3 || p.ksize == 5); }
+
+// Token splits of the state kernel: two CTAs per multiprocessor, at least one tile each.  Up to kF32ApplyParts of them need
+// no reduction in between.
+int f32_choose_splits(int BH, int N) {
+    const int tiles = (N + kTok - 1) / kTok;
+    int P = 2 * device_sm_count() / BH;
+    if (P > tiles) P = tiles;
+    if (P > 64) P = 64;
+    return P < 1 ? 1 : P;
+}
+
+cudaError_t f32_forward(const Problem& p, float* ws_state, float* ws_partial, int P, cudaStream_t stream, int* launches,
+                        KernelTimer* timer) {
+    *launches = 0;
+    if (p.d == 32) return launch_f32_d<32>(p, ws_state, ws_partial, P, stream, launches, timer);
+    if (p.d == 64) return launch_f32_d<64>(p, ws_state, ws_partial, P, stream, launches, timer);
+    return launch_f32_d<128>(p, ws_state, ws_partial, P, stream, launches, timer);
+}
+
+}  // namespace castling

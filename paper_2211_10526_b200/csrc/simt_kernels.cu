@@ -1,7 +1,8 @@
 // CUDA-core (FMA) kernels of the linear-angular attention core.
 //
-// These cover every supported dtype, head width and filter size; the fp32 I/O
-// path always runs here because its 1e-5 tolerance rules out bf16 operands.
+// These cover every supported dtype, head width and filter size; fp32 heads of width
+// 32, 64 and 128 with 3x3 or 5x5 filters have kernels of their own (f32_kernels.cu) unless
+// the single-launch kernel takes them.
 //
 //   state kernel  : per (b,h) and token split, k^ = k / max(||k||, eps),
 //                   S += k^^T v (d x d), s += v           (Eq. 9, K^T V and the 1/2 term)
@@ -490,6 +491,7 @@ cudaError_t launch_simt(const Problem& p, float* ws_state, float* ws_partial, in
         timer->mark(stream, "simt_fused");
         return e;
     }
+    if (f32_supports(p)) return f32_forward(p, ws_state, ws_partial, P, stream, launches, timer);
     cudaError_t e = cudaSuccess;
     if (p.phase != kPhaseApplyOnly) {
         const int tiles = (p.N + kStateTile - 1) / kStateTile;
@@ -545,7 +547,8 @@ bool simt_supports(int d, int ksize) {
 
 // Token splits of the state kernel: enough CTAs to fill the device about twice over,
 // at least four staged tiles per split, capped at 64.
-int simt_choose_splits(int BH, int N) {
+int simt_choose_splits(int BH, int N, int d, bool bf16) {
+    if (!bf16 && f32_width(d)) return f32_choose_splits(BH, N);
     const int tiles = (N + kStateTile - 1) / kStateTile;
     int P = (2 * device_sm_count() + BH - 1) / BH;
     if (P > tiles / 4) P = tiles / 4;
