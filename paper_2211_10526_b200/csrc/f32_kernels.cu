@@ -1,6 +1,6 @@
 // fp32 kernels of the linear-angular attention core for head widths 32, 64 and 128 and 3x3 or 5x5 filters (the 1e-5
 // tolerance rules out bf16 operands; every other fp32 shape runs on simt_kernels.cu):
-//   state kernel  S += k^^T v, s += v per (plane, token split): 64-token tiles, K scaled to unit rows on its way to shared
+//   state kernel  S += k^^T v, s += v per (plane, token split): tiles of 64 tokens (128 at D = 32), K scaled to unit rows on its way to shared
 //                 memory, the next tile's loads in flight; a thread owns 8 x 8 of S and every G-th token (G groups of
 //                 (D/8)^2 threads), the groups meet in shared memory at the end
 //   apply kernel  a patch of 8 rows x TX columns of tokens: Q, V with halo and S' = S / pi in shared memory (asynchronous
@@ -11,7 +11,7 @@
 // kernel, 128 per twelve in the apply kernel.
 // Measured: 2 x 8 planes of 128 x 128, d = 64: 155 us per forward (392 on the kernels of simt_kernels.cu, whose threads issued 28
 // instructions and eight 4-byte loads for 16 FMAs and read the convolution's window from global memory); 2 x 4 planes of 14 x 14,
-// d = 32: 8.5 us in a replayed graph (22.7: one CTA per plane walked through seven tiles with three barriers and a trip to
+// d = 32: 10.3 us in a replayed graph (22.7: one CTA per plane walked through seven tiles with three barriers and a trip to
 // memory each).
 #include "tc_common.cuh"
 #include "tc_host.cuh"
@@ -25,7 +25,6 @@ using tc::pdl_wait_primary;
 using tc::smem_u32;
 
 constexpr int kThreads = 256;
-constexpr int kTok = 64;          // tokens per tile of the state kernel
 constexpr int kF32ApplyParts = 4; // partial states that the apply kernel adds up itself
 
 __device__ __forceinline__ void cp_async16(void* dst, const void* src, bool valid) {   // zero-filled when not valid
@@ -38,6 +37,7 @@ template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile(
 // state kernel: grid (BH * P); CTA bh * P + p covers tokens [p * chunk, min(N, (p + 1) * chunk))
 // ---------------------------------------------------------------------------
 template <int D> struct StateGeo {
+    static constexpr int kTok = D == 32 ? 128 : 64;   // tokens per tile
     static constexpr int kSide = D / 8, kGroup = kSide * kSide, G = kThreads / kGroup;   // threads per group, groups
     static constexpr int kChunks = D / 4, kRowsPass = kThreads / kChunks, kPasses = kTok / kRowsPass;   // 16-byte chunks
     static constexpr int kTileBytes = kTok * D * 4;
@@ -49,7 +49,7 @@ __global__ void __launch_bounds__(kThreads, D == 128 ? 1 : 2)
 f32_state_kernel(const float* __restrict__ k, const float* __restrict__ v, float* __restrict__ dst, int N, int chunk, int P,
                  float eps2, Layout lk, Layout lv, int hdiv) {
     using G = StateGeo<D>;
-    constexpr int kWords = D * D + D + (RN ? D : 0);
+    constexpr int kWords = D * D + D + (RN ? D : 0), kTok = G::kTok;
     extern __shared__ __align__(16) float smem[];
     const int tid = threadIdx.x, p = blockIdx.x % P, bh = blockIdx.x / P;
     const int n_begin = p * chunk, n_end = min(N, n_begin + chunk);
@@ -363,14 +363,14 @@ cudaError_t launch_f32(const Problem& p, float* ws_state, float* ws_partial, int
     int apply_parts = 1;
     cudaError_t e;
     if (p.phase != kPhaseApplyOnly) {
-        const int tiles = (p.N + kTok - 1) / kTok, per = (tiles + P - 1) / P;
-        P = (tiles + per - 1) / per;   // every split has tokens
         using G = StateGeo<D>;
+        const int tiles = (p.N + G::kTok - 1) / G::kTok, per = (tiles + P - 1) / P;
+        P = (tiles + per - 1) / per;   // every split has tokens
         static PerDevice opt_in;
         e = opt_in_smem(f32_state_kernel<D, RN>, G::kSmem, opt_in);
         if (e != cudaSuccess) return e;
         e = launch_pdl(f32_state_kernel<D, RN>, dim3((unsigned)(p.BH * P)), G::kSmem, st, static_cast<const float*>(p.k),
-                       static_cast<const float*>(p.v), P > 1 ? ws_partial : ws_state, p.N, per * kTok, P, p.eps2, p.lk, p.lv, p.hdiv);
+                       static_cast<const float*>(p.v), P > 1 ? ws_partial : ws_state, p.N, per * G::kTok, P, p.eps2, p.lk, p.lv, p.hdiv);
         if (e != cudaSuccess) return e;
         ++*launches;
         timer->mark(st, "f32_state");
@@ -416,12 +416,11 @@ cudaError_t launch_f32_d(const Problem& p, float* s, float* part, int P, cudaStr
 
 bool f32_supports(const Problem& p) { return !p.bf16 && f32_width(p.d) && (p.ksize == 3 || p.ksize == 5); }
 
-// Token splits of the state kernel: two CTAs per multiprocessor, at least one tile each.  Up to kF32ApplyParts of them need
-// no reduction in between.
+// Token splits of the state kernel: two CTAs per multiprocessor, at least 128 tokens each (the states of smaller grids need
+// no workspace beyond the final one).  Up to kF32ApplyParts of them need no reduction in between.
 int f32_choose_splits(int BH, int N) {
-    const int tiles = (N + kTok - 1) / kTok;
     int P = 2 * device_sm_count() / BH;
-    if (P > tiles) P = tiles;
+    if (P > N / 128) P = N / 128;
     if (P > 64) P = 64;
     return P < 1 ? 1 : P;
 }
