@@ -1,11 +1,17 @@
 """Convenience wrapper: torch tensors in, torch tensor out, all arithmetic in the CUDA library."""
 from __future__ import annotations
 
+import ctypes
 from typing import Optional
 
 import torch
 
 from . import binding as _b
+from . import _torch_call   # C++: checks, strides, output and stream of a device forward (raises if it is not built)
+
+_torch_call.bind(ctypes.cast(_b.lib.castling_attn_forward, ctypes.c_void_p).value,
+                 ctypes.cast(_b.lib.castling_attn_forward_strided, ctypes.c_void_p).value)
+_forward = _torch_call.forward
 
 
 def _dtype_code(t: torch.Tensor) -> int:
@@ -64,61 +70,36 @@ class CastlingAttn:
     def handle(self) -> int:
         return self._h
 
-    def _check(self, q, k, v, w, bias, out, gridH, gridW, device_type):
-        # straight-line on purpose: this runs on every call and small shapes are bound by host time
+    def _check_host(self, q, k, v, w, bias, out, gridH, gridW):
         shape = q.shape
         if len(shape) != 4 or k.shape != shape or v.shape != shape or out.shape != shape:
             raise ValueError("q, k, v, out must share one [B, H, N, d] shape")
         B, H, N, d = shape
         if N != self.prefix_tokens + gridH * gridW:
             raise ValueError("N != prefix_tokens + gridH * gridW")
-        ks = self.ksize
-        if w.shape != (H * d, ks, ks):
+        if w.shape != (H * d, self.ksize, self.ksize):
             raise ValueError("dw_weight must be [H*d, ksize, ksize]")
-        dt = q.dtype
-        if bias is not None:
-            if bias.shape != (H * d,):
-                raise ValueError("dw_bias must be [H*d]")
-            if bias.device.type != device_type or not bias.is_contiguous() or bias.dtype != dt:
-                raise ValueError(f"dw_bias must be a contiguous {device_type} tensor of the tensors' dtype")
-        if not (q.device.type == k.device.type == v.device.type == w.device.type == out.device.type == device_type):
-            raise ValueError(f"expected {device_type} tensors")
-        if not w.is_contiguous():
-            raise ValueError("dw_weight must be contiguous")
-        if not (q.is_contiguous() and k.is_contiguous() and v.is_contiguous() and out.is_contiguous()):
-            if device_type != "cuda":
-                raise ValueError("host tensors must be contiguous")
-            for t in (q, k, v, out):
-                if t.stride(3) != 1:
-                    raise ValueError("the d elements of a token must be contiguous (stride 1 in the last dimension)")
-        if not (k.dtype == dt and v.dtype == dt and w.dtype == dt and out.dtype == dt):
-            raise TypeError("all tensors must share one dtype")
+        if bias is not None and bias.shape != (H * d,):
+            raise ValueError("dw_bias must be [H*d]")
+        for t in (q, k, v, w, out) + (() if bias is None else (bias,)):
+            if t.device.type != "cpu" or not t.is_contiguous():
+                raise ValueError("host tensors must be contiguous tensors on the cpu")
+            if t.dtype != q.dtype:
+                raise TypeError("all tensors must share one dtype")
         return B, H, N, d
 
     def forward(self, q, k, v, dw_weight, dw_bias: Optional[torch.Tensor], gridH: int, gridW: int,
                 out: Optional[torch.Tensor] = None) -> torch.Tensor:
-        if out is None:
-            out = torch.empty_like(q)
-        B, H, N, d = self._check(q, k, v, dw_weight, dw_bias, out, gridH, gridW, "cuda")
-        stream = _current_raw_stream(q.device)
-        bias_ptr = None if dw_bias is None else dw_bias.data_ptr()
-        if q.is_contiguous() and k.is_contiguous() and v.is_contiguous() and out.is_contiguous():
-            rc = _b.castling_attn_forward(self._h, q.data_ptr(), k.data_ptr(), v.data_ptr(), dw_weight.data_ptr(),
-                                          bias_ptr, out.data_ptr(), B, H, gridH, gridW, d, _dtype_code(q), stream)
-        else:  # views of token-major or fused-projection buffers: pass their strides through
-            strides = [s for t in (q, k, v, out) for s in t.stride()[:3]]
-            rc = _b.castling_attn_forward_strided(self._h, q.data_ptr(), k.data_ptr(), v.data_ptr(),
-                                                  dw_weight.data_ptr(), bias_ptr, out.data_ptr(), B, H, gridH, gridW,
-                                                  d, _dtype_code(q), strides, stream)
-        if rc != _b.OK:
-            raise _b.CastlingError(rc, "castling_attn_forward")
-        return out
+        r = _forward(self._h, self.ksize, self.prefix_tokens, q, k, v, dw_weight, dw_bias, gridH, gridW, out)
+        if r.__class__ is int:
+            raise _b.CastlingError(r, "castling_attn_forward")
+        return r
 
     def forward_host(self, q, k, v, dw_weight, dw_bias: Optional[torch.Tensor], gridH: int, gridW: int,
                      out: Optional[torch.Tensor] = None, stream: int = 0) -> torch.Tensor:
         if out is None:
             out = torch.empty_like(q)
-        B, H, N, d = self._check(q, k, v, dw_weight, dw_bias, out, gridH, gridW, "cpu")
+        B, H, N, d = self._check_host(q, k, v, dw_weight, dw_bias, out, gridH, gridW)
         rc = _b.castling_attn_forward_host(self._h, q.data_ptr(), k.data_ptr(), v.data_ptr(), dw_weight.data_ptr(),
                                            None if dw_bias is None else dw_bias.data_ptr(), out.data_ptr(),
                                            B, H, gridH, gridW, d, _dtype_code(q), stream)
