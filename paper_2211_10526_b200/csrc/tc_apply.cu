@@ -6,13 +6,16 @@
 //               the convolution's zero padding
 //   warp 1      one thread issues four UMMAs: acc[128 x 64] = Q[128 x 64] * S'[64 x 64] into TMEM,
 //               S' = S / pi in bf16; the row scale 1/||q|| commutes and is applied afterwards
-//   warps 10..17 depthwise convolution on CUDA cores, one lane per channel pair, filters in
-//               registers, sliding window along x (two rows x eight columns per warp), packed
-//               fp32x2 FMAs, result (+ 1/2 s + bias) staged in shared memory as fp32
+//   warps 10..17 depthwise convolution on CUDA cores, one lane per channel pair, filters in registers: two columns
+//               slide down the patch, every word of V is loaded (a row ahead) and unpacked once per pair of columns, sums
+//               of the KS open output rows in registers, packed fp32x2 FMAs, result (+ 1/2 s + bias) staged in shared
+//               memory as fp32
 //   warps 2..9  one thread per token and half of its channels: ||q|| from the Q patch (each of
 //               the two warps of a token sums half of the row, exchanged through shared memory),
 //               accumulator row from TMEM, out = acc / max(||q||, eps) + staged, one rounding to
 //               bf16, patch written to shared memory and stored with TMA (clipped at the grid edge)
+// Measured: 2 x 8 planes of 128 x 128 with 5 x 5 filters 56 us per forward, 8 x 8 planes of 64 x 64 53 us (75 and 73 with a window
+// that slid along x: 8 halo rows of 5 columns and the filters did not fit the registers); 3 x 3, 256 x 256: 125.0 us (127.5).
 #include "tc_common.cuh"
 #include "tc_host.cuh"
 
@@ -29,12 +32,13 @@ constexpr int kStgBytes = kTile * kStgStride;
 constexpr int kEpiWarps = 8;                   // two warps per TMEM lane quarter
 constexpr int kEpiThreads = kEpiWarps * 32;
 constexpr int kTmemCols = 128;              // two 64-column accumulators
+constexpr int kCols = 2;                    // columns a convolution warp takes down the patch at a time
 
 template <int KS> struct Geo {
-    // conv warps: each takes kConvRows patch rows x 8 columns.  3x3: 8 warps of 2 rows; 5x5: 4 warps of
-    // 4 rows (fewer redundant window loads, and the larger window fits the registers of 448 threads)
-    static constexpr int kConvRows = (KS == 3) ? 2 : 4;
-    static constexpr int kConvWarps = 2 * kTY / kConvRows, kConvThreads = kConvWarps * 32;
+    // 3 x 3: 8 convolution warps of two columns (96 registers per thread); 5 x 5: 4 warps of four columns, in two steps
+    // (the filters alone take 50 registers: 128 per thread)
+    static constexpr int kConvWarps = KS == 3 ? 8 : 4, kConvThreads = kConvWarps * 32;
+    static constexpr int kGroups = kTX / (kCols * kConvWarps);
     static constexpr int kThreads = 64 + kEpiThreads + kConvThreads;
     static constexpr int R = KS / 2;
     static constexpr int HY = kTY + 2 * R, HX = kTX + 2 * R;
@@ -306,10 +310,9 @@ tc_apply_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
         }
         if (leader) tma_store_wait_all();
     } else {
-        // ------- depthwise convolution: lane = channel pair, warp = two patch rows x eight columns -------
-        const int cw = (warp - 2 - kEpiWarps) >> 1, xh = (warp - 2 - kEpiWarps) & 1;
-        constexpr int kCX = kTX / 2;
-        constexpr int R = G::R, RO = G::kConvRows, ROWS = RO + 2 * R;
+        // ------- depthwise convolution: lane = channel pair, two columns at a time down the patch -------
+        const int cw = warp - 2 - kEpiWarps;
+        constexpr int NIN = kCols - 1 + KS;   // columns of V that kCols output columns need
         float2 wreg[KS][KS];
         float2 cinit = make_float2(0.f, 0.f), hs2 = make_float2(0.f, 0.f);
         int prev_bh = -1;
@@ -335,39 +338,46 @@ tc_apply_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
             }
             if (!mbar_wait(&full[s], use & 1, abort_flag, prm.status, kBit)) break;
             if (ub > 0 && !mbar_wait(&buf_free[b], (ub - 1) & 1, abort_flag, prm.status, kBit)) break;
-            // Window of KS columns per halo row, sliding along x; column x (relative to the first this lane needs) lives in
-            // slot x % KS (compile-time after unrolling).
-            const uint8_t* vh = stages + s * G::kStage + kQBytes + ((RO * cw) * G::HX + xh * kCX) * 128 + lane * 4;
-            uint8_t* so = stg + b * kStgBytes + ((RO * cw) * kTX + xh * kCX) * kStgStride + lane * 8;
-            float2 win[ROWS][KS];
+#pragma unroll 1
+            for (int g = 0; g < G::kGroups; ++g) {
+                const int x0 = (cw * G::kGroups + g) * kCols;   // first column
+                const uint8_t* vh = stages + s * G::kStage + kQBytes + x0 * 128 + lane * 4;
+                uint8_t* so = stg + b * kStgBytes + x0 * kStgStride + lane * 8;
+                float2 acc[KS][kCols];   // output row y in slot y % KS
+                uint32_t raw[NIN];       // the row's words, loaded a row ahead
 #pragma unroll
-            for (int t = 0; t < KS - 1; ++t)
+                for (int o = 0; o < NIN; ++o) raw[o] = lds32(vh + o * 128);
 #pragma unroll
-                for (int r = 0; r < ROWS; ++r) {
-                    const uint32_t wv = *reinterpret_cast<const uint32_t*>(vh + (r * G::HX + t) * 128);
-                    win[r][t] = make_float2(bf16lo(wv), bf16hi(wv));
-                }
+                for (int hy = 0; hy < G::HY; ++hy) {
+                    float2 in[NIN];
 #pragma unroll
-            for (int x = 0; x < kCX; ++x) {
+                    for (int o = 0; o < NIN; ++o) in[o] = make_float2(bf16lo(raw[o]), bf16hi(raw[o]));
+                    if (hy + 1 < G::HY) {
 #pragma unroll
-                for (int r = 0; r < ROWS; ++r) {
-                    const uint32_t wv = *reinterpret_cast<const uint32_t*>(vh + (r * G::HX + x + KS - 1) * 128);
-                    win[r][(x + KS - 1) % KS] = make_float2(bf16lo(wv), bf16hi(wv));
-                }
-                float2 acc[RO];
+                        for (int o = 0; o < NIN; ++o) raw[o] = lds32(vh + ((hy + 1) * G::HX + o) * 128);
+                    }
+                    if (hy < kTY) {      // output row hy starts here
 #pragma unroll
-                for (int r = 0; r < RO; ++r) acc[r] = cinit;
-#pragma unroll
-                for (int dy = 0; dy < KS; ++dy)
+                        for (int c = 0; c < kCols; ++c) acc[hy % KS][c] = cinit;
+                    }
+                    // taps in the outer loops: consecutive FMAs share the filter and go to different sums
 #pragma unroll
                     for (int dx = 0; dx < KS; ++dx)
 #pragma unroll
-                        for (int r = 0; r < RO; ++r)
-                            acc[r] = ffma2(wreg[dy][dx], win[dy + r][(x + dx) % KS], acc[r]);
+                        for (int dy = 0; dy < KS; ++dy) {
+                            const int y = hy - dy;   // compile-time after unrolling
+                            if (y < 0 || y >= kTY) continue;
 #pragma unroll
-                for (int r = 0; r < RO; ++r) *reinterpret_cast<float2*>(so + (r * kTX + x) * kStgStride) = acc[r];
+                            for (int c = 0; c < kCols; ++c) acc[y % KS][c] = ffma2(wreg[dy][dx], in[c + dx], acc[y % KS][c]);
+                        }
+                    if (hy >= KS - 1) {  // and output row hy - (KS - 1) ends here
+                        const int y = hy - (KS - 1);
+#pragma unroll
+                        for (int c = 0; c < kCols; ++c) *reinterpret_cast<float2*>(so + (y * kTX + c) * kStgStride) = acc[y % KS][c];
+                    }
+                }
             }
-            if (RN && cw == 0 && xh == 0) {
+            if (RN && cw == 0) {
                 // 1/2 s of the plane this patch belongs to, beside the staging buffer
                 *reinterpret_cast<float2*>(hs_s + b * kD + 2 * lane) = hs2;
             }

@@ -11,9 +11,10 @@
 //               word of V is loaded and unpacked once per pair of columns, sums of the KS open output rows in registers;
 //               result (+ 1/2 s + bias) staged in shared memory as fp32
 // Bound: issue slots of the convolution (per output pair of channels 9 packed FMAs and 11 other instructions at 3 x 3).
-// Measured (per forward with the state kernel): 8 x 8 planes of 50 x 75, 5 x 5 filters 39 us (245 on the CUDA-core kernels,
-// which took odd widths before); 64 x 64 32 us (37 with two tokens packed to a 128-byte row, where a lane's window slid two
-// tokens per output and loaded 4.3 words per output instead of 3.1, and two CTA-wide barriers joined the warps per patch).
+// Measured (per forward with the state kernel): 8 x 8 planes of 50 x 75, 5 x 5 filters 33 us (245 on the CUDA-core kernels,
+// which took odd widths before; 39 with the words of a row loaded right before their use: one convolution warp per scheduler
+// hides nothing); 64 x 64 28 us (37 with two tokens packed to a 128-byte row, where a lane's window slid two tokens per
+// output and loaded 4.3 words per output instead of 3.1, and two CTA-wide barriers joined the warps per patch).
 #include "tc_common.cuh"
 #include "tc_host.cuh"
 
@@ -294,26 +295,33 @@ tc_apply32_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                 const uint8_t* vh = stages + s * G::kStage + kQBytes + x0 * 64 + cp * 4;
                 uint8_t* so = stg + b * kStgBytes + x0 * kStgStride + cp * 8;
                 float2 acc[KS][kCols];   // output row y in slot y % KS
+                uint32_t raw[NIN];       // the row's words, loaded a row ahead
+#pragma unroll
+                for (int o = 0; o < NIN; ++o) raw[o] = lds32(vh + o * 64);
 #pragma unroll
                 for (int hy = 0; hy < G::HY; ++hy) {
                     float2 in[NIN];
 #pragma unroll
-                    for (int o = 0; o < NIN; ++o) {
-                        const uint32_t wv = *reinterpret_cast<const uint32_t*>(vh + (hy * G::HX + o) * 64);
-                        in[o] = make_float2(bf16lo(wv), bf16hi(wv));
+                    for (int o = 0; o < NIN; ++o) in[o] = make_float2(bf16lo(raw[o]), bf16hi(raw[o]));
+                    if (hy + 1 < G::HY) {
+#pragma unroll
+                        for (int o = 0; o < NIN; ++o) raw[o] = lds32(vh + ((hy + 1) * G::HX + o) * 64);
                     }
+                    if (hy < kTY) acc[hy % KS][0] = acc[hy % KS][1] = cinit;   // output row hy starts here
+                    // taps in the outer loop: consecutive FMAs go to different sums
 #pragma unroll
-                    for (int dy = KS - 1; dy >= 0; --dy) {
-                        const int y = hy - dy;   // compile-time after unrolling
-                        if (y < 0 || y >= kTY) continue;
+                    for (int dx = 0; dx < KS; ++dx)
 #pragma unroll
-                        for (int c = 0; c < kCols; ++c) {
-                            if (dy == 0) acc[y % KS][c] = cinit;
+                        for (int dy = 0; dy < KS; ++dy) {
+                            const int y = hy - dy;   // compile-time after unrolling
+                            if (y < 0 || y >= kTY) continue;
 #pragma unroll
-                            for (int dx = 0; dx < KS; ++dx) acc[y % KS][c] = ffma2(wreg[dy][dx], in[2 * c + dx], acc[y % KS][c]);
-                            if (dy == KS - 1)
-                                *reinterpret_cast<float2*>(so + (y * kTX + 2 * c) * kStgStride) = acc[y % KS][c];
+                            for (int c = 0; c < kCols; ++c) acc[y % KS][c] = ffma2(wreg[dy][dx], in[2 * c + dx], acc[y % KS][c]);
                         }
+                    if (hy >= KS - 1) {              // and output row hy - (KS - 1) ends here
+                        const int y = hy - (KS - 1);
+#pragma unroll
+                        for (int c = 0; c < kCols; ++c) *reinterpret_cast<float2*>(so + (y * kTX + 2 * c) * kStgStride) = acc[y % KS][c];
                     }
                 }
             }
