@@ -98,7 +98,7 @@ tc_apply_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     constexpr int kAcc = RN ? 2 * kD : kD;              // TMEM columns per accumulator
     constexpr int kAccN = RN ? kD + 16 : kD;            // columns the UMMAs write
     extern __shared__ uint8_t smem_raw[];
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    uint8_t* smem = align_smem(smem_raw);
     uint8_t* S_s = smem + G::kOffS;
     uint8_t* out_s = smem + G::kOffOut;
     uint8_t* stages = smem + G::kOffStages;

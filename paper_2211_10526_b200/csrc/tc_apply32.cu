@@ -72,7 +72,7 @@ tc_apply32_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
     constexpr int kAccTile = RN ? 2 * kD : kD, kAcc = 2 * kAccTile;
     constexpr int kTmemCols = 2 * kAcc;
     extern __shared__ uint8_t smem_raw[];
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    uint8_t* smem = align_smem(smem_raw);
     uint8_t* S_s = smem + G::kOffS;
     uint8_t* S2_s = smem + G::kOffS2;
     float* hs_s = reinterpret_cast<float*>(smem + G::kOffHs);   // [2][32]

@@ -132,7 +132,7 @@ tc_cluster_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant
     using G = Geo<KS, PAIR>;
     constexpr int NS = G::kStages, SNS = G::kSStages, NG = G::kNormGroups;
     extern __shared__ uint8_t smem_raw[];
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    uint8_t* smem = align_smem(smem_raw);
     // phase 3
     uint8_t* S_s = smem + G::kOffS;
     uint8_t* out_s = smem + G::kOffOut;

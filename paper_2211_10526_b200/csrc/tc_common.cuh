@@ -26,6 +26,10 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
+// The first 1024-byte boundary of the dynamic shared memory.  An offset, not a pointer made from an integer: that would lose
+// the address space, and every access would become a generic one (slower, and tracked with the loads from global memory).
+__device__ __forceinline__ uint8_t* align_smem(uint8_t* smem_raw) { return smem_raw + (-smem_u32(smem_raw) & 1023u); }
+
 __device__ __forceinline__ unsigned long long global_ns() {
     unsigned long long t;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));

@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                const __grid_constant__ CUtensorMap tmV, const QuadParams prm) {
     extern __shared__ uint8_t smem_raw[];
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    uint8_t* smem = align_smem(smem_raw);
     uint8_t* Q_s = smem + kOffQ;
     uint8_t* K_s = smem + kOffK;
     uint8_t* V_s = smem + kOffV;

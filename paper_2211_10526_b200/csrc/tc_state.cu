@@ -39,7 +39,7 @@ tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
                 float* __restrict__ dst, float* __restrict__ final_state, unsigned* __restrict__ counters,
                 int N, int tiles_per_cta, int P, int BH, int hdiv, int items_per_cta, float eps2, unsigned* status) {
     extern __shared__ uint8_t smem_raw[];
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    uint8_t* smem = align_smem(smem_raw);
     uint8_t* ones = smem + kStages * kStageBytes;
     uint64_t* full = reinterpret_cast<uint64_t*>(ones + kOnesBytes);  // TMA bytes landed
     uint64_t* scaled = full + kStages;                                // K rows normalised (128 arrivals)
