@@ -14,11 +14,10 @@
 //               contraction and s as fp32
 //   warp 1      apply UMMAs: acc[tile] = Q[tile] * S' into TMEM (the state's columns are reused)
 //   warps 2..9  thread = token: accumulator rows from TMEM to shared memory as fp32 (over the swizzled
-//               V tile and the Q tile, both dead by then); then lane = channel pair, warp = a run of
-//               eight tokens of one grid row: depthwise convolution with the filters in registers and a
-//               sliding window along x, out = acc / max(||q||, eps) + 1/2 s + bias + conv, one rounding
-//               to bf16, 128-byte rows stored straight to memory; leading off-grid tokens get the
-//               attention terms only
+//               V tile and the Q tile, both dead by then); then lane = channel pair, warp = a strip of two
+//               columns: depthwise convolution sliding down the strip with the filters in registers,
+//               out = acc / max(||q||, eps) + 1/2 s + bias + conv, one rounding to bf16, 128-byte rows stored
+//               straight to memory; leading off-grid tokens get the attention terms only
 #include "tc_common.cuh"
 #include "tc_host.cuh"
 
@@ -34,19 +33,18 @@ constexpr int kBufBytes = kMaxTiles * kTileBytes;
 constexpr int kWorkers = 256;                    // warps 2..9
 constexpr int kThreads = 64 + kWorkers;
 constexpr int kTmemCols = 128;                   // [0,64): state, then tile 0 of the output; [64,128): tile 1
-constexpr int kSeg = 8;                          // tokens of one grid row per convolution unit
 
-// Shared memory: K | V | Q | S' | ones | rq | s | zeros | barriers.  After their first use the buffers change
+// Shared memory: K | V | Q | S' | ones | rq | s | barriers.  After their first use the buffers change
 // role: K holds the unswizzled V plane, V and Q hold the fp32 accumulator rows of tiles 0 and 1.
 constexpr int kOffK = 0, kOffV = kBufBytes, kOffQ = 2 * kBufBytes;
 constexpr int kOffS = 3 * kBufBytes;            // S' 64 x 64 bf16
 constexpr int kOffOnes = kOffS + 8192;          // constant block of the A operand (after K: positive offset)
-constexpr int kRqStride = 256 + kSeg;           // ragged units read up to kSeg - 1 entries past token N - 1
+constexpr int kRqStride = 256;
 constexpr int kOffRq = kOffOnes + 2048;         // [2][kRqStride] 1 / max(||q||, eps); second row: second half (blockdiag)
 constexpr int kOffSum = kOffRq + 2 * kRqStride * 4;  // [64] token sum of V
-constexpr int kOffZero = kOffSum + kD * 4;      // 128 B of zeros: the convolution's padding
-constexpr int kOffBar = kOffZero + 128;
-constexpr size_t kSmemBytes = 1024 + kOffBar + 128;
+constexpr int kOffBar = kOffSum + kD * 4;
+constexpr int kOffW = kOffBar + 128;            // filters of the plane's head, [taps][64] fp32, and its bias
+constexpr size_t smem_bytes(int ks) { return 1024 + kOffW + (ks * ks + 1) * kD * 4; }
 
 struct FusedParams {
     const __nv_bfloat16* w;     // [H*64][KS][KS]
@@ -79,6 +77,7 @@ tc_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     uint8_t* ones = smem + kOffOnes;
     float* rq_s = reinterpret_cast<float*>(smem + kOffRq);
     float* sum_s = reinterpret_cast<float*>(smem + kOffSum);
+    float* w_s = reinterpret_cast<float*>(smem + kOffW);
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kOffBar);
     uint64_t* k_full = bars + 0;      // TMA: K landed
     uint64_t* v_full = bars + 1;      // TMA: V (swizzled) landed
@@ -117,7 +116,6 @@ tc_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
         uint4 val = make_uint4(0, 0, 0, 0);
         if ((c ^ (r & 7)) == 0) val.x = 0x3f80u;
         *reinterpret_cast<uint4*>(ones + r * 128 + c * 16) = val;
-        if (t < 8) *reinterpret_cast<uint4*>(smem + kOffZero + t * 16) = make_uint4(0, 0, 0, 0);
         fence_proxy_async_smem();
     }
     tcgen05_fence_before_sync();
@@ -208,24 +206,27 @@ tc_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
         const int half = ww >> 2;                   // thread = token phases: channels half*32 .. half*32 + 31
         const int r = quarter * 32 + lane;          // thread = token phases: row of both tiles
         const int Wc = TOKPAIR ? W / 2 : W;        // 128-byte columns per grid row
-        const int segs = (Wc + kSeg - 1) / kSeg, n_units = prm.gridH * segs;
+        // units of the convolution: strips of two columns, cut along y as long as there are fewer than warps
+        const int n_strips = (Wc + 1) / 2, cuts = min(prm.gridH, max(1, (kWorkers / 32) / n_strips));
+        const int seg_rows = (prm.gridH + cuts - 1) / cuts, n_units = n_strips * ((prm.gridH + seg_rows - 1) / seg_rows);
         const float2 zero2 = make_float2(0.f, 0.f);
         for (int it = 0; it < n_planes; ++it) {
             const uint32_t ph = it & 1;
             const int bh = blockIdx.x + it * gridDim.x;
             const int h = (prm.head0 + bh) % prm.H;
-            // raw filter taps and bias of this lane's channel pair: loaded now, converted right before the
-            // convolution, so that the round trip to L2 hides behind everything in between
-            unsigned short wraw[2][KS * KS], braw[2] = {0, 0};
+            // this thread's share of the head's filters (and bias): on its way while the rows are normalised, into shared memory
+            // once the state is ready.  Volatile: left to itself the compiler moves the loads down to their use.
+            constexpr int kWidth = TOKPAIR ? 32 : kD, kElems = kWidth * KS * KS, kShare = (kElems + kWorkers - 1) / kWorkers;
+            unsigned short fraw[kShare], braw = 0;
             {
-                const int ch0 = TOKPAIR ? h * 32 + 2 * (lane & 15) : h * kD + 2 * lane;  // first channel of the lane's pair
-                const unsigned short* w0 = reinterpret_cast<const unsigned short*>(prm.w) + (size_t)ch0 * (KS * KS);
+                const unsigned short* w0 = reinterpret_cast<const unsigned short*>(prm.w) + (size_t)h * kElems;
 #pragma unroll
-                for (int i = 0; i < KS * KS; ++i) { wraw[0][i] = __ldg(w0 + i); wraw[1][i] = __ldg(w0 + KS * KS + i); }
-                if (prm.bias) {
-                    const unsigned short* b0 = reinterpret_cast<const unsigned short*>(prm.bias) + ch0;
-                    braw[0] = __ldg(b0); braw[1] = __ldg(b0 + 1);
+                for (int i = 0; i < kShare; ++i) {
+                    fraw[i] = 0;
+                    if (wt + i * kWorkers < kElems) asm volatile("ld.global.nc.u16 %0, [%1];" : "=h"(fraw[i]) : "l"(w0 + wt + i * kWorkers));
                 }
+                if (prm.bias && wt < kWidth)
+                    asm volatile("ld.global.nc.u16 %0, [%1];" : "=h"(braw) : "l"(reinterpret_cast<const unsigned short*>(prm.bias) + h * kWidth + wt));
             }
             // ---- K row -> unit row, in place ----
             if (!mbar_wait(k_full, ph, abort_flag, prm.status, kBit)) break;
@@ -346,6 +347,14 @@ tc_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
             fence_proxy_async_smem();
             tcgen05_fence_before_sync();
             mbar_arrive(sp_ready);
+            // [tap][channel] as fp32, then the bias (every warp has left the previous plane's convolution: s_done followed its
+            // arrival on k_scaled)
+#pragma unroll
+            for (int i = 0; i < kShare; ++i) {
+                const int e = wt + i * kWorkers;
+                if (e < kElems) w_s[(e % (KS * KS)) * kWidth + e / (KS * KS)] = __uint_as_float((uint32_t)fraw[i] << 16);
+            }
+            if (wt < kWidth) w_s[kElems + wt] = __uint_as_float((uint32_t)braw << 16);
 
             // ---- accumulator rows out of TMEM -> fp32 rows in shared memory ----
             // Row r of tile t goes to the V buffer (t = 0) or the Q buffer (t = 1), 256 bytes per row,
@@ -376,132 +385,77 @@ tc_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
             if (!mbar_wait(vp_full, ph, abort_flag, prm.status, kBit)) break;
             named_barrier_sync(1, kWorkers);  // accumulator rows, rq and s are visible to every worker
 
-            // ---- convolution + combine: lane = channel pair, warp = up to eight tokens of one grid row ----
+            // ---- convolution + combine: lane = channel pair ----
+            // A unit is a strip of two output columns (two 128-byte columns, i.e. columns 2 c + parity and 2 c + 2 + parity of
+            // this lane, when TOKPAIR) over a run of grid rows: every word of V is loaded and unpacked once per strip, sums of
+            // the KS open output rows stay in registers.
+            const int tp = TOKPAIR ? lane >> 4 : 0, cp = TOKPAIR ? lane & 15 : lane;   // token parity, channel pair
+            constexpr int kTokBytes = TOKPAIR ? 64 : 128, STEP = TOKPAIR ? 2 : 1, NIN = STEP + KS;
+            const float2 hs2 = TOKPAIR ? make_float2(0.5f * (sum_s[2 * cp] + sum_s[32 + 2 * cp]), 0.5f * (sum_s[2 * cp + 1] + sum_s[32 + 2 * cp + 1]))
+                                       : make_float2(0.5f * sum_s[2 * lane], 0.5f * sum_s[2 * lane + 1]);   // 1/2 s
+            const float2 bias2 = *reinterpret_cast<const float2*>(w_s + kElems + 2 * cp);
+            const float2 c2 = make_float2(hs2.x + bias2.x, hs2.y + bias2.y);  // + bias: grid tokens
             float2 wreg[KS][KS];
 #pragma unroll
             for (int dy = 0; dy < KS; ++dy)
 #pragma unroll
-                for (int dx = 0; dx < KS; ++dx)
-                    wreg[dy][dx] = make_float2(__uint_as_float((uint32_t)wraw[0][dy * KS + dx] << 16),
-                                               __uint_as_float((uint32_t)wraw[1][dy * KS + dx] << 16));
-            if constexpr (TOKPAIR) {
-                // lane = (token parity, channel pair): a 128-byte row of the plain V plane, of the accumulator rows
-                // and of the output holds tokens (2c, 2c+1) of a grid row; tokens are 64 bytes apart
-                const int tp = lane >> 4, cp = lane & 15;
-                const float2 hs2 = make_float2(0.5f * (sum_s[2 * cp] + sum_s[32 + 2 * cp]),
-                                               0.5f * (sum_s[2 * cp + 1] + sum_s[32 + 2 * cp + 1]));  // 1/2 s
-                const float2 c2 = make_float2(hs2.x + __uint_as_float((uint32_t)braw[0] << 16),
-                                              hs2.y + __uint_as_float((uint32_t)braw[1] << 16));
-                uint32_t* out_plane = reinterpret_cast<uint32_t*>(prm.out + plane_offset(prm.lo, bh, prm.hdiv)) + lane;
-                const int sc = lane >> 1, sw = (lane & 1) * 8;
-                const float* rq_l = rq_s + tp * kRqStride;  // the norm of the lane's token
-                const uint32_t k_base = smem_u32(K_s) + cp * 4, z_addr = smem_u32(smem + kOffZero) + cp * 4;
-                for (int u = ww; u < n_units; u += kWorkers / 32) {
-                    const int y = u / segs, c0 = (u - y * segs) * kSeg, nc = min(kSeg, Wc - c0);
-                    uint32_t ra[KS], rstep[KS];  // address of token (y + dy - R, 0) (or the zero row) and bytes per token
+                for (int dx = 0; dx < KS; ++dx) wreg[dy][dx] = *reinterpret_cast<const float2*>(w_s + (dy * KS + dx) * kWidth + 2 * cp);
+            uint32_t* out_plane = reinterpret_cast<uint32_t*>(prm.out + plane_offset(prm.lo, bh, prm.hdiv)) + lane;
+            const long long out_tok = OUT_PACKED ? kD / 2 : prm.lo.token / 2;  // 32-bit words per 128-byte row
+            const int sc = lane >> 1, sw = (lane & 1) * 8;  // chunk and offset of the lane's pair in an fp32 row
+            // the norm of the lane's token (TOKPAIR) or head (two heads side by side)
+            const float* rq_l = rq_s + ((TOKPAIR ? tp != 0 : (prm.blockdiag && lane >= 16)) ? kRqStride : 0);
+            // row r (of 128 bytes) of the plane: accumulator (tile 1 follows tile 0 in shared memory), scale, add, store
+            auto emit = [&](int r, float2 add) {
+                const float2 a2 = *reinterpret_cast<const float2*>(V_s + r * 256 + ((sc ^ (r & 7)) << 4) + sw);
+                const float rq = rq_l[r];
+                const float2 o = ffma2(a2, make_float2(rq, rq), add);
+                out_plane[r * out_tok] = pack_bf16x2(o.x, o.y);
+            };
+            const uint32_t v_base = smem_u32(K_s) + cp * 4;
+            for (int u = ww; u < n_units; u += kWorkers / 32) {
+                const int strip = u % n_strips, y_first = (u / n_strips) * seg_rows, n_rows = min(seg_rows, prm.gridH - y_first);
+                const int x0 = strip * 2 * STEP + tp;     // grid column of the lane's first output; the next is x0 + STEP
+                const bool second = strip * 2 + 1 < Wc;   // the strip's second column exists
+                bool cv[NIN];
 #pragma unroll
-                    for (int dy = 0; dy < KS; ++dy) {
-                        const int yy = y + dy - R;
+                for (int o = 0; o < NIN; ++o) cv[o] = (unsigned)(x0 + o - R) < (unsigned)W;
+                float2 acc[KS][2];   // output row y of the unit in slot y % KS
+#pragma unroll
+                for (int k = 0; k < KS; ++k) acc[k][0] = acc[k][1] = zero2;
+                for (int h0 = 0; h0 < n_rows + KS - 1; h0 += KS) {
+#pragma unroll
+                    for (int k = 0; k < KS; ++k) {
+                        const int hy = h0 + k, yy = y_first + hy - R;    // halo row of the unit, grid row
+                        const uint32_t row = v_base + (uint32_t)((prm.prefix + yy * W + x0 - R) * kTokBytes);
                         const bool rv = (unsigned)yy < (unsigned)prm.gridH;
-                        ra[dy] = rv ? k_base + (uint32_t)((prm.prefix + yy * W) * 64) : z_addr;
-                        rstep[dy] = rv ? 64u : 0u;
-                    }
+                        float2 in[NIN];
 #pragma unroll
-                    for (int j = 0; j < kSeg; ++j) {
-                        const int x = 2 * (c0 + j) + tp;  // the lane's token in the grid row
-                        float2 part[KS];
-#pragma unroll
-                        for (int dy = 0; dy < KS; ++dy) {
-                            part[dy] = (dy == 0) ? c2 : zero2;
-#pragma unroll
-                            for (int dx = 0; dx < KS; ++dx) {
-                                const int xt = x + dx - R;
-                                const uint32_t a = ((unsigned)xt < (unsigned)W) ? ra[dy] + (uint32_t)xt * rstep[dy] : z_addr;
-                                uint32_t wv;
-                                asm volatile("ld.shared.b32 %0, [%1];" : "=r"(wv) : "r"(a));
-                                part[dy] = ffma2(wreg[dy][dx], make_float2(bf16lo(wv), bf16hi(wv)), part[dy]);
-                            }
-                        }
-                        float2 acc = part[0];
-#pragma unroll
-                        for (int dy = 1; dy < KS; ++dy) { acc.x += part[dy].x; acc.y += part[dy].y; }
-                        const int pr = (prm.prefix + y * W) / 2 + c0 + j, tr = pr & (kTile - 1);  // row of the token pair
-                        const uint8_t* srow = (pr < kTile ? V_s : Q_s) + tr * 256;
-                        const float2 a2 = *reinterpret_cast<const float2*>(srow + ((sc ^ (tr & 7)) << 4) + sw);
-                        const float rq = rq_l[pr];
-                        const float2 o = ffma2(a2, make_float2(rq, rq), acc);
-                        if (j < nc) out_plane[pr * (kD / 2)] = pack_bf16x2(o.x, o.y);
-                    }
-                }
-                for (int pr = ww; pr < prm.prefix / 2; pr += kWorkers / 32) {  // off-grid leading tokens
-                    const float2 a2 = *reinterpret_cast<const float2*>(V_s + pr * 256 + ((sc ^ (pr & 7)) << 4) + sw);
-                    const float rq = rq_l[pr];
-                    const float2 o = ffma2(a2, make_float2(rq, rq), hs2);
-                    out_plane[pr * (kD / 2)] = pack_bf16x2(o.x, o.y);
-                }
-            } else {
-                const float2 hs2 = make_float2(0.5f * sum_s[2 * lane], 0.5f * sum_s[2 * lane + 1]);  // 1/2 s
-                const float2 c2 = make_float2(hs2.x + __uint_as_float((uint32_t)braw[0] << 16),
-                                              hs2.y + __uint_as_float((uint32_t)braw[1] << 16));  // + bias: grid tokens
-                uint32_t* out_plane = reinterpret_cast<uint32_t*>(prm.out + plane_offset(prm.lo, bh, prm.hdiv)) + lane;
-                const long long out_tok = OUT_PACKED ? kD / 2 : prm.lo.token / 2;  // 32-bit words per token step
-                const int sc = lane >> 1, sw = (lane & 1) * 8;  // chunk and offset of the lane's pair in an fp32 row
-                const float* rq_l = rq_s + ((prm.blockdiag && lane >= 16) ? kRqStride : 0);  // the norm of the lane's head
-                // Branch-free inside a unit: a neighbour outside the grid is read from a row of zeros, the
-                // columns of a ragged last unit are computed (from in-bounds shared memory) and not stored.
-                const uint32_t k_base = smem_u32(K_s) + lane * 4, z_addr = smem_u32(smem + kOffZero) + lane * 4;
-                for (int u = ww; u < n_units; u += kWorkers / 32) {
-                    const int y = u / segs, x0 = (u - y * segs) * kSeg, nx = min(kSeg, W - x0);
-                    uint32_t ra[KS];  // address of the lane's word of token (y + dy - R, x0); rows outside the grid: the zero row
-                    uint32_t rstep[KS];  // bytes per column in that row (0 for the zero row)
-    #pragma unroll
-                    for (int dy = 0; dy < KS; ++dy) {
-                        const int yy = y + dy - R;
-                        const bool rv = (unsigned)yy < (unsigned)prm.gridH;
-                        ra[dy] = rv ? k_base + (uint32_t)((prm.prefix + yy * W + x0) * 128) : z_addr;
-                        rstep[dy] = rv ? 128u : 0u;
-                    }
-                    float2 win[KS][KS];  // column x0 - R + jj lives in slot jj % KS
-    #pragma unroll
-                    for (int jj = 0; jj < KS - 1 + kSeg; ++jj) {
-                        // load column jj of the window (grid column x0 - R + jj), then finish output column jj - (KS - 1)
-                        const bool cv = (unsigned)(x0 + jj - R) < (unsigned)W;
-    #pragma unroll
-                        for (int dy = 0; dy < KS; ++dy) {
-                            const uint32_t a = cv ? ra[dy] + (uint32_t)(jj - R) * rstep[dy] : z_addr;
+                        for (int o = 0; o < NIN; ++o) {
                             uint32_t wv;
-                            asm volatile("ld.shared.b32 %0, [%1];" : "=r"(wv) : "r"(a));
-                            win[dy][jj % KS] = make_float2(bf16lo(wv), bf16hi(wv));
+                            asm("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %2, 0;\n\tmov.b32 %0, 0;\n\t@p ld.shared.b32 %0, [%1];\n\t}"
+                                : "=r"(wv) : "r"(row + (uint32_t)(o * kTokBytes)), "r"((int)(rv && cv[o])) : "memory");
+                            in[o] = make_float2(bf16lo(wv), bf16hi(wv));
                         }
-                        if (jj >= KS - 1) {  // compile-time
-                            const int j = jj - (KS - 1);
-                            float2 part[KS];  // one chain per filter row
-    #pragma unroll
-                            for (int dy = 0; dy < KS; ++dy) {
-                                part[dy] = (dy == 0) ? c2 : zero2;
-    #pragma unroll
-                                for (int dx = 0; dx < KS; ++dx) part[dy] = ffma2(wreg[dy][dx], win[dy][(j + dx) % KS], part[dy]);
-                            }
-                            float2 acc = part[0];
-    #pragma unroll
-                            for (int dy = 1; dy < KS; ++dy) { acc.x += part[dy].x; acc.y += part[dy].y; }
-                            const int t = prm.prefix + y * W + x0 + j, tr = t & (kTile - 1);  // t < N + kSeg: inside a row of rq_s
-                            const uint8_t* srow = (t < kTile ? V_s : Q_s) + tr * 256;
-                            const float2 a2 = *reinterpret_cast<const float2*>(srow + ((sc ^ (tr & 7)) << 4) + sw);
-                            const float rq = rq_l[t];
-                            const float2 o = ffma2(a2, make_float2(rq, rq), acc);
-                            if (j < nx) out_plane[t * out_tok] = pack_bf16x2(o.x, o.y);
+                        acc[k][0] = acc[k][1] = c2;   // output row hy starts here; it ends KS - 1 rows on
+#pragma unroll
+                        for (int dy = 0; dy < KS; ++dy)
+#pragma unroll
+                            for (int c = 0; c < 2; ++c)
+#pragma unroll
+                                for (int dx = 0; dx < KS; ++dx)
+                                    acc[(k - dy + KS) % KS][c] = ffma2(wreg[dy][dx], in[STEP * c + dx], acc[(k - dy + KS) % KS][c]);
+                        const int y = hy - (KS - 1);
+                        if (y >= 0 && y < n_rows) {
+                            const int r = (TOKPAIR ? (prm.prefix + (y_first + y) * W) / 2 : prm.prefix + (y_first + y) * W) + strip * 2;
+                            emit(r, acc[(k + 1) % KS][0]);
+                            if (second) emit(r + 1, acc[(k + 1) % KS][1]);
                         }
                     }
-                }
-                // off-grid leading tokens: the attention terms only
-                for (int t = ww; t < prm.prefix; t += kWorkers / 32) {
-                    const float2 a2 = *reinterpret_cast<const float2*>(V_s + t * 256 + ((sc ^ (t & 7)) << 4) + sw);
-                    const float rq = rq_l[t];
-                    const float2 o = ffma2(a2, make_float2(rq, rq), hs2);
-                    out_plane[t * out_tok] = pack_bf16x2(o.x, o.y);
                 }
             }
+            // off-grid leading tokens: the attention terms only
+            for (int r = ww; r < (TOKPAIR ? prm.prefix / 2 : prm.prefix); r += kWorkers / 32) emit(r, hs2);
             fence_proxy_async_smem();
             mbar_arrive(plane_free);
         }
@@ -538,18 +492,18 @@ cudaError_t launch_fused_ks(const Problem& p, unsigned* status, cudaStream_t st)
     prm.eps2 = p.eps2; prm.status = status;
     static PerDevice opt_in[3];  // per instantiation
     const bool packed = (p.lo.token == kD);
-    const cudaError_t e = pair     ? opt_in_smem(tc_fused_kernel<KS, true, true>, kSmemBytes, opt_in[2])
-                          : packed ? opt_in_smem(tc_fused_kernel<KS, true, false>, kSmemBytes, opt_in[1])
-                                   : opt_in_smem(tc_fused_kernel<KS, false, false>, kSmemBytes, opt_in[0]);
+    const cudaError_t e = pair     ? opt_in_smem(tc_fused_kernel<KS, true, true>, smem_bytes(KS), opt_in[2])
+                          : packed ? opt_in_smem(tc_fused_kernel<KS, true, false>, smem_bytes(KS), opt_in[1])
+                                   : opt_in_smem(tc_fused_kernel<KS, false, false>, smem_bytes(KS), opt_in[0]);
     if (e != cudaSuccess) return e;
     const int resident = 2 * device_sm_count();  // two CTAs per multiprocessor
     const int grid = p.BH < resident ? p.BH : resident;
     if (pair)
-        tc_fused_kernel<KS, true, true><<<(unsigned)grid, kThreads, kSmemBytes, st>>>(tmK, tmV, tmQ, tmVplain, prm);
+        tc_fused_kernel<KS, true, true><<<(unsigned)grid, kThreads, smem_bytes(KS), st>>>(tmK, tmV, tmQ, tmVplain, prm);
     else if (packed)
-        tc_fused_kernel<KS, true, false><<<(unsigned)grid, kThreads, kSmemBytes, st>>>(tmK, tmV, tmQ, tmVplain, prm);
+        tc_fused_kernel<KS, true, false><<<(unsigned)grid, kThreads, smem_bytes(KS), st>>>(tmK, tmV, tmQ, tmVplain, prm);
     else
-        tc_fused_kernel<KS, false, false><<<(unsigned)grid, kThreads, kSmemBytes, st>>>(tmK, tmV, tmQ, tmVplain, prm);
+        tc_fused_kernel<KS, false, false><<<(unsigned)grid, kThreads, smem_bytes(KS), st>>>(tmK, tmV, tmQ, tmVplain, prm);
     return cudaGetLastError();
 }
 
