@@ -423,30 +423,36 @@ tc_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
                 float2 acc[KS][2];   // output row y of the unit in slot y % KS
 #pragma unroll
                 for (int k = 0; k < KS; ++k) acc[k][0] = acc[k][1] = zero2;
+                uint32_t raw[NIN];   // the words of the next halo row, loaded a row ahead
+                auto load_row = [&](int hy) {
+                    const int yy = y_first + hy - R;
+                    const uint32_t row = v_base + (uint32_t)((prm.prefix + yy * W + x0 - R) * kTokBytes);
+                    const bool rv = (unsigned)yy < (unsigned)prm.gridH;
+#pragma unroll
+                    for (int o = 0; o < NIN; ++o)
+                        asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %2, 0;\n\tmov.b32 %0, 0;\n\t@p ld.shared.b32 %0, [%1];\n\t}"
+                                     : "=r"(raw[o]) : "r"(row + (uint32_t)(o * kTokBytes)), "r"((int)(rv && cv[o])));
+                };
+                load_row(0);
                 for (int h0 = 0; h0 < n_rows + KS - 1; h0 += KS) {
 #pragma unroll
                     for (int k = 0; k < KS; ++k) {
-                        const int hy = h0 + k, yy = y_first + hy - R;    // halo row of the unit, grid row
-                        const uint32_t row = v_base + (uint32_t)((prm.prefix + yy * W + x0 - R) * kTokBytes);
-                        const bool rv = (unsigned)yy < (unsigned)prm.gridH;
+                        const int hy = h0 + k;    // halo row of the unit
+                        if (hy >= n_rows + KS - 1) break;
                         float2 in[NIN];
 #pragma unroll
-                        for (int o = 0; o < NIN; ++o) {
-                            uint32_t wv;
-                            asm("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %2, 0;\n\tmov.b32 %0, 0;\n\t@p ld.shared.b32 %0, [%1];\n\t}"
-                                : "=r"(wv) : "r"(row + (uint32_t)(o * kTokBytes)), "r"((int)(rv && cv[o])) : "memory");
-                            in[o] = make_float2(bf16lo(wv), bf16hi(wv));
-                        }
+                        for (int o = 0; o < NIN; ++o) in[o] = make_float2(bf16lo(raw[o]), bf16hi(raw[o]));
+                        load_row(hy + 1);
                         acc[k][0] = acc[k][1] = c2;   // output row hy starts here; it ends KS - 1 rows on
 #pragma unroll
-                        for (int dy = 0; dy < KS; ++dy)
+                        for (int dx = 0; dx < KS; ++dx)
 #pragma unroll
-                            for (int c = 0; c < 2; ++c)
+                            for (int dy = 0; dy < KS; ++dy)
 #pragma unroll
-                                for (int dx = 0; dx < KS; ++dx)
+                                for (int c = 0; c < 2; ++c)
                                     acc[(k - dy + KS) % KS][c] = ffma2(wreg[dy][dx], in[STEP * c + dx], acc[(k - dy + KS) % KS][c]);
                         const int y = hy - (KS - 1);
-                        if (y >= 0 && y < n_rows) {
+                        if (y >= 0) {
                             const int r = (TOKPAIR ? (prm.prefix + (y_first + y) * W) / 2 : prm.prefix + (y_first + y) * W) + strip * 2;
                             emit(r, acc[(k + 1) % KS][0]);
                             if (second) emit(r + 1, acc[(k + 1) % KS][1]);
