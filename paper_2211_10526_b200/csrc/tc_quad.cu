@@ -241,7 +241,7 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                     }
                 }
                 if (moved) { idle = 0; continue; }
-                __nanosleep(20);
+                __nanosleep(100);
                 if ((++idle & 255u) == 0) {
                     const unsigned long long now = global_ns();
                     if (idle == 256u) t_last = now;
@@ -350,13 +350,13 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     } else if (warp < 8) {
         // ---- unit rows ----
         const int t = tid - 128;
-        auto scale_row = [&](uint8_t* row) {   // row t of a tile
-            uint4 c[8];
+        auto scale_row = [&](uint8_t* row) {   // row t of a tile, read twice: the whole row does not fit beside the rest
+            auto chunk = [&](int j) { return reinterpret_cast<uint4*>(row + ((j ^ (t & 7)) << 4)); };
             float2 ss[4] = {dup2(0.f), dup2(0.f), dup2(0.f), dup2(0.f)};
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
-                c[j] = *reinterpret_cast<const uint4*>(row + ((j ^ (t & 7)) << 4));
-                const uint32_t w[4] = {c[j].x, c[j].y, c[j].z, c[j].w};
+                const uint4 c = *chunk(j);
+                const uint32_t w[4] = {c.x, c.y, c.z, c.w};
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
                     const float2 p = make_float2(bf16lo(w[e]), bf16hi(w[e]));
@@ -365,16 +365,17 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
             }
             const float2 sum = fadd2(fadd2(ss[0], ss[1]), fadd2(ss[2], ss[3]));
             const float2 rk2 = dup2(1.0f / sqrtf(fmaxf(sum.x + sum.y, prm.eps2)));
-#pragma unroll
+#pragma unroll 4
             for (int j = 0; j < 8; ++j) {
-                const uint32_t w[4] = {c[j].x, c[j].y, c[j].z, c[j].w};
+                const uint4 c = *chunk(j);
+                const uint32_t w[4] = {c.x, c.y, c.z, c.w};
                 uint32_t o[4];
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
                     const float2 p = ffma2(make_float2(bf16lo(w[e]), bf16hi(w[e])), rk2, dup2(0.f));
                     o[e] = pack_bf16x2(p.x, p.y);
                 }
-                *reinterpret_cast<uint4*>(row + ((j ^ (t & 7)) << 4)) = make_uint4(o[0], o[1], o[2], o[3]);
+                *chunk(j) = make_uint4(o[0], o[1], o[2], o[3]);
             }
         };
         // The Q tiles of item i + 1 come after the first K tiles of item i: their copy starts once the cosines of item
