@@ -2,15 +2,16 @@
 //     out_t = sum_j (1 - arccos(q^_t . k^_j) / pi) v_j + bias + DWConv(V)_t
 // and / or the masked softmax branch of training (Eq. 10) on top of either base kernel; quadratic in the number of
 // tokens.  A work item is a plane and one or two tiles ("slots") of 128 queries, which share every tile of 128 keys.
-//   warp 0       one thread keeps three rings of TMA copies going: Q tiles (an item ahead), K tiles, V tiles
+//   warp 0       one thread keeps four rings of TMA copies going: Q tiles (an item ahead), K tiles, V tiles, and patches of
+//                the token grid with their halo for the convolution
 //   warps 4..7   scale every K row and every Q row to a unit row in place, as bf16
 //   warp 1       issues C[128 x 128] = Q^ K^^T, slot after slot, into three TMEM buffers in turn
 //   warps 8..23  thread = (query, 64 of the tile's keys): cosines out of TMEM, the weights back over them as bf16 (eight
 //                warps per slot)
 //   warp 2       issues O[128 x 64] += W[128 x 128] V, whose A operand W is read from TMEM
 //   warps 24..31 while the sweep over the keys runs: bias and depthwise convolution of V for the item's queries (lane =
-//                channel pair, V from global memory in coalesced rows) into shared memory as fp32; then thread = query:
-//                O out of TMEM, add, round, 128-byte rows to memory
+//                channel pair, warp = two columns of the patch) into shared memory as fp32; then thread = query: O out of
+//                TMEM, add, round, 128-byte rows to memory
 // Keys beyond the plane have k^ = 0 and v = 0 and need no mask in the weighted sum.  The masked branch takes a first
 // sweep over the keys that only forms the cosines and adds up exp(cosine) per query (keys beyond the plane excluded); in
 // the second sweep the weight of a pair is the base weight plus Mask_eps of its softmax probability.  When a plane has at
@@ -20,10 +21,13 @@
 // 64 x 64 tokens: 2.7e8 pairs, 61 us of that unit at 1.85 GHz).  Per 128 x 128 pairs that unit needs 1024 cycles and the
 // UMMAs 512 (64 each at N = 128, 32 each with A in TMEM), so two slots keep both busy.  The two contractions have an
 // issuing warp each: a ready wait costs 50 to 90 cycles and an issue 30 per UMMA, which one warp could not do in time.
-// Measured (B200, per forward): exact kernel, 2 x 8 planes of 64 x 64 tokens 143 us (338 with one issuing thread, weights
-// through shared memory and eight weight warps: 480 TFLOP/s over the two contractions against 203); masked branch, 64 x 12
-// planes of 14 x 14 74 us (303: there every item waited for its Q tiles and for a convolution of one thread per token).
-// Eight weight warps instead of sixteen: 151 and 77 us (two warps per scheduler do not hide the trips to TMEM).
+// Measured (B200, per forward): exact kernel, 2 x 8 planes of 64 x 64 tokens 135 us (338 with one issuing thread, weights
+// through shared memory and eight weight warps: 510 TFLOP/s over the two contractions against 203); masked branch, 64 x 12
+// planes of 14 x 14 62 us (303: there every item waited for its Q tiles and for a convolution of one thread per token; 67 with
+// the convolution's window read word by word from global memory).  Eight weight warps instead of sixteen: 151 and 77 us (two
+// warps per scheduler do not hide the trips to TMEM); all sixteen on one slot at a time: 139 and 68 us.  Issue slots are 70 %
+// busy in the exact kernel; what is left is the hand-over of a cosine buffer (weights, second contraction, first contraction),
+// of which TMEM has room for three.
 // No workspace; every wait is bounded.
 #include "tc_common.cuh"
 #include "tc_host.cuh"
@@ -35,7 +39,7 @@ namespace {
 constexpr int kD = 64;
 constexpr int kTile = 128;                          // queries per slot, keys per tile
 constexpr int kTileBytes = kTile * kD * 2;          // 16 KiB
-constexpr int kKStages = 3, kVStages = 2;
+constexpr int kKStages = 2, kVStages = 2;
 constexpr int kResident = 2;                        // key tiles of a plane that stay between the sweeps
 constexpr int kCBufs = 3;                           // cosine buffers
 constexpr int kNormThreads = 128, kSlotThreads = 256, kConvThreads = 256;
@@ -44,20 +48,20 @@ constexpr int kTmemCols = 512;
 constexpr int kColO = kCBufs * kTile;               // outputs of the two slots behind the cosine buffers
 constexpr int kStgStride = kD * 4 + 16;             // fp32 row + 16 B: conflict-free row-per-thread access
 constexpr int kOffQ = 0, kOffK = 4 * kTileBytes, kOffV = kOffK + kKStages * kTileBytes;   // Q: [2 items][2 slots]
-constexpr int kOffStg = kOffV + kVStages * kTileBytes;
+constexpr int kPatchX = 16, kPatchBytes = 10 * 18 * kD * 2;   // 8 rows (5 x 5 filters: 4) x 16 columns and their halo
+constexpr int kOffPatch = kOffV + kVStages * kTileBytes, kOffStg = kOffPatch + kPatchBytes;
 constexpr int kOffDen = kOffStg + 2 * kTile * kStgStride;   // softmax denominators [2 items][2 slots][2 halves][128]
 constexpr int kOffW = kOffDen + 8 * kTile * 4;              // filters of the item's head: [taps][32 lanes] channel pairs
 constexpr int kOffBar = kOffW + 25 * 32 * 4;
-constexpr size_t kSmem = 1024 + kOffBar + 512;
+constexpr size_t kSmem = 1024 + kOffBar + 384;
 static_assert(kSmem <= 227 * 1024, "shared memory");
 static_assert(kColO + 2 * kD <= kTmemCols, "tensor memory");
 
 struct QuadParams {
-    const __nv_bfloat16* v;      // for the convolution
     __nv_bfloat16* out;
     const __nv_bfloat16* w;
     const __nv_bfloat16* bias;
-    Layout lv, lo;
+    Layout lo;
     int hdiv, H, head0, N, gridH, gridW;
     int slots;                   // query tiles per item (1 or 2)
     int groups;                  // items per plane
@@ -106,20 +110,6 @@ __device__ __forceinline__ float exp2_approx(float x) {
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
-// A word of V, or 0.  Volatile: the loads of a window stay together in front of the arithmetic.  Left to itself the
-// compiler spreads them out to save registers, and every few FMAs then wait for a trip to L2 (102 us instead of 77 us for
-// the masked branch on 768 planes of 14 x 14).
-__device__ __forceinline__ uint32_t ldg_or_zero(const __nv_bfloat16* p, bool valid) {
-    uint32_t v;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %2, 0;\n\t"
-        "mov.b32 %0, 0;\n\t"
-        "@p ld.global.nc.b32 %0, [%1];\n\t}"
-        : "=r"(v) : "l"(p), "r"((int)valid));
-    return v;
-}
-
 constexpr float kLog2e = 1.4426950408889634f;
 
 // 1 - arccos(x)/pi of a pair: with t = 1 - |x| (clamped to [0, 1]: rounding can leave a cosine just outside [-1, 1]),
@@ -140,7 +130,9 @@ __device__ __forceinline__ float2 angular_weight2(float2 x) {
 template <int KS, bool SPARSE, bool EXACT>
 __global__ void __launch_bounds__(kThreads, 1)
 tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
-               const __grid_constant__ CUtensorMap tmV, const QuadParams prm) {
+               const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmP, const QuadParams prm) {
+    constexpr int R = KS / 2, kPatchY = KS == 3 ? 8 : 4, HX = kPatchX + 2 * R, HY = kPatchY + 2 * R;
+    static_assert(HX * HY * kD * 2 <= kPatchBytes, "patch");
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = align_smem(smem_raw);
     uint8_t* Q_s = smem + kOffQ;
@@ -161,7 +153,9 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     uint64_t* pv_done = p_full + kCBufs;         // [kCBufs] weights read by the second contraction
     uint64_t* o_full = pv_done + kCBufs;         // [2] by slot
     uint64_t* o_free = o_full + 2;               // [2] (128)
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(o_free + 2);
+    uint64_t* patch_full = o_free + 2;
+    uint64_t* patch_free = patch_full + 1;       // (one arrival per convolution warp)
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(patch_free + 1);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -177,6 +171,13 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
         const int item = blockIdx.x + i * gridDim.x, bh = item / prm.groups, t0 = (item - bh * prm.groups) * prm.slots * kTile;
         return {bh, t0, min(prm.slots, (N - t0 + kTile - 1) / kTile)};
     };
+    // patches of the token grid that hold an item's queries
+    struct Patches { int y0, nx, n; };
+    auto patches_of = [&](const Item& im) -> Patches {
+        const int y0 = im.t0 / prm.gridW, y1 = (min(N, im.t0 + im.slots * kTile) - 1) / prm.gridW;
+        const int nx = (prm.gridW + kPatchX - 1) / kPatchX;
+        return {y0, nx, nx * ((y1 - y0) / kPatchY + 1)};
+    };
     auto warp_wait = [&](uint64_t* bar, uint32_t parity) -> bool {
         return mbar_wait_warp(bar, parity, abort_flag, prm.status, kBit);
     };
@@ -190,9 +191,10 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
             mbar_init(&r_done[b], kSlotThreads); mbar_init(&p_full[b], kSlotThreads); mbar_init(&pv_done[b], 1);
         }
         for (int s = 0; s < 2; ++s) { mbar_init(&o_full[s], 1); mbar_init(&o_free[s], kTile); }
+        mbar_init(patch_full, 1); mbar_init(patch_free, kConvThreads / 32);
         *abort_flag = 0;
         mbar_fence_init();
-        tma_prefetch_desc(&tmQ); tma_prefetch_desc(&tmK); tma_prefetch_desc(&tmV);
+        tma_prefetch_desc(&tmQ); tma_prefetch_desc(&tmK); tma_prefetch_desc(&tmV); tma_prefetch_desc(&tmP);
     }
     if (warp == 1) tmem_alloc(tmem_slot, kTmemCols);
     tcgen05_fence_before_sync();
@@ -202,13 +204,24 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
 
     if (warp == 0) {
         if (lane == 0) {
-            // three independent rings, polled in turn: none waits behind another
+            // independent rings, polled in turn: none waits behind another
             int qi = 0, ki = 0, kj = 0, vi = 0, vj = 0;   // next item (and tile of it) of each ring
-            int kn = 0, vn = 0;                           // tiles issued
+            int pi = 0, pj = 0;                           // next item (and patch of it) of the convolution
+            int kn = 0, vn = 0, pn = 0;                   // tiles and patches issued
             unsigned long long t_last = 0;
             uint32_t idle = 0;
-            while (qi < my_items || ki < my_items || vi < my_items) {
+            while (qi < my_items || ki < my_items || vi < my_items || pi < my_items) {
                 bool moved = false;
+                if (pi < my_items && (pn == 0 || mbar_poll(patch_free, (pn - 1) & 1))) {
+                    const Item im = item_of(pi);
+                    const Patches pa = patches_of(im);
+                    const int pb = im.bh / prm.hdiv, ph = im.bh - pb * prm.hdiv, y = pj / pa.nx;
+                    mbar_expect_tx(patch_full, HX * HY * kD * 2);
+                    tma_load_5d(smem + kOffPatch, &tmP, patch_full, 0, (pj - y * pa.nx) * kPatchX - R, pa.y0 + y * kPatchY - R, ph, pb);
+                    ++pn;
+                    if (++pj == pa.n) { pj = 0; ++pi; }
+                    moved = true;
+                }
                 if (qi < my_items && (qi < 2 || mbar_poll(&q_free[qi & 1], ((qi >> 1) - 1) & 1))) {
                     const Item im = item_of(qi);
                     const int pb = im.bh / prm.hdiv, ph = im.bh - pb * prm.hdiv, b = qi & 1;
@@ -254,6 +267,7 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                     for (int spin = 0; spin < (1 << 20) && !mbar_try_wait(&k_full[i % kKStages], (i / kKStages) & 1); ++spin) {}
                 for (int i = max(0, vn - kVStages); i < vn; ++i)
                     for (int spin = 0; spin < (1 << 20) && !mbar_try_wait(&v_full[i % kVStages], (i / kVStages) & 1); ++spin) {}
+                if (pn > 0) for (int spin = 0; spin < (1 << 20) && !mbar_try_wait(patch_full, (pn - 1) & 1); ++spin) {}
                 for (int i = max(0, qi - 2); i < qi; ++i)
                     for (int spin = 0; spin < (1 << 20) && !mbar_try_wait(&q_full[i & 1], (i >> 1) & 1); ++spin) {}
             }
@@ -504,15 +518,15 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     } else {
         // ---- convolution of the item's queries, then their output rows ----
         const int cw = warp - 24, slot = cw >> 2, quarter = warp & 3;
-        constexpr int R = KS / 2, SEG = 4;
+        constexpr int NIN = KS + 1;       // columns of V that two output columns need
         uint32_t* w_s = reinterpret_cast<uint32_t*>(smem + kOffW) + lane;
+        float2 wreg[9];                   // 3 x 3: the filters in registers
         float2 bias2 = dup2(0.f);
-        int prev_head = -1, o_uses = 0;
+        int prev_head = -1, o_uses = 0, patch = 0;
         bool ok = true;
-        const int W = prm.gridW, segs = (W + SEG - 1) / SEG;
+        const int W = prm.gridW;
         for (int i = 0; i < my_items; ++i) {
             const Item im = item_of(i);
-            const int t_end = min(N, im.t0 + im.slots * kTile);
             const int head = (prm.head0 + im.bh) % prm.H;
             if (head != prev_head) {
                 prev_head = head;
@@ -524,45 +538,56 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                     bias2 = make_float2(bf16lo(bw), bf16hi(bw));
                 }
                 named_barrier_sync(1, kConvThreads);
+                if (KS == 3) {
+#pragma unroll
+                    for (int e = 0; e < 9; ++e) { const uint32_t fw = w_s[e * 32]; wreg[e] = make_float2(bf16lo(fw), bf16hi(fw)); }
+                }
             }
-            const __nv_bfloat16* vp = prm.v + plane_offset(prm.lv, im.bh, prm.hdiv) + 2 * lane;
-            const int y_first = im.t0 / W, n_units = ((t_end - 1) / W - y_first + 1) * segs;
-            for (int u = cw; u < n_units; u += kConvThreads / 32) {
-                const int y = y_first + u / segs, x0 = (u % segs) * SEG;
-                const int tl = y * W + x0 - im.t0;                        // first token of the unit, within the item
-                if (tl + SEG <= 0 || y * W + x0 >= t_end) continue;
-                uint32_t raw[KS][SEG + KS - 1];
+            const Patches pa = patches_of(im);
+            for (int pj = 0; pj < pa.n; ++pj, ++patch) {
+                ok = ok && warp_wait(patch_full, patch & 1);
+                if (!ok) break;
+                // two columns slide down the patch; the words of a row are loaded a row ahead
+                const int py = pj / pa.nx, y0 = pa.y0 + py * kPatchY, x0 = (pj - py * pa.nx) * kPatchX + 2 * cw;
+                const uint8_t* vh = smem + kOffPatch + 2 * cw * 128 + lane * 4;
+                int tl = y0 * W + x0 - im.t0;          // token of the first output, within the item
+                uint32_t raw[NIN];
+                float2 acc[KS][2];                     // output row y in slot y % KS
 #pragma unroll
-                for (int dy = 0; dy < KS; ++dy) {
-                    const int yy = y + dy - R;
-                    const bool rv = (unsigned)yy < (unsigned)prm.gridH;
-                    const __nv_bfloat16* vr = vp + (long long)(yy * W + x0 - R) * prm.lv.token;
+                for (int o = 0; o < NIN; ++o) raw[o] = lds32(vh + o * 128);
 #pragma unroll
-                    for (int c = 0; c < SEG + KS - 1; ++c) {
-                        raw[dy][c] = ldg_or_zero(vr, rv && (unsigned)(x0 + c - R) < (unsigned)W);
-                        asm volatile("add.s64 %0, %0, %1;" : "+l"(vr) : "l"(prm.lv.token * 2));   // no table of offsets
+                for (int hy = 0; hy < HY; ++hy) {
+                    float2 in[NIN];
+#pragma unroll
+                    for (int o = 0; o < NIN; ++o) in[o] = make_float2(bf16lo(raw[o]), bf16hi(raw[o]));
+                    if (hy + 1 < HY) {
+#pragma unroll
+                        for (int o = 0; o < NIN; ++o) raw[o] = lds32(vh + ((hy + 1) * HX + o) * 128);
+                    }
+                    if (hy < kPatchY) acc[hy % KS][0] = acc[hy % KS][1] = bias2;
+#pragma unroll
+                    for (int dx = 0; dx < KS; ++dx)
+#pragma unroll
+                        for (int dy = 0; dy < KS; ++dy) {
+                            const int y = hy - dy;     // compile-time after unrolling
+                            if (y < 0 || y >= kPatchY) continue;
+                            float2 f;
+                            if (KS == 3) f = wreg[(dy * KS + dx) % 9];
+                            else { const uint32_t fw = w_s[(dy * KS + dx) * 32]; f = make_float2(bf16lo(fw), bf16hi(fw)); }
+#pragma unroll
+                            for (int c = 0; c < 2; ++c) acc[y % KS][c] = ffma2(f, in[c + dx], acc[y % KS][c]);
+                        }
+                    if (hy >= KS - 1) {
+                        const int y = hy - (KS - 1);
+#pragma unroll
+                        for (int c = 0; c < 2; ++c)    // rows beyond the plane are beyond its last token
+                            if (x0 + c < W && (unsigned)(tl + c) < 2u * kTile)
+                                *reinterpret_cast<float2*>(stg + (tl + c) * kStgStride + lane * 8) = acc[y % KS][c];
+                        tl += W;
                     }
                 }
-                float2 acc[SEG];
-#pragma unroll
-                for (int j = 0; j < SEG; ++j) acc[j] = bias2;
-#pragma unroll
-                for (int dy = 0; dy < KS; ++dy) {
-                    float2 win[SEG + KS - 1];
-#pragma unroll
-                    for (int c = 0; c < SEG + KS - 1; ++c) win[c] = make_float2(bf16lo(raw[dy][c]), bf16hi(raw[dy][c]));
-#pragma unroll
-                    for (int dx = 0; dx < KS; ++dx) {
-                        const uint32_t fw = w_s[(dy * KS + dx) * 32];
-                        const float2 f = make_float2(bf16lo(fw), bf16hi(fw));
-#pragma unroll
-                        for (int j = 0; j < SEG; ++j) acc[j] = ffma2(f, win[j + dx], acc[j]);
-                    }
-                }
-#pragma unroll
-                for (int j = 0; j < SEG; ++j)
-                    if (x0 + j < W && tl + j >= 0 && tl + j < 2 * kTile)
-                        *reinterpret_cast<float2*>(stg + (tl + j) * kStgStride + lane * 8) = acc[j];
+                __syncwarp();
+                if (lane == 0) mbar_arrive(patch_free);
             }
             named_barrier_sync(1, kConvThreads);   // the item's convolution is in shared memory
             if (slot < im.slots) {
@@ -612,7 +637,7 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
 
 template <int KS, bool SPARSE, bool EXACT>
 cudaError_t launch_quad_ks(const Problem& p, unsigned* status, cudaStream_t st) {
-    CUtensorMap tmQ, tmK, tmV;
+    CUtensorMap tmQ, tmK, tmV, tmP;
     const uint64_t nb = (uint64_t)(p.BH / p.hdiv);
     const uint64_t dims[4] = {(uint64_t)kD, (uint64_t)p.N, (uint64_t)p.hdiv, nb};
     const uint32_t box[4] = {kD, kTile, 1, 1};
@@ -624,12 +649,16 @@ cudaError_t launch_quad_ks(const Problem& p, unsigned* status, cudaStream_t st) 
     if (!make_tensor_map_bf16(&tmQ, p.q, 4, dims, sq, box, 128) || !make_tensor_map_bf16(&tmK, p.k, 4, dims, sk, box, 128) ||
         !make_tensor_map_bf16(&tmV, p.v, 4, dims, sv, box, 128))
         return cudaErrorNotSupported;
+    // [64, columns, grid rows, planes per batch step, batch steps]: columns and rows outside the grid are zero-filled
+    const uint64_t dims_p[5] = {(uint64_t)kD, (uint64_t)p.gridW, (uint64_t)p.gridH, (uint64_t)p.hdiv, nb};
+    const uint64_t strides_p[4] = {(uint64_t)p.lv.token, (uint64_t)(p.lv.token * p.gridW), sv[1], sv[2]};
+    const uint32_t box_p[5] = {kD, kPatchX + 2 * (KS / 2), (KS == 3 ? 8 : 4) + 2 * (KS / 2), 1, 1};
+    if (!make_tensor_map_bf16(&tmP, p.v, 5, dims_p, strides_p, box_p, 0)) return cudaErrorNotSupported;
     QuadParams prm;
-    prm.v = static_cast<const __nv_bfloat16*>(p.v);
     prm.out = static_cast<__nv_bfloat16*>(p.out);
     prm.w = static_cast<const __nv_bfloat16*>(p.w);
     prm.bias = static_cast<const __nv_bfloat16*>(p.bias);
-    prm.lv = p.lv; prm.lo = p.lo;
+    prm.lo = p.lo;
     prm.hdiv = p.hdiv; prm.H = p.H; prm.head0 = p.head0; prm.N = p.N;
     prm.gridH = p.gridH; prm.gridW = p.gridW;
     // Two query tiles per item share the key tiles and keep both halves of the weight warps busy, but an item of one tile
@@ -649,7 +678,7 @@ cudaError_t launch_quad_ks(const Problem& p, unsigned* status, cudaStream_t st) 
         if (e != cudaSuccess) return e;
     }
     const int grid = prm.n_items < sms ? prm.n_items : sms;
-    tc_quad_kernel<KS, SPARSE, EXACT><<<(unsigned)grid, kThreads, kSmem, st>>>(tmQ, tmK, tmV, prm);
+    tc_quad_kernel<KS, SPARSE, EXACT><<<(unsigned)grid, kThreads, kSmem, st>>>(tmQ, tmK, tmV, tmP, prm);
     return cudaGetLastError();
 }
 
