@@ -16,9 +16,9 @@ constexpr long long kNarrowMinTokens = 4096;
 }
 
 namespace {
-// The single-kernel forward (and the non-default variants) put two width-32 rows side by side in one of 128 bytes: two
-// adjacent tokens of one head (tokens contiguous, even grid width), or the same token of two adjacent heads (head stride
-// 32, as in a token-major [B,N,H,32] tensor with an even number of heads).
+// The non-default variants put two width-32 rows side by side in one of 128 bytes: two adjacent tokens of one head (tokens
+// contiguous, even grid width), or the same token of two adjacent heads (head stride 32, as in a token-major [B,N,H,32]
+// tensor with an even number of heads).
 bool head_pairs(const Problem& p) {
     return p.d == 32 && p.H % 2 == 0 && p.hdiv == p.H && p.head0 == 0 && p.lq.head == 32 && p.lk.head == 32 &&
            p.lv.head == 32 && p.lo.head == 32;
@@ -73,6 +73,14 @@ cudaError_t forward(const Problem& p_in, float* ws_state, float* ws_partial, uns
                     cudaStream_t stream, int* launches, KernelTimer* timer) {
     *launches = 0;
     Problem p = p_in;
+    cudaError_t e;
+    if (!p.rownorm && fused_supports(p)) {  // a whole (b,h) fits in shared memory: one kernel, no workspace
+        e = launch_fused(p, status, stream);
+        if (e != cudaSuccess) return e;
+        ++*launches;
+        timer->mark(stream, "tc_fused");
+        return cudaSuccess;
+    }
     bool rows128 = p.d == 64 || token_pairs(p);   // every row of 128 bytes is full
     if (!rows128 && head_pairs(p)) {
         // heads (2m, 2m+1) side by side = one width-64 plane whose state is block diagonal
@@ -81,14 +89,6 @@ cudaError_t forward(const Problem& p_in, float* ws_state, float* ws_partial, uns
         rows128 = true;
     }
     rows128 = rows128 && !p.rownorm;   // the row sums are carried by the separate state and apply kernels only
-    cudaError_t e;
-    if (rows128 && fused_supports(p)) {  // a whole (b,h) fits in shared memory: one kernel, no workspace
-        e = launch_fused(p, status, stream);
-        if (e != cudaSuccess) return e;
-        ++*launches;
-        timer->mark(stream, "tc_fused");
-        return cudaSuccess;
-    }
     if (const int C = (cluster_enabled() && rows128) ? cluster_size(p) : 0) {
         e = launch_cluster(p, C, status, stream);
         if (e != cudaSuccess) return e;

@@ -92,8 +92,8 @@ cudaError_t launch_pipe(const Problem& p, float* state, float* ready, unsigned* 
 int cluster_size(const Problem& p);
 cudaError_t launch_cluster(const Problem& p, int C, unsigned* status, cudaStream_t st);
 
-// Single-kernel forward for short sequences (bf16, 3x3 or 5x5 filters, at most 256 128-byte rows per plane:
-// d = 64 with N <= 256, two width-32 heads per row with N <= 256, or width-32 token pairs with N <= 512): no workspace.
+// Single-kernel forward for short sequences (bf16, 3x3 or 5x5 filters; d = 64 with N <= 256, or d = 32 with N <= 512, 256 when
+// the tokens are not contiguous): no workspace.
 bool fused_supports(const Problem& p);
 cudaError_t launch_fused(const Problem& p, unsigned* status, cudaStream_t st);
 
