@@ -145,10 +145,10 @@ int castling_attn_create(const castling_attn_config_t* cfg, castling_attn_t** ou
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return fail_cuda(nullptr, e);
-    cudaDeviceProp prop;
-    e = cudaGetDeviceProperties(&prop, dev);
+    int major = 0;
+    e = cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev);
     if (e != cudaSuccess) return fail_cuda(nullptr, e);
-    if (prop.major != 10) return CASTLING_ERR_ARCH;
+    if (major != 10) return CASTLING_ERR_ARCH;
     castling_attn* h = new (std::nothrow) castling_attn();
     if (!h) return CASTLING_ERR_OOM;
     h->cfg = c;

@@ -24,9 +24,12 @@ int scratch_address(float** out) {
     if (dev < 0 || dev >= kMaxDevices) return CASTLING_ERR_UNSUPPORTED;
     std::lock_guard<std::mutex> lock(g_mutex);
     if (!g_scratch_addr[dev]) {
-        cudaDeviceProp prop;
-        if (cudaGetDeviceProperties(&prop, dev) != cudaSuccess) { (void)cudaGetLastError(); return CASTLING_ERR_CUDA; }
-        if (prop.major != 10) return CASTLING_ERR_ARCH;
+        int major = 0;
+        if (cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev) != cudaSuccess) {
+            (void)cudaGetLastError();
+            return CASTLING_ERR_CUDA;
+        }
+        if (major != 10) return CASTLING_ERR_ARCH;
         float* ptr = nullptr;
         if (cudaGetSymbolAddress((void**)&ptr, g_static_scratch) != cudaSuccess || !ptr) {
             (void)cudaGetLastError();
