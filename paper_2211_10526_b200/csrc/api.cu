@@ -208,7 +208,7 @@ int castling_attn_last_path(const castling_attn_t* h, int* kernel_launches) {
 namespace {
 
 // Enqueue the kernels for one validated problem whose tensors are all on the device.
-int run_device(castling_attn* h, const Problem& p, cudaStream_t stream) {
+int run_device(castling_attn* h, Problem p, cudaStream_t stream) {
     if (p.exact_kernel || p.sparse) {
         // explicit attention weights: one kernel, no workspace; quadratic in the number of tokens
         if (p.N > 16384) return CASTLING_ERR_UNSUPPORTED;
@@ -240,6 +240,7 @@ int run_device(castling_attn* h, const Problem& p, cudaStream_t stream) {
     }
     int rc = ensure_workspace(h, p.BH, p.N, p.d, p.bf16);
     if (rc != CASTLING_OK) return rc;
+    p.status = reinterpret_cast<unsigned*>(h->ws);
     const bool tensor_ok = castling::tc::supports(p);
     if (h->cfg.force_path == CASTLING_PATH_TENSOR && !tensor_ok) return CASTLING_ERR_UNSUPPORTED;
     bool use_tensor = tensor_ok && (h->cfg.force_path == CASTLING_PATH_TENSOR ||
@@ -545,6 +546,7 @@ int castling_attn_shard_apply(castling_attn_t* h, const void* q, const void* v_h
     p.v_row0 = halo_top;
     p.v_rows = halo_top + gridH_local + halo_bottom;
     p.lv.head = (long long)p.v_rows * gridW * d;   // planes of the taller V tensor
+    p.status = reinterpret_cast<unsigned*>(h->ws);
     int launches = 0;
     h->timer.begin(static_cast<cudaStream_t>(stream));
     bool tensor = h->cfg.force_path != CASTLING_PATH_SIMT && castling::tc::shard_supports(p);

@@ -54,6 +54,7 @@ struct Problem {
     int phase = 0;              // kPhaseAll / kPhaseStateOnly / kPhaseApplyOnly
     int v_row0 = 0, v_rows = 0; // apply of a shard: V holds v_rows grid rows and its row v_row0 is the shard's row 0
                                 // (v_rows = 0: V holds exactly the gridH rows)
+    unsigned* status = nullptr; // device status word for the bounded waits of the CUDA-core path's kernels, if there is one
     int hdiv;          // planes per batch step of the layouts: H for a caller's strided tensors, BH for a
                        // run of contiguous planes (one uniform plane stride)
     // Contiguous [planes][N][d] tensors; needs N, d and BH.

@@ -491,8 +491,12 @@ cudaError_t launch_simt(const Problem& p, float* ws_state, float* ws_partial, in
         timer->mark(stream, "simt_fused");
         return e;
     }
-    if (f32_supports(p)) return f32_forward(p, ws_state, ws_partial, P, stream, launches, timer);
     cudaError_t e = cudaSuccess;
+    if (f32_supports(p)) {
+        e = f32_forward(p, ws_state, ws_partial, P, stream, launches, timer);
+        if (e != cudaErrorNotSupported) return e;
+        e = cudaSuccess;   // strides that the tensor maps cannot take: the kernels below take any layout
+    }
     if (p.phase != kPhaseApplyOnly) {
         const int tiles = (p.N + kStateTile - 1) / kStateTile;
         const int chunk = ((tiles + P - 1) / P) * kStateTile;

@@ -12,6 +12,8 @@ constexpr int kCountersPerHead = 17;
 
 bool make_tensor_map_bf16(CUtensorMap* out, const void* base, int rank, const uint64_t* dims,
                           const uint64_t* strides, const uint32_t* box, int swizzle);
+bool make_tensor_map_f32(CUtensorMap* out, const void* base, int rank, const uint64_t* dims,
+                         const uint64_t* strides, const uint32_t* box);
 
 // Width-32 heads, two adjacent tokens of one head per 128-byte row: contiguous tokens, even grid width,
 // an even number of tokens per plane.

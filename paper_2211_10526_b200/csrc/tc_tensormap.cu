@@ -1,4 +1,4 @@
-// Host helper: build TMA tensor maps for bf16 tensors.  The driver entry point is looked up
+// Host helper: build TMA tensor maps for bf16 and fp32 tensors.  The driver entry point is looked up
 // through the runtime so that the library does not link against libcuda directly.
 #include "tc_host.cuh"
 
@@ -28,17 +28,17 @@ void lookup() {
 // by what they look like -- sizes, strides, box, swizzle -- and puts the tensor's address in: tensors that a caller has never
 // passed before cost the same as ones it passes again.
 struct Shape {
-    int rank = 0, swizzle = 0;
+    int rank = 0, swizzle = 0, bytes = 2;   // of an element
     uint32_t box[5] = {};
     uint64_t dims[5] = {}, strides[4] = {};
     bool operator==(const Shape& o) const {
-        if (rank != o.rank || swizzle != o.swizzle) return false;
+        if (rank != o.rank || swizzle != o.swizzle || bytes != o.bytes) return false;
         for (int i = 0; i < rank; ++i)
             if (dims[i] != o.dims[i] || box[i] != o.box[i] || (i + 1 < rank && strides[i] != o.strides[i])) return false;
         return true;
     }
     uint32_t slot() const {
-        uint64_t h = (uint64_t)rank * 131 + (uint64_t)swizzle;
+        uint64_t h = (uint64_t)rank * 131 + (uint64_t)swizzle + (uint64_t)bytes * 1009;
         for (int i = 0; i < rank; ++i) h = (h ^ dims[i] ^ ((uint64_t)box[i] << 40) ^ (i + 1 < rank ? strides[i] << 20 : 0)) * 0x9e3779b97f4a7c15ull;
         return (uint32_t)(h >> 58);   // 64 slots
     }
@@ -46,21 +46,20 @@ struct Shape {
 struct Entry { Shape shape; CUtensorMap map; };
 thread_local Entry t_maps[64];   // rank 0: empty
 
-bool encode_tensor_map_bf16(CUtensorMap* out, const void* base, const Shape& s);
-}  // namespace
+bool encode_tensor_map(CUtensorMap* out, const void* base, const Shape& s);
 
 // dims/box are innermost-first, in elements; the innermost dimension is contiguous; strides[i] is the
 // distance in elements between consecutive indices of dimension i + 1 (rank - 1 entries); swizzle: 0, 64 or 128 bytes.
-bool make_tensor_map_bf16(CUtensorMap* out, const void* base, int rank, const uint64_t* dims,
-                          const uint64_t* strides, const uint32_t* box, int swizzle) {
+bool make_tensor_map(CUtensorMap* out, const void* base, int rank, const uint64_t* dims, const uint64_t* strides,
+                     const uint32_t* box, int swizzle, int bytes) {
     if (rank < 2 || rank > 5) return false;
     Shape s;
-    s.rank = rank; s.swizzle = swizzle;
+    s.rank = rank; s.swizzle = swizzle; s.bytes = bytes;
     for (int i = 0; i < rank; ++i) {
         s.dims[i] = dims[i]; s.box[i] = box[i];
         if (i + 1 == rank) break;
         s.strides[i] = (dims[i + 1] == 1 && strides[i] == 0) ? 8 : strides[i];  // never stepped over: any legal value
-        if (s.strides[i] == 0 || (s.strides[i] * 2) % 16 != 0 || s.strides[i] * 2 >= (1ull << 40)) return false;
+        if (s.strides[i] == 0 || (s.strides[i] * bytes) % 16 != 0 || s.strides[i] * bytes >= (1ull << 40)) return false;
     }
     std::call_once(g_once, lookup);
     Entry& e = t_maps[s.slot()];
@@ -68,14 +67,13 @@ bool make_tensor_map_bf16(CUtensorMap* out, const void* base, int rank, const ui
         *out = e.map;
         return g_replace(out, const_cast<void*>(base)) == CUDA_SUCCESS;
     }
-    if (!encode_tensor_map_bf16(out, base, s)) return false;
+    if (!encode_tensor_map(out, base, s)) return false;
     e.shape = s;
     e.map = *out;
     return true;
 }
 
-namespace {
-bool encode_tensor_map_bf16(CUtensorMap* out, const void* base, const Shape& s) {
+bool encode_tensor_map(CUtensorMap* out, const void* base, const Shape& s) {
     if (!g_encode) return false;
     cuuint64_t gdim[5];
     cuuint64_t gstride[4];
@@ -84,15 +82,24 @@ bool encode_tensor_map_bf16(CUtensorMap* out, const void* base, const Shape& s) 
         gdim[i] = s.dims[i];
         bdim[i] = s.box[i];
         estride[i] = 1;
-        if (i + 1 < s.rank) gstride[i] = s.strides[i] * 2;  // bytes
+        if (i + 1 < s.rank) gstride[i] = s.strides[i] * s.bytes;
     }
-    const CUresult r = g_encode(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (cuuint32_t)s.rank, const_cast<void*>(base), gdim,
+    const CUresult r = g_encode(out, s.bytes == 2 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, (cuuint32_t)s.rank, const_cast<void*>(base), gdim,
                                 gstride, bdim, estride, CU_TENSOR_MAP_INTERLEAVE_NONE,
                                 s.swizzle == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : s.swizzle == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_NONE,
                                 CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS;
 }
 }  // namespace
+
+bool make_tensor_map_bf16(CUtensorMap* out, const void* base, int rank, const uint64_t* dims, const uint64_t* strides,
+                          const uint32_t* box, int swizzle) {
+    return make_tensor_map(out, base, rank, dims, strides, box, swizzle, 2);
+}
+bool make_tensor_map_f32(CUtensorMap* out, const void* base, int rank, const uint64_t* dims, const uint64_t* strides,
+                         const uint32_t* box) {
+    return make_tensor_map(out, base, rank, dims, strides, box, 0, 4);
+}
 
 }  // namespace tc
 }  // namespace castling
