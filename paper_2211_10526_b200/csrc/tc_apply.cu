@@ -438,11 +438,12 @@ cudaError_t launch_apply_ks(const Problem& p, const float* state, unsigned* stat
     const int grid = prm.n_tiles < sms ? prm.n_tiles : sms;
     // programmatic dependent launch: this grid's prologue and first Q / V loads overlap the tail of
     // the state kernel; the warps that read its results wait for it (griddepcontrol.wait) first
+    // (an apply pass on its own starts after what is before it in the stream: that may be writing its Q and V)
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid); cfg.blockDim = dim3(G::kThreads); cfg.dynamicSmemBytes = kSmemBytes; cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[0].val.programmaticStreamSerializationAllowed = p.phase != kPhaseApplyOnly;
     cfg.attrs = attr; cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, tc_apply_kernel<KS, RN>, tmQ, tmV, tmO, prm);
 }
