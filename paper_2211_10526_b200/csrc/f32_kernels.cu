@@ -1,7 +1,7 @@
 // fp32 kernels of the linear-angular attention core for head widths 32, 64 and 128 and 3x3 or 5x5 filters (the 1e-5
 // tolerance rules out bf16 operands; every other fp32 shape runs on simt_kernels.cu):
-//   state kernel  S += k^^T v, s += v per (plane, token split): tiles of 64 tokens (128 at D = 32), K scaled to unit rows on its way to shared
-//                 memory, the next tile's loads in flight; a thread owns 8 x 8 of S and every G-th token (G groups of
+//   state kernel  S += k^^T v, s += v per (plane, token split): tiles of 64 tokens (128 at D = 32), brought by TMA, the next one on its way,
+//                 K scaled to unit rows in place; a thread owns 8 x 8 of S and every G-th token (G groups of
 //                 (D/8)^2 threads), the groups meet in shared memory at the end
 //   apply kernel  persistent CTAs walk through patches of 8 rows x TX columns of tokens: Q and V with halo come by TMA (Q and V before
 //                 the state kernel has finished; the next Q during the convolution, the next V during the contraction), S' = S / pi
@@ -10,10 +10,10 @@
 // Bound: fp32 FMA issue (4 d^2 flop per token and head at 128 FMA per cycle and multiprocessor: 62 us for 2 x 8 planes of
 // 128 x 128, d = 64), which needs register tiles large enough for shared memory: 64 FMAs per four 16-byte loads in the state
 // kernel, 128 per twelve in the apply kernel.
-// Measured: 2 x 8 planes of 128 x 128, d = 64: 138 us per forward (392 on the kernels of simt_kernels.cu, whose threads issued 28
+// Measured: 2 x 8 planes of 128 x 128, d = 64: 133 us per forward (392 on the kernels of simt_kernels.cu, whose threads issued 28
 // instructions and eight 4-byte loads for 16 FMAs and read the convolution's window from global memory), the apply kernel 72 of
 // them (88 with a CTA per patch that copied it in with 16-byte asynchronous copies: issuing those took 5 000 of its 23 000
-// cycles); 2 x 4 planes of 14 x 14, d = 32: 10.3 us in a replayed graph (22.7: one CTA per plane walked through seven tiles with
+// cycles), the state kernel 58 (63 with K through registers); 2 x 4 planes of 14 x 14, d = 32: 10.3 us in a replayed graph (22.7: one CTA per plane walked through seven tiles with
 // three barriers and a trip to memory each).
 #include "tc_common.cuh"
 #include "tc_host.cuh"
@@ -25,16 +25,9 @@ using tc::ffma2;
 using tc::mbar_wait;
 using tc::pdl_launch_dependents;
 using tc::pdl_wait_primary;
-using tc::smem_u32;
 
 constexpr int kThreads = 256;
 constexpr int kF32ApplyParts = 4; // partial states that the apply kernel adds up itself
-
-__device__ __forceinline__ void cp_async16(void* dst, const void* src, bool valid) {   // zero-filled when not valid
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(valid ? 16 : 0) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
 // ---------------------------------------------------------------------------
 // state kernel: grid (BH * P); CTA bh * P + p covers tokens [p * chunk, min(N, (p + 1) * chunk))
@@ -44,48 +37,47 @@ template <int D> struct StateGeo {
     static constexpr int kSide = D / 8, kGroup = kSide * kSide, G = kThreads / kGroup;   // threads per group, groups
     static constexpr int kChunks = D / 4, kRowsPass = kThreads / kChunks, kPasses = kTok / kRowsPass;   // 16-byte chunks
     static constexpr int kTileBytes = kTok * D * 4;
-    static constexpr size_t kSmem = (size_t)(4 * kTileBytes > G * D * D * 4 ? 4 * kTileBytes : G * D * D * 4);   // K, V twice
+    static constexpr int kOffBar = 4 * kTileBytes > G * D * D * 4 ? 4 * kTileBytes : G * D * D * 4;   // after K, V twice
+    static constexpr size_t kSmem = 1024 + kOffBar + 32;
 };
 
 template <int D, bool RN>
 __global__ void __launch_bounds__(kThreads, D == 128 ? 1 : 2)
-f32_state_kernel(const float* __restrict__ k, const float* __restrict__ v, float* __restrict__ dst, int N, int chunk, int P,
-                 float eps2, Layout lk, Layout lv, int hdiv) {
+f32_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, float* __restrict__ dst, int N,
+                 int chunk, int P, float eps2, int hdiv, unsigned* status_word) {
     using G = StateGeo<D>;
     constexpr int kWords = D * D + D + (RN ? D : 0), kTok = G::kTok;
-    extern __shared__ __align__(16) float smem[];
+    constexpr unsigned kBit = tc::kStatusStateTimeout;
+    extern __shared__ uint8_t smem_raw[];
+    float* smem = reinterpret_cast<float*>(tc::align_smem(smem_raw));
+    uint64_t* full = reinterpret_cast<uint64_t*>(smem + G::kOffBar / 4);   // TMA: K and V of a tile landed
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(full + 2);
+    unsigned* status = status_word ? status_word : reinterpret_cast<unsigned*>(full + 2) + 1;
     const int tid = threadIdx.x, p = blockIdx.x % P, bh = blockIdx.x / P;
     const int n_begin = p * chunk, n_end = min(N, n_begin + chunk);
-    // loading: thread = 16-byte chunk lc of rows lr, lr + kRowsPass, ...
+    const int pb = bh / hdiv, ph = bh - pb * hdiv;
+    // scaling: thread = 16-byte chunk lc of rows lr, lr + kRowsPass, ...
     const int lc = tid % G::kChunks, lr = tid / G::kChunks;
-    const float* kb = k + plane_offset(lk, bh, hdiv) + lc * 4;
-    const float* vb = v + plane_offset(lv, bh, hdiv) + lc * 4;
-    float4 kreg[G::kPasses];
     float4 vsum = make_float4(0.f, 0.f, 0.f, 0.f), ksum = vsum;
-    auto fetch = [&](int n0, int buf) {   // V straight to shared memory, K to registers
-        float* vs = smem + (2 * buf + 1) * (kTok * D);
-#pragma unroll
-        for (int r = 0; r < G::kPasses; ++r) {
-            const int row = lr + r * G::kRowsPass, n = n0 + row;
-            const bool ok = n < n_end;
-            const long long off = ok ? n : n_begin;
-            kreg[r] = ok ? __ldg(reinterpret_cast<const float4*>(kb + off * lk.token)) : make_float4(0.f, 0.f, 0.f, 0.f);
-            cp_async16(vs + row * D + lc * 4, vb + off * lv.token, ok);
-        }
-        cp_async_commit();
+    auto load = [&](int n0, int buf) {   // rows beyond N arrive as zeros
+        float* ks = smem + 2 * buf * (kTok * D);
+        tc::mbar_expect_tx(&full[buf], 2 * G::kTileBytes);
+        tc::tma_load_4d(ks, &tmK, &full[buf], 0, n0, ph, pb);
+        tc::tma_load_4d(ks + kTok * D, &tmV, &full[buf], 0, n0, ph, pb);
     };
-    auto store_k = [&](int buf) {   // unit rows to shared memory
+    auto scale_k = [&](int buf) {   // unit rows, in place
         float* ks = smem + 2 * buf * (kTok * D);
 #pragma unroll
         for (int r = 0; r < G::kPasses; ++r) {
-            float4 x = kreg[r];
+            float4* at = reinterpret_cast<float4*>(ks + (lr + r * G::kRowsPass) * D + lc * 4);
+            float4 x = *at;
             float ss = fmaf(x.x, x.x, fmaf(x.y, x.y, fmaf(x.z, x.z, x.w * x.w)));
 #pragma unroll
             for (int o = G::kChunks / 2; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
             const float rk = 1.0f / sqrtf(fmaxf(ss, eps2));
             x.x *= rk; x.y *= rk; x.z *= rk; x.w *= rk;
             if (RN) { ksum.x += x.x; ksum.y += x.y; ksum.z += x.z; ksum.w += x.w; }
-            *reinterpret_cast<float4*>(ks + (lr + r * G::kRowsPass) * D + lc * 4) = x;
+            *at = x;
         }
     };
     // computing: group g takes tokens g, g + G, ...; a thread owns rows 8 ti .. and columns {4 tj .., D/2 + 4 tj ..} of S
@@ -100,15 +92,23 @@ f32_state_kernel(const float* __restrict__ k, const float* __restrict__ v, float
 #pragma unroll
         for (int b = 0; b < 4; ++b) acc[a][b] = make_float2(0.f, 0.f);
 
+    if (tid == 0) {
+        tc::mbar_init(&full[0], 1); tc::mbar_init(&full[1], 1);
+        *abort_flag = 0;
+        tc::mbar_fence_init();
+    }
     pdl_wait_primary();
     pdl_launch_dependents();
-    fetch(n_begin, 0);
+    if (tid == 0) load(n_begin, 0);
+    __syncthreads();   // the barriers are set up
     int buf = 0;
-    for (int n0 = n_begin; n0 < n_end; n0 += kTok, buf ^= 1) {
-        store_k(buf);
-        cp_async_wait<0>();
-        __syncthreads();   // this tile is in shared memory; every thread has left the previous one
-        if (n0 + kTok < n_end) fetch(n0 + kTok, buf ^ 1);
+    uint32_t phase = 0;
+    for (int n0 = n_begin; n0 < n_end; n0 += kTok, phase ^= buf, buf ^= 1) {
+        const bool ok = mbar_wait(&full[buf], phase, abort_flag, status, kBit);
+        scale_k(buf);
+        tc::fence_proxy_async_smem();       // TMA writes this buffer after the next tile's barrier
+        if (__syncthreads_or(!ok)) break;   // this tile is ready; every thread has left the previous one
+        if (tid == 0 && n0 + kTok < n_end) load(n0 + kTok, buf ^ 1);
         const float* ks = smem + 2 * buf * (kTok * D);
         const float* vs = ks + kTok * D;
 #pragma unroll 2
@@ -124,12 +124,14 @@ f32_state_kernel(const float* __restrict__ k, const float* __restrict__ v, float
 #pragma unroll
                 for (int y = 0; y < 4; ++y) acc[x][y] = ffma2(make_float2(a[x], a[x]), b[y], acc[x][y]);
         }
-        // the thread's own columns of V: rows it loaded itself, so its asynchronous copies are complete
 #pragma unroll
         for (int r = 0; r < G::kPasses; ++r) {
             const float4 x = *reinterpret_cast<const float4*>(vs + (lr + r * G::kRowsPass) * D + lc * 4);
             vsum.x += x.x; vsum.y += x.y; vsum.z += x.z; vsum.w += x.w;
         }
+    }
+    if (tid == 0 && *abort_flag) {   // giving up: let the copies in flight land before their place is used
+        for (int spin = 0; spin < (1 << 20) && !tc::mbar_try_wait(&full[buf], phase); ++spin) {}
     }
     float* out = dst + ((size_t)bh * P + p) * kWords;
     // groups meet in shared memory, in their order
@@ -415,9 +417,9 @@ cudaError_t launch_f32(const Problem& p, float* ws_state, float* ws_partial, int
     using A = ApplyGeo<D, KS>;
     CUtensorMap tmQ, tmV;
     const int v_rows = p.v_rows > 0 ? p.v_rows : p.gridH;
+    const uint64_t nb = (uint64_t)(p.BH / p.hdiv), hd = (uint64_t)p.hdiv;
     if (p.phase != kPhaseStateOnly) {
         // [d, columns, rows, planes per batch step, batch steps]: out-of-range coordinates read as zero
-        const uint64_t nb = (uint64_t)(p.BH / p.hdiv), hd = (uint64_t)p.hdiv;
         auto map = [&](CUtensorMap* m, const void* base, const Layout& l, int rows, int bx, int by) {
             const uint64_t dims[5] = {(uint64_t)D, (uint64_t)p.gridW, (uint64_t)rows, hd, nb}, token = (uint64_t)l.token;
             const uint64_t strides[4] = {token, token * p.gridW, hd > 1 ? (uint64_t)l.head : token, nb > 1 ? (uint64_t)l.batch : token};
@@ -433,11 +435,19 @@ cudaError_t launch_f32(const Problem& p, float* ws_state, float* ws_partial, int
         using G = StateGeo<D>;
         const int tiles = (p.N + G::kTok - 1) / G::kTok, per = (tiles + P - 1) / P;
         P = (tiles + per - 1) / per;   // every split has tokens
+        CUtensorMap tmK, tmV;   // [d, tokens, planes per batch step, batch steps]
+        auto map = [&](CUtensorMap* m, const void* base, const Layout& l) {
+            const uint64_t dims[4] = {(uint64_t)D, (uint64_t)p.N, hd, nb}, token = (uint64_t)l.token;
+            const uint64_t strides[3] = {token, hd > 1 ? (uint64_t)l.head : token, nb > 1 ? (uint64_t)l.batch : token};
+            const uint32_t box[4] = {(uint32_t)D, (uint32_t)G::kTok, 1, 1};
+            return tc::make_tensor_map_f32(m, base, 4, dims, strides, box);
+        };
+        if (!map(&tmK, p.k, p.lk) || !map(&tmV, p.v, p.lv)) return cudaErrorNotSupported;
         static PerDevice opt_in;
         e = opt_in_smem(f32_state_kernel<D, RN>, G::kSmem, opt_in);
         if (e != cudaSuccess) return e;
-        e = launch_pdl(f32_state_kernel<D, RN>, dim3((unsigned)(p.BH * P)), G::kSmem, st, true, static_cast<const float*>(p.k),
-                       static_cast<const float*>(p.v), P > 1 ? ws_partial : ws_state, p.N, per * G::kTok, P, p.eps2, p.lk, p.lv, p.hdiv);
+        e = launch_pdl(f32_state_kernel<D, RN>, dim3((unsigned)(p.BH * P)), G::kSmem, st, true, tmK, tmV,
+                       P > 1 ? ws_partial : ws_state, p.N, per * G::kTok, P, p.eps2, p.hdiv, p.status);
         if (e != cudaSuccess) return e;
         ++*launches;
         timer->mark(st, "f32_state");
