@@ -1,20 +1,21 @@
 // Apply kernel of the tensor-core path for width-32 heads in 64-byte rows (bf16): any grid width, any number of tokens,
 // tokens or heads next to one another in memory:
 //     out_t = (1/pi) q^_t S + 1/2 s + bias + DWConv(V)_t                         (Eq. 9)
-// The roles are those of the width-64 apply kernel, on patches of 8 x 32 tokens (256 rows of 64 bytes):
+// The roles are those of the width-64 apply kernel, on patches of 8 x 32 or 16 x 16 tokens (256 rows of 64 bytes):
 //   warp 0      TMA: Q patch (64-byte swizzle) and V patch with its halo (out-of-grid rows and columns zero-filled, which is
 //               the convolution's padding)
 //   warp 1      four UMMAs per patch: acc[2 x 128 x 32] = Q S', S' = S / pi in bf16
 //   warps 2..9  thread = token: ||q||, accumulator row from TMEM, out = acc / max(||q||, eps) + staged, one rounding; a warp
-//               holds 32 tokens of one grid row and stores them with a TMA copy of its own, so no barrier joins the warps
+//               holds 32 tokens (one row of the patch, or two) and stores them with a TMA copy of its own, so no barrier joins the warps
 //   warps 10..  depthwise convolution, lane = (column parity, channel pair): two columns at a time slide down the patch, every
 //               word of V is loaded and unpacked once per pair of columns, sums of the KS open output rows in registers;
 //               result (+ 1/2 s + bias) staged in shared memory as fp32
-// Bound: issue slots of the convolution (per output pair of channels 9 packed FMAs and 11 other instructions at 3 x 3).
-// Measured (per forward with the state kernel): 8 x 8 planes of 50 x 75, 5 x 5 filters 33 us (245 on the CUDA-core kernels,
-// which took odd widths before; 39 with the words of a row loaded right before their use: one convolution warp per scheduler
-// hides nothing); 64 x 64 28 us (37 with two tokens packed to a 128-byte row, where a lane's window slid two tokens per
-// output and loaded 4.3 words per output instead of 3.1, and two CTA-wide barriers joined the warps per patch).
+// Bound: the packed FMAs of the convolution, 2.5 to 3 cycles each (5 x 5 filters: its warps are busy 3 100 of the 3 300 cycles of
+// a patch, with four of them as with eight).
+// Measured (per forward with the state kernel): 8 x 8 planes of 50 x 75, 5 x 5 filters 31 us (245 on the CUDA-core kernels,
+// which took odd widths before; 39 with the words of a row loaded right before their use); 64 x 64 27 us (37 with two tokens
+// packed to a 128-byte row, where a lane's window slid two tokens per output and loaded 4.3 words per output instead of 3.1, and
+// two CTA-wide barriers joined the warps per patch).
 #include "tc_common.cuh"
 #include "tc_host.cuh"
 
@@ -23,8 +24,7 @@ namespace tc {
 namespace {
 
 constexpr int kD = 32;
-constexpr int kTY = 8, kTX = 32;               // patch: 8 rows x 32 columns of tokens
-constexpr int kTile = kTY * kTX;               // 256 tokens, two UMMA tiles of 128
+constexpr int kTile = 256;                     // tokens of a patch (TX columns x 256 / TX rows): two UMMA tiles of 128
 constexpr int kQBytes = kTile * kD * 2;        // 16 KiB
 constexpr int kStgStride = kD * 4 + 16;        // fp32 row + 16 B: conflict-free row-per-thread reads
 constexpr int kStgBytes = kTile * kStgStride;
@@ -32,12 +32,10 @@ constexpr int kEpiThreads = 256;
 constexpr int kStages = 3;
 constexpr int kCols = 2;                       // columns per lane of the convolution
 
-template <int KS> struct Geo {
-    static constexpr int R = KS / 2;
-    // 3 x 3: 8 convolution warps of four columns (96 registers per thread); 5 x 5: 4 warps of eight columns, in two steps
-    // (the filters alone take 50 registers: 128 per thread)
-    static constexpr int kConvWarps = KS == 3 ? 8 : 4, kConvThreads = kConvWarps * 32;
-    static constexpr int kGroups = kTX / (2 * kCols * kConvWarps);
+template <int KS, int kTX> struct Geo {
+    static constexpr int R = KS / 2, kTY = kTile / kTX;
+    // a convolution warp takes 8 rows of four columns
+    static constexpr int kConvWarps = 8, kConvThreads = kConvWarps * 32, kRows = 8, kGroups = kTX / (2 * kCols);
     static constexpr int kThreads = 64 + kEpiThreads + kConvThreads;
     static constexpr int HY = kTY + 2 * R, HX = kTX + 2 * R;
     static constexpr int kVBytes = HY * HX * kD * 2;
@@ -62,11 +60,12 @@ struct Apply32Params {
 };
 
 // RN: row-sum normalisation, as in the width-64 kernel: column 32 of the accumulator is q . sum k^ / pi.
-template <int KS, bool RN>
-__global__ void __launch_bounds__(Geo<KS>::kThreads, 1)
+template <int KS, bool RN, int kTX>
+__global__ void __launch_bounds__((Geo<KS, kTX>::kThreads), 1)
 tc_apply32_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmV,
                   const __grid_constant__ CUtensorMap tmO, const Apply32Params prm) {
-    using G = Geo<KS>;
+    using G = Geo<KS, kTX>;
+    constexpr int kTY = G::kTY;
     constexpr int kSW = kD * kD + kD + (RN ? kD : 0);   // words of one state
     constexpr int kAccN = RN ? kD + 16 : kD;            // columns the UMMAs write per tile
     constexpr int kAccTile = RN ? 2 * kD : kD, kAcc = 2 * kAccTile;
@@ -171,7 +170,7 @@ tc_apply32_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             __syncwarp();
         }
     } else if (warp < 10) {
-        // ------- epilogue: thread = token; a warp holds one grid row of the patch -------
+        // ------- epilogue: thread = token; a warp holds one grid row of the patch, or two half as long -------
         const int quarter = warp & 3, tile = (warp - 2) >> 2, row = tile * 128 + quarter * 32 + lane, et = tid - 64;
         const uint32_t acc_addr = tmem + ((uint32_t)(quarter * 32) << 16) + tile * kAccTile;
         uint8_t* orow = out_s + row * 64;
@@ -251,7 +250,7 @@ tc_apply32_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             fence_proxy_async_smem();
             __syncwarp();
             if (lane == 0) {
-                const int y = py * kTY + tile * 4 + quarter, x0 = px * kTX;   // rows below the grid are clipped by TMA
+                const int y = py * kTY + (tile * 4 + quarter) * (32 / kTX), x0 = px * kTX;   // rows below the grid are clipped by TMA
                 const uint8_t* src = out_s + (tile * 128 + quarter * 32) * 64;
                 if (prm.flat) {
                     tma_store_4d_hint(&tmO, src, 0, x0, y, bh, pol_o);
@@ -267,62 +266,63 @@ tc_apply32_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         // ------- depthwise convolution: lane = (column parity, channel pair), two columns at a time down the patch -------
         const int cw = warp - 10, par = lane >> 4, cp = lane & 15;
         constexpr int NIN = 2 * (kCols - 1) + KS;   // columns of V that two output columns (two apart) need
-        float2 wreg[KS][KS];
-        float2 cinit = make_float2(0.f, 0.f), hs2 = make_float2(0.f, 0.f);
+        const int x0 = (cw % G::kGroups) * 2 * kCols + par, y0 = cw / G::kGroups * G::kRows;   // first column of this lane; the next is x0 + 2
+        float2 wreg[KS][KS], bias2 = make_float2(0.f, 0.f);
+        float2 cinit = bias2, hs2 = bias2;
+        auto load_filters = [&]() {
+            const int ch = ((prm.head0 + bh) % prm.H) * kD + 2 * cp;
+#pragma unroll
+            for (int dy = 0; dy < KS; ++dy)
+#pragma unroll
+                for (int dx = 0; dx < KS; ++dx)
+                    wreg[dy][dx] = make_float2(__bfloat162float(prm.w[(size_t)ch * KS * KS + dy * KS + dx]),
+                                               __bfloat162float(prm.w[(size_t)(ch + 1) * KS * KS + dy * KS + dx]));
+            if (prm.bias) bias2 = make_float2(__bfloat162float(prm.bias[ch]), __bfloat162float(prm.bias[ch + 1]));
+        };
+        load_filters();      // of the first plane, while the state kernel finishes
         int prev_bh = -1;
         pdl_wait_primary();  // the token sums of the state kernel are read below
         for (int it = 0; it < my_tiles; ++it, step()) {
             const int s = it % kStages, use = it / kStages, b = it & 1, ub = it >> 1;
             if (bh != prev_bh) {
+                if (prev_bh >= 0) load_filters();
                 prev_bh = bh;
-                const int ch = ((prm.head0 + bh) % prm.H) * kD + 2 * cp;
                 const float* sv = prm.state + (size_t)bh * kSW + kD * kD + 2 * cp;
                 hs2 = make_float2(0.5f * __ldg(sv), 0.5f * __ldg(sv + 1));
-                cinit = RN ? make_float2(0.f, 0.f) : hs2;
-                if (prm.bias) { cinit.x += __bfloat162float(prm.bias[ch]); cinit.y += __bfloat162float(prm.bias[ch + 1]); }
-#pragma unroll
-                for (int dy = 0; dy < KS; ++dy)
-#pragma unroll
-                    for (int dx = 0; dx < KS; ++dx)
-                        wreg[dy][dx] = make_float2(__bfloat162float(prm.w[(size_t)ch * KS * KS + dy * KS + dx]),
-                                                   __bfloat162float(prm.w[(size_t)(ch + 1) * KS * KS + dy * KS + dx]));
+                cinit = RN ? bias2 : make_float2(hs2.x + bias2.x, hs2.y + bias2.y);
             }
             if (!mbar_wait_warp(&full[s], use & 1, abort_flag, prm.status, kBit)) break;
             if (ub > 0 && !mbar_wait_warp(&buf_free[b], (ub - 1) & 1, abort_flag, prm.status, kBit)) break;
-#pragma unroll 1
-            for (int g = 0; g < G::kGroups; ++g) {
-                const int x0 = (cw * G::kGroups + g) * 2 * kCols + par;   // first column of this lane; the next is x0 + 2
-                const uint8_t* vh = stages + s * G::kStage + kQBytes + x0 * 64 + cp * 4;
-                uint8_t* so = stg + b * kStgBytes + x0 * kStgStride + cp * 8;
-                float2 acc[KS][kCols];   // output row y in slot y % KS
-                uint32_t raw[NIN];       // the row's words, loaded a row ahead
+            const uint8_t* vh = stages + s * G::kStage + kQBytes + (y0 * G::HX + x0) * 64 + cp * 4;
+            uint8_t* so = stg + b * kStgBytes + (y0 * kTX + x0) * kStgStride + cp * 8;
+            float2 acc[KS][kCols];   // output row y in slot y % KS
+            uint32_t raw[NIN];       // the row's words, loaded a row ahead
 #pragma unroll
-                for (int o = 0; o < NIN; ++o) raw[o] = lds32(vh + o * 64);
+            for (int o = 0; o < NIN; ++o) raw[o] = lds32(vh + o * 64);
 #pragma unroll
-                for (int hy = 0; hy < G::HY; ++hy) {
-                    float2 in[NIN];
+            for (int hy = 0; hy < G::kRows + 2 * G::R; ++hy) {
+                float2 in[NIN];
 #pragma unroll
-                    for (int o = 0; o < NIN; ++o) in[o] = make_float2(bf16lo(raw[o]), bf16hi(raw[o]));
-                    if (hy + 1 < G::HY) {
+                for (int o = 0; o < NIN; ++o) in[o] = make_float2(bf16lo(raw[o]), bf16hi(raw[o]));
+                if (hy + 1 < G::kRows + 2 * G::R) {
 #pragma unroll
-                        for (int o = 0; o < NIN; ++o) raw[o] = lds32(vh + ((hy + 1) * G::HX + o) * 64);
+                    for (int o = 0; o < NIN; ++o) raw[o] = lds32(vh + ((hy + 1) * G::HX + o) * 64);
+                }
+                if (hy < G::kRows) acc[hy % KS][0] = acc[hy % KS][1] = cinit;   // output row hy starts here
+                // taps in the outer loop: consecutive FMAs go to different sums
+#pragma unroll
+                for (int dx = 0; dx < KS; ++dx)
+#pragma unroll
+                    for (int dy = 0; dy < KS; ++dy) {
+                        const int y = hy - dy;   // compile-time after unrolling
+                        if (y < 0 || y >= G::kRows) continue;
+#pragma unroll
+                        for (int c = 0; c < kCols; ++c) acc[y % KS][c] = ffma2(wreg[dy][dx], in[2 * c + dx], acc[y % KS][c]);
                     }
-                    if (hy < kTY) acc[hy % KS][0] = acc[hy % KS][1] = cinit;   // output row hy starts here
-                    // taps in the outer loop: consecutive FMAs go to different sums
+                if (hy >= KS - 1) {              // and output row hy - (KS - 1) ends here
+                    const int y = hy - (KS - 1);
 #pragma unroll
-                    for (int dx = 0; dx < KS; ++dx)
-#pragma unroll
-                        for (int dy = 0; dy < KS; ++dy) {
-                            const int y = hy - dy;   // compile-time after unrolling
-                            if (y < 0 || y >= kTY) continue;
-#pragma unroll
-                            for (int c = 0; c < kCols; ++c) acc[y % KS][c] = ffma2(wreg[dy][dx], in[2 * c + dx], acc[y % KS][c]);
-                        }
-                    if (hy >= KS - 1) {              // and output row hy - (KS - 1) ends here
-                        const int y = hy - (KS - 1);
-#pragma unroll
-                        for (int c = 0; c < kCols; ++c) *reinterpret_cast<float2*>(so + (y * kTX + 2 * c) * kStgStride) = acc[y % KS][c];
-                    }
+                    for (int c = 0; c < kCols; ++c) *reinterpret_cast<float2*>(so + (y * kTX + 2 * c) * kStgStride) = acc[y % KS][c];
                 }
             }
             if (RN && warp == 10 && par == 0) *reinterpret_cast<float2*>(hs_s + b * kD + 2 * cp) = hs2;
@@ -335,15 +335,16 @@ tc_apply32_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
     if (warp == 1) tmem_dealloc(tmem, kTmemCols);
 }
 
-template <int KS, bool RN>
+template <int KS, bool RN, int kTX>
 cudaError_t launch_apply32_ks(const Problem& p, const float* state, unsigned* status, cudaStream_t st) {
-    using G = Geo<KS>;
+    using G = Geo<KS, kTX>;
+    constexpr int kTY = G::kTY;
     CUtensorMap tmQ, tmV, tmO;
     // [32, columns, grid rows, planes per batch step, batch steps]; with a single batch step the last dimension is dropped
     const uint64_t nb = (uint64_t)(p.BH / p.hdiv);
     const int rank = nb > 1 ? 5 : 4;
     const uint64_t dims[5] = {(uint64_t)kD, (uint64_t)p.gridW, (uint64_t)p.gridH, (uint64_t)p.hdiv, nb};
-    const uint32_t boxq[5] = {kD, kTX, kTY, 1, 1}, boxv[5] = {kD, (uint32_t)G::HX, (uint32_t)G::HY, 1, 1}, boxo[5] = {kD, kTX, 1, 1, 1};
+    const uint32_t boxq[5] = {kD, kTX, kTY, 1, 1}, boxv[5] = {kD, (uint32_t)G::HX, (uint32_t)G::HY, 1, 1}, boxo[5] = {kD, kTX, 32 / kTX, 1, 1};
     auto strides = [&](const Layout& l, uint64_t (&s)[4]) {
         s[0] = (uint64_t)l.token; s[1] = (uint64_t)(l.token * p.gridW); s[2] = (uint64_t)l.head;
         s[3] = (uint64_t)(nb > 1 ? l.batch : l.head * p.hdiv);
@@ -368,7 +369,7 @@ cudaError_t launch_apply32_ks(const Problem& p, const float* state, unsigned* st
     prm.eps2 = p.eps2; prm.status = status; prm.n_tokens = p.N;
     static PerDevice opt_in;  // one per instantiation
     {
-        const cudaError_t e = opt_in_smem(tc_apply32_kernel<KS, RN>, G::kSmem, opt_in);
+        const cudaError_t e = opt_in_smem(tc_apply32_kernel<KS, RN, kTX>, G::kSmem, opt_in);
         if (e != cudaSuccess) return e;
     }
     const int sms = device_sm_count();
@@ -379,15 +380,26 @@ cudaError_t launch_apply32_ks(const Problem& p, const float* state, unsigned* st
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr; cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, tc_apply32_kernel<KS, RN>, tmQ, tmV, tmO, prm);
+    return cudaLaunchKernelEx(&cfg, tc_apply32_kernel<KS, RN, kTX>, tmQ, tmV, tmO, prm);
+}
+
+template <int KS, bool RN>
+cudaError_t launch_apply32_rn(const Problem& p, const float* state, unsigned* status, cudaStream_t st) {
+    // Patches of 16 x 16 where they need fewer rounds of the device.  Measured, 32 columns wide against 16: 8 x 8 planes of
+    // 50 x 75, 5 x 5 filters 31.4 / 30.6 us (10 rounds / 9), 25 x 38 18.0 / 16.1 (4 / 3), 3 x 3, 31 x 33 14.1 / 12.9 (4 / 3); as
+    // many rounds: 64 x 64 27.4 / 27.6; fewer with 32: 100 x 150 84.4 / 88.5 (29 / 31), 64 x 8 planes of 24 x 24 28.1 / 31.5.
+    auto rounds = [&](int tx) {
+        const long long n = (long long)p.BH * ((p.gridW + tx - 1) / tx) * ((p.gridH + kTile / tx - 1) / (kTile / tx));
+        return (n + device_sm_count() - 1) / device_sm_count();
+    };
+    return rounds(16) < rounds(32) ? launch_apply32_ks<KS, RN, 16>(p, state, status, st) : launch_apply32_ks<KS, RN, 32>(p, state, status, st);
 }
 
 }  // namespace
 
 cudaError_t launch_apply32(const Problem& p, const float* state, unsigned* status, cudaStream_t st) {
-    if (p.ksize == 3)
-        return p.rownorm ? launch_apply32_ks<3, true>(p, state, status, st) : launch_apply32_ks<3, false>(p, state, status, st);
-    return p.rownorm ? launch_apply32_ks<5, true>(p, state, status, st) : launch_apply32_ks<5, false>(p, state, status, st);
+    if (p.ksize == 3) return p.rownorm ? launch_apply32_rn<3, true>(p, state, status, st) : launch_apply32_rn<3, false>(p, state, status, st);
+    return p.rownorm ? launch_apply32_rn<5, true>(p, state, status, st) : launch_apply32_rn<5, false>(p, state, status, st);
 }
 
 }  // namespace tc

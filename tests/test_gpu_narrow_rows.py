@@ -1,6 +1,6 @@
 """Width-32 heads in 64-byte rows on the tensor-core kernels (odd grid widths, odd token counts, an odd number of heads side
 by side), against the float64 oracle at the edges of their tiles: 256-token stages of the state kernel with one token less
-or more, 8 x 32-token patches with a row or a column less or more, one column, several token splits, leading tokens, both
+or more, patches of 8 x 32 and 16 x 16 tokens with a row or a column less or more, one column, several token splits, leading tokens, both
 filter sizes, the row-sum division; and each term of Eq. 9 on its own scale.  Bound: 2e-2 of the largest output, as for
 every bf16 shape (output rounding 2^-9, operands rounded to bf16).
 """
@@ -19,7 +19,8 @@ pytestmark = pytest.mark.gpu
 CASES = [(4, 5, 15, 17, 3, "heads", 0), (4, 5, 1, 257, 3, "heads", 0), (3, 6, 7, 33, 5, "heads", 0),
          (3, 6, 9, 31, 3, "heads", 0), (20, 3, 73, 1, 3, "heads", 0), (1, 2, 90, 57, 5, "heads", 0),
          (8, 3, 16, 16, 3, "tokens", 0), (4, 5, 8, 32, 5, "fused", 0), (3, 3, 24, 40, 3, "heads", 1),
-         (5, 3, 17, 31, 5, "tokens", 2), (60, 8, 7, 7, 3, "heads", 0)]
+         (5, 3, 17, 31, 5, "tokens", 2), (60, 8, 7, 7, 3, "heads", 0),
+         (8, 9, 17, 15, 3, "heads", 0), (8, 9, 32, 17, 5, "tokens", 1), (8, 8, 31, 33, 5, "heads", 0), (8, 9, 33, 16, 3, "fused", 0)]
 
 
 def views(c, layout, dev):
