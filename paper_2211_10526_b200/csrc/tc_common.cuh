@@ -345,6 +345,16 @@ __device__ __forceinline__ uint32_t lds32(const void* p) {
     return v;
 }
 
+// The same from a shared-space address.
+__device__ __forceinline__ uint32_t lds32(uint32_t addr) {
+    uint32_t v;
+    asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(addr));
+    return v;
+}
+__device__ __forceinline__ void lds64(uint32_t addr, float2& v) {
+    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr));
+}
+
 // Packed fp32 FMA on a pair: d = a * b + c element-wise.
 __device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) {
     float2 d;

@@ -24,7 +24,9 @@
 // a call is the number of planes over those in flight.  Two shapes of CTA: 256 workers for planes of any size, two per SM;
 // 128 workers for planes of at most 128 lines, three or four per SM, which finish a plane later but more of them at a time:
 // taken when that saves a round of planes.
-// Measured: 512 planes of 7 x 7, width 32, 14.1 -> 10.3 us a call (two tokens a line and large CTAs before).
+// Measured: 512 planes of 7 x 7, width 32, 14.1 -> 10.3 us a call (two tokens a line and large CTAs before); 3000 planes of
+// 11 x 11, width 64, 69.8 -> 64.4, 768 planes of 14 x 14 and a class token 32.2 -> 31.7 with masks instead of predicated loads,
+// running addresses, and the accumulator's words loaded ahead of the FMAs.
 #include "tc_common.cuh"
 #include "tc_host.cuh"
 
@@ -42,11 +44,13 @@ template <int KS, bool NARROW, int WORKERS> struct Geo {
     static constexpr int kThreads = 64 + WORKERS;
     static constexpr int kCtas = KS != 3 ? (WORKERS == 256 ? 1 : 2) : WORKERS == 256 ? 2 : NARROW ? 4 : 3;   // per multiprocessor
     static constexpr int kTmemCols = kTokens / kTile * kW;       // outputs; the state uses the first kW columns before
-    // Shared memory: K | V | Q | S' | ones | rq | s | barriers | filters.  After their first use the buffers change role: K holds
-    // the unswizzled V plane, V and Q hold the fp32 accumulator rows.
+    // Shared memory: S' | K | V | Q | ones | rq | s | barriers | filters.  After their first use the buffers change role: K holds
+    // the unswizzled V plane, V and Q hold the fp32 accumulator rows.  The convolution's reads left of the plane's first token
+    // fall into S'.
     static constexpr int kBuf = WORKERS * 128;
-    static constexpr int kOffK = 0, kOffV = kBuf, kOffQ = 2 * kBuf, kOffS = 3 * kBuf;
-    static constexpr int kOffOnes = kOffS + kW * kRow;           // constant block of the A operand (after K: positive offset)
+    static constexpr int kOffS = 0, kOffK = kW * kRow, kOffV = kOffK + kBuf, kOffQ = kOffV + kBuf;
+    static_assert(kOffK % 1024 == 0 && kOffK >= KS / 2 * kRow, "swizzle atoms; room for the reads left of the plane");
+    static constexpr int kOffOnes = kOffQ + kBuf;                // constant block of the A operand (after K: positive offset)
     static constexpr int kOffRq = kOffOnes + 16 * kRow;          // [kTokens] 1 / max(||q||, eps)
     static constexpr int kOffSum = kOffRq + kTokens * 4;         // [kW] token sum of V
     static constexpr int kOffBar = kOffSum + kW * 4;
@@ -356,6 +360,7 @@ tc_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
             // even and the odd columns of four.
             const int par = NARROW ? lane >> 4 : 0, cp = NARROW ? lane & 15 : lane;   // column parity, channel pair
             constexpr int STEP = NARROW ? 2 : 1, NIN = STEP + KS;
+            constexpr bool kEarly = WORKERS == 256;
             const float2 hs2 = make_float2(0.5f * sum_s[2 * cp], 0.5f * sum_s[2 * cp + 1]);   // 1/2 s
             const float2 bias2 = *reinterpret_cast<const float2*>(w_s + kElems + 2 * cp);
             const float2 c2 = make_float2(hs2.x + bias2.x, hs2.y + bias2.y);  // + bias: grid tokens
@@ -366,35 +371,38 @@ tc_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
                 for (int dx = 0; dx < KS; ++dx) wreg[dy][dx] = *reinterpret_cast<const float2*>(w_s + (dy * KS + dx) * kW + 2 * cp);
             uint32_t* out_plane = reinterpret_cast<uint32_t*>(prm.out + plane_offset(prm.lo, bh, prm.hdiv)) + cp;
             const long long out_tok = OUT_PACKED ? kW / 2 : prm.lo.token / 2;  // 32-bit words per token
-            // token t: accumulator, scale, add, store
-            auto emit = [&](int t, float2 add) {
-                const float2 a2 = *reinterpret_cast<const float2*>(V_s + t * (kW * 4) + (((cp >> 1) ^ (t & 7)) << 4) + (cp & 1) * 8);
-                const float rq = rq_s[t];
+            // token t: accumulator and scale, add, store
+            auto load_acc = [&](int t, float2& a2, float& rq) {
+                lds64(smem_u32(V_s) + (uint32_t)(t * (kW * 4) + (((cp >> 1) ^ (t & 7)) << 4) + (cp & 1) * 8), a2);
+                rq = __uint_as_float(lds32(smem_u32(rq_s) + (uint32_t)t * 4));
+            };
+            auto emit = [&](uint32_t* to, float2 a2, float rq, float2 add) {
                 const float2 o = ffma2(a2, make_float2(rq, rq), add);
-                out_plane[t * out_tok] = pack_bf16x2(o.x, o.y);
+                *to = pack_bf16x2(o.x, o.y);
             };
             const uint32_t v_base = smem_u32(K_s) + cp * 4;
             for (int u = ww; u < n_units; u += kWarps) {
                 const int strip = u % n_strips, y_first = (u / n_strips) * seg_rows, n_rows = min(seg_rows, prm.gridH - y_first);
                 const int x0 = strip * 2 * STEP + par;    // grid column of the lane's first output; the next is x0 + STEP
                 const bool first = x0 < W, second = x0 + STEP < W;
-                bool cv[NIN];
+                uint32_t cmask[NIN];      // of the words that lie in the grid's columns
 #pragma unroll
-                for (int o = 0; o < NIN; ++o) cv[o] = (unsigned)(x0 + o - R) < (unsigned)W;
+                for (int o = 0; o < NIN; ++o) cmask[o] = (unsigned)(x0 + o - R) < (unsigned)W ? 0xffffffffu : 0u;
                 float2 acc[KS][2];   // output row y of the unit in slot y % KS
 #pragma unroll
                 for (int k = 0; k < KS; ++k) acc[k][0] = acc[k][1] = zero2;
-                uint32_t raw[NIN];   // the words of the next halo row
+                uint32_t raw[NIN], rmask = 0;   // the words of the next halo row, all ones if it lies in the grid
+                uint32_t v_row = v_base + (uint32_t)((prm.prefix + (y_first - R) * W + x0 - R) * kRow);
                 auto load_row = [&](int hy) {
-                    const int yy = y_first + hy - R;
-                    const uint32_t row = v_base + (uint32_t)((prm.prefix + yy * W + x0 - R) * kRow);
-                    const bool rv = (unsigned)yy < (unsigned)prm.gridH;
+                    rmask = (unsigned)(y_first + hy - R) < (unsigned)prm.gridH ? 0xffffffffu : 0u;
+                    const uint32_t from = rmask ? v_row : v_base;
 #pragma unroll
-                    for (int o = 0; o < NIN; ++o)
-                        asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %2, 0;\n\tmov.b32 %0, 0;\n\t@p ld.shared.b32 %0, [%1];\n\t}"
-                                     : "=r"(raw[o]) : "r"(row + (uint32_t)(o * kRow)), "r"((int)(rv && cv[o])));
+                    for (int o = 0; o < NIN; ++o) raw[o] = lds32(from + (uint32_t)(o * kRow));
+                    v_row += (uint32_t)(W * kRow);
                 };
                 load_row(0);
+                int t = prm.prefix + (y_first - (KS - 1)) * W + x0;        // token of the row that ends with this halo row
+                uint32_t* to = out_plane + t * out_tok;
                 for (int h0 = 0; h0 < n_rows + KS - 1; h0 += KS) {
 #pragma unroll
                     for (int k = 0; k < KS; ++k) {
@@ -402,8 +410,17 @@ tc_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
                         if (hy >= n_rows + KS - 1) break;
                         float2 in[NIN];
 #pragma unroll
-                        for (int o = 0; o < NIN; ++o) in[o] = make_float2(bf16lo(raw[o]), bf16hi(raw[o]));
+                        for (int o = 0; o < NIN; ++o) {
+                            const uint32_t word = raw[o] & cmask[o] & rmask;
+                            in[o] = make_float2(bf16lo(word), bf16hi(word));
+                        }
                         load_row(hy + 1);
+                        float2 a2[2];
+                        float rq[2];
+                        const bool ends = hy >= KS - 1;
+                        // of the outputs that end with this row (beyond the grid they are some other token's): ahead of the
+                        // FMAs where there are registers for it
+                        if (kEarly && ends) { load_acc(t, a2[0], rq[0]); load_acc(t + STEP, a2[1], rq[1]); }
                         acc[k][0] = acc[k][1] = c2;   // output row hy starts here; it ends KS - 1 rows on
 #pragma unroll
                         for (int dx = 0; dx < KS; ++dx)
@@ -412,17 +429,23 @@ tc_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
 #pragma unroll
                                 for (int c = 0; c < 2; ++c)
                                     acc[(k - dy + KS) % KS][c] = ffma2(wreg[dy][dx], in[STEP * c + dx], acc[(k - dy + KS) % KS][c]);
-                        const int y = hy - (KS - 1);
-                        if (y >= 0) {
-                            const int t = prm.prefix + (y_first + y) * W + x0;
-                            if (first) emit(t, acc[(k + 1) % KS][0]);
-                            if (second) emit(t + STEP, acc[(k + 1) % KS][1]);
+                        if (ends) {
+                            if (!kEarly) { load_acc(t, a2[0], rq[0]); load_acc(t + STEP, a2[1], rq[1]); }
+                            if (first) emit(to, a2[0], rq[0], acc[(k + 1) % KS][0]);
+                            if (second) emit(to + STEP * out_tok, a2[1], rq[1], acc[(k + 1) % KS][1]);
                         }
+                        t += W;
+                        to += W * out_tok;
                     }
                 }
             }
             // off-grid leading tokens: the attention terms only
-            for (int t = ww * STEP + par; t < prm.prefix; t += kWarps * STEP) emit(t, hs2);
+            for (int t = ww * STEP + par; t < prm.prefix; t += kWarps * STEP) {
+                float2 a2;
+                float rq;
+                load_acc(t, a2, rq);
+                emit(out_plane + t * out_tok, a2, rq, hs2);
+            }
             fence_proxy_async_smem();
             mbar_arrive(plane_free);
         }
@@ -473,8 +496,8 @@ cudaError_t launch_fused_ks(const Problem& p, unsigned* status, cudaStream_t st)
 template <int KS, bool NARROW>
 cudaError_t launch_fused_width(const Problem& p, unsigned* status, cudaStream_t st) {
     // Small CTAs when the plane fits and they need fewer rounds of planes: a plane takes them about 1.2 times as long.  Measured,
-    // large against small: 1000 planes of 7 x 7, width 32, 16.8 / 13.4 us; 3000 of 16 x 16 69.7 / 59.8; 320 of 11 x 11, width
-    // 64, 14.0 / 12.3; 5x5 filters, 450 of 11 x 11, 30.1 / 24.5.  As many rounds with either: 148 planes of 11 x 11 8.1 / 9.5,
+    // large against small: 1000 planes of 7 x 7, width 32, 17.3 / 13.5 us; 3000 of 16 x 16 71.3 / 56.9; 320 of 11 x 11, width
+    // 64, 13.7 / 11.8; 5x5 filters, 450 of 11 x 11, 29.4 / 23.8.  As many rounds with either: 148 planes of 11 x 11 8.1 / 9.5,
     // 450 15.7 / 17.9.
     auto rounds = [&](int ctas) { const int n = ctas * device_sm_count(); return (p.BH + n - 1) / n; };
     if (p.N <= Geo<KS, NARROW, 128>::kTokens && rounds(Geo<KS, NARROW, 128>::kCtas) < rounds(Geo<KS, NARROW, 256>::kCtas))
