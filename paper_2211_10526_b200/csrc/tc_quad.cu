@@ -661,12 +661,13 @@ cudaError_t launch_quad_ks(const Problem& p, unsigned* status, cudaStream_t st) 
     prm.lo = p.lo;
     prm.hdiv = p.hdiv; prm.H = p.H; prm.head0 = p.head0; prm.N = p.N;
     prm.gridH = p.gridH; prm.gridW = p.gridW;
-    // Two query tiles per item share the key tiles and keep both halves of the weight warps busy, but an item of one tile
-    // takes about 0.6 of its time: one tile each when that fills the multiprocessors in fewer rounds.
+    // Two query tiles per item share the key tiles and keep both halves of the weight warps busy; an item of one tile takes
+    // 0.7 (exact kernel) to 0.85 of its time: one tile each where that leaves (nearly) as few rounds.  Measured, one tile
+    // against two: exact, 24 planes of 32 x 64 (3 rounds / 2) 79.9 / 72.8 us; masked, 192 planes of 14 x 14 (3 / 2) 27.5 / 23.1.
     const int sms = device_sm_count();
     const int q_tiles = (p.N + kTile - 1) / kTile;
     const long long one = (long long)p.BH * q_tiles, two = (long long)p.BH * ((q_tiles + 1) / 2);
-    prm.slots = ((one + sms - 1) / sms) * 3 < ((two + sms - 1) / sms) * 5 ? 1 : 2;
+    prm.slots = ((one + sms - 1) / sms) * 3 < ((two + sms - 1) / sms) * 4 ? 1 : 2;
     prm.groups = (q_tiles + prm.slots - 1) / prm.slots;
     prm.k_tiles = q_tiles;
     prm.n_items = p.BH * prm.groups;
