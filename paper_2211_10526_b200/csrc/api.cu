@@ -88,38 +88,40 @@ int check_shape(const castling_attn* h, int B, int H, int gridH, int gridW, int 
     return CASTLING_OK;
 }
 
-int ensure_workspace(castling_attn* h, int BH, int N, int d, bool bf16) {
-    const size_t need = workspace_words(BH, N, d, bf16) * sizeof(float);
-    if (need <= h->ws_bytes) return CASTLING_OK;
-    if (h->cfg.max_workspace && need > h->cfg.max_workspace) return CASTLING_ERR_OOM;
-    cudaError_t e = cudaDeviceSynchronize();  // nothing may still be using the old buffer
-    if (e != cudaSuccess) return fail_cuda(h, e);
-    if (h->ws) cudaFree(h->ws);
+// The workspace and, where the tensor-core path wants them, its arrival counters behind it: one allocation (a second one
+// cost a new handle's first call 0.25 ms).
+int ensure_workspace(castling_attn* h, int BH, int N, int d, bool bf16, bool counters = false) {
+    size_t need = workspace_words(BH, N, d, bf16) * sizeof(float), want = 0;
+    if (counters) {
+        // either variant of the tensor-core path: 17 words per plane, or a header and 4 words per plane
+        const size_t a = (size_t)BH * castling::tc::kCountersPerHead;
+        const size_t b = castling::tc::kPipeCtrHeader + (size_t)BH * castling::tc::kPipeCtrPerPlane;
+        want = a > b ? a : b;
+    }
+    if (need <= h->ws_bytes && want <= h->counters_cap) return CASTLING_OK;
+    if (need > h->ws_bytes && h->cfg.max_workspace && need > h->cfg.max_workspace) return CASTLING_ERR_OOM;
+    if (need < h->ws_bytes) need = h->ws_bytes;
+    size_t cap = h->counters_cap;
+    if (want > cap) for (cap = 4096; cap < want;) cap *= 2;
+    unsigned status = 0;   // an error not reported yet outlives the buffer
+    if (h->ws) {
+        cudaError_t e = cudaDeviceSynchronize();  // nothing may still be using the old buffer
+        if (e == cudaSuccess) e = cudaMemcpy(&status, h->ws, sizeof(status), cudaMemcpyDeviceToHost);
+        if (e != cudaSuccess) return fail_cuda(h, e);
+        cudaFree(h->ws);
+    }
     h->ws = nullptr; h->ws_bytes = 0;
-    e = cudaMalloc((void**)&h->ws, need);
-    if (e != cudaSuccess) return fail_cuda(h, e, CASTLING_ERR_OOM);
+    h->counters = nullptr; h->counters_cap = 0;
+    cudaError_t e = cudaMalloc((void**)&h->ws, need + cap * sizeof(unsigned));
+    if (e != cudaSuccess) { h->ws = nullptr; return fail_cuda(h, e, CASTLING_ERR_OOM); }
     e = cudaMemset(h->ws, 0, castling::kHeaderWords * sizeof(float));
+    if (e == cudaSuccess && cap) e = cudaMemset(reinterpret_cast<char*>(h->ws) + need, 0, cap * sizeof(unsigned));
+    if (e == cudaSuccess && status) e = cudaMemcpy(h->ws, &status, sizeof(status), cudaMemcpyHostToDevice);
+    // the caller's stream may be one that does not wait for the default stream's memsets
+    if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
     if (e != cudaSuccess) return fail_cuda(h, e);
     h->ws_bytes = need;
-    return CASTLING_OK;
-}
-
-int ensure_counters(castling_attn* h, int BH) {
-    // either variant of the tensor-core path: 17 words per plane, or a header and 4 words per plane
-    const size_t a = (size_t)BH * castling::tc::kCountersPerHead;
-    const size_t b = castling::tc::kPipeCtrHeader + (size_t)BH * castling::tc::kPipeCtrPerPlane;
-    const size_t want = a > b ? a : b;
-    if (want <= h->counters_cap) return CASTLING_OK;
-    size_t cap = 4096;
-    while (cap < want) cap *= 2;
-    cudaError_t e = cudaDeviceSynchronize();
-    if (e != cudaSuccess) return fail_cuda(h, e);
-    if (h->counters) cudaFree(h->counters);
-    h->counters = nullptr; h->counters_cap = 0;
-    e = cudaMalloc((void**)&h->counters, cap * sizeof(unsigned));
-    if (e != cudaSuccess) return fail_cuda(h, e, CASTLING_ERR_OOM);
-    e = cudaMemset(h->counters, 0, cap * sizeof(unsigned));
-    if (e != cudaSuccess) return fail_cuda(h, e);
+    if (cap) h->counters = reinterpret_cast<unsigned*>(reinterpret_cast<char*>(h->ws) + need);
     h->counters_cap = cap;
     return CASTLING_OK;
 }
@@ -161,7 +163,6 @@ int castling_attn_destroy(castling_attn_t* h) {
     if (!h) return CASTLING_OK;
     if (h->ws) cudaFree(h->ws);
     if (h->stage) cudaFree(h->stage);
-    if (h->counters) cudaFree(h->counters);
     if (h->copy_in) cudaStreamDestroy(h->copy_in);
     if (h->copy_out) cudaStreamDestroy(h->copy_out);
     if (h->ev_start) cudaEventDestroy(h->ev_start);
@@ -238,13 +239,13 @@ int run_device(castling_attn* h, Problem p, cudaStream_t stream) {
         h->last_launches = launches;
         return CASTLING_OK;
     }
-    int rc = ensure_workspace(h, p.BH, p.N, p.d, p.bf16);
-    if (rc != CASTLING_OK) return rc;
-    p.status = reinterpret_cast<unsigned*>(h->ws);
     const bool tensor_ok = castling::tc::supports(p);
-    if (h->cfg.force_path == CASTLING_PATH_TENSOR && !tensor_ok) return CASTLING_ERR_UNSUPPORTED;
     bool use_tensor = tensor_ok && (h->cfg.force_path == CASTLING_PATH_TENSOR ||
                                     (h->cfg.force_path == CASTLING_PATH_AUTO && castling::tc::preferred(p)));
+    int rc = ensure_workspace(h, p.BH, p.N, p.d, p.bf16, use_tensor);
+    if (rc != CASTLING_OK) return rc;
+    p.status = reinterpret_cast<unsigned*>(h->ws);
+    if (h->cfg.force_path == CASTLING_PATH_TENSOR && !tensor_ok) return CASTLING_ERR_UNSUPPORTED;
     float* state = h->ws + castling::kHeaderWords;
     const size_t simt_words = p.rownorm ? castling::state_words_rownorm(p.d) : castling::state_words(p.d);
     float* partial = state + (size_t)p.BH * (use_tensor ? (size_t)castling::tc::state_words_of(p) : simt_words);
@@ -252,8 +253,6 @@ int run_device(castling_attn* h, Problem p, cudaStream_t stream) {
     h->timer.begin(stream);
     cudaError_t e;
     if (use_tensor) {
-        rc = ensure_counters(h, p.BH);
-        if (rc != CASTLING_OK) return rc;
         e = castling::tc::forward(p, state, partial, h->counters, reinterpret_cast<unsigned*>(h->ws), stream, &launches, &h->timer);
     } else {
         e = castling::simt_forward(p, state, partial, castling::simt_choose_splits(p.BH, p.N, p.d, p.bf16), stream, &launches,
@@ -430,9 +429,7 @@ int castling_attn_forward_host(castling_attn_t* h, const void* q, const void* k,
     // workspace and counters for every run length, before anything is in flight: growing them later
     // would synchronise the device in the middle of the pipeline (and clear the status word)
     for (int c = 0; c < chunks; ++c) {
-        rc = ensure_workspace(h, b0[c + 1] - b0[c], (int)n_tok, d, dtype == CASTLING_BF16);
-        if (rc != CASTLING_OK) return rc;
-        rc = ensure_counters(h, b0[c + 1] - b0[c]);
+        rc = ensure_workspace(h, b0[c + 1] - b0[c], (int)n_tok, d, dtype == CASTLING_BF16, true);
         if (rc != CASTLING_OK) return rc;
     }
     for (int c = 0; c < chunks; ++c) {
@@ -504,16 +501,14 @@ int castling_attn_shard_state(castling_attn_t* h, const void* k, const void* v, 
     if (((uintptr_t)k | (uintptr_t)v | (uintptr_t)state_out) & 15) return CASTLING_ERR_ALIGNMENT;
     Problem p = make_problem(h, nullptr, k, v, nullptr, nullptr, nullptr, B, H, 1, n_tokens, d, dtype);
     p.phase = castling::kPhaseStateOnly;
-    rc = ensure_workspace(h, p.BH, p.N, p.d, p.bf16);
+    bool tensor = h->cfg.force_path != CASTLING_PATH_SIMT && castling::tc::shard_supports(p);
+    rc = ensure_workspace(h, p.BH, p.N, p.d, p.bf16, tensor);
     if (rc != CASTLING_OK) return rc;
     float* partial = h->ws + castling::kHeaderWords + (size_t)p.BH * castling::state_words(p.d);
     int launches = 0;
     h->timer.begin(static_cast<cudaStream_t>(stream));
-    bool tensor = h->cfg.force_path != CASTLING_PATH_SIMT && castling::tc::shard_supports(p);
     cudaError_t e = cudaSuccess;
     if (tensor) {
-        rc = ensure_counters(h, p.BH);
-        if (rc != CASTLING_OK) return rc;
         // the partial states of the tensor-core kernel follow BH final-state slots of its own size
         partial = h->ws + castling::kHeaderWords + (size_t)p.BH * castling::tc::kStateWords;
         e = castling::tc::shard_state(p, state_out, partial, h->counters, reinterpret_cast<unsigned*>(h->ws),
