@@ -534,9 +534,9 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                 const unsigned short* w0 = reinterpret_cast<const unsigned short*>(prm.w) + (size_t)(head * kD + 2 * lane) * (KS * KS);
                 for (int e = cw; e < KS * KS; e += kConvThreads / 32)
                     w_s[e * 32] = (uint32_t)__ldg(w0 + e) | ((uint32_t)__ldg(w0 + KS * KS + e) << 16);
-                if (prm.bias) {
-                    const uint32_t bw = __ldg(reinterpret_cast<const uint32_t*>(prm.bias + head * kD) + lane);
-                    bias2 = make_float2(bf16lo(bw), bf16hi(bw));
+                if (prm.bias) {   // element by element, like the filters: neither need begin on a word boundary
+                    const unsigned short* b0 = reinterpret_cast<const unsigned short*>(prm.bias) + head * kD + 2 * lane;
+                    bias2 = make_float2(bf16lo(__ldg(b0)), bf16lo(__ldg(b0 + 1)));
                 }
                 named_barrier_sync(1, kConvThreads);
                 if (KS == 3) {
