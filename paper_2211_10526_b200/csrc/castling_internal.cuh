@@ -44,6 +44,7 @@ struct Problem {
                              // side (heads h, h+1 of a layout whose head stride is 32): rows are normalised per
                              // half and only the two diagonal 32 x 32 blocks of the state are used
     bool narrow = false;     // tensor-core path only: width-32 heads in 64-byte rows of their own
+    bool fine = false;       // with `narrow`: unit keys and scaled states as two bf16 each (value and rest), as precise as fp32
     // Variants beyond the inference-time core (all off by default):
     bool rownorm = false;       // every row of attention weights divided by its sum (Eq. 3's denominator)
     bool exact_kernel = false;  // 1 - arccos(x)/pi (Eq. 4-5) instead of its kept part 1/2 + x/pi (Eq. 8)

@@ -10,14 +10,17 @@
 //   warps 10..  depthwise convolution, lane = (column parity, channel pair): two columns at a time slide down the patch, every
 //               word of V is loaded and unpacked once per pair of columns, sums of the KS open output rows in registers;
 //               result (+ 1/2 s + bias) staged in shared memory as fp32
+// FINE: S' is held as two bf16, the value and what rounding it left off, and contracted with Q (which is exact) one after the other.
 // Bound: the packed FMAs of the convolution, 2.5 to 3 cycles each (5 x 5 filters: its warps are busy 3 100 of the 3 300 cycles of
 // a patch, with four of them as with eight).
-// Measured (per forward with the state kernel): 8 x 8 planes of 50 x 75, 5 x 5 filters 31 us (245 on the CUDA-core kernels,
-// which took odd widths before; 39 with the words of a row loaded right before their use); 64 x 64 27 us (37 with two tokens
+// Measured (per forward with the state kernel): 8 x 8 planes of 50 x 75, 5 x 5 filters 33 us (FINE; 31 otherwise; 245 on the
+// CUDA-core kernels; 39 with the words of a row loaded right before their use); 64 x 64 27 us (37 with two tokens
 // packed to a 128-byte row, where a lane's window slid two tokens per output and loaded 4.3 words per output instead of 3.1, and
 // two CTA-wide barriers joined the warps per patch).
 #include "tc_common.cuh"
 #include "tc_host.cuh"
+
+#include <type_traits>
 
 namespace castling {
 namespace tc {
@@ -32,7 +35,7 @@ constexpr int kEpiThreads = 256;
 constexpr int kStages = 3;
 constexpr int kCols = 2;                       // columns per lane of the convolution
 
-template <int KS, int kTX> struct Geo {
+template <int KS, int kTX, bool FINE> struct Geo {
     static constexpr int R = KS / 2, kTY = kTile / kTX;
     // a convolution warp takes 8 rows of four columns
     static constexpr int kConvWarps = 8, kConvThreads = kConvWarps * 32, kRows = 8, kGroups = kTX / (2 * kCols);
@@ -40,8 +43,10 @@ template <int KS, int kTX> struct Geo {
     static constexpr int HY = kTY + 2 * R, HX = kTX + 2 * R;
     static constexpr int kVBytes = HY * HX * kD * 2;
     static constexpr int kStage = ((kQBytes + kVBytes + 1023) / 1024) * 1024;
-    // S' | its second block (row sums) | 1/2 s (row sums) | out rows | stages | staging x2 | barriers
-    static constexpr int kOffS = 0, kOffS2 = 2048, kOffHs = 4096, kOffOut = 5120, kOffStages = kOffOut + kQBytes;
+    // S' | its second block (row sums) | the rest of both (FINE) | 1/2 s (row sums) | out rows | stages | staging x2 | barriers; the
+    // swizzle repeats every 512 bytes
+    static constexpr int kOffS = 0, kOffS2 = 2048, kRest = 4096, kOffHs = FINE ? 8192 : 4096;
+    static constexpr int kOffOut = FINE ? kOffHs + 512 : 5120, kOffStages = kOffOut + kQBytes;
     static constexpr int kOffStg = kOffStages + kStages * kStage;
     static constexpr int kOffBar = kOffStg + 2 * kStgBytes;
     static constexpr size_t kSmem = 1024 + kOffBar + 256;
@@ -60,11 +65,11 @@ struct Apply32Params {
 };
 
 // RN: row-sum normalisation, as in the width-64 kernel: column 32 of the accumulator is q . sum k^ / pi.
-template <int KS, bool RN, int kTX>
-__global__ void __launch_bounds__((Geo<KS, kTX>::kThreads), 1)
+template <int KS, bool RN, int kTX, bool FINE>
+__global__ void __launch_bounds__((Geo<KS, kTX, FINE>::kThreads), 1)
 tc_apply32_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmV,
                   const __grid_constant__ CUtensorMap tmO, const Apply32Params prm) {
-    using G = Geo<KS, kTX>;
+    using G = Geo<KS, kTX, FINE>;
     constexpr int kTY = G::kTY;
     constexpr int kSW = kD * kD + kD + (RN ? kD : 0);   // words of one state
     constexpr int kAccN = RN ? kD + 16 : kD;            // columns the UMMAs write per tile
@@ -146,6 +151,7 @@ tc_apply32_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         constexpr uint32_t idesc = umma_idesc_bf16(128, kAccN, false, true);
         const uint32_t s_addr = smem_u32(S_s);
         const uint32_t s_low = desc_low(s_addr, RN ? smem_u32(S2_s) - s_addr : 0);
+        constexpr uint32_t kRest = G::kRest >> 4;   // to the rest of S'
         int prev_bh = -1, seg = 0;
         for (int it = 0; it < my_tiles; ++it, step()) {
             const int s = it % kStages, use = it / kStages, b = it & 1, ub = it >> 1;
@@ -161,9 +167,11 @@ tc_apply32_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
 #pragma unroll
                 for (int t = 0; t < 2; ++t)
 #pragma unroll
-                    for (int k = 0; k < kD / 16; ++k)   // the operand is N-major, 16 K-rows of 64 B per step
-                        umma_bf16_low<kDescHigh64>(tmem + b * kAcc + t * kAccTile, q_low + t * (kQBytes / 2 >> 4) + k * 2,
-                                                   s_low + k * (1024u >> 4), idesc, k != 0);
+                    for (int k = 0; k < (FINE ? 2 : 1) * kD / 16; ++k) {   // the operand is N-major, 16 K-rows of 64 B per step
+                        const int kk = k % (kD / 16);
+                        umma_bf16_low<kDescHigh64>(tmem + b * kAcc + t * kAccTile, q_low + t * (kQBytes / 2 >> 4) + kk * 2,
+                                                   s_low + kk * (1024u >> 4) + (k < kD / 16 ? 0u : kRest), idesc, k != 0);
+                    }
                 umma_commit(&acc_full[b]);
                 umma_commit(&empty[s]);  // the same UMMAs have finished reading the Q patch
             }
@@ -191,10 +199,20 @@ tc_apply32_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                     const float4 hi = __ldg(reinterpret_cast<const float4*>(st + i * kD + part * 8 + 4));
                     o.x = pack_bf16x2(lo.x * kInvPi, lo.y * kInvPi); o.y = pack_bf16x2(lo.z * kInvPi, lo.w * kInvPi);
                     o.z = pack_bf16x2(hi.x * kInvPi, hi.y * kInvPi); o.w = pack_bf16x2(hi.z * kInvPi, hi.w * kInvPi);
-                    *reinterpret_cast<uint4*>(S_s + i * 64 + ((part ^ ((i >> 1) & 3)) << 4)) = o;
+                    uint8_t* at = S_s + i * 64 + ((part ^ ((i >> 1) & 3)) << 4);
+                    *reinterpret_cast<uint4*>(at) = o;
+                    if (FINE) *reinterpret_cast<uint4*>(at + G::kRest) =
+                        make_uint4(rest_bf16x2(lo.x, lo.y, kInvPi, o.x), rest_bf16x2(lo.z, lo.w, kInvPi, o.y),
+                                   rest_bf16x2(hi.x, hi.y, kInvPi, o.z), rest_bf16x2(hi.z, hi.w, kInvPi, o.w));
                 } else if (RN) {   // second block of the operand: sum k^ / pi in column 0
-                    if (part == 0) o.x = pack_bf16x2(__ldg(st + kD * kD + kD + i) * kInvPi, 0.f) & 0xffffu;
-                    *reinterpret_cast<uint4*>(S2_s + i * 64 + ((part ^ ((i >> 1) & 3)) << 4)) = o;
+                    const float z = __ldg(st + kD * kD + kD + i);
+                    if (part == 0) o.x = pack_bf16x2(z * kInvPi, 0.f) & 0xffffu;
+                    uint8_t* at = S2_s + i * 64 + ((part ^ ((i >> 1) & 3)) << 4);
+                    *reinterpret_cast<uint4*>(at) = o;
+                    if (FINE) {
+                        if (part == 0) o.x = rest_bf16x2(z, 0.f, kInvPi, o.x) & 0xffffu;
+                        *reinterpret_cast<uint4*>(at + G::kRest) = o;
+                    }
                 }
                 fence_proxy_async_smem();
                 mbar_arrive(s_ready);
@@ -335,9 +353,9 @@ tc_apply32_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
     if (warp == 1) tmem_dealloc(tmem, kTmemCols);
 }
 
-template <int KS, bool RN, int kTX>
+template <int KS, bool RN, int kTX, bool FINE>
 cudaError_t launch_apply32_ks(const Problem& p, const float* state, unsigned* status, cudaStream_t st) {
-    using G = Geo<KS, kTX>;
+    using G = Geo<KS, kTX, FINE>;
     constexpr int kTY = G::kTY;
     CUtensorMap tmQ, tmV, tmO;
     // [32, columns, grid rows, planes per batch step, batch steps]; with a single batch step the last dimension is dropped
@@ -369,7 +387,7 @@ cudaError_t launch_apply32_ks(const Problem& p, const float* state, unsigned* st
     prm.eps2 = p.eps2; prm.status = status; prm.n_tokens = p.N;
     static PerDevice opt_in;  // one per instantiation
     {
-        const cudaError_t e = opt_in_smem(tc_apply32_kernel<KS, RN, kTX>, G::kSmem, opt_in);
+        const cudaError_t e = opt_in_smem(tc_apply32_kernel<KS, RN, kTX, FINE>, G::kSmem, opt_in);
         if (e != cudaSuccess) return e;
     }
     const int sms = device_sm_count();
@@ -380,10 +398,10 @@ cudaError_t launch_apply32_ks(const Problem& p, const float* state, unsigned* st
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr; cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, tc_apply32_kernel<KS, RN, kTX>, tmQ, tmV, tmO, prm);
+    return cudaLaunchKernelEx(&cfg, tc_apply32_kernel<KS, RN, kTX, FINE>, tmQ, tmV, tmO, prm);
 }
 
-template <int KS, bool RN>
+template <int KS, bool RN, bool FINE>
 cudaError_t launch_apply32_rn(const Problem& p, const float* state, unsigned* status, cudaStream_t st) {
     // Patches of 16 x 16 where they need fewer rounds of the device.  Measured, 32 columns wide against 16: 8 x 8 planes of
     // 50 x 75, 5 x 5 filters 31.4 / 30.6 us (10 rounds / 9), 25 x 38 18.0 / 16.1 (4 / 3), 3 x 3, 31 x 33 14.1 / 12.9 (4 / 3); as
@@ -392,14 +410,18 @@ cudaError_t launch_apply32_rn(const Problem& p, const float* state, unsigned* st
         const long long n = (long long)p.BH * ((p.gridW + tx - 1) / tx) * ((p.gridH + kTile / tx - 1) / (kTile / tx));
         return (n + device_sm_count() - 1) / device_sm_count();
     };
-    return rounds(16) < rounds(32) ? launch_apply32_ks<KS, RN, 16>(p, state, status, st) : launch_apply32_ks<KS, RN, 32>(p, state, status, st);
+    return rounds(16) < rounds(32) ? launch_apply32_ks<KS, RN, 16, FINE>(p, state, status, st) : launch_apply32_ks<KS, RN, 32, FINE>(p, state, status, st);
 }
 
 }  // namespace
 
 cudaError_t launch_apply32(const Problem& p, const float* state, unsigned* status, cudaStream_t st) {
-    if (p.ksize == 3) return p.rownorm ? launch_apply32_rn<3, true>(p, state, status, st) : launch_apply32_rn<3, false>(p, state, status, st);
-    return p.rownorm ? launch_apply32_rn<5, true>(p, state, status, st) : launch_apply32_rn<5, false>(p, state, status, st);
+    auto launch = [&](auto fine) {
+        constexpr bool F = decltype(fine)::value;
+        if (p.ksize == 3) return p.rownorm ? launch_apply32_rn<3, true, F>(p, state, status, st) : launch_apply32_rn<3, false, F>(p, state, status, st);
+        return p.rownorm ? launch_apply32_rn<5, true, F>(p, state, status, st) : launch_apply32_rn<5, false, F>(p, state, status, st);
+    };
+    return p.fine ? launch(std::true_type{}) : launch(std::false_type{});
 }
 
 }  // namespace tc

@@ -338,6 +338,15 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
     return r;
 }
 
+// What rounding x * r and y * r to bf16 left off, as bf16: `rounded` is the word that pack_bf16x2 made of the products.  Value and
+// rest together carry 16 bits or more.  (The second form: x and y are the two bf16 of a word.)
+__device__ __forceinline__ uint32_t rest_bf16x2(float x, float y, float r, uint32_t rounded) {
+    return pack_bf16x2(fmaf(x, r, -bf16lo(rounded)), fmaf(y, r, -bf16hi(rounded)));
+}
+__device__ __forceinline__ uint32_t rest_bf16x2(uint32_t xy, float r, uint32_t rounded) {
+    return rest_bf16x2(bf16lo(xy), bf16hi(xy), r, rounded);
+}
+
 // A word from shared memory; volatile keeps loads that are issued ahead in front of the arithmetic they are to overlap.
 __device__ __forceinline__ uint32_t lds32(const void* p) {
     uint32_t v;

@@ -73,6 +73,13 @@ cudaError_t forward(const Problem& p_in, float* ws_state, float* ws_partial, uns
                     cudaStream_t stream, int* launches, KernelTimer* timer) {
     *launches = 0;
     Problem p = p_in;
+    // What the packed 128-byte rows do not take, and planes too small to fill their tiles, have the precision of fp32 operands, as
+    // on the CUDA cores: unit keys and scaled states as pairs.  Relative error against 64 bits of the bf16 outputs, CUDA
+    // cores / single bf16 / pairs: 64 x 8 planes of 7 x 7 1.65499e-3 / 1.67565e-3 / 1.65499e-3, 8 x 8 of 50 x 75, 5 x 5 filters,
+    // 1.66210e-3 / 1.68312e-3 / 1.66210e-3, 64 x 8 of 8 x 8 1.65823e-3 / 1.67885e-3 / 1.65823e-3.  Time: 18.4 / 10.3 / 11.7 us,
+    // 245 / 30.6 / 33.2, 21.4 / 10.7 / 12.6.
+    p.fine = p.d == 32 && !head_pairs(p) && (!token_pairs(p) || p.N < 96);
+    const bool fine = p.fine;
     cudaError_t e;
     if (!p.rownorm && fused_supports(p)) {  // a whole (b,h) fits in shared memory: one kernel, no workspace
         e = launch_fused(p, status, stream);
@@ -105,6 +112,7 @@ cudaError_t forward(const Problem& p_in, float* ws_state, float* ws_partial, uns
     } else {
         p = p_in;   // width-32 heads in 64-byte rows of their own
         p.narrow = p.d == 32;
+        p.fine = fine;
         const int rows = rows_per_head(p.N, p.d), P = choose_splits(p.BH, rows);
         const int tiles = (rows + kStateTile - 1) / kStateTile;
         e = launch_state(p, ws_partial, ws_state, counters, P, (tiles + P - 1) / P, status, stream);

@@ -19,6 +19,10 @@
 //               strip of two columns (four): depthwise convolution sliding down the strip with the filters in registers,
 //               out = acc / max(||q||, eps) + 1/2 s + bias + conv, one rounding to bf16, rows stored
 //               straight to memory; leading off-grid tokens get the attention terms only
+// FINE (width 32 only): the unit keys and S' are two bf16 each, the value and what rounding it left off, contracted one after the
+// other: as precise as fp32 operands.  The rest of K lies in the Q buffer, so Q comes with the second copy of V, once the state
+// UMMAs have retired; the rest of S' lies in the V buffer, which is dead by then.  512 planes of 7 x 7: 11.7 us a call, 10.3
+// with single operands.
 //
 // A plane is a serial chain of about 15 000 cycles (14 x 14 tokens, width 64, 7 000 of them the convolution), so the time of
 // a call is the number of planes over those in flight.  Two shapes of CTA: 256 workers for planes of any size, two per SM;
@@ -70,7 +74,7 @@ struct FusedParams {
 
 // OUT_PACKED: the output's token rows are contiguous, which keeps the row addresses of the
 // store loop compile-time offsets.
-template <int KS, bool OUT_PACKED, bool NARROW, int WORKERS>
+template <int KS, bool OUT_PACKED, bool NARROW, int WORKERS, bool FINE>
 __global__ void __launch_bounds__((Geo<KS, NARROW, WORKERS>::kThreads), (Geo<KS, NARROW, WORKERS>::kCtas))
 tc_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
                 const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmVplain,
@@ -142,11 +146,15 @@ tc_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
                 for (int t = 0; t < tiles; ++t) tma_load_4d_hint(K_s + t * kTileBytes, &tmK, k_full, 0, t * kTile, ph, pb, pol);
                 mbar_expect_tx(v_full, tiles * kTileBytes);
                 for (int t = 0; t < tiles; ++t) tma_load_4d(V_s + t * kTileBytes, &tmV, v_full, 0, t * kTile, ph, pb);
-                mbar_expect_tx(q_full, tiles * kTileBytes);
-                for (int t = 0; t < tiles; ++t) tma_load_4d_hint(Q_s + t * kTileBytes, &tmQ, q_full, 0, t * kTile, ph, pb, pol);
+                auto load_q = [&]() {
+                    mbar_expect_tx(q_full, tiles * kTileBytes);
+                    for (int t = 0; t < tiles; ++t) tma_load_4d_hint(Q_s + t * kTileBytes, &tmQ, q_full, 0, t * kTile, ph, pb, pol);
+                };
+                if (!FINE) load_q();
                 ++issued;
                 // the K tiles are dead once the state UMMAs have retired: bring V in again, unswizzled
                 if (!mbar_wait(s_done, it & 1, abort_flag, prm.status, kBit)) break;
+                if (FINE) load_q();   // over the rest of K
                 mbar_expect_tx(vp_full, tiles * kTileBytes);
                 for (int t = 0; t < tiles; ++t) tma_load_4d(K_s + t * kTileBytes, &tmVplain, vp_full, 0, t * kTile, ph, pb);
                 ++issued_vp;
@@ -157,8 +165,9 @@ tc_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
                     const uint32_t ph = (issued - 1) & 1;
                     for (int spin = 0; spin < (1 << 20) && !mbar_try_wait(k_full, ph); ++spin) {}
                     for (int spin = 0; spin < (1 << 20) && !mbar_try_wait(v_full, ph); ++spin) {}
-                    for (int spin = 0; spin < (1 << 20) && !mbar_try_wait(q_full, ph); ++spin) {}
                 }
+                const int issued_q = FINE ? issued_vp : issued;
+                if (issued_q) for (int spin = 0; spin < (1 << 20) && !mbar_try_wait(q_full, (issued_q - 1) & 1); ++spin) {}
                 if (issued_vp) for (int spin = 0; spin < (1 << 20) && !mbar_try_wait(vp_full, (issued_vp - 1) & 1); ++spin) {}
             }
         }
@@ -180,9 +189,12 @@ tc_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
             tcgen05_fence_after_sync();
             if (elect_one()) {
                 uint32_t a = desc_low(k_addr, ones_addr - k_addr), b = desc_low(v_addr);
+                uint32_t rest = FINE ? desc_low(q_addr, ones_addr - q_addr) : 0;   // its row of ones counts the tokens a second time
 #pragma unroll 4
-                for (int j = 0; j < steps; ++j, a += kStepA, b += kStepB)  // one UMMA per 16 tokens (K = 16)
+                for (int j = 0; j < steps; ++j, a += kStepA, b += kStepB) {  // one UMMA per 16 tokens (K = 16)
                     umma_bf16_low<kHigh>(tmem, a, b, idesc_state, j != 0);
+                    if (FINE) { umma_bf16_low<kHigh>(tmem, rest, b, idesc_state, 1u); rest += kStepA; }
+                }
                 umma_commit(s_done);
             }
             __syncwarp();
@@ -190,11 +202,13 @@ tc_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
             if (!mbar_wait_warp(sp_ready, ph, abort_flag, prm.status, kBit)) break;
             tcgen05_fence_after_sync();
             if (elect_one()) {
-                const uint32_t sl = desc_low(s_addr);
+                const uint32_t sl = desc_low(s_addr), sl_rest = desc_low(v_addr);
                 for (int t = 0; t < tiles; ++t) {
                     const uint32_t q = desc_low(q_addr + t * kTileBytes);
 #pragma unroll
                     for (int k = 0; k < kW / 16; ++k) umma_bf16_low<kHigh>(tmem + t * kW, q + k * 2, sl + k * kStepB, idesc_apply, k != 0);
+#pragma unroll
+                    for (int k = 0; FINE && k < kW / 16; ++k) umma_bf16_low<kHigh>(tmem + t * kW, q + k * 2, sl_rest + k * kStepB, idesc_apply, 1u);
                 }
                 umma_commit(o_done);
             }
@@ -267,14 +281,24 @@ tc_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
                         o4[e] = pack_bf16x2(p.x, p.y);
                     }
                     *reinterpret_cast<uint4*>(row + ((j ^ (wt & 7)) << 4)) = make_uint4(o4[0], o4[1], o4[2], o4[3]);
+                    if (FINE) {
+                        uint32_t r4[4];
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) r4[e] = rest_bf16x2(w4[e], rk2.x, o4[e]);
+                        *reinterpret_cast<uint4*>(Q_s + wt * 128 + ((j ^ (wt & 7)) << 4)) = make_uint4(r4[0], r4[1], r4[2], r4[3]);
+                    }
                 }
+                fence_proxy_async_smem();
+            } else if (FINE && wt * 2 < (N + 15) / 16 * 16) {   // tokens beyond the plane that the UMMAs take along
+#pragma unroll
+                for (int j = 0; j < 8; ++j) *reinterpret_cast<uint4*>(Q_s + wt * 128 + (j << 4)) = make_uint4(0, 0, 0, 0);
                 fence_proxy_async_smem();
             }
             mbar_arrive(k_scaled);
 
             // ---- 1 / max(||q||, eps) ----
-            if (!mbar_wait(q_full, ph, abort_flag, prm.status, kBit)) break;
-            if (has_line) {
+            auto q_norms = [&]() {
+                if (!has_line) return;
                 const uint8_t* row = Q_s + wt * 128;
                 uint4 c[8];
 #pragma unroll
@@ -288,6 +312,10 @@ tc_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
                 } else {
                     rq_s[wt] = rsqrtf(fmaxf(sa + sb, prm.eps2));
                 }
+            };
+            if (!FINE) {
+                if (!mbar_wait(q_full, ph, abort_flag, prm.status, kBit)) break;
+                q_norms();
             }
 
             // ---- S, s out of TMEM -> S' (bf16 operand) and s ----
@@ -312,6 +340,9 @@ tc_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
                             o.w = pack_bf16x2(a[8 * e + 6] * kInvPi, a[8 * e + 7] * kInvPi);
                             const int chunk = (col / 8 + e) ^ (NARROW ? (row >> 1) & 3 : row & 7);
                             *reinterpret_cast<uint4*>(S_s + row * kRow + (chunk << 4)) = o;
+                            if (FINE) *reinterpret_cast<uint4*>(V_s + row * kRow + (chunk << 4)) =
+                                make_uint4(rest_bf16x2(a[8 * e + 0], a[8 * e + 1], kInvPi, o.x), rest_bf16x2(a[8 * e + 2], a[8 * e + 3], kInvPi, o.y),
+                                           rest_bf16x2(a[8 * e + 4], a[8 * e + 5], kInvPi, o.z), rest_bf16x2(a[8 * e + 6], a[8 * e + 7], kInvPi, o.w));
                         }
                     } else if (row == kW) {   // the token sum of V
 #pragma unroll
@@ -319,6 +350,10 @@ tc_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
                             *reinterpret_cast<float4*>(sum_s + col + 4 * e) = make_float4(a[4 * e], a[4 * e + 1], a[4 * e + 2], a[4 * e + 3]);
                     }
                 }
+            }
+            if (FINE) {
+                if (!mbar_wait(q_full, ph, abort_flag, prm.status, kBit)) break;
+                q_norms();
             }
             fence_proxy_async_smem();
             tcgen05_fence_before_sync();
@@ -361,7 +396,8 @@ tc_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
             const int par = NARROW ? lane >> 4 : 0, cp = NARROW ? lane & 15 : lane;   // column parity, channel pair
             constexpr int STEP = NARROW ? 2 : 1, NIN = STEP + KS;
             constexpr bool kEarly = WORKERS == 256;
-            const float2 hs2 = make_float2(0.5f * sum_s[2 * cp], 0.5f * sum_s[2 * cp + 1]);   // 1/2 s
+            const float half = FINE ? 0.25f : 0.5f;   // FINE: the sums are of every token twice
+            const float2 hs2 = make_float2(half * sum_s[2 * cp], half * sum_s[2 * cp + 1]);   // 1/2 s
             const float2 bias2 = *reinterpret_cast<const float2*>(w_s + kElems + 2 * cp);
             const float2 c2 = make_float2(hs2.x + bias2.x, hs2.y + bias2.y);  // + bias: grid tokens
             float2 wreg[KS][KS];
@@ -455,7 +491,7 @@ tc_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     if (warp == 1) tmem_dealloc(tmem, G::kTmemCols);
 }
 
-template <int KS, bool NARROW, int WORKERS>
+template <int KS, bool NARROW, int WORKERS, bool FINE>
 cudaError_t launch_fused_ks(const Problem& p, unsigned* status, cudaStream_t st) {
     using G = Geo<KS, NARROW, WORKERS>;
     CUtensorMap tmK, tmV, tmQ, tmVplain;
@@ -481,19 +517,19 @@ cudaError_t launch_fused_ks(const Problem& p, unsigned* status, cudaStream_t st)
     prm.eps2 = p.eps2; prm.status = status;
     static PerDevice opt_in[2];  // per instantiation
     const bool packed = (p.lo.token == G::kW);
-    const cudaError_t e = packed ? opt_in_smem(tc_fused_kernel<KS, true, NARROW, WORKERS>, G::kSmem, opt_in[1])
-                                 : opt_in_smem(tc_fused_kernel<KS, false, NARROW, WORKERS>, G::kSmem, opt_in[0]);
+    const cudaError_t e = packed ? opt_in_smem(tc_fused_kernel<KS, true, NARROW, WORKERS, FINE>, G::kSmem, opt_in[1])
+                                 : opt_in_smem(tc_fused_kernel<KS, false, NARROW, WORKERS, FINE>, G::kSmem, opt_in[0]);
     if (e != cudaSuccess) return e;
     const int resident = G::kCtas * device_sm_count();
     const int grid = p.BH < resident ? p.BH : resident;
     if (packed)
-        tc_fused_kernel<KS, true, NARROW, WORKERS><<<(unsigned)grid, G::kThreads, G::kSmem, st>>>(tmK, tmV, tmQ, tmVplain, prm);
+        tc_fused_kernel<KS, true, NARROW, WORKERS, FINE><<<(unsigned)grid, G::kThreads, G::kSmem, st>>>(tmK, tmV, tmQ, tmVplain, prm);
     else
-        tc_fused_kernel<KS, false, NARROW, WORKERS><<<(unsigned)grid, G::kThreads, G::kSmem, st>>>(tmK, tmV, tmQ, tmVplain, prm);
+        tc_fused_kernel<KS, false, NARROW, WORKERS, FINE><<<(unsigned)grid, G::kThreads, G::kSmem, st>>>(tmK, tmV, tmQ, tmVplain, prm);
     return cudaGetLastError();
 }
 
-template <int KS, bool NARROW>
+template <int KS, bool NARROW, bool FINE>
 cudaError_t launch_fused_width(const Problem& p, unsigned* status, cudaStream_t st) {
     // Small CTAs when the plane fits and they need fewer rounds of planes: a plane takes them about 1.2 times as long.  Measured,
     // large against small: 1000 planes of 7 x 7, width 32, 17.3 / 13.5 us; 3000 of 16 x 16 71.3 / 56.9; 320 of 11 x 11, width
@@ -501,8 +537,8 @@ cudaError_t launch_fused_width(const Problem& p, unsigned* status, cudaStream_t 
     // 450 15.7 / 17.9.
     auto rounds = [&](int ctas) { const int n = ctas * device_sm_count(); return (p.BH + n - 1) / n; };
     if (p.N <= Geo<KS, NARROW, 128>::kTokens && rounds(Geo<KS, NARROW, 128>::kCtas) < rounds(Geo<KS, NARROW, 256>::kCtas))
-        return launch_fused_ks<KS, NARROW, 128>(p, status, st);
-    return launch_fused_ks<KS, NARROW, 256>(p, status, st);
+        return launch_fused_ks<KS, NARROW, 128, FINE>(p, status, st);
+    return launch_fused_ks<KS, NARROW, 256, FINE>(p, status, st);
 }
 
 }  // namespace
@@ -514,8 +550,9 @@ bool fused_supports(const Problem& p) {
 }
 
 cudaError_t launch_fused(const Problem& p, unsigned* status, cudaStream_t st) {
-    if (p.d == 32) return p.ksize == 3 ? launch_fused_width<3, true>(p, status, st) : launch_fused_width<5, true>(p, status, st);
-    return p.ksize == 3 ? launch_fused_width<3, false>(p, status, st) : launch_fused_width<5, false>(p, status, st);
+    if (p.fine) return p.ksize == 3 ? launch_fused_width<3, true, true>(p, status, st) : launch_fused_width<5, true, true>(p, status, st);
+    if (p.d == 32) return p.ksize == 3 ? launch_fused_width<3, true, false>(p, status, st) : launch_fused_width<5, true, false>(p, status, st);
+    return p.ksize == 3 ? launch_fused_width<3, false, false>(p, status, st) : launch_fused_width<5, false, false>(p, status, st);
 }
 
 }  // namespace tc

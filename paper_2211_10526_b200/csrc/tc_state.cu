@@ -27,20 +27,26 @@ constexpr int kOnesBytes = 2048;             // 16 token rows x 128 B: feature 6
 constexpr int kThreads = 192;                // warp 0 TMA, warp 1 UMMA, warps 2..5 scale + epilogue
 constexpr int kTmemCols = 128;                // two 64-column accumulators: a CTA may serve several (b,h) (RN: twice that)
 constexpr int kGroup = 4;                    // splits per first-level reduction group
-constexpr size_t kSmemBytes = 1024 + kStages * kStageBytes + kOnesBytes + 256;
+constexpr int kFineStages = 2, kFineStageBytes = kStageBytes + kTileBytes;   // K, V, the rest of K
+constexpr int kStagesBytes = kStages * kStageBytes;
+static_assert(kFineStages * kFineStageBytes == kStagesBytes, "one size of shared memory");
+constexpr size_t kSmemBytes = 1024 + kStagesBytes + kOnesBytes + 256;
 
 // NARROW serves width-32 heads: rows of 64 bytes, 64-byte swizzle, 256 tokens per stage (any grid width, any number of
 // tokens), UMMAs of M = 64 (32 key features, then the row of ones) and N = 32, states of 32 x 32 + 32 words.  Two tokens
 // packed to a 128-byte row instead, which wastes half of the contraction and needs an even grid width, took 19.8 us against
 // 17.6 us (8 x 8 planes of 64 x 64 tokens).
-template <bool NARROW, bool RN>
+// FINE (NARROW only): the unit keys are kept as two bf16, the value and what rounding it left off, and contracted one after the
+// other, so that the state is as precise as one from fp32 keys; the second tile of K takes the place of a stage.
+template <bool NARROW, bool RN, bool FINE>
 __global__ void __launch_bounds__(kThreads, 2)
 tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
                 float* __restrict__ dst, float* __restrict__ final_state, unsigned* __restrict__ counters,
                 int N, int tiles_per_cta, int P, int BH, int hdiv, int items_per_cta, float eps2, unsigned* status) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = align_smem(smem_raw);
-    uint8_t* ones = smem + kStages * kStageBytes;
+    constexpr int kStages = FINE ? kFineStages : castling::tc::kStages, kStageBytes = FINE ? kFineStageBytes : castling::tc::kStageBytes;
+    uint8_t* ones = smem + kStagesBytes;
     uint64_t* full = reinterpret_cast<uint64_t*>(ones + kOnesBytes);  // TMA bytes landed
     uint64_t* scaled = full + kStages;                                // K rows normalised (128 arrivals)
     uint64_t* empty = scaled + kStages;                               // UMMAs of the stage retired
@@ -89,12 +95,14 @@ tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     if (warp >= 2) {
         // constant block of A: for each of 16 token rows, element 64 (first of the second 64-wide
         // block along M) is 1.0 and the rest 0; 16-byte chunk c of row r sits at chunk c ^ (r & 7)
-        // (rows of 64 bytes: element 32, chunk c of row r at chunk c ^ ((r >> 1) & 3), half as many threads)
+        // (rows of 64 bytes: element 32, chunk c of row r at chunk c ^ ((r >> 1) & 3), half as many threads; FINE: the other
+        // half of the place is a block of zeros, which goes with the rest of K)
         const int t = tid - 64;  // 0..127 -> one 16-byte chunk each
         const int r = NARROW ? t >> 2 : t >> 3, c = NARROW ? t & 3 : t & 7;
         uint4 val = make_uint4(0, 0, 0, 0);
         if ((c ^ (NARROW ? (r >> 1) & 3 : r & 7)) == 0) val.x = 0x3f80u;  // logical chunk 0: bf16 1.0 in its first element
-        if (!NARROW || r < 16) *reinterpret_cast<uint4*>(ones + t * 16) = val;
+        if (NARROW && r >= 16) val.x = 0u;
+        if (!NARROW || FINE || r < 16) *reinterpret_cast<uint4*>(ones + t * 16) = val;
         fence_proxy_async_smem();
     }
     tcgen05_fence_before_sync();
@@ -123,7 +131,7 @@ tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
                     const int s = issued % kStages, use = issued / kStages;
                     if (use > 0 && !mbar_wait(&empty[s], (use - 1) & 1, abort_flag, status, kStatusStateTimeout)) { ok = false; break; }
                     uint8_t* ks = smem + s * kStageBytes;
-                    mbar_expect_tx(&full[s], kStageBytes);
+                    mbar_expect_tx(&full[s], 2 * kTileBytes);
                     const int plane = bh0 + item, pb = plane / hdiv, ph = plane - pb * hdiv;
                     tma_load_4d_hint(ks, &tmK, &full[s], 0, (t_begin + it) * kTok, ph, pb, pol_k);
                     tma_load_4d_hint(ks + kTileBytes, &tmV, &full[s], 0, (t_begin + it) * kTok, ph, pb, pol_v);
@@ -155,10 +163,13 @@ tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
                 if (elect_one()) {
                     const uint32_t ka = smem_u32(smem + s * kStageBytes), va = ka + kTileBytes;
                     const uint32_t a = desc_low(ka, ones_addr - ka), b = desc_low(va, RN ? ones_addr - va : 0);
+                    const uint32_t rest = FINE ? desc_low(va + kTileBytes, ones_addr + kOnesBytes / 2 - (va + kTileBytes)) : 0;
 #pragma unroll
-                    for (int j = 0; j < kTok / 16; ++j)  // one UMMA per 16 tokens (K = 16)
+                    for (int j = 0; j < kTok / 16; ++j) {  // one UMMA per 16 tokens (K = 16)
                         umma_bf16_low<NARROW ? kDescHigh64 : kDescHigh>(tmem + buf * kAcc, a + j * kStep,
                                                                         b + j * (RN ? kStep : kStepB), idesc, (it | j) != 0);
+                        if (FINE) umma_bf16_low<kDescHigh64>(tmem + buf * kAcc, rest + j * kStep, b + j * (RN ? kStep : kStepB), idesc, 1u);
+                    }
                     umma_commit(&empty[s]);
                     if (it == n_tiles - 1) umma_commit(&accum[buf]);
                 }
@@ -243,6 +254,8 @@ tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
                     o.z = pack_bf16x2(bf16lo(c[j].z) * rk, bf16hi(c[j].z) * rk);
                     o.w = pack_bf16x2(bf16lo(c[j].w) * rk, bf16hi(c[j].w) * rk);
                     *reinterpret_cast<uint4*>(row + ((j ^ (t & 7)) << 4)) = o;
+                    if (FINE) *reinterpret_cast<uint4*>(row + 2 * kTileBytes + ((j ^ (t & 7)) << 4)) =
+                        make_uint4(rest_bf16x2(c[j].x, rk, o.x), rest_bf16x2(c[j].y, rk, o.y), rest_bf16x2(c[j].z, rk, o.z), rest_bf16x2(c[j].w, rk, o.w));
                 }
                 fence_proxy_async_smem();
                 mbar_arrive(&scaled[s]);
@@ -371,7 +384,7 @@ cudaError_t launch_state(const Problem& p, float* partial, float* final_state, u
     const int swizzle = narrow ? 64 : 128;
     if (!make_tensor_map_bf16(&tmK, p.k, 4, dims, sk, box, swizzle) || !make_tensor_map_bf16(&tmV, p.v, 4, dims, sv, box, swizzle))
         return cudaErrorNotSupported;
-    static PerDevice opt_in[4];
+    static PerDevice opt_in[6];
     float* dst = P > 1 ? partial : final_state;
     // P == 1: a CTA serves several consecutive (b,h); at most two CTAs per multiprocessor so all are resident
     int grid = p.BH * P, items = 1;
@@ -387,13 +400,14 @@ cudaError_t launch_state(const Problem& p, float* partial, float* final_state, u
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr; cfg.numAttrs = 1;
     auto launch = [&](auto kernel) {
-        const cudaError_t e = opt_in_smem(kernel, kSmemBytes, opt_in[(narrow ? 2 : 0) + (p.rownorm ? 1 : 0)]);
+        const cudaError_t e = opt_in_smem(kernel, kSmemBytes, opt_in[(p.fine ? 4 : narrow ? 2 : 0) + (p.rownorm ? 1 : 0)]);
         if (e != cudaSuccess) return e;
         return cudaLaunchKernelEx(&cfg, kernel, tmK, tmV, dst, final_state, counters, p.N, tiles_per_cta, P, p.BH, p.hdiv, items,
                                   p.eps2, status);
     };
-    if (narrow) return p.rownorm ? launch(tc_state_kernel<true, true>) : launch(tc_state_kernel<true, false>);
-    return p.rownorm ? launch(tc_state_kernel<false, true>) : launch(tc_state_kernel<false, false>);
+    if (p.fine) return p.rownorm ? launch(tc_state_kernel<true, true, true>) : launch(tc_state_kernel<true, false, true>);
+    if (narrow) return p.rownorm ? launch(tc_state_kernel<true, true, false>) : launch(tc_state_kernel<true, false, false>);
+    return p.rownorm ? launch(tc_state_kernel<false, true, false>) : launch(tc_state_kernel<false, false, false>);
 }
 
 }  // namespace tc
