@@ -116,6 +116,18 @@ __device__ __forceinline__ void tcgen05_fence_after_sync() {
 __device__ __forceinline__ void named_barrier_sync(uint32_t id, uint32_t threads) {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
+// The same, and whether any of the threads says so.  It has no time limit: where threads may give up a wait, all of them come
+// here all the same and leave together on the answer.
+__device__ __forceinline__ bool named_barrier_any(uint32_t id, uint32_t threads, bool flag) {
+    uint32_t any;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.u32 p, %3, 0;\n\t"
+        "bar.red.or.pred q, %1, %2, p;\n\t"
+        "selp.u32 %0, 1, 0, q;\n\t}"
+        : "=r"(any) : "r"(id), "r"(threads), "r"((uint32_t)flag) : "memory");
+    return any != 0;
+}
 
 // ---- TMA ------------------------------------------------------------------------------
 __device__ __forceinline__ void tma_prefetch_desc(const CUtensorMap* m) {

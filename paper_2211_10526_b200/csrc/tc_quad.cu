@@ -429,7 +429,8 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
             return done;
         };
         bool ok = true;
-        for (int i = 0; i < my_items && ok; ++i) {
+        // with the mask, a warp that has given up still meets the others at the next item's denominators, where all leave
+        for (int i = 0; i < my_items && (ok || SPARSE); ++i) {
             const Item im = item_of(i);
             if (slot >= im.slots) { skip(kSweeps * T * im.slots); continue; }
             const bool live = im.t0 + slot * kTile + quarter * 32 < N;   // some row of this warp is a token
@@ -438,7 +439,7 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
             if (SPARSE) {
                 float2 den = dup2(0.f);
                 for (int jt = 0; jt < T; ++jt) {
-                    if (!(ok = wait_cosines())) break;
+                    if (!(ok = ok && wait_cosines())) break;
                     const int left = N - jt * kTile - half * (kTile / 2);   // keys of the plane from this half on
                     if (live && left > 0) {
                         tcgen05_fence_after_sync();
@@ -466,11 +467,10 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                     mbar_arrive(&r_done[b]);
                     skip(im.slots);
                 }
-                if (!ok) break;
                 // the two halves of a query meet in shared memory (by item parity: a thread is never two items ahead)
                 float* den_s = reinterpret_cast<float*>(smem + kOffDen) + ((i & 1) * 4 + slot * 2) * kTile + quarter * 32 + lane;
                 den_s[half * kTile] = den.x + den.y;
-                named_barrier_sync(2 + slot, kSlotThreads);
+                if (named_barrier_any(2 + slot, kSlotThreads, !ok)) break;
                 ebias = -kLog2e - __log2f(den_s[0] + den_s[kTile]);
             }
             for (int jt = 0; jt < T; ++jt) {
