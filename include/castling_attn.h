@@ -74,7 +74,9 @@ typedef struct {
     double eps;           /* floor on ||q||, ||k||; <= 0 selects the default 1e-12.  A zero    */
                           /* row therefore has cosine 0 with everything (similarity 1/2).     */
     int force_path;       /* CASTLING_PATH_*; AUTO picks by dtype, d and N                     */
-    size_t max_workspace; /* cap on handle-owned device memory in bytes; 0 = no cap            */
+    size_t max_workspace; /* cap on the handle's workspace (castling_attn_workspace_bytes) and on  */
+                          /* the staging buffers of castling_attn_forward_host, each, in bytes; 0 = no */
+                          /* cap.  Arrival counters (16 KB, or up to 136 bytes per (b,h)) come on top.   */
     int prefix_tokens;    /* 0..16 leading tokens per sequence that have no grid position (class */
                           /* / distillation tokens).  N becomes prefix_tokens + gridH*gridW in     */
                           /* every forward call.  The paper does not say how such tokens meet the */

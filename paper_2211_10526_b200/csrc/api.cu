@@ -15,6 +15,7 @@ struct castling_attn {
     size_t ws_bytes = 0;
     unsigned* counters = nullptr;  // arrival counters of the split reduction, zero between calls
     size_t counters_cap = 0;
+    unsigned* more_counters = nullptr;  // an allocation of their own, where those behind the workspace became too few
     char* stage = nullptr;      // device staging for castling_attn_forward_host
     size_t stage_bytes = 0;
     // castling_attn_forward_host pipelines batch chunks: copies in, kernels and copies out overlap
@@ -88,40 +89,52 @@ int check_shape(const castling_attn* h, int B, int H, int gridH, int gridW, int 
     return CASTLING_OK;
 }
 
-// The workspace and, where the tensor-core path wants them, its arrival counters behind it: one allocation (a second one
-// cost a new handle's first call 0.25 ms).
-int ensure_workspace(castling_attn* h, int BH, int N, int d, bool bf16, bool counters = false) {
-    size_t need = workspace_words(BH, N, d, bf16) * sizeof(float), want = 0;
-    if (counters) {
-        // either variant of the tensor-core path: 17 words per plane, or a header and 4 words per plane
-        const size_t a = (size_t)BH * castling::tc::kCountersPerHead;
-        const size_t b = castling::tc::kPipeCtrHeader + (size_t)BH * castling::tc::kPipeCtrPerPlane;
-        want = a > b ? a : b;
-    }
-    if (need <= h->ws_bytes && want <= h->counters_cap) return CASTLING_OK;
-    if (need > h->ws_bytes && h->cfg.max_workspace && need > h->cfg.max_workspace) return CASTLING_ERR_OOM;
-    if (need < h->ws_bytes) need = h->ws_bytes;
-    size_t cap = h->counters_cap;
-    if (want > cap) for (cap = 4096; cap < want;) cap *= 2;
+// Arrival counters: either variant of the tensor-core path, 17 words per plane, or a header and 4 words per plane.
+size_t counter_words(int BH) {
+    const size_t a = (size_t)BH * castling::tc::kCountersPerHead;
+    const size_t b = castling::tc::kPipeCtrHeader + (size_t)BH * castling::tc::kPipeCtrPerPlane;
+    const size_t want = a > b ? a : b;
+    size_t cap = 4096;
+    while (cap < want) cap *= 2;
+    return cap;
+}
+
+// The workspace and, behind it in the same allocation, the arrival counters (a second allocation cost a new handle's first call
+// 0.25 ms), whichever kernels the call takes.  Only a shape that needs a larger workspace moves it: captured graphs of
+// earlier calls hold its address.  Where the planes alone have become more, the counters get an allocation of their own.
+int ensure_workspace(castling_attn* h, int BH, int N, int d, bool bf16) {
+    const size_t need = workspace_words(BH, N, d, bf16) * sizeof(float);
+    const size_t cap = counter_words(BH) > h->counters_cap ? counter_words(BH) : h->counters_cap;
+    if (need <= h->ws_bytes && cap == h->counters_cap) return CASTLING_OK;
+    const bool grow = need > h->ws_bytes;
+    if (grow && h->cfg.max_workspace && need > h->cfg.max_workspace) return CASTLING_ERR_OOM;
     unsigned status = 0;   // an error not reported yet outlives the buffer
+    cudaError_t e = cudaSuccess;
     if (h->ws) {
-        cudaError_t e = cudaDeviceSynchronize();  // nothing may still be using the old buffer
-        if (e == cudaSuccess) e = cudaMemcpy(&status, h->ws, sizeof(status), cudaMemcpyDeviceToHost);
+        e = cudaDeviceSynchronize();  // nothing may still be using the old buffers
+        if (e == cudaSuccess && grow) e = cudaMemcpy(&status, h->ws, sizeof(status), cudaMemcpyDeviceToHost);
         if (e != cudaSuccess) return fail_cuda(h, e);
-        cudaFree(h->ws);
     }
-    h->ws = nullptr; h->ws_bytes = 0;
-    h->counters = nullptr; h->counters_cap = 0;
-    cudaError_t e = cudaMalloc((void**)&h->ws, need + cap * sizeof(unsigned));
-    if (e != cudaSuccess) { h->ws = nullptr; return fail_cuda(h, e, CASTLING_ERR_OOM); }
-    e = cudaMemset(h->ws, 0, castling::kHeaderWords * sizeof(float));
-    if (e == cudaSuccess && cap) e = cudaMemset(reinterpret_cast<char*>(h->ws) + need, 0, cap * sizeof(unsigned));
-    if (e == cudaSuccess && status) e = cudaMemcpy(h->ws, &status, sizeof(status), cudaMemcpyHostToDevice);
+    if (h->more_counters) cudaFree(h->more_counters);
+    h->more_counters = nullptr; h->counters = nullptr; h->counters_cap = 0;
+    if (grow) {
+        if (h->ws) cudaFree(h->ws);
+        h->ws = nullptr; h->ws_bytes = 0;
+        e = cudaMalloc((void**)&h->ws, need + cap * sizeof(unsigned));
+        if (e != cudaSuccess) { h->ws = nullptr; return fail_cuda(h, e, CASTLING_ERR_OOM); }
+        e = cudaMemset(h->ws, 0, castling::kHeaderWords * sizeof(float));
+        if (e == cudaSuccess && status) e = cudaMemcpy(h->ws, &status, sizeof(status), cudaMemcpyHostToDevice);
+    } else {
+        e = cudaMalloc((void**)&h->more_counters, cap * sizeof(unsigned));
+        if (e != cudaSuccess) { h->more_counters = nullptr; return fail_cuda(h, e, CASTLING_ERR_OOM); }
+    }
+    unsigned* counters = grow ? reinterpret_cast<unsigned*>(reinterpret_cast<char*>(h->ws) + need) : h->more_counters;
+    if (e == cudaSuccess) e = cudaMemset(counters, 0, cap * sizeof(unsigned));
     // the caller's stream may be one that does not wait for the default stream's memsets
     if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
     if (e != cudaSuccess) return fail_cuda(h, e);
-    h->ws_bytes = need;
-    if (cap) h->counters = reinterpret_cast<unsigned*>(reinterpret_cast<char*>(h->ws) + need);
+    if (grow) h->ws_bytes = need;
+    h->counters = counters;
     h->counters_cap = cap;
     return CASTLING_OK;
 }
@@ -162,6 +175,7 @@ int castling_attn_create(const castling_attn_config_t* cfg, castling_attn_t** ou
 int castling_attn_destroy(castling_attn_t* h) {
     if (!h) return CASTLING_OK;
     if (h->ws) cudaFree(h->ws);
+    if (h->more_counters) cudaFree(h->more_counters);
     if (h->stage) cudaFree(h->stage);
     if (h->copy_in) cudaStreamDestroy(h->copy_in);
     if (h->copy_out) cudaStreamDestroy(h->copy_out);
@@ -242,7 +256,7 @@ int run_device(castling_attn* h, Problem p, cudaStream_t stream) {
     const bool tensor_ok = castling::tc::supports(p);
     bool use_tensor = tensor_ok && (h->cfg.force_path == CASTLING_PATH_TENSOR ||
                                     (h->cfg.force_path == CASTLING_PATH_AUTO && castling::tc::preferred(p)));
-    int rc = ensure_workspace(h, p.BH, p.N, p.d, p.bf16, use_tensor);
+    int rc = ensure_workspace(h, p.BH, p.N, p.d, p.bf16);
     if (rc != CASTLING_OK) return rc;
     p.status = reinterpret_cast<unsigned*>(h->ws);
     if (h->cfg.force_path == CASTLING_PATH_TENSOR && !tensor_ok) return CASTLING_ERR_UNSUPPORTED;
@@ -429,7 +443,7 @@ int castling_attn_forward_host(castling_attn_t* h, const void* q, const void* k,
     // workspace and counters for every run length, before anything is in flight: growing them later
     // would synchronise the device in the middle of the pipeline (and clear the status word)
     for (int c = 0; c < chunks; ++c) {
-        rc = ensure_workspace(h, b0[c + 1] - b0[c], (int)n_tok, d, dtype == CASTLING_BF16, true);
+        rc = ensure_workspace(h, b0[c + 1] - b0[c], (int)n_tok, d, dtype == CASTLING_BF16);
         if (rc != CASTLING_OK) return rc;
     }
     for (int c = 0; c < chunks; ++c) {
@@ -502,7 +516,7 @@ int castling_attn_shard_state(castling_attn_t* h, const void* k, const void* v, 
     Problem p = make_problem(h, nullptr, k, v, nullptr, nullptr, nullptr, B, H, 1, n_tokens, d, dtype);
     p.phase = castling::kPhaseStateOnly;
     bool tensor = h->cfg.force_path != CASTLING_PATH_SIMT && castling::tc::shard_supports(p);
-    rc = ensure_workspace(h, p.BH, p.N, p.d, p.bf16, tensor);
+    rc = ensure_workspace(h, p.BH, p.N, p.d, p.bf16);
     if (rc != CASTLING_OK) return rc;
     float* partial = h->ws + castling::kHeaderWords + (size_t)p.BH * castling::state_words(p.d);
     int launches = 0;
