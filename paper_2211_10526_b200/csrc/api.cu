@@ -139,6 +139,20 @@ int ensure_workspace(castling_attn* h, int BH, int N, int d, bool bf16) {
     return CASTLING_OK;
 }
 
+// A status word for a call that needs no workspace.  A call without one is not refused: during a capture, or under a cap that
+// leaves no room, it takes the kernels that do not wait.
+unsigned* status_word(castling_attn* h, cudaStream_t stream) {
+    if (!h->ws) {
+        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(stream, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone ||
+            ensure_workspace(h, 1, 1, 16, false) != CASTLING_OK) {
+            (void)cudaGetLastError();
+            return nullptr;
+        }
+    }
+    return reinterpret_cast<unsigned*>(h->ws);
+}
+
 }  // namespace
 
 extern "C" {
@@ -518,6 +532,7 @@ int castling_attn_shard_state(castling_attn_t* h, const void* k, const void* v, 
     bool tensor = h->cfg.force_path != CASTLING_PATH_SIMT && castling::tc::shard_supports(p);
     rc = ensure_workspace(h, p.BH, p.N, p.d, p.bf16);
     if (rc != CASTLING_OK) return rc;
+    p.status = reinterpret_cast<unsigned*>(h->ws);
     float* partial = h->ws + castling::kHeaderWords + (size_t)p.BH * castling::state_words(p.d);
     int launches = 0;
     h->timer.begin(static_cast<cudaStream_t>(stream));
@@ -555,7 +570,6 @@ int castling_attn_shard_apply(castling_attn_t* h, const void* q, const void* v_h
     p.v_row0 = halo_top;
     p.v_rows = halo_top + gridH_local + halo_bottom;
     p.lv.head = (long long)p.v_rows * gridW * d;   // planes of the taller V tensor
-    p.status = reinterpret_cast<unsigned*>(h->ws);
     int launches = 0;
     h->timer.begin(static_cast<cudaStream_t>(stream));
     bool tensor = h->cfg.force_path != CASTLING_PATH_SIMT && castling::tc::shard_supports(p);
@@ -567,9 +581,11 @@ int castling_attn_shard_apply(castling_attn_t* h, const void* q, const void* v_h
                                       &launches, &h->timer);
         if (e == cudaErrorNotSupported) { (void)cudaGetLastError(); tensor = false; h->timer.begin(static_cast<cudaStream_t>(stream)); }
     }
-    if (!tensor)
+    if (!tensor) {
+        if (!p.bf16) p.status = status_word(h, static_cast<cudaStream_t>(stream));
         e = castling::simt_forward(p, const_cast<float*>(state), nullptr, 1, static_cast<cudaStream_t>(stream), &launches,
                                    &h->timer);
+    }
     if (e != cudaSuccess) return fail_cuda(h, e);
     h->last_path = tensor ? CASTLING_PATH_TENSOR : CASTLING_PATH_SIMT; h->last_launches = launches;
     return CASTLING_OK;

@@ -55,7 +55,8 @@ struct Problem {
     int phase = 0;              // kPhaseAll / kPhaseStateOnly / kPhaseApplyOnly
     int v_row0 = 0, v_rows = 0; // apply of a shard: V holds v_rows grid rows and its row v_row0 is the shard's row 0
                                 // (v_rows = 0: V holds exactly the gridH rows)
-    unsigned* status = nullptr; // device status word for the bounded waits of the CUDA-core path's kernels, if there is one
+    unsigned* status = nullptr; // device status word for the bounded waits of the CUDA-core path's kernels; without one the call
+                                // takes kernels that do not wait
     int hdiv;          // planes per batch step of the layouts: H for a caller's strided tensors, BH for a
                        // run of contiguous planes (one uniform plane stride)
     // Contiguous [planes][N][d] tensors; needs N, d and BH.
@@ -121,9 +122,10 @@ int device_sm_count();
 // CUDA-core path.  simt_forward returns the cudaError_t of its launches.
 cudaError_t simt_forward(const Problem& p, float* ws_state, float* ws_partial, int P,
                          cudaStream_t stream, int* launches, KernelTimer* timer);
-int simt_choose_splits(int BH, int N, int d, bool bf16);
+// waits: the call has a status word, so that it may take kernels whose waits can give up.
+int simt_choose_splits(int BH, int N, int d, bool bf16, bool waits = true);
 // fp32 kernels for head widths 32, 64 and 128 and 3x3 or 5x5 filters (csrc/f32_kernels.cu); simt_forward takes them where
-// they apply.
+// they apply and there is a status word for their waits.
 inline bool f32_width(int d) { return d == 32 || d == 64 || d == 128; }
 bool f32_supports(const Problem& p);
 int f32_choose_splits(int BH, int N);

@@ -44,7 +44,7 @@ template <int D> struct StateGeo {
 template <int D, bool RN>
 __global__ void __launch_bounds__(kThreads, D == 128 ? 1 : 2)
 f32_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, float* __restrict__ dst, int N,
-                 int chunk, int P, float eps2, int hdiv, unsigned* status_word) {
+                 int chunk, int P, float eps2, int hdiv, unsigned* status) {
     using G = StateGeo<D>;
     constexpr int kWords = D * D + D + (RN ? D : 0), kTok = G::kTok;
     constexpr unsigned kBit = tc::kStatusStateTimeout;
@@ -52,7 +52,6 @@ f32_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
     float* smem = reinterpret_cast<float*>(tc::align_smem(smem_raw));
     uint64_t* full = reinterpret_cast<uint64_t*>(smem + G::kOffBar / 4);   // TMA: K and V of a tile landed
     volatile int* abort_flag = reinterpret_cast<volatile int*>(full + 2);
-    unsigned* status = status_word ? status_word : reinterpret_cast<unsigned*>(full + 2) + 1;
     const int tid = threadIdx.x, p = blockIdx.x % P, bh = blockIdx.x / P;
     const int n_begin = p * chunk, n_end = min(N, n_begin + chunk);
     const int pb = bh / hdiv, ph = bh - pb * hdiv;
@@ -206,7 +205,7 @@ struct F32ApplyParams {
     int P;                 // partial states per plane to be summed here (1: the state is final)
     float eps2;
     int v_row0;            // row v_row0 of V is grid row 0
-    unsigned* status;      // device status word, or nullptr
+    unsigned* status;      // device status word
 };
 
 template <int D, int KS, bool RN>
@@ -223,7 +222,6 @@ f32_apply_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     uint64_t* q_full = reinterpret_cast<uint64_t*>(smem + G::kOffBar);   // TMA: Q of the patch landed
     uint64_t* v_full = q_full + 1;                                       // TMA: V of the patch landed
     volatile int* abort_flag = reinterpret_cast<volatile int*>(q_full + 2);
-    unsigned* status = prm.status ? prm.status : reinterpret_cast<unsigned*>(q_full + 2) + 1;
     const int tid = threadIdx.x, W = prm.gridW;
     // this CTA's run of patches, counted through all planes
     const int i_begin = (int)((long long)prm.total * blockIdx.x / gridDim.x), i_end = (int)((long long)prm.total * (blockIdx.x + 1) / gridDim.x);
@@ -297,7 +295,7 @@ f32_apply_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
                 *reinterpret_cast<float4*>(q_s + c * 4) = __ldg(reinterpret_cast<const float4*>(qp + (c / G::kCG) * prm.lq.token + (c % G::kCG) * 4));
         }
         __syncthreads();
-        bool ok = lead || mbar_wait(q_full, phase, abort_flag, status, kBit);
+        bool ok = lead || mbar_wait(q_full, phase, abort_flag, prm.status, kBit);
         {   // 1 / max(||q||, eps) of every token, one to four threads each; they walk a row from different chunks on, which lie in
             // different banks
             constexpr int L = kThreads / G::kTokens;
@@ -345,7 +343,7 @@ f32_apply_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
                 }
             }
         }
-        ok = ok && (lead || mbar_wait(v_full, phase, abort_flag, status, kBit));
+        ok = ok && (lead || mbar_wait(v_full, phase, abort_flag, prm.status, kBit));
         tc::fence_proxy_async_smem();          // a leading patch wrote Q, which TMA writes next
         if (__syncthreads_or(!ok)) break;      // the factors of every token are there, Q is dead
         if (tid == 0) load_q(it + 1);
@@ -495,7 +493,7 @@ cudaError_t launch_f32_d(const Problem& p, float* s, float* part, int P, cudaStr
 
 }  // namespace
 
-bool f32_supports(const Problem& p) { return !p.bf16 && f32_width(p.d) && (p.ksize == 3 || p.ksize == 5); }
+bool f32_supports(const Problem& p) { return !p.bf16 && f32_width(p.d) && (p.ksize == 3 || p.ksize == 5) && p.status; }
 
 // Token splits of the state kernel: two CTAs per multiprocessor, at least 128 tokens each (the states of smaller grids need
 // no workspace beyond the final one).  Up to kF32ApplyParts of them need no reduction in between.

@@ -73,7 +73,8 @@ extern "C" int castling_attn_forward_static(const void* q, const void* k, const 
     // per (b,h).  If the split version does not fit, fall back to one split; if that does not fit
     // either, the problem is beyond what this entry point serves.
     const size_t words = castling::state_words(d);
-    int P = castling::simt_choose_splits((int)BH, (int)N, d, dtype == CASTLING_BF16);
+    // No handle, no status word: the kernels without waits.
+    int P = castling::simt_choose_splits((int)BH, (int)N, d, dtype == CASTLING_BF16, false);
     if ((size_t)BH * words * (1 + (P > 1 ? P : 0)) > kStaticScratchWords) P = 1;
     if ((size_t)BH * words > kStaticScratchWords) return CASTLING_ERR_SCRATCH_LIMIT;
 

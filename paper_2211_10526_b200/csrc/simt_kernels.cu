@@ -2,7 +2,7 @@
 //
 // These cover every supported dtype, head width and filter size; fp32 heads of width
 // 32, 64 and 128 with 3x3 or 5x5 filters have kernels of their own (f32_kernels.cu) unless
-// the single-launch kernel takes them.
+// the single-launch kernel takes them or there is no status word to report a wait that ran out.
 //
 //   state kernel  : per (b,h) and token split, k^ = k / max(||k||, eps),
 //                   S += k^^T v (d x d), s += v           (Eq. 9, K^T V and the 1/2 term)
@@ -551,8 +551,8 @@ bool simt_supports(int d, int ksize) {
 
 // Token splits of the state kernel: enough CTAs to fill the device about twice over,
 // at least four staged tiles per split, capped at 64.
-int simt_choose_splits(int BH, int N, int d, bool bf16) {
-    if (!bf16 && f32_width(d)) return f32_choose_splits(BH, N);
+int simt_choose_splits(int BH, int N, int d, bool bf16, bool waits) {
+    if (waits && !bf16 && f32_width(d)) return f32_choose_splits(BH, N);
     const int tiles = (N + kStateTile - 1) / kStateTile;
     int P = (2 * device_sm_count() + BH - 1) / BH;
     if (P > tiles / 4) P = tiles / 4;
