@@ -309,7 +309,7 @@ Problem make_problem(const castling_attn* h, const void* q, const void* k, const
     p.prefix = h->cfg.prefix_tokens;
     p.N = p.prefix + gridH * gridW; p.BH = B * H; p.head0 = 0;
     p.bf16 = (dtype == CASTLING_BF16);
-    p.eps2 = (float)(h->cfg.eps * h->cfg.eps);
+    p.eps2 = castling::squared_floor(h->cfg.eps);
     p.rownorm = h->cfg.normalize_rows != 0;
     p.exact_kernel = h->cfg.exact_kernel != 0;
     p.sparse = h->cfg.sparse_branch != 0;

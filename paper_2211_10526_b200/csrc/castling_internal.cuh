@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
 #include <atomic>
+#include <limits>
 #include <stddef.h>
 #include <stdint.h>
 
@@ -22,6 +23,13 @@ struct Layout {
 __host__ __device__ inline long long plane_offset(const Layout& l, int i, int hdiv) {
     const int b = i / hdiv;
     return (long long)b * l.batch + (long long)(i - b * hdiv) * l.head;
+}
+
+// eps^2 as the kernels take it, the floor under a row's sum of squares.  Never zero, even where the square is: the rows of zeros
+// that fill up a tile are scaled like all others, and by infinity would become NaN.
+inline float squared_floor(double eps) {
+    const float e = (float)(eps * eps);
+    return e > 0.f ? e : std::numeric_limits<float>::denorm_min();
 }
 
 // One forward call, as the kernels see it.

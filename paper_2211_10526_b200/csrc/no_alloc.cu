@@ -89,7 +89,7 @@ extern "C" int castling_attn_forward_static(const void* q, const void* k, const 
     p.set_contiguous();
     p.bf16 = (dtype == CASTLING_BF16);
     if (eps <= 0.0) eps = 1e-12;
-    p.eps2 = (float)(eps * eps);
+    p.eps2 = castling::squared_floor(eps);
     castling::KernelTimer timer;  // off: records nothing, creates nothing
     int launches = 0;
     // Nothing in the scratch has to start at zero: the state kernel overwrites every word that the
