@@ -82,20 +82,22 @@ PyObject* forward(PyObject*, PyObject* const* a, Py_ssize_t n) {
     if (B > INT32_MAX || H > INT32_MAX || d > INT32_MAX || gridH > INT32_MAX || gridW > INT32_MAX) return value_error("size out of range");
     const castling_dtype_t code = dt == at::kFloat ? CASTLING_F32 : CASTLING_BF16;
     void* stream = c10::cuda::getCurrentCUDAStream(q->get_device()).stream();
-    const void* b = bias ? bias->const_data_ptr() : nullptr;
+    // addresses while the lock is held: a tensor without storage (inside vmap or grad, a fake one) raises here
+    const void *qp = q->const_data_ptr(), *kp = k->const_data_ptr(), *vp = v->const_data_ptr(), *wp = w->const_data_ptr();
+    const void* bp = bias ? bias->const_data_ptr() : nullptr;
+    void* op = out->mutable_data_ptr();
     int rc;
     PyThreadState* gil = PyEval_SaveThread();   // a first call of a larger shape allocates and waits for the device
     if (contiguous) {
-        rc = g_forward(static_cast<castling_attn_t*>(handle), q->const_data_ptr(), k->const_data_ptr(), v->const_data_ptr(),
-                       w->const_data_ptr(), b, out->mutable_data_ptr(), (int)B, (int)H, (int)gridH, (int)gridW, (int)d, code, stream);
+        rc = g_forward(static_cast<castling_attn_t*>(handle), qp, kp, vp, wp, bp, op, (int)B, (int)H, (int)gridH, (int)gridW, (int)d,
+                       code, stream);
     } else {   // views of token-major or fused-projection buffers: pass their strides through
         long long s[12];
         for (int i = 0; i < 4; ++i)
             for (int j = 0; j < 3; ++j) s[3 * i + j] = t[i]->stride(j);
         const castling_attn_layout_t layout = {s[0], s[1], s[2], s[3], s[4], s[5], s[6], s[7], s[8], s[9], s[10], s[11]};
-        rc = g_strided(static_cast<castling_attn_t*>(handle), q->const_data_ptr(), k->const_data_ptr(), v->const_data_ptr(),
-                       w->const_data_ptr(), b, out->mutable_data_ptr(), (int)B, (int)H, (int)gridH, (int)gridW, (int)d, code, &layout,
-                       stream);
+        rc = g_strided(static_cast<castling_attn_t*>(handle), qp, kp, vp, wp, bp, op, (int)B, (int)H, (int)gridH, (int)gridW, (int)d,
+                       code, &layout, stream);
     }
     PyEval_RestoreThread(gil);
     if (rc != CASTLING_OK) return PyLong_FromLong(rc);
