@@ -81,11 +81,13 @@ class CastlingAttn:
             raise ValueError("dw_weight must be [H*d, ksize, ksize]")
         if bias is not None and bias.shape != (H * d,):
             raise ValueError("dw_bias must be [H*d]")
-        for t in (q, k, v, w, out) + (() if bias is None else (bias,)):
-            if t.device.type != "cpu" or not t.is_contiguous():
-                raise ValueError("host tensors must be contiguous tensors on the cpu")
-            if t.dtype != q.dtype:
-                raise TypeError("all tensors must share one dtype")
+        if bias is not None and (bias.device.type != "cpu" or not bias.is_contiguous() or bias.dtype != q.dtype):
+            raise ValueError("dw_bias must be a contiguous cpu tensor of the tensors' dtype")
+        tensors = (q, k, v, w, out)
+        if any(t.device.type != "cpu" or not t.is_contiguous() for t in tensors):
+            raise ValueError("host tensors must be contiguous tensors on the cpu")
+        if any(t.dtype != q.dtype for t in tensors):
+            raise TypeError("all tensors must share one dtype")
         return B, H, N, d
 
     def forward(self, q, k, v, dw_weight, dw_bias: Optional[torch.Tensor], gridH: int, gridW: int,
