@@ -170,8 +170,8 @@ typedef struct {
  *
  * The tensor-core kernels read such layouts directly through strided TMA descriptors: width-64
  * heads with any strides; width-32 heads whose tokens (token stride 32) or heads (head stride 32, as in
- * token-major [B,N,H,32]) lie next to one another, except small calls whose 64-byte rows do not fill 128-byte
- * ones (odd gridW, N or H).  Everything else, and any layout a descriptor cannot express, runs on the CUDA-core
+ * token-major [B,N,H,32]) lie next to one another; automatic dispatch leaves small calls whose 64-byte rows do not
+ * fill 128-byte ones (odd gridW, N or H) to the CUDA cores.  Everything else, and any layout a descriptor cannot express, runs on the CUDA-core
  * kernels.  The tensor-core kernels round unit keys and the scaled state to bf16 between the contractions -- except for
  * width-32 heads whose rows do not fill 128-byte ones and for planes of under 96 width-32 tokens, where both are held as
  * pairs of bf16 and results are as close to exact arithmetic as those of the CUDA-core kernels.

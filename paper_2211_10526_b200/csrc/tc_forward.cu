@@ -9,9 +9,9 @@ namespace tc {
 
 namespace {
 constexpr int kStateTile = 128;  // 128-byte rows per UMMA stage of the state kernel
-// Width-32 shapes that fit no 128-byte rows (odd grid widths or token counts, an odd number of heads side by side) come
-// here from this many tokens in all planes on.  The kernels are faster below it too (300 tokens: 6 us against 17 us on the
-// CUDA cores; 2 x 6 planes of 33 x 21: 8 us against 25 us), but the tests hold the smallest shapes to the CUDA-core family.
+// Automatic dispatch takes width-32 shapes that fit no 128-byte rows (odd grid widths or token counts, an odd number of heads
+// side by side) from this many tokens in all planes on.  The kernels are faster below it too (300 tokens: 6 us against 17 us on
+// the CUDA cores; 2 x 6 planes of 33 x 21: 8 us against 25 us), but the tests hold the smallest shapes to the CUDA-core family.
 constexpr long long kNarrowMinTokens = 4096;
 }
 
@@ -30,10 +30,10 @@ static bool dense_rows(const Problem& p) {
     return p.d == 32 && (p.contiguous_tokens() || (p.hdiv == p.H && p.lq.head == 32 && p.lk.head == 32 && p.lv.head == 32 && p.lo.head == 32));
 }
 
-// bf16, 3x3 or 5x5 filters, head width 64, one of the two width-32 arrangements above, or enough dense 64-byte rows.
+// bf16, 3x3 or 5x5 filters, head width 64, or one of the width-32 arrangements above.
 bool supports(const Problem& p) {
     if (!p.bf16 || (p.ksize != 3 && p.ksize != 5)) return false;
-    return p.d == 64 || token_pairs(p) || head_pairs(p) || (dense_rows(p) && (long long)p.BH * p.N >= kNarrowMinTokens);
+    return p.d == 64 || dense_rows(p);
 }
 
 int rows_per_head(int N, int d) { return d == 32 ? (N + 1) / 2 : N; }
@@ -41,7 +41,9 @@ int rows_per_head(int N, int d) { return d == 32 ? (N + 1) / 2 : N; }
 // With fewer than 48 tokens per (b,h) the tiles of the tensor-core kernels are mostly padding and the CUDA-core kernels
 // are faster (measured: 4x4 grids of width-32 heads, 20 us against 33 us); from 7x7 on they are not (64 x 8 planes: 17.0 us
 // against 14.6 us).
-bool preferred(const Problem& p) { return supports(p) && p.N >= 48; }
+bool preferred(const Problem& p) {
+    return supports(p) && p.N >= 48 && (p.d == 64 || token_pairs(p) || head_pairs(p) || (long long)p.BH * p.N >= kNarrowMinTokens);
+}
 
 // Two state CTAs fit on an SM: as many splits as keep all CTAs of the launch resident at once
 // (two per multiprocessor), every split non-empty, at most 64 splits.
