@@ -44,7 +44,7 @@ def _start_torch_call(verbose: bool) -> subprocess.Popen:
     root = os.path.dirname(torch.__file__)
     cuda = os.path.dirname(os.path.dirname(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")))
     cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
-           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", "-I", INCLUDE,
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", f'-DBUILT_AGAINST="{_torch_tag().decode()}"', "-I", INCLUDE,
            "-isystem", os.path.join(root, "include"), "-isystem", os.path.join(root, "include", "torch", "csrc", "api", "include"),
            "-isystem", os.path.join(cuda, "include"), "-I", sysconfig.get_paths()["include"], CALL_SOURCE, "-o",
            f"{CALL_PATH}.{os.getpid()}.tmp", "-L", os.path.join(root, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"]
@@ -53,9 +53,17 @@ def _start_torch_call(verbose: bool) -> subprocess.Popen:
     return subprocess.Popen(cmd)
 
 
+def _torch_tag() -> bytes:
+    import torch
+    return f"built against torch {torch.__version__}".encode()
+
+
 def _call_stale() -> bool:
     if not os.path.exists(CALL_PATH):
         return True
+    with open(CALL_PATH, "rb") as f:   # another torch may have another C++ interface
+        if _torch_tag() + b"\0" not in f.read():
+            return True
     built = os.path.getmtime(CALL_PATH)
     return any(os.path.getmtime(p) > built for p in [CALL_SOURCE] + glob.glob(os.path.join(INCLUDE, "*.h")))
 

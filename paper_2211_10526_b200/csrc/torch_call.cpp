@@ -114,4 +114,8 @@ PyModuleDef module = {PyModuleDef_HEAD_INIT, "_torch_call", nullptr, -1, methods
 
 }  // namespace
 
-PyMODINIT_FUNC PyInit__torch_call() { return PyModule_Create(&module); }
+PyMODINIT_FUNC PyInit__torch_call() {
+    PyObject* m = PyModule_Create(&module);
+    if (m && PyModule_AddStringConstant(m, "built_against", BUILT_AGAINST) != 0) { Py_DECREF(m); return nullptr; }
+    return m;
+}
