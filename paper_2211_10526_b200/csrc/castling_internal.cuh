@@ -136,6 +136,8 @@ int simt_choose_splits(int BH, int N, int d, bool bf16, bool waits = true);
 // they apply and there is a status word for their waits.
 inline bool f32_width(int d) { return d == 32 || d == 64 || d == 128; }
 bool f32_supports(const Problem& p);
+// Grids so thin that the apply kernel's patches would be mostly empty: simt_forward's own apply kernel follows the state kernel.
+bool f32_thin(const Problem& p);
 int f32_choose_splits(int BH, int N);
 cudaError_t f32_forward(const Problem& p, float* ws_state, float* ws_partial, int P, cudaStream_t stream, int* launches,
                         KernelTimer* timer);

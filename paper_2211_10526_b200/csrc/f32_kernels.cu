@@ -495,6 +495,17 @@ cudaError_t launch_f32_d(const Problem& p, float* s, float* part, int P, cudaStr
 
 bool f32_supports(const Problem& p) { return !p.bf16 && f32_width(p.d) && (p.ksize == 3 || p.ksize == 5) && p.status; }
 
+// The apply kernel takes a patch of 8 rows x TX columns whole, the one of simt_kernels.cu 64 tokens whatever their grid.  Where the
+// patches hold much more than the grid, and there are more of them than run at a time, the latter is the faster one.  Whole
+// forwards of 2 x 8 planes, this kernel / that one, us: 1 x 16384, d = 64 552 / 218, 2 x 8192 310 / 247, 4096 x 4 309 / 269 (patches four
+// times the grid), 4096 x 4, d = 32 200 / 130 (eight times); apply kernels alone on this side of the line: 3 x 5461, d = 64 177 / 197 (2.7
+// times), 2048 x 8, d = 32 96 / 102 (four times), 5 x 5 filters 119 / 171.
+bool f32_thin(const Problem& p) {
+    const long long tx = 4 * kThreads / p.d;   // ApplyGeo's TX
+    const long long patches = ((p.gridW + tx - 1) / tx) * ((p.gridH + 7) / 8), places = patches * tx * 8, tokens = (long long)p.gridH * p.gridW;
+    return p.BH * patches > 2 * device_sm_count() && (p.d == 32 ? places > 4 * tokens : 2 * places > 7 * tokens);
+}
+
 // Token splits of the state kernel: two CTAs per multiprocessor, at least 128 tokens each (the states of smaller grids need
 // no workspace beyond the final one).  Up to kF32ApplyParts of them need no reduction in between.
 int f32_choose_splits(int BH, int N) {

@@ -492,12 +492,17 @@ cudaError_t launch_simt(const Problem& p, float* ws_state, float* ws_partial, in
         return e;
     }
     cudaError_t e = cudaSuccess;
-    if (f32_supports(p)) {
-        e = f32_forward(p, ws_state, ws_partial, P, stream, launches, timer);
-        if (e != cudaErrorNotSupported) return e;
+    int phase = p.phase;
+    const bool thin = phase != kPhaseStateOnly && f32_thin(p);   // the apply kernel below in place of the one of fixed patches
+    if (f32_supports(p) && !(thin && phase == kPhaseApplyOnly)) {
+        Problem part = p;
+        if (thin) part.phase = kPhaseStateOnly;
+        e = f32_forward(part, ws_state, ws_partial, P, stream, launches, timer);
+        if (e == cudaSuccess && thin) phase = kPhaseApplyOnly;
+        else if (e != cudaErrorNotSupported) return e;
         e = cudaSuccess;   // strides that the tensor maps cannot take: the kernels below take any layout
     }
-    if (p.phase != kPhaseApplyOnly) {
+    if (phase != kPhaseApplyOnly) {
         const int tiles = (p.N + kStateTile - 1) / kStateTile;
         const int chunk = ((tiles + P - 1) / P) * kStateTile;
         float* dst = (P > 1) ? ws_partial : ws_state;
@@ -514,7 +519,7 @@ cudaError_t launch_simt(const Problem& p, float* ws_state, float* ws_partial, in
             ++*launches;
             timer->mark(stream, "simt_reduce");
         }
-        if (p.phase == kPhaseStateOnly) return cudaSuccess;
+        if (phase == kPhaseStateOnly) return cudaSuccess;
     }
     const size_t smem = simt_apply_smem<D>(p.ksize);
     static PerDevice apply_opt_in;
