@@ -63,6 +63,7 @@ struct QuadParams {
     const __nv_bfloat16* bias;
     Layout lo;
     int hdiv, H, head0, N, gridH, gridW;
+    int column;                  // the grid is one column, taken as a row (kOneRow): the filters are read transposed
     int slots;                   // query tiles per item (1 or 2)
     int groups;                  // items per plane
     int k_tiles, n_items;
@@ -127,11 +128,16 @@ __device__ __forceinline__ float2 angular_weight2(float2 x) {
                              __uint_as_float((__float_as_uint(h.y) & 0x7fffffffu) | sy)), dup2(0.5f));
 }
 
-template <int KS, bool SPARSE, bool EXACT>
+// GRID.  kWide: rows longer than an item's queries, which then lie in one row, or at the end of one and the beginning of the next,
+// and need not all columns of patches: 16 planes of 2 x 2048 (exact kernel) 155 us, 460 with all columns.  kOneRow: the same with
+// patches of one row; a grid of one column is taken as one row: 16 planes of 1 x 4096 138 us (809 in patches of eight rows and all
+// columns), 768 planes of 196 x 1 105 us (254 in patches of which one column is used).
+enum { kOrdinary, kWide, kOneRow };
+template <int KS, bool SPARSE, bool EXACT, int GRID>
 __global__ void __launch_bounds__(kThreads, 1)
 tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmP, const QuadParams prm) {
-    constexpr int R = KS / 2, kPatchY = KS == 3 ? 8 : 4, HX = kPatchX + 2 * R, HY = kPatchY + 2 * R;
+    constexpr int R = KS / 2, kPatchY = GRID == kOneRow ? 1 : KS == 3 ? 8 : 4, HX = kPatchX + 2 * R, HY = kPatchY + 2 * R;
     static_assert(HX * HY * kD * 2 <= kPatchBytes, "patch");
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = align_smem(smem_raw);
@@ -176,7 +182,16 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     auto patches_of = [&](const Item& im) -> Patches {
         const int y0 = im.t0 / prm.gridW, y1 = (min(N, im.t0 + im.slots * kTile) - 1) / prm.gridW;
         const int nx = (prm.gridW + kPatchX - 1) / kPatchX;
+        if (GRID != kOrdinary) {   // from the first query's column of patches on; y1 - y0 is 0 or 1
+            const int first = (im.t0 - y0 * prm.gridW) / kPatchX, last = (min(N, im.t0 + im.slots * kTile) - 1 - y1 * prm.gridW) / kPatchX;
+            return {y0, nx, min(nx, last - first + 1 + (y1 - y0) * nx)};
+        }
         return {y0, nx, nx * ((y1 - y0) / kPatchY + 1)};
+    };
+    // column of patch j of an item on such a grid: past the last one from the first on
+    auto wide_column = [&](const Item& im, const Patches& pa, int j) -> int {
+        const int c = (im.t0 - pa.y0 * prm.gridW) / kPatchX + j;
+        return c < pa.nx ? c : c - pa.nx;
     };
     auto warp_wait = [&](uint64_t* bar, uint32_t parity) -> bool {
         return mbar_wait_warp(bar, parity, abort_flag, prm.status, kBit);
@@ -215,9 +230,10 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                 if (pi < my_items && (pn == 0 || mbar_poll(patch_free, (pn - 1) & 1))) {
                     const Item im = item_of(pi);
                     const Patches pa = patches_of(im);
-                    const int pb = im.bh / prm.hdiv, ph = im.bh - pb * prm.hdiv, y = pj / pa.nx;
+                    const int pb = im.bh / prm.hdiv, ph = im.bh - pb * prm.hdiv, y = GRID == kOrdinary ? pj / pa.nx : 0;
+                    const int x = GRID == kOrdinary ? pj - y * pa.nx : wide_column(im, pa, pj);
                     mbar_expect_tx(patch_full, HX * HY * kD * 2);
-                    tma_load_5d(smem + kOffPatch, &tmP, patch_full, 0, (pj - y * pa.nx) * kPatchX - R, pa.y0 + y * kPatchY - R, ph, pb);
+                    tma_load_5d(smem + kOffPatch, &tmP, patch_full, 0, x * kPatchX - R, pa.y0 + y * kPatchY - R, ph, pb);
                     ++pn;
                     if (++pj == pa.n) { pj = 0; ++pi; }
                     moved = true;
@@ -532,8 +548,10 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
             if (head != prev_head) {
                 prev_head = head;
                 const unsigned short* w0 = reinterpret_cast<const unsigned short*>(prm.w) + (size_t)(head * kD + 2 * lane) * (KS * KS);
-                for (int e = cw; e < KS * KS; e += kConvThreads / 32)
-                    w_s[e * 32] = (uint32_t)__ldg(w0 + e) | ((uint32_t)__ldg(w0 + KS * KS + e) << 16);
+                for (int e = cw; e < KS * KS; e += kConvThreads / 32) {
+                    const int tap = GRID == kOneRow && prm.column ? e % KS * KS + e / KS : e;
+                    w_s[e * 32] = (uint32_t)__ldg(w0 + tap) | ((uint32_t)__ldg(w0 + KS * KS + tap) << 16);
+                }
                 if (prm.bias) {   // element by element, like the filters: neither need begin on a word boundary
                     const unsigned short* b0 = reinterpret_cast<const unsigned short*>(prm.bias) + head * kD + 2 * lane;
                     bias2 = make_float2(bf16lo(__ldg(b0)), bf16lo(__ldg(b0 + 1)));
@@ -549,7 +567,8 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                 ok = ok && warp_wait(patch_full, patch & 1);
                 if (!ok) break;
                 // two columns slide down the patch; the words of a row are loaded a row ahead
-                const int py = pj / pa.nx, y0 = pa.y0 + py * kPatchY, x0 = (pj - py * pa.nx) * kPatchX + 2 * cw;
+                const int py = GRID == kOrdinary ? pj / pa.nx : 0, y0 = pa.y0 + py * kPatchY;
+                const int x0 = (GRID == kOrdinary ? pj - py * pa.nx : wide_column(im, pa, pj)) * kPatchX + 2 * cw;
                 const uint8_t* vh = smem + kOffPatch + 2 * cw * 128 + lane * 4;
                 int tl = y0 * W + x0 - im.t0;          // token of the first output, within the item
                 uint32_t raw[NIN];
@@ -636,8 +655,8 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     if (warp == 1) tmem_dealloc(tmem, kTmemCols);
 }
 
-template <int KS, bool SPARSE, bool EXACT>
-cudaError_t launch_quad_ks(const Problem& p, unsigned* status, cudaStream_t st) {
+template <int KS, bool SPARSE, bool EXACT, int GRID>
+cudaError_t launch_quad_grid(const Problem& p, int gridH, int gridW, int slots, unsigned* status, cudaStream_t st) {
     CUtensorMap tmQ, tmK, tmV, tmP;
     const uint64_t nb = (uint64_t)(p.BH / p.hdiv);
     const uint64_t dims[4] = {(uint64_t)kD, (uint64_t)p.N, (uint64_t)p.hdiv, nb};
@@ -651,9 +670,9 @@ cudaError_t launch_quad_ks(const Problem& p, unsigned* status, cudaStream_t st) 
         !make_tensor_map_bf16(&tmV, p.v, 4, dims, sv, box, 128))
         return cudaErrorNotSupported;
     // [64, columns, grid rows, planes per batch step, batch steps]: columns and rows outside the grid are zero-filled
-    const uint64_t dims_p[5] = {(uint64_t)kD, (uint64_t)p.gridW, (uint64_t)p.gridH, (uint64_t)p.hdiv, nb};
-    const uint64_t strides_p[4] = {(uint64_t)p.lv.token, (uint64_t)(p.lv.token * p.gridW), sv[1], sv[2]};
-    const uint32_t box_p[5] = {kD, kPatchX + 2 * (KS / 2), (KS == 3 ? 8 : 4) + 2 * (KS / 2), 1, 1};
+    const uint64_t dims_p[5] = {(uint64_t)kD, (uint64_t)gridW, (uint64_t)gridH, (uint64_t)p.hdiv, nb};
+    const uint64_t strides_p[4] = {(uint64_t)p.lv.token, (uint64_t)(p.lv.token * gridW), sv[1], sv[2]};
+    const uint32_t box_p[5] = {kD, kPatchX + 2 * (KS / 2), (GRID == kOneRow ? 1 : KS == 3 ? 8 : 4) + 2 * (KS / 2), 1, 1};
     if (!make_tensor_map_bf16(&tmP, p.v, 5, dims_p, strides_p, box_p, 0)) return cudaErrorNotSupported;
     QuadParams prm;
     prm.out = static_cast<__nv_bfloat16*>(p.out);
@@ -661,14 +680,9 @@ cudaError_t launch_quad_ks(const Problem& p, unsigned* status, cudaStream_t st) 
     prm.bias = static_cast<const __nv_bfloat16*>(p.bias);
     prm.lo = p.lo;
     prm.hdiv = p.hdiv; prm.H = p.H; prm.head0 = p.head0; prm.N = p.N;
-    prm.gridH = p.gridH; prm.gridW = p.gridW;
-    // Two query tiles per item share the key tiles and keep both halves of the weight warps busy; an item of one tile takes
-    // 0.7 (exact kernel) to 0.85 of its time: one tile each where that leaves (nearly) as few rounds.  Measured, one tile
-    // against two: exact, 24 planes of 32 x 64 (3 rounds / 2) 79.9 / 72.8 us; masked, 192 planes of 14 x 14 (3 / 2) 27.5 / 23.1.
-    const int sms = device_sm_count();
-    const int q_tiles = (p.N + kTile - 1) / kTile;
-    const long long one = (long long)p.BH * q_tiles, two = (long long)p.BH * ((q_tiles + 1) / 2);
-    prm.slots = ((one + sms - 1) / sms) * 3 < ((two + sms - 1) / sms) * 4 ? 1 : 2;
+    prm.gridH = gridH; prm.gridW = gridW; prm.column = gridW != p.gridW ? 1 : 0;
+    const int sms = device_sm_count(), q_tiles = (p.N + kTile - 1) / kTile;
+    prm.slots = slots;
     prm.groups = (q_tiles + prm.slots - 1) / prm.slots;
     prm.k_tiles = q_tiles;
     prm.n_items = p.BH * prm.groups;
@@ -676,12 +690,30 @@ cudaError_t launch_quad_ks(const Problem& p, unsigned* status, cudaStream_t st) 
     prm.sparse_eps = p.sparse_eps;
     static PerDevice opt_in;
     {
-        const cudaError_t e = opt_in_smem(tc_quad_kernel<KS, SPARSE, EXACT>, kSmem, opt_in);
+        const cudaError_t e = opt_in_smem(tc_quad_kernel<KS, SPARSE, EXACT, GRID>, kSmem, opt_in);
         if (e != cudaSuccess) return e;
     }
     const int grid = prm.n_items < sms ? prm.n_items : sms;
-    tc_quad_kernel<KS, SPARSE, EXACT><<<(unsigned)grid, kThreads, kSmem, st>>>(tmQ, tmK, tmV, tmP, prm);
+    tc_quad_kernel<KS, SPARSE, EXACT, GRID><<<(unsigned)grid, kThreads, kSmem, st>>>(tmQ, tmK, tmV, tmP, prm);
     return cudaGetLastError();
+}
+
+template <int KS, bool SPARSE, bool EXACT>
+cudaError_t launch_quad_ks(const Problem& p, unsigned* status, cudaStream_t st) {
+    // Two query tiles per item share the key tiles and keep both halves of the weight warps busy; an item of one tile takes
+    // 0.7 (exact kernel) to 0.85 of its time: one tile each where that leaves (nearly) as few rounds.  Over 26 shapes of 1 to 768
+    // planes and 128 to 4096 tokens this is the faster one with either kernel; closest to the line, one tile against two: exact, 24
+    // planes of 32 x 64 (3 rounds / 2) 77.4 / 74.4 us, 16 of 32 x 32 (1 / 1) 18.3 / 23.9; masked, 192 planes of 14 x 14 (3 / 2)
+    // 29.2 / 23.6, 48 of 14 x 14 (1 / 1) 12.0 / 14.7.
+    const int sms = device_sm_count();
+    const int q_tiles = (p.N + kTile - 1) / kTile;
+    const long long one = (long long)p.BH * q_tiles, two = (long long)p.BH * ((q_tiles + 1) / 2);
+    const int slots = ((one + sms - 1) / sms) * 3 < ((two + sms - 1) / sms) * 4 ? 1 : 2;
+    const bool column = p.gridW == 1 && p.gridH > 1;
+    const int gridH = column ? 1 : p.gridH, gridW = column ? p.gridH : p.gridW;
+    if (gridH == 1) return launch_quad_grid<KS, SPARSE, EXACT, kOneRow>(p, gridH, gridW, slots, status, st);
+    if (gridW > slots * kTile) return launch_quad_grid<KS, SPARSE, EXACT, kWide>(p, gridH, gridW, slots, status, st);
+    return launch_quad_grid<KS, SPARSE, EXACT, kOrdinary>(p, gridH, gridW, slots, status, st);
 }
 
 }  // namespace

@@ -39,6 +39,17 @@ def worst(got, ref):
     return float(np.max(np.abs(got - ref)) / np.max(np.abs(ref)))
 
 
+@pytest.mark.parametrize("shape", [(1, 2, 1, 600, 64, 3), (1, 2, 600, 1, 64, 3), (1, 2, 2, 331, 64, 5), (1, 2, 3, 700, 64, 3), (2, 2, 1, 40, 64, 5),
+                                   (2, 2, 40, 1, 64, 5), (1, 1, 2, 129, 64, 3), (1, 1, 1, 2000, 64, 5), (1, 2, 2000, 1, 64, 5), (1, 2, 7, 90, 64, 3),
+                                   (1, 2, 257, 2, 64, 3), (40, 8, 196, 1, 64, 3), (1, 2, 5, 257, 64, 5), (1, 3, 3, 256, 64, 3), (1, 70, 3, 300, 64, 3)],
+                         ids=lambda c: "x".join(map(str, c)))
+def test_explicit_weights(shape):
+    c = thin((*shape, "bf16"), 2200 + sum(shape))
+    s = c.shape
+    ref = oracle.forward_matrix(c.q, c.k, c.v, c.dw_weight, c.dw_bias, s.gridH, s.gridW, s.ksize, threads=8, kernel=oracle.KERNEL_EXACT)
+    assert worst(run(c, 2, exact_kernel=True), ref) <= 2e-2
+
+
 # on both sides of the rule: patches four times (3.5 times) as large as the grid, more of them than run at a time
 @pytest.mark.parametrize("rownorm", [False, True], ids=["core", "rownorm"])
 @pytest.mark.parametrize("shape", [(1, 4, 1, 2000, 64, 3), (1, 4, 2000, 1, 64, 5), (4, 12, 2, 331, 64, 3), (4, 12, 331, 4, 64, 3), (4, 12, 331, 5, 64, 5),
