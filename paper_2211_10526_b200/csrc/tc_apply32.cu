@@ -57,6 +57,7 @@ struct Apply32Params {
     const float* state;            // [BH][32*32 + 32 (+ 32)]
     const __nv_bfloat16* w;        // [H*32][KS][KS]
     const __nv_bfloat16* bias;     // [H*32] or nullptr
+    int column;                    // the grid is one column, taken as a row
     int flat;                      // the planes have one uniform stride: the tensor maps are 4-D, [.., plane]
     int H, head0, hdiv, tilesX, tilesY, n_tiles;
     float eps2;
@@ -295,6 +296,12 @@ tc_apply32_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                 for (int dx = 0; dx < KS; ++dx)
                     wreg[dy][dx] = make_float2(__bfloat162float(prm.w[(size_t)ch * KS * KS + dy * KS + dx]),
                                                __bfloat162float(prm.w[(size_t)(ch + 1) * KS * KS + dy * KS + dx]));
+            if (prm.column) {   // the filters' middle column, as the middle row: the only taps that meet the grid
+#pragma unroll
+                for (int dx = 0; dx < KS; ++dx)
+                    wreg[G::R][dx] = make_float2(__bfloat162float(prm.w[(size_t)ch * KS * KS + dx * KS + G::R]),
+                                                 __bfloat162float(prm.w[(size_t)(ch + 1) * KS * KS + dx * KS + G::R]));
+            }
             if (prm.bias) bias2 = make_float2(__bfloat162float(prm.bias[ch]), __bfloat162float(prm.bias[ch + 1]));
         };
         load_filters();      // of the first plane, while the state kernel finishes
@@ -354,7 +361,7 @@ tc_apply32_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
 }
 
 template <int KS, bool RN, int kTX, bool FINE>
-cudaError_t launch_apply32_ks(const Problem& p, const float* state, unsigned* status, cudaStream_t st) {
+cudaError_t launch_apply32_ks(const Problem& p, bool column, const float* state, unsigned* status, cudaStream_t st) {
     using G = Geo<KS, kTX, FINE>;
     constexpr int kTY = G::kTY;
     CUtensorMap tmQ, tmV, tmO;
@@ -378,6 +385,7 @@ cudaError_t launch_apply32_ks(const Problem& p, const float* state, unsigned* st
         return cudaErrorNotSupported;
     Apply32Params prm;
     prm.state = state;
+    prm.column = column ? 1 : 0;
     prm.w = static_cast<const __nv_bfloat16*>(p.w);
     prm.bias = static_cast<const __nv_bfloat16*>(p.bias);
     prm.flat = (rank == 4) ? 1 : 0;
@@ -402,7 +410,7 @@ cudaError_t launch_apply32_ks(const Problem& p, const float* state, unsigned* st
 }
 
 template <int KS, bool RN, bool FINE>
-cudaError_t launch_apply32_rn(const Problem& p, const float* state, unsigned* status, cudaStream_t st) {
+cudaError_t launch_apply32_rn(const Problem& p, bool column, const float* state, unsigned* status, cudaStream_t st) {
     // Patches of 16 x 16 where they need fewer rounds of the device.  Measured, 32 columns wide against 16: 8 x 8 planes of
     // 50 x 75, 5 x 5 filters 31.4 / 30.6 us (10 rounds / 9), 25 x 38 18.0 / 16.1 (4 / 3), 3 x 3, 31 x 33 14.1 / 12.9 (4 / 3); as
     // many rounds: 64 x 64 27.4 / 27.6; fewer with 32: 100 x 150 84.4 / 88.5 (29 / 31), 64 x 8 planes of 24 x 24 28.1 / 31.5.
@@ -410,16 +418,22 @@ cudaError_t launch_apply32_rn(const Problem& p, const float* state, unsigned* st
         const long long n = (long long)p.BH * ((p.gridW + tx - 1) / tx) * ((p.gridH + kTile / tx - 1) / (kTile / tx));
         return (n + device_sm_count() - 1) / device_sm_count();
     };
-    return rounds(16) < rounds(32) ? launch_apply32_ks<KS, RN, 16, FINE>(p, state, status, st) : launch_apply32_ks<KS, RN, 32, FINE>(p, state, status, st);
+    return rounds(16) < rounds(32) ? launch_apply32_ks<KS, RN, 16, FINE>(p, column, state, status, st)
+                                   : launch_apply32_ks<KS, RN, 32, FINE>(p, column, state, status, st);
 }
 
 }  // namespace
 
-cudaError_t launch_apply32(const Problem& p, const float* state, unsigned* status, cudaStream_t st) {
+cudaError_t launch_apply32(const Problem& given, const float* state, unsigned* status, cudaStream_t st) {
+    // A grid of one column is taken as one row, of which a patch holds 32 tokens or 16 instead of 8 or 16: 8 x 8 planes of
+    // 16383 x 1, 5 x 5 filters 455 us (895 as a column), 3 x 3 319 (595).
+    Problem p = given;
+    const bool column = given.gridW == 1 && given.gridH > 1;
+    if (column) { p.gridH = 1; p.gridW = given.gridH; }
     auto launch = [&](auto fine) {
         constexpr bool F = decltype(fine)::value;
-        if (p.ksize == 3) return p.rownorm ? launch_apply32_rn<3, true, F>(p, state, status, st) : launch_apply32_rn<3, false, F>(p, state, status, st);
-        return p.rownorm ? launch_apply32_rn<5, true, F>(p, state, status, st) : launch_apply32_rn<5, false, F>(p, state, status, st);
+        if (p.ksize == 3) return p.rownorm ? launch_apply32_rn<3, true, F>(p, column, state, status, st) : launch_apply32_rn<3, false, F>(p, column, state, status, st);
+        return p.rownorm ? launch_apply32_rn<5, true, F>(p, column, state, status, st) : launch_apply32_rn<5, false, F>(p, column, state, status, st);
     };
     return p.fine ? launch(std::true_type{}) : launch(std::false_type{});
 }

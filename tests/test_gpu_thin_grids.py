@@ -50,6 +50,16 @@ def test_explicit_weights(shape):
     assert worst(run(c, 2, exact_kernel=True), ref) <= 2e-2
 
 
+@pytest.mark.parametrize("rownorm", [False, True], ids=["core", "rownorm"])
+@pytest.mark.parametrize("shape", [(8, 8, 1, 601, 32, 5), (8, 8, 601, 1, 32, 5), (8, 8, 600, 1, 32, 3), (5, 9, 1031, 1, 32, 3), (8, 8, 301, 2, 32, 3)],
+                         ids=lambda c: "x".join(map(str, c)))
+def test_width_32(shape, rownorm):
+    c = thin((*shape, "bf16"), 2300 + sum(shape))
+    s = c.shape
+    ref = (oracle.forward_rownorm if rownorm else oracle.forward)(c.q, c.k, c.v, c.dw_weight, c.dw_bias, s.gridH, s.gridW, s.ksize, threads=8)
+    assert worst(run(c, 2, normalize_rows=rownorm), ref) <= 2e-2
+
+
 # on both sides of the rule: patches four times (3.5 times) as large as the grid, more of them than run at a time
 @pytest.mark.parametrize("rownorm", [False, True], ids=["core", "rownorm"])
 @pytest.mark.parametrize("shape", [(1, 4, 1, 2000, 64, 3), (1, 4, 2000, 1, 64, 5), (4, 12, 2, 331, 64, 3), (4, 12, 331, 4, 64, 3), (4, 12, 331, 5, 64, 5),
