@@ -259,6 +259,9 @@ tc_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
                 if (prm.bias && wt < kW)
                     asm volatile("ld.global.nc.u16 %0, [%1];" : "=h"(braw) : "l"(reinterpret_cast<const unsigned short*>(prm.bias) + h * kW + wt));
             }
+            // A thread whose wait has run out goes straight to the barrier behind this block, where all of them leave.
+            bool ok = false;
+            do {
             // ---- K rows -> unit rows, in place ----
             if (!mbar_wait(k_full, ph, abort_flag, prm.status, kBit)) break;
             if (has_line) {
@@ -386,8 +389,9 @@ tc_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
             }
             tcgen05_fence_before_sync();
             mbar_arrive(tm_free);
-            if (!mbar_wait(vp_full, ph, abort_flag, prm.status, kBit)) break;
-            named_barrier_sync(1, WORKERS);  // accumulator rows, rq, s and filters are visible to every worker
+            ok = mbar_wait(vp_full, ph, abort_flag, prm.status, kBit);
+            } while (false);
+            if (named_barrier_any(1, WORKERS, !ok)) break;  // accumulator rows, rq, s and filters are visible to every worker
 
             // ---- convolution + combine ----
             // A unit is a strip of two output columns per lane over a run of grid rows: every word of V is loaded (a row ahead)
