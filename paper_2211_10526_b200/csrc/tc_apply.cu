@@ -227,9 +227,10 @@ tc_apply_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                 fence_proxy_async_smem();
                 mbar_arrive(s_ready);
             }
+            bool ok;   // a thread whose wait has run out goes on to the barrier below, which all of them leave the loop at
             {   // this thread's half of sum(q^2) for its token; the other half comes from the partner warp
                 const int s = it % NS, use = it / NS;
-                if (!mbar_wait(&full[s], use & 1, abort_flag, prm.status, kBit)) break;
+                ok = mbar_wait(&full[s], use & 1, abort_flag, prm.status, kBit);
                 const uint8_t* qrow = stages + s * G::kStage + row * 128;
                 float ss[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
@@ -245,7 +246,7 @@ tc_apply_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                 rq_s[half * kTile + row] = (ss[0] + ss[1]) + (ss[2] + ss[3]);
                 mbar_arrive(&empty[s]);  // the Q rows of this stage have been read
             }
-            if (!mbar_wait(&acc_full[b], ub & 1, abort_flag, prm.status, kBit)) break;
+            ok &= mbar_wait(&acc_full[b], ub & 1, abort_flag, prm.status, kBit);
             tcgen05_fence_after_sync();
             float a[32];
             {
@@ -263,11 +264,11 @@ tc_apply_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
                 tmem_ld_wait();
                 qk = x[0];
             }
-            if (!mbar_wait(&conv_full[b], ub & 1, abort_flag, prm.status, kBit)) break;
+            ok &= mbar_wait(&conv_full[b], ub & 1, abort_flag, prm.status, kBit);
             // the previous patch's TMA store must have read out_s before it is rewritten; the same
             // barrier makes both halves of every row's sum of squares visible
             if (it > 0 && leader) tma_store_wait_read();
-            named_barrier_sync(1, kEpiThreads);
+            if (named_barrier_any(1, kEpiThreads, !ok)) break;
             const float rq = rsqrtf(fmaxf(rq_s[row] + rq_s[kTile + row], prm.eps2));
             const uint8_t* srow = stg + b * kStgBytes + row * kStgStride + half * 128;
             uint8_t* orow = out_s + row * 128;
