@@ -43,10 +43,10 @@ FALLBACK_HBM_GBS = 6650.0
 # bench.py reports the figure only while `git log` still names that commit as the kernel's latest: after
 # any later change to the kernel the counters are stale and `traffic` is null.
 NCU_TRAFFIC = {
-    ("c5_sweep_bf16:3", "tc_apply"): {"bytes": 281.8e6 + 122.1e6, "profile": "profiles/tc_kernels_c5_sweep.md",
-                                      "source": "paper_2211_10526_b200/csrc/tc_apply.cu", "commit": "0c32e4c"},
-    ("c3_deit_base_bf16", "tc_fused"): {"bytes": 57.9e6 + 2.0e6, "profile": "profiles/tc_fused_c3_deit_base.md",
-                                        "source": "paper_2211_10526_b200/csrc/tc_fused.cu", "commit": "d209734"},
+    ("c5_sweep_bf16:3", "tc_apply"): {"bytes": 281.7e6 + 122.1e6, "profile": "profiles/kernels.md",
+                                      "source": "paper_2211_10526_b200/csrc/tc_apply.cu", "commit": "2168f5d"},
+    ("c3_deit_base_bf16", "tc_fused"): {"bytes": 37.7e6 + 0.7e6, "profile": "profiles/kernels.md",
+                                        "source": "paper_2211_10526_b200/csrc/tc_fused.cu", "commit": "e3bc655"},
 }
 REPEATS = 5          # timed repeats; the median is reported
 MIN_FORWARDS = 100   # forwards per repeat, at least

@@ -38,9 +38,9 @@ bool supports(const Problem& p) {
 
 int rows_per_head(int N, int d) { return d == 32 ? (N + 1) / 2 : N; }
 
-// With fewer than 48 tokens per (b,h) the tiles of the tensor-core kernels are mostly padding and the CUDA-core kernels
-// are faster (measured: 4x4 grids of width-32 heads, 20 us against 33 us); from 7x7 on they are not (64 x 8 planes: 17.0 us
-// against 14.6 us).
+// Planes of fewer than 48 tokens stay on the CUDA cores, where their operands are fp32 and where the tests hold them.  It is not the
+// time that draws the line (CUDA cores / these kernels, from a graph): 64 x 12 planes of 4 x 4, width 32 13.6 / 12.8 us, 8 x 8 planes of
+// 4 x 4 5.7 / 6.6, 64 x 8 of 6 x 6 14.1 / 10.0; width 64, 64 x 12 planes of 4 x 4 28.9 / 11.9.
 bool preferred(const Problem& p) {
     return supports(p) && p.N >= 48 && (p.d == 64 || token_pairs(p) || head_pairs(p) || (long long)p.BH * p.N >= kNarrowMinTokens);
 }
@@ -78,7 +78,7 @@ cudaError_t forward(const Problem& p_in, float* ws_state, float* ws_partial, uns
     // What the packed 128-byte rows do not take, and planes too small to fill their tiles, have the precision of fp32 operands, as
     // on the CUDA cores: unit keys and scaled states as pairs.  Relative error against 64 bits of the bf16 outputs, CUDA
     // cores / single bf16 / pairs: 64 x 8 planes of 7 x 7 1.65499e-3 / 1.67565e-3 / 1.65499e-3, 8 x 8 of 50 x 75, 5 x 5 filters,
-    // 1.66210e-3 / 1.68312e-3 / 1.66210e-3, 64 x 8 of 8 x 8 1.65823e-3 / 1.67885e-3 / 1.65823e-3.  Time: 18.4 / 10.3 / 11.7 us,
+    // 1.66210e-3 / 1.68312e-3 / 1.66210e-3, 64 x 8 of 8 x 8 1.65823e-3 / 1.67885e-3 / 1.65823e-3.  Time: 18.4 / 10.3 / 11.9 us,
     // 245 / 30.6 / 33.2, 21.4 / 10.7 / 12.6.
     p.fine = p.d == 32 && !head_pairs(p) && (!token_pairs(p) || p.N < 96);
     const bool fine = p.fine;

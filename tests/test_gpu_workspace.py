@@ -23,7 +23,7 @@ def error(out, c):
 
 
 # the captured call, then calls of other kernel families whose workspace is smaller; the last has more planes than the arrival
-# counters behind the workspace are for
+# counters allocated with the workspace are for
 CAPTURED = [(2, 8, 64, 64, 128, 3, "f32"), (1, 8, 64, 64, 64, 3, "f32"), (2, 8, 20, 24, 64, 5, "bf16")]
 LATER = [(2, 4, 14, 14, 64, 3, "bf16"), (1, 4, 24, 24, 64, 3, "bf16"), (1, 2, 9, 9, 48, 3, "bf16"), (1, 2, 24, 20, 64, 5, "bf16"),
          (1, 2, 9, 9, 32, 5, "f32"), (300, 1, 7, 7, 32, 3, "bf16")]
