@@ -186,7 +186,7 @@ tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
         // normalisation of the next item's tiles.
         auto flush = [&](int item) -> bool {
             const int buf = item & 1;
-            if (!mbar_wait(&accum[buf], (item >> 1) & 1, abort_flag, status, kStatusStateTimeout)) return false;
+            if (!mbar_wait_warp(&accum[buf], (item >> 1) & 1, abort_flag, status, kStatusStateTimeout)) return false;
             tcgen05_fence_after_sync();
             if (quarter < 3) {
                 float* out = dst + ((size_t)(bh0 + item) * P + p) * kStateW;
@@ -218,7 +218,7 @@ tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
         for (int item = 0; item < n_items && ok; ++item) {
             for (int it = 0; it < n_tiles; ++it, ++gt) {
                 const int s = gt % kStages, use = gt / kStages;
-                ok = mbar_wait(&full[s], use & 1, abort_flag, status, kStatusStateTimeout);
+                ok = mbar_wait_warp(&full[s], use & 1, abort_flag, status, kStatusStateTimeout);   // as a whole: flush() reads tensor memory
                 if (!ok) break;
                 // NARROW: the 128 bytes are tokens 2 t and 2 t + 1, whose chunk c sits at chunk c ^ (t & 3) of their half; the
                 // same walk over the eight chunks as for a 128-byte swizzle meets all chunks of one of them first
