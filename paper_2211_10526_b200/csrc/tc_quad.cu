@@ -17,20 +17,23 @@
 // the second sweep the weight of a pair is the base weight plus Mask_eps of its softmax probability.  When a plane has at
 // most kResident key tiles they stay in shared memory between the two sweeps.
 //
-// What bounds it: the weight function, 16 square roots or exponentials per cycle and multiprocessor (2 x 8 planes of
-// 64 x 64 tokens: 2.7e8 pairs, 61 us of that unit at 1.85 GHz).  Per 128 x 128 pairs that unit needs 1024 cycles and the
-// UMMAs 512 (64 each at N = 128, 32 each with A in TMEM), so two slots keep both busy.  The two contractions have an
-// issuing warp each: a ready wait costs 50 to 90 cycles and an issue 30 per UMMA, which one warp could not do in time.
-// Measured (B200, per forward): exact kernel, 2 x 8 planes of 64 x 64 tokens 135 us (338 with one issuing thread, weights
-// through shared memory and eight weight warps: 510 TFLOP/s over the two contractions against 203); masked branch, 64 x 12
-// planes of 14 x 14 62 us (303: there every item waited for its Q tiles and for a convolution of one thread per token; 67 with
-// the convolution's window read word by word from global memory).  Eight weight warps instead of sixteen: 151 and 77 us (two
-// warps per scheduler do not hide the trips to TMEM); all sixteen on one slot at a time: 139 and 68 us.  Issue slots are 70 %
-// busy in the exact kernel; what is left is the hand-over of a cosine buffer (weights, second contraction, first contraction),
-// of which TMEM has room for three.
+// What bounds it: the issue slots of the warps that turn cosines into weights and rows into unit rows, on top of the hand-over of a
+// cosine buffer (first contraction, weights, second contraction), of which tensor memory has room for three.  2 x 8 planes of 64 x 64
+// tokens, exact kernel: 119 us; in working copies 97 with cosines written back as they are, 76 with rows left as they are as well: what
+// the weights and the rows take comes on top of the chain, which waits for tensor memory and barriers.  So a weight has no square root where the cosines
+// of a step are small (127 us with the old scaling of rows and 5 packed operations a pair, 135.5 with the square roots, whose unit has 16 lanes), and a row
+// is read once and scaled by two packed bf16 operations a word instead of two conversions, a product and a rounding (127 -> 119 together
+// with one operation less a pair).  K scaled by the weight warps instead (its norms beside it, cosines not before a packed product): 133 against 127, as
+// sixteen warps pay for what four did.  Four K stages, the convolution staged for one slot at a time: 117 against 119, but the masked branch 66 against 62.
+// The two contractions have an issuing warp each: a ready wait costs 50 to 90 cycles and an issue 30 per UMMA, which one warp could not do in time.
+// Eight weight warps instead of sixteen (with square roots): 151 us against 135; all sixteen on one slot at a time: 139.
+// Masked branch, 64 x 12 planes of 14 x 14: 62 us (303 where every item waited for its Q tiles and for a convolution of one thread per
+// token; 67 with the convolution's window read word by word from global memory).
 // No workspace; every wait is bounded.
 #include "tc_common.cuh"
 #include "tc_host.cuh"
+
+#include <type_traits>
 
 namespace castling {
 namespace tc {
@@ -111,9 +114,19 @@ __device__ __forceinline__ float exp2_approx(float x) {
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
+__device__ __forceinline__ uint32_t hmul2_bf16(uint32_t a, uint32_t b) {
+    uint32_t d;
+    asm("mul.rn.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
+    return d;
+}
+__device__ __forceinline__ uint32_t hfma2_bf16(uint32_t a, uint32_t b, uint32_t c) {
+    uint32_t d;
+    asm("fma.rn.bf16x2 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
+    return d;
+}
 constexpr float kLog2e = 1.4426950408889634f;
 
-// 1 - arccos(x)/pi of a pair: with t = 1 - |x| (clamped to [0, 1]: rounding can leave a cosine just outside [-1, 1]),
+// 1 - arccos(x)/pi of a pair, any cosine: with t = 1 - |x| (clamped to [0, 1]: rounding can leave a cosine just outside [-1, 1]),
 // arccos(|x|) = sqrt(t) * cubic(t) -- Abramowitz & Stegun 4.4.45 with its cubic in |x| expanded about |x| = 1, |error| <
 // 7e-5 rad, far below the bf16 rounding of the weights -- and 1 - arccos(x)/pi = 1/2 + sign(x) (1/2 - arccos(|x|)/pi).
 __device__ __forceinline__ float2 angular_weight2(float2 x) {
@@ -126,6 +139,23 @@ __device__ __forceinline__ float2 angular_weight2(float2 x) {
     const uint32_t sx = __float_as_uint(x.x) & 0x80000000u, sy = __float_as_uint(x.y) & 0x80000000u;
     return fadd2(make_float2(__uint_as_float((__float_as_uint(h.x) & 0x7fffffffu) | sx),
                              __uint_as_float((__float_as_uint(h.y) & 0x7fffffffu) | sy)), dup2(0.5f));
+}
+// The same where both |x| <= kNearLimit: 1/2 + arcsin(x)/pi with arcsin(x)/x quadratic in x^2 (|error| < 5e-5 rad, 1.2e-5 in the
+// root mean square over cosines of independent rows; the general form 4.5e-5).  No square root and less than half the instructions
+// of the general form, which is left to the few steps that hold a larger cosine: between independent rows of 64 elements 0.6 is
+// 4.8 standard deviations, and one step of 512 cosines in 15 000 has one.
+constexpr float kNearLimit = 0.6f;
+__device__ __forceinline__ float2 angular_weight2_near(float2 x) {
+    const float2 u = ffma2(x, x, dup2(0.f));
+    float2 p = ffma2(dup2(0.03577495f), u, dup2(0.05099359f));
+    p = ffma2(p, u, dup2(0.31836814f));
+    return ffma2(p, x, dup2(0.5f));
+}
+// Largest magnitude of three.
+__device__ __forceinline__ float max3_abs(float a, float b, float c) {
+    float r;
+    asm("max.NaN.abs.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
 }
 
 // GRID.  kWide: rows longer than an item's queries, which then lie in one row, or at the end of one and the beginning of the next,
@@ -146,19 +176,19 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     uint8_t* V_s = smem + kOffV;
     uint8_t* stg = smem + kOffStg;
     uint64_t* q_full = reinterpret_cast<uint64_t*>(smem + kOffBar);   // [2] by item
-    uint64_t* q_ready = q_full + 2;              // [2] Q rows scaled (kNormThreads)
+    uint64_t* q_ready = q_full + 2;              // [2] Q rows scaled (one arrival per warp, here and below)
     uint64_t* q_free = q_ready + 2;              // [2] the item's last cosine UMMAs have read Q
     uint64_t* k_full = q_free + 2;               // [kKStages]
-    uint64_t* k_scaled = k_full + kKStages;      // [kKStages] (kNormThreads)
+    uint64_t* k_scaled = k_full + kKStages;      // [kKStages]
     uint64_t* k_empty = k_scaled + kKStages;     // [kKStages]
     uint64_t* v_full = k_empty + kKStages;       // [kVStages]
     uint64_t* v_empty = v_full + kVStages;       // [kVStages]
     uint64_t* c_full = v_empty + kVStages;       // [2][kCBufs] by slot: cosines written
-    uint64_t* r_done = c_full + 2 * kCBufs;      // [kCBufs] cosines of a first sweep read (kSlotThreads)
-    uint64_t* p_full = r_done + kCBufs;          // [kCBufs] weights written (kSlotThreads)
+    uint64_t* r_done = c_full + 2 * kCBufs;      // [kCBufs] cosines of a first sweep read
+    uint64_t* p_full = r_done + kCBufs;          // [kCBufs] weights written
     uint64_t* pv_done = p_full + kCBufs;         // [kCBufs] weights read by the second contraction
     uint64_t* o_full = pv_done + kCBufs;         // [2] by slot
-    uint64_t* o_free = o_full + 2;               // [2] (128)
+    uint64_t* o_free = o_full + 2;               // [2]
     uint64_t* patch_full = o_free + 2;
     uint64_t* patch_free = patch_full + 1;       // (one arrival per convolution warp)
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(patch_free + 1);
@@ -193,19 +223,20 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
         const int c = (im.t0 - pa.y0 * prm.gridW) / kPatchX + j;
         return c < pa.nx ? c : c - pa.nx;
     };
+    auto warp_arrive = [&](uint64_t* bar) { __syncwarp(); if (lane == 0) mbar_arrive(bar); };   // for all lanes of a warp
     auto warp_wait = [&](uint64_t* bar, uint32_t parity) -> bool {
         return mbar_wait_warp(bar, parity, abort_flag, prm.status, kBit);
     };
 
     if (tid == 0) {
-        for (int b = 0; b < 2; ++b) { mbar_init(&q_full[b], 1); mbar_init(&q_ready[b], kNormThreads); mbar_init(&q_free[b], 1); }
-        for (int s = 0; s < kKStages; ++s) { mbar_init(&k_full[s], 1); mbar_init(&k_scaled[s], kNormThreads); mbar_init(&k_empty[s], 1); }
+        for (int b = 0; b < 2; ++b) { mbar_init(&q_full[b], 1); mbar_init(&q_ready[b], kNormThreads / 32); mbar_init(&q_free[b], 1); }
+        for (int s = 0; s < kKStages; ++s) { mbar_init(&k_full[s], 1); mbar_init(&k_scaled[s], kNormThreads / 32); mbar_init(&k_empty[s], 1); }
         for (int s = 0; s < kVStages; ++s) { mbar_init(&v_full[s], 1); mbar_init(&v_empty[s], 1); }
         for (int b = 0; b < kCBufs; ++b) {
             mbar_init(&c_full[b], 1); mbar_init(&c_full[kCBufs + b], 1);
-            mbar_init(&r_done[b], kSlotThreads); mbar_init(&p_full[b], kSlotThreads); mbar_init(&pv_done[b], 1);
+            mbar_init(&r_done[b], kSlotThreads / 32); mbar_init(&p_full[b], kSlotThreads / 32); mbar_init(&pv_done[b], 1);
         }
-        for (int s = 0; s < 2; ++s) { mbar_init(&o_full[s], 1); mbar_init(&o_free[s], kTile); }
+        for (int s = 0; s < 2; ++s) { mbar_init(&o_full[s], 1); mbar_init(&o_free[s], kTile / 32); }
         mbar_init(patch_full, 1); mbar_init(patch_free, kConvThreads / 32);
         *abort_flag = 0;
         mbar_fence_init();
@@ -380,32 +411,30 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     } else if (warp < 8) {
         // ---- unit rows ----
         const int t = tid - 128;
-        auto scale_row = [&](uint8_t* row) {   // row t of a tile, read twice: the whole row does not fit beside the rest
-            auto chunk = [&](int j) { return reinterpret_cast<uint4*>(row + ((j ^ (t & 7)) << 4)); };
+        // Row t of a tile times r = 1 / max(norm, eps), r as the sum of two bf16: x r_hi + (x r_lo), the product in brackets rounded,
+        // the rest in one rounding.  That is the rounding of x r itself but for 1 case in 256, where x r lies next to the middle between two bf16.
+        auto scale_row = [&](uint8_t* row) {
+            uint32_t w[32];
             float2 ss[4] = {dup2(0.f), dup2(0.f), dup2(0.f), dup2(0.f)};
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
-                const uint4 c = *chunk(j);
-                const uint32_t w[4] = {c.x, c.y, c.z, c.w};
+                const uint4 c = *reinterpret_cast<const uint4*>(row + ((j ^ (t & 7)) << 4));
+                w[4 * j] = c.x; w[4 * j + 1] = c.y; w[4 * j + 2] = c.z; w[4 * j + 3] = c.w;
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
-                    const float2 p = make_float2(bf16lo(w[e]), bf16hi(w[e]));
+                    const float2 p = make_float2(bf16lo(w[4 * j + e]), bf16hi(w[4 * j + e]));
                     ss[e] = ffma2(p, p, ss[e]);
                 }
             }
             const float2 sum = fadd2(fadd2(ss[0], ss[1]), fadd2(ss[2], ss[3]));
-            const float2 rk2 = dup2(1.0f / sqrtf(fmaxf(sum.x + sum.y, prm.eps2)));
-#pragma unroll 4
+            const float r = 1.0f / sqrtf(fmaxf(sum.x + sum.y, prm.eps2));
+            const uint32_t hi = pack_bf16x2(r, r), lo = pack_bf16x2(r - bf16lo(hi), r - bf16lo(hi));
+#pragma unroll
             for (int j = 0; j < 8; ++j) {
-                const uint4 c = *chunk(j);
-                const uint32_t w[4] = {c.x, c.y, c.z, c.w};
                 uint32_t o[4];
 #pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const float2 p = ffma2(make_float2(bf16lo(w[e]), bf16hi(w[e])), rk2, dup2(0.f));
-                    o[e] = pack_bf16x2(p.x, p.y);
-                }
-                *chunk(j) = make_uint4(o[0], o[1], o[2], o[3]);
+                for (int e = 0; e < 4; ++e) o[e] = hfma2_bf16(w[4 * j + e], hi, hmul2_bf16(w[4 * j + e], lo));
+                *reinterpret_cast<uint4*>(row + ((j ^ (t & 7)) << 4)) = make_uint4(o[0], o[1], o[2], o[3]);
             }
         };
         // The Q tiles of item i + 1 come after the first K tiles of item i: their copy starts once the cosines of item
@@ -415,7 +444,7 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
             const int slots = item_of(i).slots;
             for (int s = 0; s < slots; ++s) scale_row(Q_s + (2 * (i & 1) + s) * kTileBytes + t * 128);
             fence_proxy_async_smem();
-            mbar_arrive(&q_ready[i & 1]);
+            warp_arrive(&q_ready[i & 1]);
             return true;
         };
         int ks = 0;
@@ -427,7 +456,7 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                 if (!(ok = warp_wait(&k_full[ks], k_par))) break;
                 scale_row(K_s + ks * kTileBytes + t * 128);
                 fence_proxy_async_smem();
-                mbar_arrive(&k_scaled[ks]);
+                warp_arrive(&k_scaled[ks]);
                 if (++ks == kKStages) { ks = 0; k_par ^= 1; }
                 if (j == q_after && i + 1 < my_items && !(ok = scale_q(i + 1))) break;
             }
@@ -480,7 +509,7 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                         }
                         tcgen05_fence_before_sync();
                     }
-                    mbar_arrive(&r_done[b]);
+                    warp_arrive(&r_done[b]);
                     skip(im.slots);
                 }
                 // the two halves of a query meet in shared memory (by item parity: a thread is never two items ahead)
@@ -503,20 +532,33 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                         if (cc < 3) tmem_ld16(cb + (cc + 1) * 16, x[(cc + 1) & 1]);
                         uint32_t o[8];
                         if (cc * 16 < left) {
+                            auto weigh = [&](auto near) {
 #pragma unroll
-                            for (int e = 0; e < 8; ++e) {
-                                const float2 xe = make_float2(x[cc & 1][2 * e], x[cc & 1][2 * e + 1]);
-                                float2 wv;
-                                if (EXACT) wv = angular_weight2(xe);
-                                if (SPARSE) {
-                                    const float2 y = make_float2(__saturatef(fmaf(xe.x, 0.5f, 0.5f)), __saturatef(fmaf(xe.y, 0.5f, 0.5f)));
-                                    if (!EXACT) wv = ffma2(y, dup2(2.0f * kInvPi), dup2(0.5f - kInvPi));   // 1/2 + x / pi
-                                    const float2 a = ffma2(y, dup2(2.0f * kLog2e), dup2(ebias));
-                                    const float px = exp2_approx(a.x), py = exp2_approx(a.y);
-                                    if (px > prm.sparse_eps) wv.x += px;   // predicated adds: 51.5 us against 52.6 with selects and a
-                                    if (py > prm.sparse_eps) wv.y += py;   // packed add (16 planes of 40 x 40)
+                                for (int e = 0; e < 8; ++e) {
+                                    const float2 xe = make_float2(x[cc & 1][2 * e], x[cc & 1][2 * e + 1]);
+                                    float2 wv;
+                                    if (EXACT) wv = decltype(near)::value ? angular_weight2_near(xe) : angular_weight2(xe);
+                                    if (SPARSE) {
+                                        const float2 y = make_float2(__saturatef(fmaf(xe.x, 0.5f, 0.5f)), __saturatef(fmaf(xe.y, 0.5f, 0.5f)));
+                                        if (!EXACT) wv = ffma2(y, dup2(2.0f * kInvPi), dup2(0.5f - kInvPi));   // 1/2 + x / pi
+                                        const float2 a = ffma2(y, dup2(2.0f * kLog2e), dup2(ebias));
+                                        const float px = exp2_approx(a.x), py = exp2_approx(a.y);
+                                        if (px > prm.sparse_eps) wv.x += px;   // predicated adds: 51.5 us against 52.6 with selects and a
+                                        if (py > prm.sparse_eps) wv.y += py;   // packed add (16 planes of 40 x 40)
+                                    }
+                                    o[e] = pack_bf16x2(wv.x, wv.y);
                                 }
-                                o[e] = pack_bf16x2(wv.x, wv.y);
+                            };
+                            weigh(std::bool_constant<EXACT>{});
+                            if (EXACT) {
+                                // whether that held is known only now: the answer need not be waited for before
+                                float m = 0.f, n = 0.f;   // NaN goes the general way
+#pragma unroll
+                                for (int e = 0; e < 16; e += 4) {
+                                    m = max3_abs(m, x[cc & 1][e], x[cc & 1][e + 1]);
+                                    n = max3_abs(n, x[cc & 1][e + 2], x[cc & 1][e + 3]);
+                                }
+                                if (!__all_sync(0xffffffffu, max3_abs(m, n, 0.f) <= kNearLimit)) weigh(std::false_type{});
                             }
                         } else {
 #pragma unroll
@@ -527,7 +569,7 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                     tmem_st_wait();
                     tcgen05_fence_before_sync();
                 }
-                mbar_arrive(&p_full[b]);
+                warp_arrive(&p_full[b]);
                 if (jt < T - 1) skip(im.slots);
             }
             skip(im.slots - slot);   // to the first step of the next item
@@ -636,7 +678,7 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                         *reinterpret_cast<uint4*>(srow + c * 32 + 16) = pk[1];
                     }
                     tcgen05_fence_before_sync();
-                    mbar_arrive(&o_free[slot]);
+                    warp_arrive(&o_free[slot]);
                     __syncwarp();
                     __nv_bfloat16* op = prm.out + plane_offset(prm.lo, im.bh, prm.hdiv) + (lane & 7) * 8;
 #pragma unroll
