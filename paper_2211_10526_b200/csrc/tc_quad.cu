@@ -27,8 +27,8 @@
 // sixteen warps pay for what four did.  Four K stages, the convolution staged for one slot at a time: 117 against 119, but the masked branch 66 against 62.
 // The two contractions have an issuing warp each: a ready wait costs 50 to 90 cycles and an issue 30 per UMMA, which one warp could not do in time.
 // Eight weight warps instead of sixteen (with square roots): 151 us against 135; all sixteen on one slot at a time: 139.
-// Masked branch, 64 x 12 planes of 14 x 14: 62 us (303 where every item waited for its Q tiles and for a convolution of one thread per
-// token; 67 with the convolution's window read word by word from global memory).
+// Masked branch, 64 x 12 planes of 14 x 14: 57 us.  62 with the cosines clamped and turned into exponents pair by pair, in both
+// sweeps, and the keys that pad a tile left out one by one; now the rows of Q bring the factor log2(e) along, and the padding's ones are taken off the sum.
 // No workspace; every wait is bounded.
 #include "tc_common.cuh"
 #include "tc_host.cuh"
@@ -151,6 +151,16 @@ __device__ __forceinline__ float2 angular_weight2_near(float2 x) {
     p = ffma2(p, u, dup2(0.31836814f));
     return ffma2(p, x, dup2(0.5f));
 }
+// (x + 1) log2(e) + bias of a pair of cosines, clamped to [-1, 1].
+__device__ __forceinline__ float2 exponent2(float2 x, float bias) {
+    const float2 y = make_float2(__saturatef(fmaf(x.x, 0.5f, 0.5f)), __saturatef(fmaf(x.y, 0.5f, 0.5f)));
+    return ffma2(y, dup2(2.0f * kLog2e), dup2(bias));
+}
+__device__ __forceinline__ float one_if_greater(float a, float b) {
+    float r;
+    asm("set.gt.f32.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+    return r;
+}
 // Largest magnitude of three.
 __device__ __forceinline__ float max3_abs(float a, float b, float c) {
     float r;
@@ -198,6 +208,9 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     const int my_items = ((int)blockIdx.x < prm.n_items) ? (prm.n_items - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
     const int T = prm.k_tiles, N = prm.N;
     constexpr int kSweeps = SPARSE ? 2 : 1;
+    // Mask alone: the rows of Q have the length log2(e), so that the first contraction gives the exponents of exp2.  What pads a
+    // tile then still counts as exp2(0) = 1.
+    constexpr float kUnitQ = SPARSE && !EXACT ? kLog2e : 1.0f;
     const bool resident = SPARSE && T <= kResident;
     const int k_loads = resident ? T : kSweeps * T;   // K tiles loaded per item
     constexpr unsigned kBit = kStatusFusedTimeout;
@@ -411,9 +424,9 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     } else if (warp < 8) {
         // ---- unit rows ----
         const int t = tid - 128;
-        // Row t of a tile times r = 1 / max(norm, eps), r as the sum of two bf16: x r_hi + (x r_lo), the product in brackets rounded,
+        // Row t of a tile times r = factor / max(norm, eps), r as the sum of two bf16: x r_hi + (x r_lo), the product in brackets rounded,
         // the rest in one rounding.  That is the rounding of x r itself but for 1 case in 256, where x r lies next to the middle between two bf16.
-        auto scale_row = [&](uint8_t* row) {
+        auto scale_row = [&](uint8_t* row, float factor) {
             uint32_t w[32];
             float2 ss[4] = {dup2(0.f), dup2(0.f), dup2(0.f), dup2(0.f)};
 #pragma unroll
@@ -427,7 +440,7 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                 }
             }
             const float2 sum = fadd2(fadd2(ss[0], ss[1]), fadd2(ss[2], ss[3]));
-            const float r = 1.0f / sqrtf(fmaxf(sum.x + sum.y, prm.eps2));
+            const float r = factor / sqrtf(fmaxf(sum.x + sum.y, prm.eps2));
             const uint32_t hi = pack_bf16x2(r, r), lo = pack_bf16x2(r - bf16lo(hi), r - bf16lo(hi));
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
@@ -442,7 +455,7 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
         auto scale_q = [&](int i) -> bool {
             if (!warp_wait(&q_full[i & 1], (i >> 1) & 1)) return false;
             const int slots = item_of(i).slots;
-            for (int s = 0; s < slots; ++s) scale_row(Q_s + (2 * (i & 1) + s) * kTileBytes + t * 128);
+            for (int s = 0; s < slots; ++s) scale_row(Q_s + (2 * (i & 1) + s) * kTileBytes + t * 128, kUnitQ);
             fence_proxy_async_smem();
             warp_arrive(&q_ready[i & 1]);
             return true;
@@ -454,7 +467,7 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
         for (int i = 0; i < my_items && ok; ++i) {
             for (int j = 0; j < k_loads; ++j) {
                 if (!(ok = warp_wait(&k_full[ks], k_par))) break;
-                scale_row(K_s + ks * kTileBytes + t * 128);
+                scale_row(K_s + ks * kTileBytes + t * 128, 1.0f);
                 fence_proxy_async_smem();
                 warp_arrive(&k_scaled[ks]);
                 if (++ks == kKStages) { ks = 0; k_par ^= 1; }
@@ -479,7 +492,7 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
             const Item im = item_of(i);
             if (slot >= im.slots) { skip(kSweeps * T * im.slots); continue; }
             const bool live = im.t0 + slot * kTile + quarter * 32 < N;   // some row of this warp is a token
-            float ebias = 0.f;   // exp(x) / den = exp2(y * 2 log2(e) + ebias), y = (x + 1) / 2
+            float ebias = 0.f;   // exp(x) / den = exp2(x log2(e) + ebias); EXACT: exp2(y * 2 log2(e) + ebias), y = (x + 1) / 2
             skip(slot);
             if (SPARSE) {
                 float2 den = dup2(0.f);
@@ -498,15 +511,12 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
 #pragma unroll
                             for (int e = 0; e < 16; e += 2) {
                                 const float* xe = &x[cc & 1][e];
-                                const float2 y = make_float2(__saturatef(fmaf(xe[0], 0.5f, 0.5f)), __saturatef(fmaf(xe[1], 0.5f, 0.5f)));
-                                const float2 a = ffma2(y, dup2(2.0f * kLog2e), dup2(-kLog2e));
-                                float2 p = make_float2(exp2_approx(a.x), exp2_approx(a.y));
-                                if (cc * 16 + 16 > left) {   // the chunk that reaches beyond the plane
-                                    p.x = cc * 16 + e < left ? p.x : 0.f; p.y = cc * 16 + e + 1 < left ? p.y : 0.f;
-                                }
-                                den = fadd2(den, p);
+                                const float2 a = EXACT ? exponent2(make_float2(xe[0], xe[1]), -kLog2e) : make_float2(xe[0], xe[1]);
+                                den = fadd2(den, make_float2(exp2_approx(a.x), exp2_approx(a.y)));
                             }
                         }
+                        // keys beyond the plane: cosine 0, an exponential of 1 each
+                        if (left < kTile / 2) den.x -= (float)(-left & 15);
                         tcgen05_fence_before_sync();
                     }
                     warp_arrive(&r_done[b]);
@@ -516,7 +526,7 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                 float* den_s = reinterpret_cast<float*>(smem + kOffDen) + ((i & 1) * 4 + slot * 2) * kTile + quarter * 32 + lane;
                 den_s[half * kTile] = den.x + den.y;
                 if (named_barrier_any(2 + slot, kSlotThreads, !ok)) break;
-                ebias = -kLog2e - __log2f(den_s[0] + den_s[kTile]);
+                ebias = (EXACT ? -kLog2e : 0.f) - __log2f(den_s[0] + den_s[kTile]);
             }
             for (int jt = 0; jt < T; ++jt) {
                 if (!(ok = wait_cosines())) break;
@@ -539,12 +549,16 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                                     float2 wv;
                                     if (EXACT) wv = decltype(near)::value ? angular_weight2_near(xe) : angular_weight2(xe);
                                     if (SPARSE) {
-                                        const float2 y = make_float2(__saturatef(fmaf(xe.x, 0.5f, 0.5f)), __saturatef(fmaf(xe.y, 0.5f, 0.5f)));
-                                        if (!EXACT) wv = ffma2(y, dup2(2.0f * kInvPi), dup2(0.5f - kInvPi));   // 1/2 + x / pi
-                                        const float2 a = ffma2(y, dup2(2.0f * kLog2e), dup2(ebias));
-                                        const float px = exp2_approx(a.x), py = exp2_approx(a.y);
-                                        if (px > prm.sparse_eps) wv.x += px;   // predicated adds: 51.5 us against 52.6 with selects and a
-                                        if (py > prm.sparse_eps) wv.y += py;   // packed add (16 planes of 40 x 40)
+                                        float2 a;
+                                        if (EXACT) {
+                                            a = exponent2(xe, ebias);
+                                        } else {
+                                            wv = ffma2(xe, dup2(kInvPi / kLog2e), dup2(0.5f));   // 1/2 + x / pi
+                                            a = fadd2(xe, dup2(ebias));
+                                        }
+                                        const float2 p = make_float2(exp2_approx(a.x), exp2_approx(a.y));
+                                        // masked by a factor of 1 or 0: a pair takes three instructions, a predicate and an addition each four
+                                        wv = ffma2(p, make_float2(one_if_greater(p.x, prm.sparse_eps), one_if_greater(p.y, prm.sparse_eps)), wv);
                                     }
                                     o[e] = pack_bf16x2(wv.x, wv.y);
                                 }
