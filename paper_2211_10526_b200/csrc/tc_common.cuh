@@ -387,6 +387,58 @@ __device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) {
         : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
     return d;
 }
+// The same where the order of the operations is to stay: one that takes the result of another waits 8 cycles for it, and left to
+// itself the compiler puts the taps of one sum one after the other.
+__device__ __forceinline__ float2 ffma2_in_order(float2 a, float2 b, float2 c) {
+    float2 d;
+    asm volatile("{\n\t.reg .b64 ra, rb, rc, rd;\n\t"
+        "mov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\tmov.b64 rc, {%6, %7};\n\t"
+        "fma.rn.f32x2 rd, ra, rb, rc;\n\t"
+        "mov.b64 {%0, %1}, rd;\n\t}"
+        : "=f"(d.x), "=f"(d.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+    return d;
+}
+
+__device__ __forceinline__ float2 fadd2(float2 a, float2 b) {
+    float2 d;
+    asm("{\n\t.reg .b64 ra, rb, rd;\n\t"
+        "mov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\t"
+        "add.rn.f32x2 rd, ra, rb;\n\t"
+        "mov.b64 {%0, %1}, rd;\n\t}"
+        : "=f"(d.x), "=f"(d.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return d;
+}
+
+__device__ __forceinline__ uint32_t hmul2_bf16(uint32_t a, uint32_t b) {
+    uint32_t d;
+    asm("mul.rn.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
+    return d;
+}
+__device__ __forceinline__ uint32_t hfma2_bf16(uint32_t a, uint32_t b, uint32_t c) {
+    uint32_t d;
+    asm("fma.rn.bf16x2 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
+    return d;
+}
+// Pairs of bf16 times r, r as the sum of two bf16: x r_hi + (x r_lo), the product in brackets rounded, the rest in one rounding.
+// That is the rounding of x r itself but for 1 case in 256, where x r lies next to the middle between two bf16.
+struct Bf16Scale {
+    uint32_t hi, lo;
+    __device__ __forceinline__ explicit Bf16Scale(float r) {
+        hi = pack_bf16x2(r, r);
+        lo = pack_bf16x2(r - bf16lo(hi), r - bf16lo(hi));
+    }
+    __device__ __forceinline__ uint32_t operator()(uint32_t x) const { return hfma2_bf16(x, hi, hmul2_bf16(x, lo)); }
+};
+
+// A word to global memory if `store` says so, as a predicated instruction.
+__device__ __forceinline__ void stg32_if(bool store, uint32_t* p, uint32_t v) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.u32 p, %2, 0;\n\t"
+        "@p st.global.b32 [%0], %1;\n\t}"
+        ::"l"(p), "r"(v), "r"((uint32_t)store) : "memory");
+}
 
 }  // namespace tc
 }  // namespace castling

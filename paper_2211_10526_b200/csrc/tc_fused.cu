@@ -6,7 +6,8 @@
 // walks over planes blockIdx.x, blockIdx.x + gridDim.x, ...  Per plane
 //   warp 0      TMA: K, V and Q as 128-token tiles (128-byte rows and swizzle, 64 bytes for width 32; rows beyond N are
 //               zero-filled); once the state UMMAs have retired, V again without swizzle into
-//               the K buffer (an L2 hit), which is what the convolution reads
+//               the K buffer (an L2 hit), which is what the convolution reads: the token grid with its halo, zero-filled outside (ROOMY),
+//               or where that does not fit the tokens as they are, and words outside the grid are masked
 //   workers     thread = 128-byte line (one token, or two of width 32): scale K rows by 1 / max(||k||, eps) in place;
 //               1 / max(||q||, eps)
 //   warp 1      one elected lane issues the state UMMAs, A = [K^ ; 1 0 0 ...] (M-major, the ones row makes
@@ -14,23 +15,23 @@
 //   workers     read S and s from TMEM, write S' = S / pi as the bf16 B operand of the second
 //               contraction and s as fp32
 //   warp 1      apply UMMAs: acc[tile] = Q[tile] * S' into TMEM (the state's columns are reused)
-//   workers     thread = token: accumulator rows from TMEM to shared memory as fp32 (over the swizzled
+//   workers     thread = token: accumulator rows from TMEM, times 1 / max(||q||, eps), to shared memory as fp32 (over the swizzled
 //               V tiles and the Q tiles, both dead by then); then lane = channel pair (width 32: and column parity), warp = a
-//               strip of two columns (four): depthwise convolution sliding down the strip with the filters in registers,
-//               out = acc / max(||q||, eps) + 1/2 s + bias + conv, one rounding to bf16, rows stored
+//               strip of two columns (four): depthwise convolution sliding down the strip with the filters in registers, the sums
+//               of an output row starting from its accumulator + 1/2 s + bias, one rounding to bf16, rows stored
 //               straight to memory; leading off-grid tokens get the attention terms only
 // FINE (width 32 only): the unit keys and S' are two bf16 each, the value and what rounding it left off, contracted one after the
 // other: as precise as fp32 operands.  The rest of K lies in the Q buffer, so Q comes with the second copy of V, once the state
 // UMMAs have retired; the rest of S' lies in the V buffer, which is dead by then.  512 planes of 7 x 7: 11.7 us a call, 10.3
 // with single operands.
 //
-// A plane is a serial chain of about 15 000 cycles (14 x 14 tokens, width 64, 7 000 of them the convolution), so the time of
+// A plane is a serial chain of about 10 500 cycles (14 x 14 tokens, width 64, 4 600 of them the convolution), so the time of
 // a call is the number of planes over those in flight.  Two shapes of CTA: 256 workers for planes of any size, two per SM;
 // 128 workers for planes of at most 128 lines, three or four per SM, which finish a plane later but more of them at a time:
 // taken when that saves a round of planes.
-// Measured: 512 planes of 7 x 7, width 32, 14.1 -> 10.3 us a call (two tokens a line and large CTAs before); 3000 planes of
-// 11 x 11, width 64, 69.8 -> 64.4, 768 planes of 14 x 14 and a class token 32.2 -> 31.7 with masks instead of predicated loads,
-// running addresses, and the accumulator's words loaded ahead of the FMAs.
+// Measured (from a graph): 768 planes of 14 x 14 and a class token 28.1 us, 31.2 with every word of V masked, accumulators scaled one by one in the
+// convolution, branches around its loads and stores and each tap's sum waiting for the last (12 300 cycles a plane); 12 planes 7.4 / 8.1; 256 planes
+// of width 32 7.9 / 9.0; 512 planes of 7 x 7, width 32, 14.1 us a call with two tokens a line and large CTAs.
 #include "tc_common.cuh"
 #include "tc_host.cuh"
 
@@ -41,7 +42,7 @@ namespace {
 constexpr int kTile = 128;                       // tokens per UMMA tile
 
 // NARROW: width-32 heads in 64-byte rows, two tokens to a line.  WORKERS: worker threads, and lines a plane may have.
-template <int KS, bool NARROW, int WORKERS> struct Geo {
+template <int KS, bool NARROW, int WORKERS, bool ROOMY = false> struct Geo {
     static constexpr int kW = NARROW ? 32 : 64;                  // head width
     static constexpr int kRow = kW * 2;                          // bytes of a token
     static constexpr int kTokens = WORKERS * (NARROW ? 2 : 1);   // tokens a plane may have
@@ -52,6 +53,8 @@ template <int KS, bool NARROW, int WORKERS> struct Geo {
     // the unswizzled V plane, V and Q hold the fp32 accumulator rows.  The convolution's reads left of the plane's first token
     // fall into S'.
     static constexpr int kBuf = WORKERS * 128;
+    // Bytes of an accumulator row.  ROOMY: the plane with its halo fits the K buffer, and its accumulator rows with 16 bytes of padding V's and Q's.
+    static constexpr int kAccRow = kW * 4 + (ROOMY ? 16 : 0);
     static constexpr int kOffS = 0, kOffK = kW * kRow, kOffV = kOffK + kBuf, kOffQ = kOffV + kBuf;
     static_assert(kOffK % 1024 == 0 && kOffK >= KS / 2 * kRow, "swizzle atoms; room for the reads left of the plane");
     static constexpr int kOffOnes = kOffQ + kBuf;                // constant block of the A operand (after K: positive offset)
@@ -74,12 +77,12 @@ struct FusedParams {
 
 // OUT_PACKED: the output's token rows are contiguous, which keeps the row addresses of the
 // store loop compile-time offsets.
-template <int KS, bool OUT_PACKED, bool NARROW, int WORKERS, bool FINE>
+template <int KS, bool OUT_PACKED, bool NARROW, int WORKERS, bool FINE, bool ROOMY>
 __global__ void __launch_bounds__((Geo<KS, NARROW, WORKERS>::kThreads), (Geo<KS, NARROW, WORKERS>::kCtas))
 tc_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
                 const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmVplain,
                 const FusedParams prm) {
-    using G = Geo<KS, NARROW, WORKERS>;
+    using G = Geo<KS, NARROW, WORKERS, ROOMY>;
     constexpr int R = KS / 2, kW = G::kW, kRow = G::kRow, kTileBytes = kTile * kRow, kWarps = WORKERS / 32, kHalves = WORKERS / 128;
     constexpr uint32_t kHigh = NARROW ? kDescHigh64 : kDescHigh;
     extern __shared__ uint8_t smem_raw[];
@@ -155,8 +158,13 @@ tc_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
                 // the K tiles are dead once the state UMMAs have retired: bring V in again, unswizzled
                 if (!mbar_wait(s_done, it & 1, abort_flag, prm.status, kBit)) break;
                 if (FINE) load_q();   // over the rest of K
-                mbar_expect_tx(vp_full, tiles * kTileBytes);
-                for (int t = 0; t < tiles; ++t) tma_load_4d(K_s + t * kTileBytes, &tmVplain, vp_full, 0, t * kTile, ph, pb);
+                if (ROOMY) {
+                    mbar_expect_tx(vp_full, (W + 2 * R) * (prm.gridH + 2 * R) * kRow);
+                    tma_load_5d(K_s, &tmVplain, vp_full, 0, -R, -R, ph, pb);
+                } else {
+                    mbar_expect_tx(vp_full, tiles * kTileBytes);
+                    for (int t = 0; t < tiles; ++t) tma_load_4d(K_s + t * kTileBytes, &tmVplain, vp_full, 0, t * kTile, ph, pb);
+                }
                 ++issued_vp;
             }
             if (*abort_flag) {
@@ -224,6 +232,7 @@ tc_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
         // units of the convolution: strips of two output columns per lane, cut along y as long as there are fewer than warps
         const int n_strips = NARROW ? (W + 3) / 4 : (W + 1) / 2, cuts = min(prm.gridH, max(1, kWarps / n_strips));
         const int seg_rows = (prm.gridH + cuts - 1) / cuts, n_units = n_strips * ((prm.gridH + seg_rows - 1) / seg_rows);
+        const int first_strip = ww % n_strips, first_seg = ww / n_strips;
         // 1 / max(norm, eps) of each half of this thread's line of K or Q: c[j] is 16-byte chunk j ^ (wt & 7) of the 128 bytes.
         // Two tokens: chunk c of token 2 wt (+ 1) sits at c ^ (wt & 3) of its half, so the walk meets all four chunks of token
         // 2 wt + bit 2 of wt first.
@@ -245,6 +254,7 @@ tc_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
             const uint32_t ph = it & 1;
             const int bh = blockIdx.x + it * gridDim.x;
             const int h = (prm.head0 + bh) % prm.H;
+            __nv_bfloat16* const out_bh = prm.out + plane_offset(prm.lo, bh, prm.hdiv);
             // this thread's share of the head's filters (and bias): on its way while the rows are normalised, into shared memory
             // once the state is ready.  Volatile: left to itself the compiler moves the loads down to their use.
             constexpr int kElems = kW * KS * KS, kShare = (kElems + WORKERS - 1) / WORKERS;
@@ -271,24 +281,29 @@ tc_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
                 for (int j = 0; j < 8; ++j) c[j] = *reinterpret_cast<const uint4*>(row + ((j ^ (wt & 7)) << 4));
                 float sa, sb;
                 sums(c, sa, sb);
-                const float rka = 1.0f / sqrtf(fmaxf(NARROW ? sa : sa + sb, prm.eps2));
-                const float rkb = NARROW ? 1.0f / sqrtf(fmaxf(sb, prm.eps2)) : rka;
+                const float rka = rsqrtf(fmaxf(NARROW ? sa : sa + sb, prm.eps2));
+                const float rkb = NARROW ? rsqrtf(fmaxf(sb, prm.eps2)) : rka;
+                if (FINE) {
 #pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    const uint32_t w4[4] = {c[j].x, c[j].y, c[j].z, c[j].w};
-                    const float2 rk2 = (j < 4) ? make_float2(rka, rka) : make_float2(rkb, rkb);
-                    uint32_t o4[4];
+                    for (int j = 0; j < 8; ++j) {
+                        const uint32_t w4[4] = {c[j].x, c[j].y, c[j].z, c[j].w};
+                        const float2 rk2 = (j < 4) ? make_float2(rka, rka) : make_float2(rkb, rkb);
+                        uint32_t o4[4], r4[4];
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const float2 p = ffma2(make_float2(bf16lo(w4[e]), bf16hi(w4[e])), rk2, zero2);
-                        o4[e] = pack_bf16x2(p.x, p.y);
-                    }
-                    *reinterpret_cast<uint4*>(row + ((j ^ (wt & 7)) << 4)) = make_uint4(o4[0], o4[1], o4[2], o4[3]);
-                    if (FINE) {
-                        uint32_t r4[4];
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) r4[e] = rest_bf16x2(w4[e], rk2.x, o4[e]);
+                        for (int e = 0; e < 4; ++e) {
+                            const float2 p = ffma2(make_float2(bf16lo(w4[e]), bf16hi(w4[e])), rk2, zero2);
+                            o4[e] = pack_bf16x2(p.x, p.y);
+                            r4[e] = rest_bf16x2(w4[e], rk2.x, o4[e]);
+                        }
+                        *reinterpret_cast<uint4*>(row + ((j ^ (wt & 7)) << 4)) = make_uint4(o4[0], o4[1], o4[2], o4[3]);
                         *reinterpret_cast<uint4*>(Q_s + wt * 128 + ((j ^ (wt & 7)) << 4)) = make_uint4(r4[0], r4[1], r4[2], r4[3]);
+                    }
+                } else {
+                    const Bf16Scale fa(rka), fb(rkb);
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        const Bf16Scale& f = j < 4 ? fa : fb;
+                        *reinterpret_cast<uint4*>(row + ((j ^ (wt & 7)) << 4)) = make_uint4(f(c[j].x), f(c[j].y), f(c[j].z), f(c[j].w));
                     }
                 }
                 fence_proxy_async_smem();
@@ -371,21 +386,34 @@ tc_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
             if (wt < kW) w_s[kElems + wt] = __uint_as_float((uint32_t)braw << 16);
 
             // ---- accumulator rows out of TMEM -> fp32 rows in shared memory ----
-            // Row t (4 kW bytes) from the start of the V buffer on, through the Q buffer, which follows it;
-            // 16-byte chunk c at chunk c ^ (t & 7): conflict-free for these row-per-thread writes and for
+            // Row t, times 1 / max(||q_t||, eps), from the start of the V buffer on, through the Q buffer, which follows it.  ROOMY: rows
+            // of 16 bytes more; else 16-byte chunk c at chunk c ^ (t & 7): conflict-free for these row-per-thread writes and for
             // the reads below.  All UMMAs and all row-norm reads of those buffers are done:
             // o_done follows sp_ready, which every worker reaches after its reads of Q.
-            if (!mbar_wait(o_done, ph, abort_flag, prm.status, kBit)) break;
+            if (!mbar_wait(o_done, ph, abort_flag, prm.status, kBit) || !mbar_wait(sp_ready, ph, abort_flag, prm.status, kBit)) break;
             tcgen05_fence_after_sync();
-            for (int i = half; i < tiles * (kW / 16); i += kHalves) {
-                const int t = i / (kW / 16), cc = i % (kW / 16), r = t * kTile + quarter * 32 + lane;
-                float a[16];
-                tmem_ld16(tmem + ((uint32_t)(quarter * 32) << 16) + i * 16, a);
-                tmem_ld_wait();
-                uint8_t* srow = V_s + r * (kW * 4);
+            {
+                const uint32_t lanes = tmem + ((uint32_t)(quarter * 32) << 16);
+                const int n = tiles * (kW / 16);
+                auto write = [&](int i, const float (&a)[16]) {
+                    const int t = i / (kW / 16), cc = i % (kW / 16), r = t * kTile + quarter * 32 + lane;
+                    if (r >= N) return;
+                    const float rq = rq_s[r];
+                    uint8_t* srow = V_s + r * G::kAccRow;
 #pragma unroll
-                for (int e = 0; e < 4; ++e)
-                    *reinterpret_cast<float4*>(srow + (((cc * 4 + e) ^ (r & 7)) << 4)) = make_float4(a[4 * e], a[4 * e + 1], a[4 * e + 2], a[4 * e + 3]);
+                    for (int e = 0; e < 4; ++e)
+                        *reinterpret_cast<float4*>(srow + (((cc * 4 + e) ^ (ROOMY ? 0 : r & 7)) << 4)) =
+                            make_float4(a[4 * e] * rq, a[4 * e + 1] * rq, a[4 * e + 2] * rq, a[4 * e + 3] * rq);
+                };
+                for (int i = half; i < n; i += 2 * kHalves) {   // two loads under way
+                    float a[16], b[16];
+                    const bool two = i + kHalves < n;
+                    tmem_ld16(lanes + i * 16, a);
+                    if (two) tmem_ld16(lanes + (i + kHalves) * 16, b);
+                    tmem_ld_wait();
+                    write(i, a);
+                    if (two) write(i + kHalves, b);
+                }
             }
             tcgen05_fence_before_sync();
             mbar_arrive(tm_free);
@@ -399,7 +427,6 @@ tc_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
             // even and the odd columns of four.
             const int par = NARROW ? lane >> 4 : 0, cp = NARROW ? lane & 15 : lane;   // column parity, channel pair
             constexpr int STEP = NARROW ? 2 : 1, NIN = STEP + KS;
-            constexpr bool kEarly = WORKERS == 256;
             const float half = FINE ? 0.25f : 0.5f;   // FINE: the sums are of every token twice
             const float2 hs2 = make_float2(half * sum_s[2 * cp], half * sum_s[2 * cp + 1]);   // 1/2 s
             const float2 bias2 = *reinterpret_cast<const float2*>(w_s + kElems + 2 * cp);
@@ -409,20 +436,16 @@ tc_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
             for (int dy = 0; dy < KS; ++dy)
 #pragma unroll
                 for (int dx = 0; dx < KS; ++dx) wreg[dy][dx] = *reinterpret_cast<const float2*>(w_s + (dy * KS + dx) * kW + 2 * cp);
-            uint32_t* out_plane = reinterpret_cast<uint32_t*>(prm.out + plane_offset(prm.lo, bh, prm.hdiv)) + cp;
+            uint32_t* out_plane = reinterpret_cast<uint32_t*>(out_bh) + cp;
             const long long out_tok = OUT_PACKED ? kW / 2 : prm.lo.token / 2;  // 32-bit words per token
-            // token t: accumulator and scale, add, store
-            auto load_acc = [&](int t, float2& a2, float& rq) {
-                lds64(smem_u32(V_s) + (uint32_t)(t * (kW * 4) + (((cp >> 1) ^ (t & 7)) << 4) + (cp & 1) * 8), a2);
-                rq = __uint_as_float(lds32(smem_u32(rq_s) + (uint32_t)t * 4));
+            const uint32_t acc_s = smem_u32(V_s) + (ROOMY ? cp * 8 : 0);
+            auto load_acc = [&](int t, float2& a2) {   // of token t, scaled
+                lds64(acc_s + (uint32_t)(t * G::kAccRow + (ROOMY ? 0 : (((cp >> 1) ^ (t & 7)) << 4) + (cp & 1) * 8)), a2);
             };
-            auto emit = [&](uint32_t* to, float2 a2, float rq, float2 add) {
-                const float2 o = ffma2(a2, make_float2(rq, rq), add);
-                *to = pack_bf16x2(o.x, o.y);
-            };
+            const int pitch = ROOMY ? W + 2 * R : W;      // tokens of a row of V in the K buffer
             const uint32_t v_base = smem_u32(K_s) + cp * 4;
             for (int u = ww; u < n_units; u += kWarps) {
-                const int strip = u % n_strips, y_first = (u / n_strips) * seg_rows, n_rows = min(seg_rows, prm.gridH - y_first);
+                const int strip = u < kWarps ? first_strip : u % n_strips, y_first = (u < kWarps ? first_seg : u / n_strips) * seg_rows, n_rows = min(seg_rows, prm.gridH - y_first);
                 const int x0 = strip * 2 * STEP + par;    // grid column of the lane's first output; the next is x0 + STEP
                 const bool first = x0 < W, second = x0 + STEP < W;
                 uint32_t cmask[NIN];      // of the words that lie in the grid's columns
@@ -432,59 +455,75 @@ tc_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
 #pragma unroll
                 for (int k = 0; k < KS; ++k) acc[k][0] = acc[k][1] = zero2;
                 uint32_t raw[NIN], rmask = 0;   // the words of the next halo row, all ones if it lies in the grid
-                uint32_t v_row = v_base + (uint32_t)((prm.prefix + (y_first - R) * W + x0 - R) * kRow);
+                float2 next[2] = {zero2, zero2};   // the attention terms of the output row that starts with it
+                uint32_t v_row = v_base + (uint32_t)((ROOMY ? y_first * pitch + x0 : prm.prefix + (y_first - R) * W + x0 - R) * kRow);
+                const int t0 = prm.prefix + y_first * W + x0, t_last = t0 + (n_rows - 1) * W;   // tokens of the unit's first and last output row
+                int t = t0;                                // of the output row that starts with the next halo row
                 auto load_row = [&](int hy) {
-                    rmask = (unsigned)(y_first + hy - R) < (unsigned)prm.gridH ? 0xffffffffu : 0u;
-                    const uint32_t from = rmask ? v_row : v_base;
+                    uint32_t from = v_row;
+                    if (!ROOMY) {
+                        rmask = (unsigned)(y_first + hy - R) < (unsigned)prm.gridH ? 0xffffffffu : 0u;
+                        from = rmask ? v_row : v_base;
+                    }
 #pragma unroll
                     for (int o = 0; o < NIN; ++o) raw[o] = lds32(from + (uint32_t)(o * kRow));
-                    v_row += (uint32_t)(W * kRow);
+                    v_row += (uint32_t)(pitch * kRow);
+                    load_acc(t, next[0]);
+                    load_acc(t + STEP, next[1]);   // beyond the row it is some other token's
+                    t = min(t + W, t_last);        // no output row starts with the last halo rows
                 };
                 load_row(0);
-                int t = prm.prefix + (y_first - (KS - 1)) * W + x0;        // token of the row that ends with this halo row
-                uint32_t* to = out_plane + t * out_tok;
-                for (int h0 = 0; h0 < n_rows + KS - 1; h0 += KS) {
+                uint32_t* to = out_plane + (t0 - (KS - 1) * W) * out_tok;   // of the output row that ends with the halo row
+                const int last = n_rows + KS - 2;
+                // halo row hy of the unit: the output row that started dy rows ago, in slot (k - dy) % KS, takes filter row dy
+                auto row = [&](int hy, int k, bool ends) {
+                    float2 in[NIN];
 #pragma unroll
-                    for (int k = 0; k < KS; ++k) {
-                        const int hy = h0 + k;    // halo row of the unit
-                        if (hy >= n_rows + KS - 1) break;
-                        float2 in[NIN];
+                    for (int o = 0; o < NIN; ++o) {
+                        const uint32_t word = ROOMY ? raw[o] : raw[o] & cmask[o] & rmask;
+                        in[o] = make_float2(bf16lo(word), bf16hi(word));
+                    }
+                    // output row hy starts here; it ends KS - 1 rows on
+                    acc[k][0] = fadd2(next[0], c2);
+                    acc[k][1] = fadd2(next[1], c2);
+                    load_row(hy + 1);
 #pragma unroll
-                        for (int o = 0; o < NIN; ++o) {
-                            const uint32_t word = raw[o] & cmask[o] & rmask;
-                            in[o] = make_float2(bf16lo(word), bf16hi(word));
+                    for (int dx = 0; dx < KS; ++dx)
+#pragma unroll
+                        for (int dy = 0; dy < KS; ++dy)
+#pragma unroll
+                            for (int c = 0; c < 2; ++c)
+                                acc[(k - dy + KS) % KS][c] = ffma2_in_order(wreg[dy][dx], in[STEP * c + dx], acc[(k - dy + KS) % KS][c]);
+                    // predicates, no branches
+                    stg32_if(ends && first, to, pack_bf16x2(acc[(k + 1) % KS][0].x, acc[(k + 1) % KS][0].y));
+                    stg32_if(ends && second, to + STEP * out_tok, pack_bf16x2(acc[(k + 1) % KS][1].x, acc[(k + 1) % KS][1].y));
+                    to += W * out_tok;
+                };
+                if (NARROW && !FINE) {
+                    // one row of code and moving sums: units of width 32 have few rows.  1024 planes of 16 x 16 22.8 us, 25.5 unrolled; with 5 x 5
+                    // filters, 14 x 14, 29.8 / 31.9; width 64 (768 planes of 14 x 14) 28.8 / 28.1
+#pragma unroll 1
+                    for (int hy = 0; hy <= last; ++hy) {
+                        row(hy, KS - 1, hy >= KS - 1);
+#pragma unroll
+                        for (int j = 0; j + 1 < KS; ++j) { acc[j][0] = acc[j + 1][0]; acc[j][1] = acc[j + 1][1]; }
+                    }
+                } else {
+                    bool done = false;
+                    for (int h0 = 0; !done; h0 += KS) {
+#pragma unroll
+                        for (int k = 0; k < KS; ++k) {
+                            row(h0 + k, k, h0 > 0 || k == KS - 1);
+                            if (h0 + k == last) { done = true; break; }
                         }
-                        load_row(hy + 1);
-                        float2 a2[2];
-                        float rq[2];
-                        const bool ends = hy >= KS - 1;
-                        // of the outputs that end with this row (beyond the grid they are some other token's): ahead of the
-                        // FMAs where there are registers for it
-                        if (kEarly && ends) { load_acc(t, a2[0], rq[0]); load_acc(t + STEP, a2[1], rq[1]); }
-                        acc[k][0] = acc[k][1] = c2;   // output row hy starts here; it ends KS - 1 rows on
-#pragma unroll
-                        for (int dx = 0; dx < KS; ++dx)
-#pragma unroll
-                            for (int dy = 0; dy < KS; ++dy)
-#pragma unroll
-                                for (int c = 0; c < 2; ++c)
-                                    acc[(k - dy + KS) % KS][c] = ffma2(wreg[dy][dx], in[STEP * c + dx], acc[(k - dy + KS) % KS][c]);
-                        if (ends) {
-                            if (!kEarly) { load_acc(t, a2[0], rq[0]); load_acc(t + STEP, a2[1], rq[1]); }
-                            if (first) emit(to, a2[0], rq[0], acc[(k + 1) % KS][0]);
-                            if (second) emit(to + STEP * out_tok, a2[1], rq[1], acc[(k + 1) % KS][1]);
-                        }
-                        t += W;
-                        to += W * out_tok;
                     }
                 }
             }
             // off-grid leading tokens: the attention terms only
             for (int t = ww * STEP + par; t < prm.prefix; t += kWarps * STEP) {
                 float2 a2;
-                float rq;
-                load_acc(t, a2, rq);
-                emit(out_plane + t * out_tok, a2, rq, hs2);
+                load_acc(t, a2);
+                out_plane[t * out_tok] = pack_bf16x2(a2.x + hs2.x, a2.y + hs2.y);
             }
             fence_proxy_async_smem();
             mbar_arrive(plane_free);
@@ -495,9 +534,9 @@ tc_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     if (warp == 1) tmem_dealloc(tmem, G::kTmemCols);
 }
 
-template <int KS, bool NARROW, int WORKERS, bool FINE>
-cudaError_t launch_fused_ks(const Problem& p, unsigned* status, cudaStream_t st) {
-    using G = Geo<KS, NARROW, WORKERS>;
+template <int KS, bool NARROW, int WORKERS, bool FINE, bool ROOMY>
+cudaError_t launch_fused_room(const Problem& p, unsigned* status, cudaStream_t st) {
+    using G = Geo<KS, NARROW, WORKERS, ROOMY>;
     CUtensorMap tmK, tmV, tmQ, tmVplain;
     // [d, tokens, planes per batch step, batch steps]
     const uint64_t nb = (uint64_t)(p.BH / p.hdiv);
@@ -509,8 +548,17 @@ cudaError_t launch_fused_ks(const Problem& p, unsigned* status, cudaStream_t st)
     uint64_t sq[3], sk[3], sv[3];
     strides(p.lq, sq); strides(p.lk, sk); strides(p.lv, sv);
     if (!make_tensor_map_bf16(&tmK, p.k, 4, dims, sk, box, G::kRow) || !make_tensor_map_bf16(&tmV, p.v, 4, dims, sv, box, G::kRow) ||
-        !make_tensor_map_bf16(&tmQ, p.q, 4, dims, sq, box, G::kRow) || !make_tensor_map_bf16(&tmVplain, p.v, 4, dims, sv, box, 0))
+        !make_tensor_map_bf16(&tmQ, p.q, 4, dims, sq, box, G::kRow))
         return cudaErrorNotSupported;
+    if (ROOMY) {   // the token grid, after the off-grid leading tokens of every plane: what lies outside is zero-filled
+        const uint64_t dims_g[5] = {(uint64_t)G::kW, (uint64_t)p.gridW, (uint64_t)p.gridH, (uint64_t)p.hdiv, nb};
+        const uint64_t sg[4] = {sv[0], sv[0] * (uint64_t)p.gridW, sv[1], sv[2]};
+        const uint32_t box_g[5] = {(uint32_t)G::kW, (uint32_t)(p.gridW + KS - 1), (uint32_t)(p.gridH + KS - 1), 1, 1};
+        if (!make_tensor_map_bf16(&tmVplain, static_cast<const __nv_bfloat16*>(p.v) + p.prefix * p.lv.token, 5, dims_g, sg, box_g, 0))
+            return cudaErrorNotSupported;
+    } else if (!make_tensor_map_bf16(&tmVplain, p.v, 4, dims, sv, box, 0)) {
+        return cudaErrorNotSupported;
+    }
     FusedParams prm;
     prm.w = static_cast<const __nv_bfloat16*>(p.w);
     prm.bias = static_cast<const __nv_bfloat16*>(p.bias);
@@ -521,16 +569,24 @@ cudaError_t launch_fused_ks(const Problem& p, unsigned* status, cudaStream_t st)
     prm.eps2 = p.eps2; prm.status = status;
     static PerDevice opt_in[2];  // per instantiation
     const bool packed = (p.lo.token == G::kW);
-    const cudaError_t e = packed ? opt_in_smem(tc_fused_kernel<KS, true, NARROW, WORKERS, FINE>, G::kSmem, opt_in[1])
-                                 : opt_in_smem(tc_fused_kernel<KS, false, NARROW, WORKERS, FINE>, G::kSmem, opt_in[0]);
+    const cudaError_t e = packed ? opt_in_smem(tc_fused_kernel<KS, true, NARROW, WORKERS, FINE, ROOMY>, G::kSmem, opt_in[1])
+                                 : opt_in_smem(tc_fused_kernel<KS, false, NARROW, WORKERS, FINE, ROOMY>, G::kSmem, opt_in[0]);
     if (e != cudaSuccess) return e;
     const int resident = G::kCtas * device_sm_count();
     const int grid = p.BH < resident ? p.BH : resident;
     if (packed)
-        tc_fused_kernel<KS, true, NARROW, WORKERS, FINE><<<(unsigned)grid, G::kThreads, G::kSmem, st>>>(tmK, tmV, tmQ, tmVplain, prm);
+        tc_fused_kernel<KS, true, NARROW, WORKERS, FINE, ROOMY><<<(unsigned)grid, G::kThreads, G::kSmem, st>>>(tmK, tmV, tmQ, tmVplain, prm);
     else
-        tc_fused_kernel<KS, false, NARROW, WORKERS, FINE><<<(unsigned)grid, G::kThreads, G::kSmem, st>>>(tmK, tmV, tmQ, tmVplain, prm);
+        tc_fused_kernel<KS, false, NARROW, WORKERS, FINE, ROOMY><<<(unsigned)grid, G::kThreads, G::kSmem, st>>>(tmK, tmV, tmQ, tmVplain, prm);
     return cudaGetLastError();
+}
+
+template <int KS, bool NARROW, int WORKERS, bool FINE>
+cudaError_t launch_fused_ks(const Problem& p, unsigned* status, cudaStream_t st) {
+    using G = Geo<KS, NARROW, WORKERS, true>;
+    const bool roomy = (p.gridW + KS - 1) * (p.gridH + KS - 1) * G::kRow <= G::kBuf && p.gridW + KS - 1 <= 256 && p.gridH + KS - 1 <= 256 &&
+                       p.N * G::kAccRow <= 2 * G::kBuf;
+    return roomy ? launch_fused_room<KS, NARROW, WORKERS, FINE, true>(p, status, st) : launch_fused_room<KS, NARROW, WORKERS, FINE, false>(p, status, st);
 }
 
 template <int KS, bool NARROW, bool FINE>

@@ -94,15 +94,6 @@ __device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&r)[8])
 }
 __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
-__device__ __forceinline__ float2 fadd2(float2 a, float2 b) {
-    float2 d;
-    asm("{\n\t.reg .b64 ra, rb, rd;\n\t"
-        "mov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\t"
-        "add.rn.f32x2 rd, ra, rb;\n\t"
-        "mov.b64 {%0, %1}, rd;\n\t}"
-        : "=f"(d.x), "=f"(d.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
-    return d;
-}
 __device__ __forceinline__ float2 dup2(float x) { return make_float2(x, x); }
 __device__ __forceinline__ float sqrt_approx(float x) {
     float r;
@@ -113,16 +104,6 @@ __device__ __forceinline__ float exp2_approx(float x) {
     float r;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
-}
-__device__ __forceinline__ uint32_t hmul2_bf16(uint32_t a, uint32_t b) {
-    uint32_t d;
-    asm("mul.rn.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
-    return d;
-}
-__device__ __forceinline__ uint32_t hfma2_bf16(uint32_t a, uint32_t b, uint32_t c) {
-    uint32_t d;
-    asm("fma.rn.bf16x2 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
-    return d;
 }
 constexpr float kLog2e = 1.4426950408889634f;
 
@@ -424,8 +405,7 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     } else if (warp < 8) {
         // ---- unit rows ----
         const int t = tid - 128;
-        // Row t of a tile times r = factor / max(norm, eps), r as the sum of two bf16: x r_hi + (x r_lo), the product in brackets rounded,
-        // the rest in one rounding.  That is the rounding of x r itself but for 1 case in 256, where x r lies next to the middle between two bf16.
+        // row t of a tile times factor / max(norm, eps)
         auto scale_row = [&](uint8_t* row, float factor) {
             uint32_t w[32];
             float2 ss[4] = {dup2(0.f), dup2(0.f), dup2(0.f), dup2(0.f)};
@@ -440,14 +420,11 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                 }
             }
             const float2 sum = fadd2(fadd2(ss[0], ss[1]), fadd2(ss[2], ss[3]));
-            const float r = factor / sqrtf(fmaxf(sum.x + sum.y, prm.eps2));
-            const uint32_t hi = pack_bf16x2(r, r), lo = pack_bf16x2(r - bf16lo(hi), r - bf16lo(hi));
+            const Bf16Scale scale(factor / sqrtf(fmaxf(sum.x + sum.y, prm.eps2)));
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
-                uint32_t o[4];
-#pragma unroll
-                for (int e = 0; e < 4; ++e) o[e] = hfma2_bf16(w[4 * j + e], hi, hmul2_bf16(w[4 * j + e], lo));
-                *reinterpret_cast<uint4*>(row + ((j ^ (t & 7)) << 4)) = make_uint4(o[0], o[1], o[2], o[3]);
+                *reinterpret_cast<uint4*>(row + ((j ^ (t & 7)) << 4)) =
+                    make_uint4(scale(w[4 * j]), scale(w[4 * j + 1]), scale(w[4 * j + 2]), scale(w[4 * j + 3]));
             }
         };
         // The Q tiles of item i + 1 come after the first K tiles of item i: their copy starts once the cosines of item
