@@ -137,9 +137,13 @@ tc_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     __syncthreads();
     tcgen05_fence_after_sync();
     const uint32_t tmem = *tmem_slot;
+    // Launched programmatically dependent on whatever precedes it in the stream: all of the above ran while that kernel drained; the
+    // threads that touch global memory wait for it first.  The next forward may set itself up in the same way.
+    pdl_launch_dependents();
 
     if (warp == 0) {
         if (lane == 0) {
+            pdl_wait_primary();
             const uint64_t pol = l2_policy_evict_first();  // K and Q are read once
             int issued = 0, issued_vp = 0;
             for (int it = 0; it < n_planes; ++it) {
@@ -250,6 +254,7 @@ tc_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
             sa = (ss[0].x + ss[0].y) + (ss[1].x + ss[1].y);
             sb = (ss[2].x + ss[2].y) + (ss[3].x + ss[3].y);
         };
+        pdl_wait_primary();   // filters and output
         for (int it = 0; it < n_planes; ++it) {
             const uint32_t ph = it & 1;
             const int bh = blockIdx.x + it * gridDim.x;
@@ -574,11 +579,17 @@ cudaError_t launch_fused_room(const Problem& p, unsigned* status, cudaStream_t s
     if (e != cudaSuccess) return e;
     const int resident = G::kCtas * device_sm_count();
     const int grid = p.BH < resident ? p.BH : resident;
-    if (packed)
-        tc_fused_kernel<KS, true, NARROW, WORKERS, FINE, ROOMY><<<(unsigned)grid, G::kThreads, G::kSmem, st>>>(tmK, tmV, tmQ, tmVplain, prm);
-    else
-        tc_fused_kernel<KS, false, NARROW, WORKERS, FINE, ROOMY><<<(unsigned)grid, G::kThreads, G::kSmem, st>>>(tmK, tmV, tmQ, tmVplain, prm);
-    return cudaGetLastError();
+    // CTAs that start while the kernel before drains lie on the multiprocessors in the order in which these became free, not one by one in
+    // turn, so that some get more of the CTAs with a plane more than others.  Width 64 gains all the same; width 32, whose planes take
+    // the issue slots of a whole multiprocessor, where no CTA has a second plane.  From a graph, started early / not: 12 planes of 14 x 14,
+    // width 64, 6.4 / 7.4 us, 768 of 11 x 11 19.8 / 20.2, 768 of 14 x 14 28.5 / 28.1 (with a new output per call 29.4 / 30.7), 768 of
+    // 16 x 16 34.3 / 33.6; width 32, 256 of 14 x 14 6.8 / 7.9, 1024 of 16 x 16 24.1 / 22.8, 1024 of 16 x 32 44.0 / 40.0.  Planes handed out
+    // by a counter instead: 7.2 against 6.9 and 30.2 against 29.4 for the first and the third.
+    const bool early = !NARROW || grid == p.BH;
+    auto launch = [&](auto kernel) {
+        return launch_programmatic(kernel, early, dim3((unsigned)grid), dim3(G::kThreads), G::kSmem, st, tmK, tmV, tmQ, tmVplain, prm);
+    };
+    return packed ? launch(tc_fused_kernel<KS, true, NARROW, WORKERS, FINE, ROOMY>) : launch(tc_fused_kernel<KS, false, NARROW, WORKERS, FINE, ROOMY>);
 }
 
 template <int KS, bool NARROW, int WORKERS, bool FINE>

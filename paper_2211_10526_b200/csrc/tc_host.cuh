@@ -55,6 +55,18 @@ cudaError_t shard_state(const Problem& p, float* state_out, float* ws_partial, u
 cudaError_t shard_apply(const Problem& p, const float* state, unsigned* status, cudaStream_t stream, int* launches,
                         KernelTimer* timer);
 
+// Launch of a kernel that, if `early`, may start while the one before it in the stream drains (it waits for that itself).
+template <typename Kernel, typename... Args>
+inline cudaError_t launch_programmatic(Kernel kernel, bool early, dim3 grid, dim3 block, size_t smem, cudaStream_t st, const Args&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = early ? 1 : 0;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 // Launchers of the individual kernels (each in its own file).
 cudaError_t launch_state(const Problem& p, float* partial, float* final_state, unsigned* counters, int P,
                          int tiles_per_cta, unsigned* status, cudaStream_t st);
