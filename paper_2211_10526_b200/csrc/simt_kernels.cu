@@ -476,6 +476,13 @@ cudaError_t launch_simt(const Problem& p, float* ws_state, float* ws_partial, in
                         cudaStream_t stream, int* launches, KernelTimer* timer) {
     const int zsum = p.rownorm ? 1 : 0;
     const int words = D * D + D + (zsum ? D : 0);
+    if (f32_plane_supports(p)) {
+        const cudaError_t e = f32_plane_forward(p, stream);
+        if (e == cudaSuccess) *launches = 1;
+        if (e == cudaSuccess) timer->mark(stream, "f32_plane");
+        if (e != cudaErrorNotSupported) return e;
+        (void)cudaGetLastError();   // strides that the tensor maps cannot take
+    }
     if (!zsum && p.phase == kPhaseAll && p.N <= kFusedMaxTokens && p.BH >= kFusedMinPlanes &&
         simt_fused_smem<D>(p.N, p.ksize) <= kFusedSmemLimit) {
         const size_t smem = simt_fused_smem<D>(p.N, p.ksize);
