@@ -19,6 +19,9 @@ namespace castling {
 namespace {
 
 using tc::ffma2;
+using tc::cluster_arrive;
+using tc::cluster_wait;
+using tc::ld_peer;
 using tc::mbar_wait;
 
 constexpr int kThreads = 256;
@@ -43,17 +46,6 @@ struct F32PlaneParams {
     float eps2;
     unsigned* status;
 };
-
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
-// Four floats at the same place of another CTA's shared memory.
-__device__ __forceinline__ float4 ld_peer(const float* p, uint32_t rank) {
-    uint32_t at;
-    float4 v;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"(tc::smem_u32(p)), "r"(rank));
-    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(at) : "memory");
-    return v;
-}
 
 template <int D, int KS>
 __global__ void __launch_bounds__(kThreads, D == 32 ? 2 : 1)
@@ -204,9 +196,9 @@ f32_plane_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
         if (prm.bands > 1) { cluster_arrive(); cluster_wait(); } else { __syncthreads(); }
         for (int i = tid * 4; i < D * D + D; i += kThreads * 4) {
             const float* at = i < D * D ? k_s + i : smem + G::kOffSum + i - D * D;
-            float4 s = prm.bands > 1 ? ld_peer(at, 0) : *reinterpret_cast<const float4*>(at);
+            float4 s = prm.bands > 1 ? ld_peer(reinterpret_cast<const float4*>(at), 0) : *reinterpret_cast<const float4*>(at);
             for (int p = 1; p < prm.bands; ++p) {
-                const float4 x = ld_peer(at, p);
+                const float4 x = ld_peer(reinterpret_cast<const float4*>(at), p);
                 s.x += x.x; s.y += x.y; s.z += x.z; s.w += x.w;
             }
             const float f = i < D * D ? kInvPi : 0.5f;

@@ -440,5 +440,17 @@ __device__ __forceinline__ void stg32_if(bool store, uint32_t* p, uint32_t v) {
         ::"l"(p), "r"(v), "r"((uint32_t)store) : "memory");
 }
 
+// ---- clusters -------------------------------------------------------------------------
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+// Four floats at the same place of another CTA's shared memory.
+__device__ __forceinline__ float4 ld_peer(const float4* p, uint32_t rank) {
+    uint32_t at;
+    float4 v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"(smem_u32(p)), "r"(rank));
+    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(at) : "memory");
+    return v;
+}
+
 }  // namespace tc
 }  // namespace castling

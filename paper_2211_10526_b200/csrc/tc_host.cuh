@@ -39,6 +39,8 @@ inline int state_words_of(const Problem& p) { return p.rownorm ? kStateWordsRown
 
 // Token splits of the tensor-core state kernel and the workspace words it needs beyond the state.
 int choose_splits(int BH, int N);
+// The splits of a plane are one cluster, whose CTAs add their states through distributed shared memory.
+bool splits_in_cluster(int BH, int P);
 
 // Enqueue state build, split reduction and apply for one problem.  `status` is the device status
 // word; `counters` holds kCountersPerHead zero-initialised arrival counters per (b,h), left at zero by every call.  Returns the cudaError_t of the launches; cudaErrorNotSupported if a tensor map could not

@@ -44,7 +44,7 @@ template <bool NARROW, bool RN, bool FINE>
 __global__ void __launch_bounds__(kThreads, 2)
 tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
                 float* __restrict__ dst, float* __restrict__ final_state, unsigned* __restrict__ counters,
-                int N, int tiles_per_cta, int P, int BH, int hdiv, int items_per_cta, float eps2, unsigned* status) {
+                int N, int tiles_per_cta, int P, int clustered, int BH, int hdiv, int items_per_cta, float eps2, unsigned* status) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = align_smem(smem_raw);
     constexpr int kStages = FINE ? kFineStages : castling::tc::kStages, kStageBytes = FINE ? kFineStageBytes : castling::tc::kStageBytes;
@@ -191,7 +191,8 @@ tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
             if (!mbar_wait_warp(&accum[buf], (item >> 1) & 1, abort_flag, status, kStatusStateTimeout)) return false;
             tcgen05_fence_after_sync();
             if (quarter < 3) {
-                float* out = dst + ((size_t)(bh0 + item) * P + p) * kStateW;
+                // a cluster's partial state stays in shared memory, over the stages, which the UMMAs have read
+                float* out = clustered ? reinterpret_cast<float*>(smem) : dst + ((size_t)(bh0 + item) * P + p) * kStateW;
                 // M = 64 keeps rows 16 q .. 16 q + 15 in lanes 32 q .. 32 q + 15
                 const int row = NARROW ? (lane < 16 ? quarter * 16 + lane : kW + 1) : quarter * 32 + lane;
 #pragma unroll
@@ -268,6 +269,25 @@ tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     tcgen05_fence_before_sync();
     __syncthreads();  // every thread's part of this split's partial state has been stored
     if (warp == 1) tmem_dealloc(tmem, RN ? 2 * kTmemCols : kTmemCols);
+
+    if (clustered) {   // the splits of a (b,h) are one cluster: each CTA adds its share of the words, in the splits' order
+        constexpr int kWords4 = kStateW / 4;
+        const int share = (kWords4 + P - 1) / P, end = min(kWords4, (p + 1) * share);
+        cluster_arrive();
+        cluster_wait();
+        for (int i = p * share + tid; i < end; i += kThreads) {
+            const float4* at = reinterpret_cast<const float4*>(smem) + i;
+            float4 sum = ld_peer(at, 0);
+            for (int m = 1; m < P; ++m) {
+                const float4 x = ld_peer(at, m);
+                sum.x += x.x; sum.y += x.y; sum.z += x.z; sum.w += x.w;
+            }
+            reinterpret_cast<float4*>(final_state + (size_t)bh * kStateW)[i] = sum;
+        }
+        cluster_arrive();   // this partial state has been read
+        cluster_wait();
+        return;
+    }
 
     // Cross-split reduction without a second launch and without any waiting, as a two-level tree
     // driven by arrival counters: the splits of a (b,h) form groups of kGroup; the CTA that arrives
@@ -396,14 +416,17 @@ cudaError_t launch_state(const Problem& p, float* partial, float* final_state, u
     }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = kSmemBytes; cfg.stream = st;
-    cudaLaunchAttribute attr[1];
+    const int clustered = splits_in_cluster(p.BH, P) ? 1 : 0;
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr; cfg.numAttrs = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)P; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr; cfg.numAttrs = clustered ? 2 : 1;
     auto launch = [&](auto kernel) {
         const cudaError_t e = opt_in_smem(kernel, kSmemBytes, opt_in[(p.fine ? 4 : narrow ? 2 : 0) + (p.rownorm ? 1 : 0)]);
         if (e != cudaSuccess) return e;
-        return cudaLaunchKernelEx(&cfg, kernel, tmK, tmV, dst, final_state, counters, p.N, tiles_per_cta, P, p.BH, p.hdiv, items,
+        return cudaLaunchKernelEx(&cfg, kernel, tmK, tmV, dst, final_state, counters, p.N, tiles_per_cta, P, clustered, p.BH, p.hdiv, items,
                                   p.eps2, status);
     };
     if (p.fine) return p.rownorm ? launch(tc_state_kernel<true, true, true>) : launch(tc_state_kernel<true, false, true>);
