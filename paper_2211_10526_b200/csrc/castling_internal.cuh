@@ -141,9 +141,9 @@ bool f32_thin(const Problem& p);
 int f32_choose_splits(int BH, int N);
 cudaError_t f32_forward(const Problem& p, float* ws_state, float* ws_partial, int P, cudaStream_t stream, int* launches,
                         KernelTimer* timer);
-// Whole fp32 forward of short planes in one kernel (csrc/f32_planes.cu).
+// fp32 forward of short planes, one kernel or two (csrc/f32_planes.cu).
 bool f32_plane_supports(const Problem& p);
-cudaError_t f32_plane_forward(const Problem& p, cudaStream_t stream);
+cudaError_t f32_plane_forward(const Problem& p, float* state, cudaStream_t stream, int* launches, KernelTimer* timer);
 // Explicit-weights forward (csrc/quad_kernels.cu): exact kernel and / or masked softmax branch; O(N^2 d).
 cudaError_t quad_forward(const Problem& p, cudaStream_t stream, int* launches, KernelTimer* timer);
 bool simt_supports(int d, int ksize);

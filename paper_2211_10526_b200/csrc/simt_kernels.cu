@@ -477,9 +477,7 @@ cudaError_t launch_simt(const Problem& p, float* ws_state, float* ws_partial, in
     const int zsum = p.rownorm ? 1 : 0;
     const int words = D * D + D + (zsum ? D : 0);
     if (f32_plane_supports(p)) {
-        const cudaError_t e = f32_plane_forward(p, stream);
-        if (e == cudaSuccess) *launches = 1;
-        if (e == cudaSuccess) timer->mark(stream, "f32_plane");
+        const cudaError_t e = f32_plane_forward(p, ws_state, stream, launches, timer);
         if (e != cudaErrorNotSupported) return e;
         (void)cudaGetLastError();   // strides that the tensor maps cannot take
     }
