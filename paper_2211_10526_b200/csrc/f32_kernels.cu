@@ -55,7 +55,7 @@ f32_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
     const int tid = threadIdx.x, p = blockIdx.x % P, bh = blockIdx.x / P;
     const int n_begin = p * chunk, n_end = min(N, n_begin + chunk);
     const int pb = bh / hdiv, ph = bh - pb * hdiv;
-    // scaling: thread = 16-byte chunk lc of rows lr, lr + kRowsPass, ...
+    // sums over tokens: thread = 16-byte chunk lc of rows lr, lr + kRowsPass, ...
     const int lc = tid % G::kChunks, lr = tid / G::kChunks;
     float4 vsum = make_float4(0.f, 0.f, 0.f, 0.f), ksum = vsum;
     auto load = [&](int n0, int buf) {   // rows beyond N arrive as zeros
@@ -64,20 +64,23 @@ f32_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
         tc::tma_load_4d(ks, &tmK, &full[buf], 0, n0, ph, pb);
         tc::tma_load_4d(ks + kTok * D, &tmV, &full[buf], 0, n0, ph, pb);
     };
-    auto scale_k = [&](int buf) {   // unit rows, in place
-        float* ks = smem + 2 * buf * (kTok * D);
+    auto scale_k = [&](int buf) {   // unit rows, in place; two or four lanes per row, neighbouring rows from different chunks on (banks)
+        constexpr int L = kThreads / kTok, kPer = G::kChunks / L;
+        const int row = tid / L, l = tid % L;
+        float* ks = smem + 2 * buf * (kTok * D) + row * D;
+        float4 x[kPer];
+        float ss = 0.f;
 #pragma unroll
-        for (int r = 0; r < G::kPasses; ++r) {
-            float4* at = reinterpret_cast<float4*>(ks + (lr + r * G::kRowsPass) * D + lc * 4);
-            float4 x = *at;
-            float ss = fmaf(x.x, x.x, fmaf(x.y, x.y, fmaf(x.z, x.z, x.w * x.w)));
-#pragma unroll
-            for (int o = G::kChunks / 2; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-            const float rk = 1.0f / sqrtf(fmaxf(ss, eps2));
-            x.x *= rk; x.y *= rk; x.z *= rk; x.w *= rk;
-            if (RN) { ksum.x += x.x; ksum.y += x.y; ksum.z += x.z; ksum.w += x.w; }
-            *at = x;
+        for (int i = 0; i < kPer; ++i) {
+            x[i] = *reinterpret_cast<const float4*>(ks + (l + L * ((i + row) % kPer)) * 4);
+            ss = fmaf(x[i].x, x[i].x, fmaf(x[i].y, x[i].y, fmaf(x[i].z, x[i].z, fmaf(x[i].w, x[i].w, ss))));
         }
+#pragma unroll
+        for (int o = L / 2; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+        const float rk = inv_sqrt(fmaxf(ss, eps2));
+#pragma unroll
+        for (int i = 0; i < kPer; ++i)
+            *reinterpret_cast<float4*>(ks + (l + L * ((i + row) % kPer)) * 4) = make_float4(x[i].x * rk, x[i].y * rk, x[i].z * rk, x[i].w * rk);
     };
     // computing: group g takes tokens g, g + G, ...; a thread owns rows 8 ti .. and columns {4 tj .., D/2 + 4 tj ..} of S
     const int g = tid / G::kGroup, t = tid % G::kGroup, ti = t / G::kSide, tj = t % G::kSide;
@@ -127,6 +130,10 @@ f32_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
         for (int r = 0; r < G::kPasses; ++r) {
             const float4 x = *reinterpret_cast<const float4*>(vs + (lr + r * G::kRowsPass) * D + lc * 4);
             vsum.x += x.x; vsum.y += x.y; vsum.z += x.z; vsum.w += x.w;
+            if (RN) {
+                const float4 z = *reinterpret_cast<const float4*>(ks + (lr + r * G::kRowsPass) * D + lc * 4);
+                ksum.x += z.x; ksum.y += z.y; ksum.z += z.z; ksum.w += z.w;
+            }
         }
     }
     if (tid == 0 && *abort_flag) {   // giving up: let the copies in flight land before their place is used
@@ -317,7 +324,7 @@ f32_apply_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
                 if (RN) dot += __shfl_xor_sync(0xffffffffu, dot, o);
             }
             if (l == 0) {
-                const float rq = 1.0f / sqrtf(fmaxf(ss, prm.eps2));
+                const float rq = inv_sqrt(fmaxf(ss, prm.eps2));
                 smem[G::kOffRq + r] = rq;
                 // Eq. 3's denominator for the kept kernel of Eq. 8: N/2 + q^ . (sum_j k^_j) / pi
                 if (RN) smem[G::kOffDen + r] = 1.0f / fmaf(dot * rq, kInvPi, 0.5f * (float)(prm.prefix + prm.gridH * W));

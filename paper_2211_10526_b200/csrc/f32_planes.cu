@@ -121,7 +121,7 @@ f32_plane_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 const int r = r0 + u * G::kRowsPass + lr;
-                const float f1 = 1.0f / sqrtf(fmaxf(ss[u], prm.eps2));
+                const float f1 = inv_sqrt(fmaxf(ss[u], prm.eps2));
                 if (r < N) f(r, x[u], f1);
             }
         }
