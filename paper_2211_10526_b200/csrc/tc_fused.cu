@@ -137,13 +137,14 @@ tc_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     __syncthreads();
     tcgen05_fence_after_sync();
     const uint32_t tmem = *tmem_slot;
-    // Launched programmatically dependent on whatever precedes it in the stream: all of the above ran while that kernel drained; the
-    // threads that touch global memory wait for it first.  The next forward may set itself up in the same way.
+    // Launched programmatically dependent on whatever precedes it in the stream: all of the above ran while that kernel drained.  Every
+    // thread waits for it here, also those that touch no memory: the limits of their waits are for this kernel's own work.  The next
+    // forward may set itself up in the same way.
     pdl_launch_dependents();
+    pdl_wait_primary();
 
     if (warp == 0) {
         if (lane == 0) {
-            pdl_wait_primary();
             const uint64_t pol = l2_policy_evict_first();  // K and Q are read once
             int issued = 0, issued_vp = 0;
             for (int it = 0; it < n_planes; ++it) {
@@ -254,7 +255,6 @@ tc_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
             sa = (ss[0].x + ss[0].y) + (ss[1].x + ss[1].y);
             sb = (ss[2].x + ss[2].y) + (ss[3].x + ss[3].y);
         };
-        pdl_wait_primary();   // filters and output
         for (int it = 0; it < n_planes; ++it) {
             const uint32_t ph = it & 1;
             const int bh = blockIdx.x + it * gridDim.x;

@@ -241,12 +241,13 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     __syncthreads();
     tcgen05_fence_after_sync();
     const uint32_t tmem = *tmem_slot;
-    // Launched programmatically dependent on whatever precedes it in the stream; the threads that touch global memory wait for it.
+    // Launched programmatically dependent on whatever precedes it in the stream, which every thread waits for here: the limits of the
+    // waits below are for this kernel's own work.
     pdl_launch_dependents();
+    pdl_wait_primary();
 
     if (warp == 0) {
         if (lane == 0) {
-            pdl_wait_primary();
             // independent rings, polled in turn: none waits behind another
             int qi = 0, ki = 0, kj = 0, vi = 0, vj = 0;   // next item (and tile of it) of each ring
             int pi = 0, pj = 0;                           // next item (and patch of it) of the convolution
@@ -578,7 +579,6 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
         int prev_head = -1, o_uses = 0, patch = 0;
         bool ok = true;
         const int W = prm.gridW;
-        pdl_wait_primary();   // filters and output
         for (int i = 0; i < my_items; ++i) {
             const Item im = item_of(i);
             const int head = (prm.head0 + im.bh) % prm.H;

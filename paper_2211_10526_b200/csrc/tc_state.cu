@@ -111,6 +111,10 @@ tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     __syncthreads();
     tcgen05_fence_after_sync();
     const uint32_t tmem = *tmem_slot;
+    // Launched programmatically dependent on the kernel before it in the stream (which may let its dependents start long before it
+    // ends): everything above ran while that kernel drained.  Every thread waits for it here; the limits of the waits below are for this
+    // kernel's own work.  Global memory is first touched after this.
+    pdl_wait_primary();
 
     if (warp == 0) {
         if (lane == 0) {
@@ -120,11 +124,6 @@ tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
             // of both kernels (measured: 132 -> 125 us per forward at 2 x 8 planes of 256 x 256 tokens).
             const uint64_t pol_k = l2_policy_evict_first(), pol_v = l2_policy_evict_first();
             bool ok = true;
-            // Launched programmatically dependent on the kernel before it in the stream (the apply kernel of the
-            // previous forward lets its dependents start early): everything above ran while that kernel drained.
-            // Global memory is first touched here; the partial states and arrival counters are written only after
-            // these loads have landed.
-            pdl_wait_primary();
             // Only now may the apply kernel begin its prologue: it loads Q and V, which may be the output of the kernel
             // this grid has just waited for, as soon as it runs.
             pdl_launch_dependents();
