@@ -410,27 +410,6 @@ __device__ __forceinline__ float2 fadd2(float2 a, float2 b) {
     return d;
 }
 
-__device__ __forceinline__ uint32_t hmul2_bf16(uint32_t a, uint32_t b) {
-    uint32_t d;
-    asm("mul.rn.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
-    return d;
-}
-__device__ __forceinline__ uint32_t hfma2_bf16(uint32_t a, uint32_t b, uint32_t c) {
-    uint32_t d;
-    asm("fma.rn.bf16x2 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
-    return d;
-}
-// Pairs of bf16 times r, r as the sum of two bf16: x r_hi + (x r_lo), the product in brackets rounded, the rest in one rounding.
-// That is the rounding of x r itself but for 1 case in 256, where x r lies next to the middle between two bf16.
-struct Bf16Scale {
-    uint32_t hi, lo;
-    __device__ __forceinline__ explicit Bf16Scale(float r) {
-        hi = pack_bf16x2(r, r);
-        lo = pack_bf16x2(r - bf16lo(hi), r - bf16lo(hi));
-    }
-    __device__ __forceinline__ uint32_t operator()(uint32_t x) const { return hfma2_bf16(x, hi, hmul2_bf16(x, lo)); }
-};
-
 // A word to global memory if `store` says so, as a predicated instruction.
 __device__ __forceinline__ void stg32_if(bool store, uint32_t* p, uint32_t v) {
     asm volatile(

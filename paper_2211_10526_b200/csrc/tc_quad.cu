@@ -21,9 +21,9 @@
 // cosine buffer (first contraction, weights, second contraction), of which tensor memory has room for three.  2 x 8 planes of 64 x 64
 // tokens, exact kernel: 119 us; in working copies 97 with cosines written back as they are, 76 with rows left as they are as well: what
 // the weights and the rows take comes on top of the chain, which waits for tensor memory and barriers.  So a weight has no square root where the cosines
-// of a step are small (127 us with the old scaling of rows and 5 packed operations a pair, 135.5 with the square roots, whose unit has 16 lanes), and a row
-// is read once and scaled by two packed bf16 operations a word instead of two conversions, a product and a rounding (127 -> 119 together
-// with one operation less a pair).  K scaled by the weight warps instead (its norms beside it, cosines not before a packed product): 133 against 127, as
+// of a step are small (127 us with 5 packed operations a pair, 135.5 with the square roots, whose unit has 16 lanes; 119 with one operation less a
+// pair and rows scaled by a refined reciprocal root, 121.4 with a root and a quotient).  Rows are scaled in fp32 with one rounding, as they are
+// everywhere.  K scaled by the weight warps instead (its norms beside it, cosines not before a packed product): 133 against 127, as
 // sixteen warps pay for what four did.  Four K stages, the convolution staged for one slot at a time: 117 against 119, but the masked branch 66 against 62.
 // The two contractions have an issuing warp each: a ready wait costs 50 to 90 cycles and an issue 30 per UMMA, which one warp could not do in time.
 // Eight weight warps instead of sixteen (with square roots): 151 us against 135; all sixteen on one slot at a time: 139.
@@ -409,26 +409,33 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     } else if (warp < 8) {
         // ---- unit rows ----
         const int t = tid - 128;
-        // row t of a tile times factor / max(norm, eps)
+        // row t of a tile times factor / max(norm, eps); read twice: the whole row does not fit beside the rest
         auto scale_row = [&](uint8_t* row, float factor) {
-            uint32_t w[32];
+            auto chunk = [&](int j) { return reinterpret_cast<uint4*>(row + ((j ^ (t & 7)) << 4)); };
             float2 ss[4] = {dup2(0.f), dup2(0.f), dup2(0.f), dup2(0.f)};
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
-                const uint4 c = *reinterpret_cast<const uint4*>(row + ((j ^ (t & 7)) << 4));
-                w[4 * j] = c.x; w[4 * j + 1] = c.y; w[4 * j + 2] = c.z; w[4 * j + 3] = c.w;
+                const uint4 c = *chunk(j);
+                const uint32_t w[4] = {c.x, c.y, c.z, c.w};
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
-                    const float2 p = make_float2(bf16lo(w[4 * j + e]), bf16hi(w[4 * j + e]));
+                    const float2 p = make_float2(bf16lo(w[e]), bf16hi(w[e]));
                     ss[e] = ffma2(p, p, ss[e]);
                 }
             }
             const float2 sum = fadd2(fadd2(ss[0], ss[1]), fadd2(ss[2], ss[3]));
-            const Bf16Scale scale(factor / sqrtf(fmaxf(sum.x + sum.y, prm.eps2)));
-#pragma unroll
+            const float2 rk2 = dup2(factor * inv_sqrt(fmaxf(sum.x + sum.y, prm.eps2)));
+#pragma unroll 4
             for (int j = 0; j < 8; ++j) {
-                *reinterpret_cast<uint4*>(row + ((j ^ (t & 7)) << 4)) =
-                    make_uint4(scale(w[4 * j]), scale(w[4 * j + 1]), scale(w[4 * j + 2]), scale(w[4 * j + 3]));
+                const uint4 c = *chunk(j);
+                const uint32_t w[4] = {c.x, c.y, c.z, c.w};
+                uint32_t o[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const float2 p = ffma2(make_float2(bf16lo(w[e]), bf16hi(w[e])), rk2, dup2(0.f));
+                    o[e] = pack_bf16x2(p.x, p.y);
+                }
+                *chunk(j) = make_uint4(o[0], o[1], o[2], o[3]);
             }
         };
         // The Q tiles of item i + 1 come after the first K tiles of item i: their copy starts once the cosines of item

@@ -32,8 +32,9 @@ constexpr int kStagesBytes = kStages * kStageBytes;
 static_assert(kFineStages * kFineStageBytes == kStagesBytes, "one size of shared memory");
 constexpr size_t kSmemBytes = 1024 + kStagesBytes + kOnesBytes + 256;
 
-// Rows are scaled by two packed bf16 operations a word (FINE: in fp32, for the rest): 16 planes of 64 x 64 20.2 -> 19.9 us a forward, 64 of
-// 50 x 75, width 32, 33.2 -> 33.0, both from a graph.
+// Rows are scaled in fp32, with one rounding to bf16; the factor as two bf16, packed bf16 operations, rounds one element in 1 300 another way and gains
+// 0.1 us.  Sums and products in pairs and a refined reciprocal root instead of a root and a quotient, us per forward from a graph: 16 planes of 64 x 64
+// 18.2 -> 17.9, of 128 x 128 42.9 -> 42.3, 64 of 50 x 75, width 32, 33.4 -> 33.1.
 // NARROW serves width-32 heads: rows of 64 bytes, 64-byte swizzle, 256 tokens per stage (any grid width, any number of
 // tokens), UMMAs of M = 64 (32 key features, then the row of ones) and N = 32, states of 32 x 32 + 32 words.  Two tokens
 // packed to a 128-byte row instead, which wastes half of the contraction and needs an even grid width, took 19.8 us against
@@ -239,24 +240,18 @@ tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
                     }
                 }
                 const float ssa = (sq[0].x + sq[0].y) + (sq[1].x + sq[1].y), ssb = (sq[2].x + sq[2].y) + (sq[3].x + sq[3].y);
-                const float rka = rsqrtf(fmaxf(NARROW ? ssa : ssa + ssb, eps2)), rkb = NARROW ? rsqrtf(fmaxf(ssb, eps2)) : rka;
-                const Bf16Scale fa(rka), fb(rkb);
+                const float rka = inv_sqrt(fmaxf(NARROW ? ssa : ssa + ssb, eps2)), rkb = NARROW ? inv_sqrt(fmaxf(ssb, eps2)) : rka;
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
-                    uint4 o;
-                    if (FINE) {
-                        const float rk = j < 4 ? rka : rkb;
-                        o.x = pack_bf16x2(bf16lo(c[j].x) * rk, bf16hi(c[j].x) * rk);
-                        o.y = pack_bf16x2(bf16lo(c[j].y) * rk, bf16hi(c[j].y) * rk);
-                        o.z = pack_bf16x2(bf16lo(c[j].z) * rk, bf16hi(c[j].z) * rk);
-                        o.w = pack_bf16x2(bf16lo(c[j].w) * rk, bf16hi(c[j].w) * rk);
-                        *reinterpret_cast<uint4*>(row + 2 * kTileBytes + ((j ^ (t & 7)) << 4)) =
-                            make_uint4(rest_bf16x2(c[j].x, rk, o.x), rest_bf16x2(c[j].y, rk, o.y), rest_bf16x2(c[j].z, rk, o.z), rest_bf16x2(c[j].w, rk, o.w));
-                    } else {
-                        const Bf16Scale& f = j < 4 ? fa : fb;
-                        o = make_uint4(f(c[j].x), f(c[j].y), f(c[j].z), f(c[j].w));
-                    }
+                    const float rk = j < 4 ? rka : rkb;
+                    auto times_rk = [&](uint32_t w) {
+                        const float2 x = ffma2(make_float2(bf16lo(w), bf16hi(w)), make_float2(rk, rk), zero2);
+                        return pack_bf16x2(x.x, x.y);
+                    };
+                    const uint4 o = make_uint4(times_rk(c[j].x), times_rk(c[j].y), times_rk(c[j].z), times_rk(c[j].w));
                     *reinterpret_cast<uint4*>(row + ((j ^ (t & 7)) << 4)) = o;
+                    if (FINE) *reinterpret_cast<uint4*>(row + 2 * kTileBytes + ((j ^ (t & 7)) << 4)) =
+                        make_uint4(rest_bf16x2(c[j].x, rk, o.x), rest_bf16x2(c[j].y, rk, o.y), rest_bf16x2(c[j].z, rk, o.z), rest_bf16x2(c[j].w, rk, o.w));
                 }
                 fence_proxy_async_smem();
                 mbar_arrive(&scaled[s]);
