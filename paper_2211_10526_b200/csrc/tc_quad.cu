@@ -27,8 +27,9 @@
 // sixteen warps pay for what four did.  Four K stages, the convolution staged for one slot at a time: 117 against 119, but the masked branch 66 against 62.
 // The two contractions have an issuing warp each: a ready wait costs 50 to 90 cycles and an issue 30 per UMMA, which one warp could not do in time.
 // Eight weight warps instead of sixteen (with square roots): 151 us against 135; all sixteen on one slot at a time: 139.
-// Masked branch, 64 x 12 planes of 14 x 14: 57 us.  62 with the cosines clamped and turned into exponents pair by pair, in both
-// sweeps, and the keys that pad a tile left out one by one; now the rows of Q bring the factor log2(e) along, and the padding's ones are taken off the sum.
+// Masked branch, 64 x 12 planes of 14 x 14: 56.2 us.  61 with the cosines clamped pair by pair in both sweeps, and the keys that pad a tile left
+// out one by one; now the padding's ones are taken off the sum.  Rows of Q that bring the factor log2(e) along to the contraction save 0.2 us, but
+// round it to bf16 with them.
 // No workspace; every wait is bounded.
 #include "tc_common.cuh"
 #include "tc_host.cuh"
@@ -189,9 +190,6 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     const int my_items = ((int)blockIdx.x < prm.n_items) ? (prm.n_items - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
     const int T = prm.k_tiles, N = prm.N;
     constexpr int kSweeps = SPARSE ? 2 : 1;
-    // Mask alone: the rows of Q have the length log2(e), so that the first contraction gives the exponents of exp2.  What pads a
-    // tile then still counts as exp2(0) = 1.
-    constexpr float kUnitQ = SPARSE && !EXACT ? kLog2e : 1.0f;
     const bool resident = SPARSE && T <= kResident;
     const int k_loads = resident ? T : kSweeps * T;   // K tiles loaded per item
     constexpr unsigned kBit = kStatusFusedTimeout;
@@ -409,8 +407,8 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     } else if (warp < 8) {
         // ---- unit rows ----
         const int t = tid - 128;
-        // row t of a tile times factor / max(norm, eps); read twice: the whole row does not fit beside the rest
-        auto scale_row = [&](uint8_t* row, float factor) {
+        // row t of a tile times 1 / max(norm, eps); read twice: the whole row does not fit beside the rest
+        auto scale_row = [&](uint8_t* row) {
             auto chunk = [&](int j) { return reinterpret_cast<uint4*>(row + ((j ^ (t & 7)) << 4)); };
             float2 ss[4] = {dup2(0.f), dup2(0.f), dup2(0.f), dup2(0.f)};
 #pragma unroll
@@ -424,7 +422,7 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                 }
             }
             const float2 sum = fadd2(fadd2(ss[0], ss[1]), fadd2(ss[2], ss[3]));
-            const float2 rk2 = dup2(factor * inv_sqrt(fmaxf(sum.x + sum.y, prm.eps2)));
+            const float2 rk2 = dup2(inv_sqrt(fmaxf(sum.x + sum.y, prm.eps2)));
 #pragma unroll 4
             for (int j = 0; j < 8; ++j) {
                 const uint4 c = *chunk(j);
@@ -443,7 +441,7 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
         auto scale_q = [&](int i) -> bool {
             if (!warp_wait(&q_full[i & 1], (i >> 1) & 1)) return false;
             const int slots = item_of(i).slots;
-            for (int s = 0; s < slots; ++s) scale_row(Q_s + (2 * (i & 1) + s) * kTileBytes + t * 128, kUnitQ);
+            for (int s = 0; s < slots; ++s) scale_row(Q_s + (2 * (i & 1) + s) * kTileBytes + t * 128);
             fence_proxy_async_smem();
             warp_arrive(&q_ready[i & 1]);
             return true;
@@ -455,7 +453,7 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
         for (int i = 0; i < my_items && ok; ++i) {
             for (int j = 0; j < k_loads; ++j) {
                 if (!(ok = warp_wait(&k_full[ks], k_par))) break;
-                scale_row(K_s + ks * kTileBytes + t * 128, 1.0f);
+                scale_row(K_s + ks * kTileBytes + t * 128);
                 fence_proxy_async_smem();
                 warp_arrive(&k_scaled[ks]);
                 if (++ks == kKStages) { ks = 0; k_par ^= 1; }
@@ -499,7 +497,7 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
 #pragma unroll
                             for (int e = 0; e < 16; e += 2) {
                                 const float* xe = &x[cc & 1][e];
-                                const float2 a = EXACT ? exponent2(make_float2(xe[0], xe[1]), -kLog2e) : make_float2(xe[0], xe[1]);
+                                const float2 a = EXACT ? exponent2(make_float2(xe[0], xe[1]), -kLog2e) : ffma2(make_float2(xe[0], xe[1]), dup2(kLog2e), dup2(0.f));
                                 den = fadd2(den, make_float2(exp2_approx(a.x), exp2_approx(a.y)));
                             }
                         }
@@ -541,8 +539,8 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                                         if (EXACT) {
                                             a = exponent2(xe, ebias);
                                         } else {
-                                            wv = ffma2(xe, dup2(kInvPi / kLog2e), dup2(0.5f));   // 1/2 + x / pi
-                                            a = fadd2(xe, dup2(ebias));
+                                            wv = ffma2(xe, dup2(kInvPi), dup2(0.5f));   // 1/2 + x / pi
+                                            a = ffma2(xe, dup2(kLog2e), dup2(ebias));
                                         }
                                         const float2 p = make_float2(exp2_approx(a.x), exp2_approx(a.y));
                                         // masked by a factor of 1 or 0: a pair takes three instructions, a predicate and an addition each four
