@@ -549,8 +549,9 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                                     o[e] = pack_bf16x2(wv.x, wv.y);
                                 }
                             };
-                            weigh(std::bool_constant<EXACT>{});
-                            if (EXACT) {
+                            // with the mask too, both forms in turn take more registers than there are: 16 planes of 64 x 64 334 us, 295 with the general one
+                            weigh(std::bool_constant<EXACT && !SPARSE>{});
+                            if (EXACT && !SPARSE) {
                                 // whether that held is known only now: the answer need not be waited for before
                                 float m = 0.f, n = 0.f;   // NaN goes the general way
 #pragma unroll
