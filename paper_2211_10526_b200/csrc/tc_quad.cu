@@ -19,10 +19,10 @@
 //
 // What bounds it: the issue slots of the warps that turn cosines into weights and rows into unit rows, on top of the hand-over of a
 // cosine buffer (first contraction, weights, second contraction), of which tensor memory has room for three.  2 x 8 planes of 64 x 64
-// tokens, exact kernel: 119 us; in working copies 97 with cosines written back as they are, 76 with rows left as they are as well: what
+// tokens, exact kernel: 115 us; in working copies, when it took 119, 97 with cosines written back as they are, 76 with rows left as they are as well: what
 // the weights and the rows take comes on top of the chain, which waits for tensor memory and barriers.  So a weight has no square root where the cosines
-// of a step are small (127 us with 5 packed operations a pair, 135.5 with the square roots, whose unit has 16 lanes; 119 with one operation less a
-// pair and rows scaled by a refined reciprocal root, 121.4 with a root and a quotient).  Rows are scaled in fp32 with one rounding, as they are
+// of a tile are small (127 us with 5 packed operations a pair, 135.5 with the square roots, whose unit has 16 lanes; 119 with one operation less a
+// pair and rows scaled by a refined reciprocal root, 121.4 with a root and a quotient; 115 where a tile is looked through before, not step by step after).  Rows are scaled in fp32 with one rounding, as they are
 // everywhere.  K scaled by the weight warps instead (its norms beside it, cosines not before a packed product): 133 against 127, as
 // sixteen warps pay for what four did.  Four K stages, the convolution staged for one slot at a time: 117 against 119, but the masked branch 66 against 62.
 // The two contractions have an issuing warp each: a ready wait costs 50 to 90 cycles and an issue 30 per UMMA, which one warp could not do in time.
@@ -124,8 +124,8 @@ __device__ __forceinline__ float2 angular_weight2(float2 x) {
 }
 // The same where both |x| <= kNearLimit: 1/2 + arcsin(x)/pi with arcsin(x)/x quadratic in x^2 (|error| < 5e-5 rad, 1.2e-5 in the
 // root mean square over cosines of independent rows; the general form 4.5e-5).  No square root and less than half the instructions
-// of the general form, which is left to the few steps that hold a larger cosine: between independent rows of 64 elements 0.6 is
-// 4.8 standard deviations, and one step of 512 cosines in 15 000 has one.
+// of the general form, which is left to tiles that hold a larger cosine: between independent rows of 64 elements 0.6 is
+// 4.8 standard deviations, and one tile in 4 000 has one.
 constexpr float kNearLimit = 0.6f;
 __device__ __forceinline__ float2 angular_weight2_near(float2 x) {
     const float2 u = ffma2(x, x, dup2(0.f));
@@ -133,6 +133,11 @@ __device__ __forceinline__ float2 angular_weight2_near(float2 x) {
     p = ffma2(p, u, dup2(0.31836814f));
     return ffma2(p, x, dup2(0.5f));
 }
+// A warp looks a tile's cosines through, 64 keys of 32 queries, before it takes one form or the other for all of them; once it has met a large
+// one it takes the general form unseen for this many tiles, or to the item's end.  16 planes of 64 x 64, us a call: independent rows 115.1,
+// cosines about 0.95 137.7, about 0.3 139.6, a large one in every 40th key 137.9; with the general form alone, in the kernel before there were two,
+// 135.5.  Both forms in turn in every step of 16 keys with a large cosine instead: 117.7, 181.9, 145.6, 138.8.
+constexpr int kLookAgain = 16;
 // (x + 1) log2(e) + bias of a pair of cosines, clamped to [-1, 1].
 __device__ __forceinline__ float2 exponent2(float2 x, float bias) {
     const float2 y = make_float2(__saturatef(fmaf(x.x, 0.5f, 0.5f)), __saturatef(fmaf(x.y, 0.5f, 0.5f)));
@@ -472,6 +477,8 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
             par ^= 1u << b;
             return done;
         };
+        // with the mask too, both forms take more registers than there are: 16 planes of 64 x 64 334 us, 295 with the general one alone
+        constexpr bool kNear = EXACT && !SPARSE;
         bool ok = true;
         // with the mask, a warp that has given up still meets the others at the next item's denominators, where all leave
         for (int i = 0; i < my_items && (ok || SPARSE); ++i) {
@@ -514,6 +521,7 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                 if (named_barrier_any(2 + slot, kSlotThreads, !ok)) break;
                 ebias = (EXACT ? -kLog2e : 0.f) - __log2f(den_s[0] + den_s[kTile]);
             }
+            [[maybe_unused]] int unseen = 0;   // tiles of the item that take the general form without a look
             for (int jt = 0; jt < T; ++jt) {
                 if (!(ok = wait_cosines())) break;
                 if (live) {
@@ -521,51 +529,78 @@ tc_quad_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
                     const uint32_t cb = col0 + b * kTile;
                     const int left = N - jt * kTile - half * (kTile / 2);
                     float x[2][16];
-                    tmem_ld16(cb, x[0]);
+                    auto tile = [&](auto near_form) {
 #pragma unroll
-                    for (int cc = 0; cc < 4; ++cc) {
-                        tmem_ld_wait();
-                        if (cc < 3) tmem_ld16(cb + (cc + 1) * 16, x[(cc + 1) & 1]);
-                        uint32_t o[8];
-                        if (cc * 16 < left) {
-                            auto weigh = [&](auto near) {
+                        for (int cc = 0; cc < 4; ++cc) {
+                            if (!kNear || cc == 2) tmem_ld_wait();
+                            if (!kNear && cc < 3) tmem_ld16(cb + (cc + 1) * 16, x[(cc + 1) & 1]);
+                            uint32_t o[8];
+                            if (cc * 16 < left) {
+                                auto weigh = [&](auto near) {
 #pragma unroll
-                                for (int e = 0; e < 8; ++e) {
-                                    const float2 xe = make_float2(x[cc & 1][2 * e], x[cc & 1][2 * e + 1]);
-                                    float2 wv;
-                                    if (EXACT) wv = decltype(near)::value ? angular_weight2_near(xe) : angular_weight2(xe);
-                                    if (SPARSE) {
-                                        float2 a;
-                                        if (EXACT) {
-                                            a = exponent2(xe, ebias);
-                                        } else {
-                                            wv = ffma2(xe, dup2(kInvPi), dup2(0.5f));   // 1/2 + x / pi
-                                            a = ffma2(xe, dup2(kLog2e), dup2(ebias));
+                                    for (int e = 0; e < 8; ++e) {
+                                        const float2 xe = make_float2(x[cc & 1][2 * e], x[cc & 1][2 * e + 1]);
+                                        float2 wv;
+                                        if (EXACT) wv = decltype(near)::value ? angular_weight2_near(xe) : angular_weight2(xe);
+                                        if (SPARSE) {
+                                            float2 a;
+                                            if (EXACT) {
+                                                a = exponent2(xe, ebias);
+                                            } else {
+                                                wv = ffma2(xe, dup2(kInvPi), dup2(0.5f));   // 1/2 + x / pi
+                                                a = ffma2(xe, dup2(kLog2e), dup2(ebias));
+                                            }
+                                            const float2 p = make_float2(exp2_approx(a.x), exp2_approx(a.y));
+                                            // masked by a factor of 1 or 0: a pair takes three instructions, a predicate and an addition each four
+                                            wv = ffma2(p, make_float2(one_if_greater(p.x, prm.sparse_eps), one_if_greater(p.y, prm.sparse_eps)), wv);
                                         }
-                                        const float2 p = make_float2(exp2_approx(a.x), exp2_approx(a.y));
-                                        // masked by a factor of 1 or 0: a pair takes three instructions, a predicate and an addition each four
-                                        wv = ffma2(p, make_float2(one_if_greater(p.x, prm.sparse_eps), one_if_greater(p.y, prm.sparse_eps)), wv);
+                                        o[e] = pack_bf16x2(wv.x, wv.y);
                                     }
-                                    o[e] = pack_bf16x2(wv.x, wv.y);
-                                }
-                            };
-                            // with the mask too, both forms in turn take more registers than there are: 16 planes of 64 x 64 334 us, 295 with the general one
-                            weigh(std::bool_constant<EXACT && !SPARSE>{});
-                            if (EXACT && !SPARSE) {
-                                // whether that held is known only now: the answer need not be waited for before
-                                float m = 0.f, n = 0.f;   // NaN goes the general way
+                                };
+                                weigh(near_form);
+                            } else {
 #pragma unroll
-                                for (int e = 0; e < 16; e += 4) {
-                                    m = max3_abs(m, x[cc & 1][e], x[cc & 1][e + 1]);
-                                    n = max3_abs(n, x[cc & 1][e + 2], x[cc & 1][e + 3]);
-                                }
-                                if (!__all_sync(0xffffffffu, max3_abs(m, n, 0.f) <= kNearLimit)) weigh(std::false_type{});
+                                for (int e = 0; e < 8; ++e) o[e] = 0u;   // keys beyond the plane: finite, times v = 0
                             }
-                        } else {
-#pragma unroll
-                            for (int e = 0; e < 8; ++e) o[e] = 0u;   // keys beyond the plane: finite, times v = 0
+                            if (kNear && cc < 2) tmem_ld16(cb + (cc + 2) * 16, x[cc]);
+                            tmem_st8(cb + cc * 8, o);   // over cosines that this thread has already read
                         }
-                        tmem_st8(cb + cc * 8, o);   // over cosines that this thread has already read
+                    };
+                    if constexpr (kNear) {
+                        // the tile's cosines are looked through first; those of the first two steps stay
+                        float m = 0.f, n = 0.f;   // NaN goes the general way
+                        if (unseen == 0) {
+                            tmem_ld16(cb + 32, x[0]);
+                            tmem_ld16(cb + 48, x[1]);
+                            tmem_ld_wait();
+#pragma unroll
+                            for (int e = 0; e < 16; e += 2) {
+                                m = max3_abs(m, x[0][e], x[0][e + 1]);
+                                n = max3_abs(n, x[1][e], x[1][e + 1]);
+                            }
+                        }
+                        tmem_ld16(cb, x[0]);
+                        tmem_ld16(cb + 16, x[1]);
+                        tmem_ld_wait();
+                        bool near = false;
+                        if (unseen == 0) {
+#pragma unroll
+                            for (int e = 0; e < 16; e += 2) {
+                                m = max3_abs(m, x[0][e], x[0][e + 1]);
+                                n = max3_abs(n, x[1][e], x[1][e + 1]);
+                            }
+                            near = __all_sync(0xffffffffu, max3_abs(m, n, 0.f) <= kNearLimit);
+                            if (!near) unseen = kLookAgain;
+                        }
+                        if (near) {
+                            tile(std::true_type{});
+                        } else {
+                            --unseen;
+                            tile(std::false_type{});
+                        }
+                    } else {
+                        tmem_ld16(cb, x[0]);
+                        tile(std::false_type{});
                     }
                     tmem_st_wait();
                     tcgen05_fence_before_sync();
