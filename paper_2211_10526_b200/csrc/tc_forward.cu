@@ -1,6 +1,7 @@
 // Orchestration of the tensor-core path: state build -> split reduction -> apply, in stream order
 // (the stream is the only synchronisation between the phases; no kernel waits on another).
 #include "tc_host.cuh"
+#include "state_splits.cuh"
 
 #include <cstdlib>
 
@@ -45,33 +46,14 @@ bool preferred(const Problem& p) {
     return supports(p) && p.N >= 48 && (p.d == 64 || token_pairs(p) || head_pairs(p) || (long long)p.BH * p.N >= kNarrowMinTokens);
 }
 
-// Two state CTAs fit on an SM: as many splits as keep all CTAs of the launch resident at once
-// (two per multiprocessor), every split non-empty, at most 64 splits.
-int choose_splits(int BH, int N) {
-    const int tiles = (N + kStateTile - 1) / kStateTile;
-    if (tiles < 1) return 1;
-    int P = (2 * device_sm_count()) / BH;
-    if (P > tiles) P = tiles;
-    if (P > 64) P = 64;
-    if (P < 1) P = 1;
-    const int per = (tiles + P - 1) / P;
-    return (tiles + per - 1) / per;
-}
+int choose_splits(int BH, int N) { return most_splits(BH, (N + kStateTile - 1) / kStateTile, device_sm_count()); }
 
-// The state kernel's own number: at most the above, which the workspace is sized for.  Eight splits that meet in a cluster are faster than
-// more of them that meet in memory as long as none has many tiles.  More splits through memory / eight in a cluster, us per forward
-// from a graph, 16 planes, width 64: 48 x 48 17.4 / 13.7, 64 x 64 20.0 / 17.5, 90 x 90 27.9 / 26.2, 128 x 128 43.4 / 41.9; one plane of 64 x 64 12.4 / 10.0.
-int launch_splits(int BH, int N) {
-    const int tiles = (N + kStateTile - 1) / kStateTile;
-    int P = choose_splits(BH, N);
-    if (P > 8 && 8 * BH <= device_sm_count() && tiles <= 8 * 16) P = 8;
-    const int per = (tiles + P - 1) / P;
-    return tiles < 1 ? 1 : (tiles + per - 1) / per;
+// The state kernel on rows of 128 bytes per plane, split as the device holds the clusters.
+static cudaError_t launch_split_state(const Problem& p, int rows, float* partial, float* state, unsigned* counters, unsigned* status, cudaStream_t stream) {
+    const int tiles = (rows + kStateTile - 1) / kStateTile;
+    const StateSplits s = state_splits(p.BH, tiles, device_sm_count(), p.d == 32, [](int P) { return state_clusters_at_once(P); });
+    return launch_state(p, partial, state, counters, s.P, (tiles + s.P - 1) / s.P, s.clustered, status, stream);
 }
-
-// Clusters of eight want multiprocessors of their own: 37 planes of 64 x 64, two CTAs each, 33.3 us (29.6 through memory); 16 planes of
-// 32 x 32, one each, 10.4 (13.8).  Up to four fit anywhere: 100 planes of 40 x 40 (two) 30.9 (31.5), 48 of 64 x 64 (four) 35.8 (37.2).
-bool splits_in_cluster(int BH, int P) { return P > 1 && (P <= 4 || (P <= 8 && BH * P <= device_sm_count())); }
 
 // CASTLING_TC_ONE_KERNEL=1 in the environment selects the one-kernel forward (state and apply pipelines side
 // by side in every CTA) instead of the separate state and apply kernels, which measure faster (read once).
@@ -130,9 +112,7 @@ cudaError_t forward(const Problem& p_in, float* ws_state, float* ws_partial, uns
         p = p_in;   // width-32 heads in 64-byte rows of their own
         p.narrow = p.d == 32;
         p.fine = fine;
-        const int rows = rows_per_head(p.N, p.d), P = launch_splits(p.BH, rows);
-        const int tiles = (rows + kStateTile - 1) / kStateTile;
-        e = launch_state(p, ws_partial, ws_state, counters, P, (tiles + P - 1) / P, status, stream);
+        e = launch_split_state(p, rows_per_head(p.N, p.d), ws_partial, ws_state, counters, status, stream);
         if (e != cudaSuccess) return e;
         ++*launches;
         timer->mark(stream, "tc_state");
@@ -157,9 +137,7 @@ bool shard_supports(const Problem& p) {
 cudaError_t shard_state(const Problem& p, float* state_out, float* ws_partial, unsigned* counters, unsigned* status,
                         cudaStream_t stream, int* launches, KernelTimer* timer) {
     *launches = 0;
-    const int P = launch_splits(p.BH, p.N);
-    const int tiles = (p.N + kStateTile - 1) / kStateTile;
-    const cudaError_t e = launch_state(p, ws_partial, state_out, counters, P, (tiles + P - 1) / P, status, stream);
+    const cudaError_t e = launch_split_state(p, p.N, ws_partial, state_out, counters, status, stream);
     if (e != cudaSuccess) return e;
     ++*launches;
     timer->mark(stream, "tc_state");

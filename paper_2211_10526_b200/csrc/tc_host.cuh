@@ -37,10 +37,8 @@ constexpr int kStateWords = 64 * 64 + 64;
 constexpr int kStateWordsRownorm = kStateWords + 64;
 inline int state_words_of(const Problem& p) { return p.rownorm ? kStateWordsRownorm : kStateWords; }
 
-// Token splits of the tensor-core state kernel and the workspace words it needs beyond the state.
+// Token splits of the tensor-core state kernel, at most (csrc/state_splits.cuh).
 int choose_splits(int BH, int N);
-// The splits of a plane are one cluster, whose CTAs add their states through distributed shared memory.
-bool splits_in_cluster(int BH, int P);
 
 // Enqueue state build, split reduction and apply for one problem.  `status` is the device status
 // word; `counters` holds kCountersPerHead zero-initialised arrival counters per (b,h), left at zero by every call.  Returns the cudaError_t of the launches; cudaErrorNotSupported if a tensor map could not
@@ -70,8 +68,11 @@ inline cudaError_t launch_programmatic(Kernel kernel, bool early, dim3 grid, dim
 }
 
 // Launchers of the individual kernels (each in its own file).
+// The state kernel; clustered: the P splits of a plane are one cluster.
 cudaError_t launch_state(const Problem& p, float* partial, float* final_state, unsigned* counters, int P,
-                         int tiles_per_cta, unsigned* status, cudaStream_t st);
+                         int tiles_per_cta, bool clustered, unsigned* status, cudaStream_t st);
+// Clusters of P state CTAs, P up to 8, that the current device holds at once; 0 if it does not say.
+int state_clusters_at_once(int P);
 cudaError_t launch_apply(const Problem& p, const float* state, unsigned* status, cudaStream_t st);
 // The apply kernel for width-32 heads in 64-byte rows (csrc/tc_apply32.cu).
 cudaError_t launch_apply32(const Problem& p, const float* state, unsigned* status, cudaStream_t st);

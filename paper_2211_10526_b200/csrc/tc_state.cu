@@ -385,8 +385,32 @@ tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
 
 }  // namespace
 
+// What a state CTA takes of a multiprocessor but for tensor memory: asked about a kernel that allocates some, the runtime counts one CTA per
+// multiprocessor, and two of the state kernel's run on each.  Never launched.
+static __global__ void __launch_bounds__(kThreads, 2) footprint_kernel() {}
+
+int state_clusters_at_once(int P) {
+    static std::atomic<int> known[kMaxDevices][9];   // the number and one more
+    static PerDevice opt_in;
+    int dev = 0, n = 0;
+    if (P < 1 || P > 8 || cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) { (void)cudaGetLastError(); return 0; }
+    if ((n = known[dev][P].load(std::memory_order_relaxed)) > 0) return n - 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)P); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = kSmemBytes;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)P; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    if (opt_in_smem(footprint_kernel, kSmemBytes, opt_in) != cudaSuccess || cudaOccupancyMaxActiveClusters(&n, footprint_kernel, &cfg) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return 0;
+    }
+    known[dev][P].store(n + 1, std::memory_order_relaxed);
+    return n;
+}
+
 cudaError_t launch_state(const Problem& p, float* partial, float* final_state, unsigned* counters, int P,
-                         int tiles_per_cta, unsigned* status, cudaStream_t st) {
+                         int tiles_per_cta, bool clustered, unsigned* status, cudaStream_t st) {
     const bool narrow = p.d == 32;
     CUtensorMap tmK, tmV;
     // [row, tokens, planes per batch step, batch steps]
@@ -410,7 +434,6 @@ cudaError_t launch_state(const Problem& p, float* partial, float* final_state, u
     }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = kSmemBytes; cfg.stream = st;
-    const int clustered = splits_in_cluster(p.BH, P) ? 1 : 0;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -420,7 +443,7 @@ cudaError_t launch_state(const Problem& p, float* partial, float* final_state, u
     auto launch = [&](auto kernel) {
         const cudaError_t e = opt_in_smem(kernel, kSmemBytes, opt_in[(p.fine ? 4 : narrow ? 2 : 0) + (p.rownorm ? 1 : 0)]);
         if (e != cudaSuccess) return e;
-        return cudaLaunchKernelEx(&cfg, kernel, tmK, tmV, dst, final_state, counters, p.N, tiles_per_cta, P, clustered, p.BH, p.hdiv, items,
+        return cudaLaunchKernelEx(&cfg, kernel, tmK, tmV, dst, final_state, counters, p.N, tiles_per_cta, P, clustered ? 1 : 0, p.BH, p.hdiv, items,
                                   p.eps2, status);
     };
     if (p.fine) return p.rownorm ? launch(tc_state_kernel<true, true, true>) : launch(tc_state_kernel<true, false, true>);
