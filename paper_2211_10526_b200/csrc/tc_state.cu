@@ -71,17 +71,8 @@ tc_state_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
     const int bh0 = (P > 1) ? blockIdx.x / P : blockIdx.x * items_per_cta;
     const int n_items = (P > 1) ? 1 : min(items_per_cta, BH - bh0);
     const int t_begin = p * tiles_per_cta;
-    const int n_tiles = min(total_tiles, t_begin + tiles_per_cta) - t_begin;  // per item
+    const int n_tiles = min(total_tiles, t_begin + tiles_per_cta) - t_begin;  // per item, at least one
     const int bh = bh0;  // the (b,h) of the split reduction below (P > 1: the only item)
-    if (n_tiles <= 0 || n_items <= 0) {  // the host never makes such a CTA; keep the partial well defined anyway
-        pdl_wait_primary();
-        if (P > 1) {
-            float* out = dst + ((size_t)bh * P + p) * kStateW;
-            for (int i = tid; i < kStateW; i += kThreads) out[i] = 0.f;
-        }
-        return;
-    }
-
     if (tid == 0) {
         for (int s = 0; s < kStages; ++s) {
             mbar_init(&full[s], 1);
@@ -412,6 +403,8 @@ int state_clusters_at_once(int P) {
 cudaError_t launch_state(const Problem& p, float* partial, float* final_state, unsigned* counters, int P,
                          int tiles_per_cta, bool clustered, unsigned* status, cudaStream_t st) {
     const bool narrow = p.d == 32;
+    const int stage = narrow ? 2 * kTile : kTile;   // tokens
+    if (P > 1 && (P - 1) * tiles_per_cta >= (p.N + stage - 1) / stage) return cudaErrorInvalidValue;   // a split without tokens: the kernel takes none
     CUtensorMap tmK, tmV;
     // [row, tokens, planes per batch step, batch steps]
     const uint64_t nb = (uint64_t)(p.BH / p.hdiv);
