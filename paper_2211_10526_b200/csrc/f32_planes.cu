@@ -2,7 +2,7 @@
 //     out_t = (1/pi) q^_t (K^^T V) + 1/2 sum_n v_n + bias + DWConv(V)_t                    (Eq. 9)
 // A cluster of 1, 2 or 4 CTAs per plane, each with a band of its grid rows (the first one with the leading off-grid tokens too) in
 // shared memory: K and Q as tokens, V as the band with its halo (zero outside the grid), all by TMA.  One kernel does the following for its
-// plane; where planes are few, one kernel stops after 2 and the other does 3, with bands and runs of its own.
+// plane; where planes are few or of a column or two, one kernel stops after 2 and the other does 3, with bands and runs of its own.
 //   1. rows of K to unit rows in place, the token sum of V, 1 / max(||q||, eps)
 //   2. the band's state: a thread owns 8 x 8 of S and every G-th token (G groups of (D/8)^2 threads); the groups meet in shared memory,
 //      the bands through distributed shared memory, both in a fixed order
@@ -384,16 +384,28 @@ cudaError_t launch_plane(const Problem& p, float* state, cudaStream_t st) {
     return cudaLaunchKernelEx(&cfg, f32_plane_kernel<D, KS, PART>, tmK, tmQ, tmV, tmLead, prm);
 }
 
+// A few planes: the second kernel's copies and convolution run beside the first one, on other multiprocessors.  14 x 14, two kernels / one, us
+// from a graph: width 32, 8 planes 6.7 / 7.7, 16 planes 6.9 / 7.8, 32 planes 9.9 / 7.9; width 64, 8 planes 10.0 / 11.1, 24 planes 13.5 / 11.3.
+// A run of the one kernel is eight tokens of a row, one of the two kernels' two, so these also take grids of one column (two at width 64, up to 64
+// planes): 20 planes of 64 x 1, width 64, two kernels / one 9.2 / 20.5, 148 of 128 x 1, width 32, 12.1 / 16.1.
+bool one_kernel(const Problem& p) {
+    const bool thin = p.gridW == 1 ? p.BH <= device_sm_count() : p.gridW == 2 && p.d == 64 && p.BH < 64;
+    return p.BH >= 20 && !thin;
+}
+
 template <int D, int KS> bool fits(const Problem& p) {
     F32PlaneParams prm;
-    return plane_layout<D, KS>(p, kWhole, &prm) <= kSmemLimit && plane_layout<D, KS>(p, kRows, &prm) <= kSmemLimit;
+    for (int part : {kWhole, kRows}) {
+        if (plane_layout<D, KS>(p, part, &prm) > kSmemLimit) return false;
+    }
+    // A band is one grid row at least: where that is more than three rounds of runs, the patches of the other kernels are faster.
+    // From a graph, they / this one, us: width 32, 8 planes of 1 x 128 8.8 / 8.2, 1 x 200 10.4 / 11.2, 1 x 250 10.4 / 12.5; width 64, 1 x 128 13.9 / 17.5.
+    return one_kernel(p) || prm.band_rows * ((p.gridW + 1) / 2) <= 3 * PlaneGeo<D, KS>::kRuns;
 }
 
 template <int D, int KS>
 cudaError_t launch(const Problem& p, float* state, cudaStream_t st, int* launches, KernelTimer* timer) {
-    // A few planes: the second kernel's copies and convolution run beside the first one, on other multiprocessors.  14 x 14, two kernels / one, us
-    // from a graph: width 32, 8 planes 6.7 / 7.7, 16 planes 6.9 / 7.8, 32 planes 9.9 / 7.9; width 64, 8 planes 10.0 / 11.1, 24 planes 13.5 / 11.3.
-    const bool whole = p.BH >= 20;
+    const bool whole = one_kernel(p);
     cudaError_t e = whole ? launch_plane<D, KS, kWhole>(p, state, st) : launch_plane<D, KS, kState>(p, state, st);
     if (e != cudaSuccess) return e;
     *launches = 1;
@@ -415,6 +427,13 @@ bool f32_plane_supports(const Problem& p) {
     // width 64.  768 planes, the kernels there were / this one, us: width 32, 5 x 5 17.1 / 21.5, 7 x 7 (3072 planes) 80.7 / 79.6, 11 x 11 54.7 / 35.5,
     // 16 x 16 64.7 / 65.9; width 64, 6 x 6 44.9 / 45.2, 8 x 8 69.6 / 53.5, 10 x 10 133 / 89, 11 x 11 89 / 95, 14 x 14 112 / 129.
     if (p.BH > device_sm_count() && (p.N < 49 || (p.d == 64 && p.N > 100))) return false;
+    // From 64 planes on the CUDA cores have one kernel too.  It is faster for the smallest planes of width 32 (96 of 1 x 16 5.4 / 6.2, 4 x 4 5.5 / 6.3)
+    // and for many planes of one column (1536 of 64 x 1 50.9 / 79.4, width 64 116 / 226) or two (1536 of 25 x 2 45.5 / 52.8, 40 x 2 65.8 / 69.6, but 50 x 2
+    // 78.4 / 80.7, 64 x 2 101 / 88, 149 of 120 x 2 28.8 / 33.3; width 64, 400 of 30 x 2 32.7 / 39.4, 40 x 2 72 / 51).
+    if (p.BH >= 64 && p.d == 32 && p.N <= 16) return false;
+    if (p.gridW == 1 && p.BH > device_sm_count()) return false;
+    if (p.gridW == 2 && p.BH > (p.d == 32 ? 2 : 1) * device_sm_count() && p.N <= (p.d == 32 ? 80 : 64)) return false;
+    if (p.gridW == 2 && p.BH > device_sm_count() && p.d == 32 && p.N >= 240) return false;
     if (p.d == 32) return p.ksize == 3 ? fits<32, 3>(p) : fits<32, 5>(p);
     return p.ksize == 3 ? fits<64, 3>(p) : fits<64, 5>(p);
 }
