@@ -396,7 +396,7 @@ bool one_kernel(const Problem& p) {
 template <int D, int KS> bool fits(const Problem& p) {
     F32PlaneParams prm;
     for (int part : {kWhole, kRows}) {
-        if (plane_layout<D, KS>(p, part, &prm) > kSmemLimit) return false;
+        if (plane_layout<D, KS>(p, part, &prm) > kSmemLimit || prm.band_rows + KS - 1 > 256) return false;   // 256: boxes of TMA copies
     }
     // A band is one grid row at least: where that is more than three rounds of runs, the patches of the other kernels are faster.
     // From a graph, they / this one, us: width 32, 8 planes of 1 x 128 8.8 / 8.2, 1 x 200 10.4 / 11.2, 1 x 250 10.4 / 12.5; width 64, 1 x 128 13.9 / 17.5.

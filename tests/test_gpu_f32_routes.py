@@ -16,7 +16,7 @@ pytestmark = pytest.mark.gpu
 TWO, ONE, CORES = ["f32_state", "f32_apply"], ["f32_plane"], ["simt_fused"]
 #        B, H, gridH, gridW, d, ksize, layout, prefix, kernels (None: not told apart by their names)
 CASES = [(5, 4, 64, 1, 64, 3, "heads", 0, TWO), (5, 4, 64, 1, 32, 5, "tokens", 1, TWO), (37, 4, 128, 1, 32, 3, "heads", 0, TWO), (12, 4, 251, 1, 32, 3, "fused", 2, TWO),
-         (50, 3, 64, 1, 32, 3, "heads", 0, CORES), (50, 3, 64, 1, 64, 3, "heads", 0, CORES), (90, 1, 254, 1, 32, 3, "heads", 1, TWO), (100, 1, 254, 1, 32, 3, "heads", 1, None),
+         (50, 3, 64, 1, 32, 3, "heads", 0, CORES), (50, 3, 64, 1, 64, 3, "heads", 0, CORES), (90, 1, 254, 1, 32, 3, "heads", 1, TWO), (100, 1, 254, 1, 32, 3, "heads", 1, None), (100, 1, 256, 1, 32, 3, "heads", 0, None),
          (5, 4, 30, 2, 64, 3, "heads", 0, TWO), (16, 4, 30, 2, 64, 5, "tokens", 0, ONE), (100, 4, 25, 2, 32, 3, "heads", 0, CORES), (75, 4, 60, 2, 32, 3, "heads", 1, ONE),
          (75, 4, 25, 2, 64, 3, "heads", 0, CORES), (32, 3, 4, 4, 32, 3, "heads", 0, CORES), (32, 3, 3, 6, 32, 3, "heads", 0, ONE), (2, 4, 1, 250, 32, 3, "heads", 0, None),
          (2, 4, 1, 128, 64, 3, "tokens", 0, None), (2, 4, 2, 128, 64, 3, "heads", 0, None), (2, 4, 1, 192, 32, 5, "heads", 0, None), (2, 4, 1, 193, 32, 5, "heads", 0, None)]
