@@ -97,7 +97,8 @@ typedef struct {
                           /* weights: Mask_eps(Softmax_j(q^_t . k^_j)), Mask_eps(p) = p if p > eps else */
                           /* 0; softmax over the keys of a query on the cosines of the unit rows, no    */
                           /* 1/sqrt(d), survivors not renormalised.  Quadratic in N.  The comparison    */
-                          /* p > eps is taken in fp32.                                                 */
+                          /* p > eps is taken in fp32.  A row of q with a NaN or an infinity makes its  */
+                          /* own output row NaN, such a row of k every output row of its (b,h).         */
     double sparse_eps;    /* the mask's threshold (the paper uses 0.02 for classification)             */
 } castling_attn_config_t;
 
