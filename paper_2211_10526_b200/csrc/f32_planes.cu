@@ -387,9 +387,10 @@ cudaError_t launch_plane(const Problem& p, float* state, cudaStream_t st) {
 // A few planes: the second kernel's copies and convolution run beside the first one, on other multiprocessors.  14 x 14, two kernels / one, us
 // from a graph: width 32, 8 planes 6.7 / 7.7, 16 planes 6.9 / 7.8, 32 planes 9.9 / 7.9; width 64, 8 planes 10.0 / 11.1, 24 planes 13.5 / 11.3.
 // A run of the one kernel is eight tokens of a row, one of the two kernels' two, so these also take grids of one column (two at width 64, up to 64
-// planes): 20 planes of 64 x 1, width 64, two kernels / one 9.2 / 20.5, 148 of 128 x 1, width 32, 12.1 / 16.1.
+// planes): 20 planes of 64 x 1, width 64, two kernels / one 9.2 / 20.5, 148 of 128 x 1, width 32, 12.1 / 16.1.  Not where many have few tokens:
+// 96 of 4 x 1, width 64, 7.5 / 6.3, 148 of 16 x 1, 5x5 filters, 12.8 / 10.3.
 bool one_kernel(const Problem& p) {
-    const bool thin = p.gridW == 1 ? p.BH <= device_sm_count() : p.gridW == 2 && p.d == 64 && p.BH < 64;
+    const bool thin = p.N <= 16 && p.BH >= 64 ? false : p.gridW == 1 ? p.BH <= device_sm_count() : p.gridW == 2 && p.d == 64 && p.BH < 64;
     return p.BH >= 20 && !thin;
 }
 
