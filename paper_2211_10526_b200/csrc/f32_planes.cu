@@ -426,7 +426,7 @@ bool f32_plane_supports(const Problem& p) {
     if (p.N > 256 || p.gridW + p.ksize - 1 > 256) return false;   // boxes of TMA copies
     // With more planes than multiprocessors their number over those in flight decides, two per multiprocessor at width 32 and mostly one at
     // width 64.  768 planes, the kernels there were / this one, us: width 32, 5 x 5 17.1 / 21.5, 7 x 7 (3072 planes) 80.7 / 79.6, 11 x 11 54.7 / 35.5,
-    // 16 x 16 64.7 / 65.9; width 64, 6 x 6 44.9 / 45.2, 8 x 8 69.6 / 53.5, 10 x 10 133 / 89, 11 x 11 89 / 95, 14 x 14 112 / 129.
+    // 16 x 16 65.9 / 63.3; width 64, 6 x 6 44.9 / 45.2, 8 x 8 69.6 / 53.5, 10 x 10 133 / 89, 11 x 11 89 / 95, 14 x 14 112 / 129.
     if (p.BH > device_sm_count() && (p.N < 49 || (p.d == 64 && p.N > 100))) return false;
     // From 64 planes on the CUDA cores have one kernel too.  It is faster for the smallest planes of width 32 (96 of 1 x 16 5.4 / 6.2, 4 x 4 5.5 / 6.3)
     // and for many planes of one column (1536 of 64 x 1 50.9 / 79.4, width 64 116 / 226) or two (1536 of 25 x 2 45.5 / 52.8, 40 x 2 65.8 / 69.6, but 50 x 2

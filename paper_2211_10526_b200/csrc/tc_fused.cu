@@ -29,9 +29,9 @@
 // a call is the number of planes over those in flight.  Two shapes of CTA: 256 workers for planes of any size, two per SM;
 // 128 workers for planes of at most 128 lines, three or four per SM, which finish a plane later but more of them at a time:
 // taken when that saves a round of planes.
-// Measured (from a graph): 768 planes of 14 x 14 and a class token 28.1 us, 31.2 with every word of V masked, accumulators scaled one by one in the
-// convolution, branches around its loads and stores and each tap's sum waiting for the last (12 300 cycles a plane); 12 planes 7.4 / 8.1; 256 planes
-// of width 32 7.9 / 9.0; 512 planes of 7 x 7, width 32, 14.1 us a call with two tokens a line and large CTAs.
+// Measured (from a graph, early launch included): 768 planes of 14 x 14 and a class token 28.7 us, 31.3 with every word of V masked, accumulators scaled one by one in the
+// convolution, branches around its loads and stores and each tap's sum waiting for the last (12 300 cycles a plane); 12 planes 6.7 / 8.0; 256 planes
+// of width 32 7.2 / 8.7; 512 planes of 7 x 7, width 32, 14.1 us a call with two tokens a line and large CTAs.
 #include "tc_common.cuh"
 #include "tc_host.cuh"
 
