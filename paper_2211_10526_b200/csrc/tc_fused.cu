@@ -71,6 +71,7 @@ struct FusedParams {
     __nv_bfloat16* out;         // token n of plane i at plane_offset(lo, i, hdiv) + n * lo.token
     Layout lo;
     int H, head0, BH, hdiv, prefix, N, gridH, gridW;  // N = prefix + gridH * gridW
+    bool turned;                // filters with rows and columns exchanged
     float eps2;
     unsigned* status;
 };
@@ -384,7 +385,8 @@ tc_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
 #pragma unroll
             for (int i = 0; i < kShare; ++i) {
                 const int e = wt + i * WORKERS;
-                if (e < kElems) w_s[(e % (KS * KS)) * kW + e / (KS * KS)] = __uint_as_float((uint32_t)fraw[i] << 16);
+                const int tap = e % (KS * KS);
+                if (e < kElems) w_s[(prm.turned ? tap % KS * KS + tap / KS : tap) * kW + e / (KS * KS)] = __uint_as_float((uint32_t)fraw[i] << 16);
             }
             if (wt < kW) w_s[kElems + wt] = __uint_as_float((uint32_t)braw << 16);
 
@@ -538,7 +540,7 @@ tc_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
 }
 
 template <int KS, bool NARROW, int WORKERS, bool FINE, bool ROOMY>
-cudaError_t launch_fused_room(const Problem& p, unsigned* status, cudaStream_t st) {
+cudaError_t launch_fused_room(const Problem& p, bool turned, unsigned* status, cudaStream_t st) {
     using G = Geo<KS, NARROW, WORKERS, ROOMY>;
     CUtensorMap tmK, tmV, tmQ, tmVplain;
     // [d, tokens, planes per batch step, batch steps]
@@ -568,7 +570,7 @@ cudaError_t launch_fused_room(const Problem& p, unsigned* status, cudaStream_t s
     prm.out = static_cast<__nv_bfloat16*>(p.out);
     prm.lo = p.lo;
     prm.H = p.H; prm.head0 = p.head0; prm.BH = p.BH; prm.hdiv = p.hdiv; prm.prefix = p.prefix; prm.N = p.N;
-    prm.gridH = p.gridH; prm.gridW = p.gridW;
+    prm.gridH = p.gridH; prm.gridW = p.gridW; prm.turned = turned;
     prm.eps2 = p.eps2; prm.status = status;
     static PerDevice opt_in[2];  // per instantiation
     const bool packed = (p.lo.token == G::kW);
@@ -578,12 +580,15 @@ cudaError_t launch_fused_room(const Problem& p, unsigned* status, cudaStream_t s
     const int resident = G::kCtas * device_sm_count();
     const int grid = p.BH < resident ? p.BH : resident;
     // CTAs that start while the kernel before drains lie on the multiprocessors in the order in which these became free, not one by one in
-    // turn, so that some get more of the CTAs with a plane more than others.  Width 64 gains all the same; width 32, whose planes take
-    // the issue slots of a whole multiprocessor, where no CTA has a second plane.  From a graph, started early / not: 12 planes of 14 x 14,
-    // width 64, 6.4 / 7.4 us, 768 of 11 x 11 19.8 / 20.2, 768 of 14 x 14 28.5 / 28.1 (with a new output per call 29.4 / 30.7), 768 of
-    // 16 x 16 34.3 / 33.6; width 32, 256 of 14 x 14 6.8 / 7.9, 1024 of 16 x 16 24.1 / 22.8, 1024 of 16 x 32 44.0 / 40.0.  Planes handed out
-    // by a counter instead: 7.2 against 6.9 and 30.2 against 29.4 for the first and the third.
-    const bool early = !NARROW || grid == p.BH;
+    // turn, so that some get more of the CTAs with a plane more than others.  Width 32, whose planes take the issue slots of a whole multiprocessor, gains
+    // only where no CTA has a second plane; width 64 unless the last round has few enough planes for each multiprocessor to keep a CTA without one,
+    // and not just a few.  Us a call with a new output, started early / not (width 64): 330 planes of 14 x 14 15.5 / 16.6, 444 19.1 / 18.6, 700 29.0 / 26.8, 768
+    // 29.6 / 31.0, 1000 37.6 / 35.2, 1536 49.2 / 51.5, 444 of 16 x 16 24.0 / 22.0 (22.7 before there were early starts), 700 35.6 / 31.3 (32.0), 1184 of
+    // 11 x 11, three to a multiprocessor, 31.1 / 29.1 (30.9); width 32 from a graph, 256 of 14 x 14 6.8 / 7.9, 1024 of 16 x 16 24.1 / 22.8, 1024 of
+    // 16 x 32 44.0 / 40.0.  Planes handed out by a counter instead: 12 planes 7.2 against 6.9, 768 30.2 against 29.4.
+    const int last = p.BH % grid;   // planes of the last round, 0 if it is full
+    const bool uneven = 4 * last > grid && last <= grid * (G::kCtas - 1) / G::kCtas + grid / 20;
+    const bool early = grid == p.BH || (!NARROW && !uneven);
     auto launch = [&](auto kernel) {
         return launch_programmatic(kernel, early, dim3((unsigned)grid), dim3(G::kThreads), G::kSmem, st, tmK, tmV, tmQ, tmVplain, prm);
     };
@@ -591,11 +596,18 @@ cudaError_t launch_fused_room(const Problem& p, unsigned* status, cudaStream_t s
 }
 
 template <int KS, bool NARROW, int WORKERS, bool FINE>
-cudaError_t launch_fused_ks(const Problem& p, unsigned* status, cudaStream_t st) {
+cudaError_t launch_fused_ks(const Problem& p_in, unsigned* status, cudaStream_t st) {
+    // A grid of one row is taken as one of one column, its filters turned to match: the strips of the convolution slide down columns.  From a graph, row /
+    // column, us: 64 planes of 1 x 200 15.3 / 11.4, 1536 of 1 x 100 55.6 / 38.9, 768 with 5x5 filters 60.8 / 35.2.  Width 32, whose strips are twice as
+    // wide, gains nothing: 768 of 1 x 100 19.2, of 100 x 1 23.5.
+    Problem p = p_in;
+    const bool turned = !NARROW && p.gridH == 1 && p.gridW > 1;
+    if (turned) { p.gridH = p.gridW; p.gridW = 1; }
     using G = Geo<KS, NARROW, WORKERS, true>;
     const bool roomy = (p.gridW + KS - 1) * (p.gridH + KS - 1) * G::kRow <= G::kBuf && p.gridW + KS - 1 <= 256 && p.gridH + KS - 1 <= 256 &&
                        p.N * G::kAccRow <= 2 * G::kBuf;
-    return roomy ? launch_fused_room<KS, NARROW, WORKERS, FINE, true>(p, status, st) : launch_fused_room<KS, NARROW, WORKERS, FINE, false>(p, status, st);
+    return roomy ? launch_fused_room<KS, NARROW, WORKERS, FINE, true>(p, turned, status, st)
+                 : launch_fused_room<KS, NARROW, WORKERS, FINE, false>(p, turned, status, st);
 }
 
 template <int KS, bool NARROW, bool FINE>

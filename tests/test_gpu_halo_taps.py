@@ -13,9 +13,11 @@ import torch
 import oracle
 import workloads
 from test_gpu_narrow_rows import views
-from test_gpu_plane_halo import CASES
+from test_gpu_plane_halo import CASES as HALO_CASES
 
 pytestmark = pytest.mark.gpu
+
+CASES = HALO_CASES + [(2, 3, 1, 100, 64, 5, "fused", 2), (2, 3, 1, 256, 64, 3, "heads", 0), (160, 2, 1, 60, 64, 5, "tokens", 0)]   # rows taken as columns
 
 
 def inputs(case):
