@@ -587,8 +587,11 @@ cudaError_t launch_fused_room(const Problem& p, bool turned, unsigned* status, c
     // 11 x 11, three to a multiprocessor, 31.1 / 29.1 (30.9); width 32 from a graph, 256 of 14 x 14 6.8 / 7.9, 1024 of 16 x 16 24.1 / 22.8, 1024 of
     // 16 x 32 44.0 / 40.0.  Planes handed out by a counter instead: 12 planes 7.2 against 6.9, 768 30.2 against 29.4.
     const int last = p.BH % grid;   // planes of the last round, 0 if it is full
-    const bool uneven = 4 * last > grid && last <= grid * (G::kCtas - 1) / G::kCtas + grid / 20;
-    const bool early = grid == p.BH || (!NARROW && !uneven);
+    const bool uneven = 4 * last >= grid && last <= grid * (G::kCtas - 1) / G::kCtas + grid / 20;
+    // In one round, CTAs that start while between a third and all of the multiprocessors are busy share some of them with one another, which only planes
+    // with their halo, whose work is short, gain from (us a call, early / not): 110 planes of 16 x 16 11.4 / 10.5, 48 8.6 / 10.5, 148 9.0 / 11.3; of 14 x 14 9.8 / 10.4.
+    const bool crowded = !ROOMY && !NARROW && 3 * p.BH > device_sm_count() && p.BH < device_sm_count();
+    const bool early = grid == p.BH ? !crowded : !NARROW && !uneven;
     auto launch = [&](auto kernel) {
         return launch_programmatic(kernel, early, dim3((unsigned)grid), dim3(G::kThreads), G::kSmem, st, tmK, tmV, tmQ, tmVplain, prm);
     };
