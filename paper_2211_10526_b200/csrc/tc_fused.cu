@@ -385,8 +385,7 @@ tc_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
 #pragma unroll
             for (int i = 0; i < kShare; ++i) {
                 const int e = wt + i * WORKERS;
-                const int tap = e % (KS * KS);
-                if (e < kElems) w_s[(prm.turned ? tap % KS * KS + tap / KS : tap) * kW + e / (KS * KS)] = __uint_as_float((uint32_t)fraw[i] << 16);
+                if (e < kElems) w_s[(e % (KS * KS)) * kW + e / (KS * KS)] = __uint_as_float((uint32_t)fraw[i] << 16);
             }
             if (wt < kW) w_s[kElems + wt] = __uint_as_float((uint32_t)braw << 16);
 
@@ -436,11 +435,13 @@ tc_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__
             const float2 hs2 = make_float2(half * sum_s[2 * cp], half * sum_s[2 * cp + 1]);   // 1/2 s
             const float2 bias2 = *reinterpret_cast<const float2*>(w_s + kElems + 2 * cp);
             const float2 c2 = make_float2(hs2.x + bias2.x, hs2.y + bias2.y);  // + bias: grid tokens
+            const bool turned = !NARROW && prm.turned;
+            const int down = turned ? kW : KS * kW, right = turned ? KS * kW : kW;   // from tap to tap
             float2 wreg[KS][KS];
 #pragma unroll
             for (int dy = 0; dy < KS; ++dy)
 #pragma unroll
-                for (int dx = 0; dx < KS; ++dx) wreg[dy][dx] = *reinterpret_cast<const float2*>(w_s + (dy * KS + dx) * kW + 2 * cp);
+                for (int dx = 0; dx < KS; ++dx) wreg[dy][dx] = *reinterpret_cast<const float2*>(w_s + dy * down + dx * right + 2 * cp);
             uint32_t* out_plane = reinterpret_cast<uint32_t*>(out_bh) + cp;
             const long long out_tok = OUT_PACKED ? kW / 2 : prm.lo.token / 2;  // 32-bit words per token
             const uint32_t acc_s = smem_u32(V_s) + (ROOMY ? cp * 8 : 0);
